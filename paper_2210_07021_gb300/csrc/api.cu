@@ -20,6 +20,7 @@ namespace sfmm {
 cudaError_t build_tree(sfmm_plan_s* P, const uint64_t* keys, int64_t n, int m, int max_depth);
 cudaError_t tree_geometry(sfmm_plan_s* P);
 cudaError_t tree_target_ranges(sfmm_plan_s* P, const uint64_t* tkeys, int64_t M);
+cudaError_t collect_items(sfmm_plan_s* P, int64_t M);
 cudaError_t collect_leaves(sfmm_plan_s* P, const int* cnt, Buf& out, int64_t* n_out, int64_t* d_out);
 cudaError_t build_lists(sfmm_plan_s* P, const TreeView& T, double c_s, double c_t, cudaStream_t s);
 void fill_tables(double* h);
@@ -66,18 +67,18 @@ cudaError_t launch_p2m_df_leaf(const TreeView& T, const int* leaves, int64_t n_l
                                const float4* doff, const float4* log_tab, int p, void* mpole, cudaStream_t s);
 cudaError_t launch_unscale(int n_nodes, const double* geom, const void* in, double* out, int p, int is_local,
                            int ek, cudaStream_t s);
-cudaError_t launch_eval32_prep(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl,
+cudaError_t launch_eval32_prep(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit,
                                const double4_32a* tgt, float4* toff, const uint64_t* p2p_t, const uint32_t* p2p_s,
                                int64_t n_p2p, const int64_t* d_np, float4* dc, cudaStream_t s);
-cudaError_t launch_eval32(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const float4* soff,
+cudaError_t launch_eval32(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const float4* soff,
                           const float4* toff, const float4* dc, const double4_32a* tgt, const uint32_t* tperm, const int64_t* p2p_off,
                           const uint32_t* p2p_src, const void* local, const void* mpole, bool dfar, int p, int zero_mean,
                           double* psi, double* alpha, bool coincide, float4* nf, int* tleaf,
                           const void* frames, int64_t M, int what, unsigned long long* leaf_ctr, cudaStream_t s);
-cudaError_t launch_count_pairs(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* p2p_off,
+cudaError_t launch_count_pairs(const TreeView& T, const int2* items, int64_t n_items, const int64_t* p2p_off,
                                const uint32_t* p2p_src, unsigned long long* out, cudaStream_t s);
 void fill_log_table(float* out);
-cudaError_t launch_eval_df(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const float4* soff,
+cudaError_t launch_eval_df(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const float4* soff,
                            const float4* toff, const float4* dc, const double4_32a* tgt, const uint32_t* tperm,
                            const int64_t* p2p_off, const uint32_t* p2p_src, const void* local, const void* mpole,
                            const float4* log_tab, int p, int zero_mean, double* psi, double* alpha,
@@ -85,12 +86,12 @@ cudaError_t launch_eval_df(const TreeView& T, const int* leaves, int64_t n_leave
                            const void* frames, int64_t M, int what, unsigned long long* leaf_ctr, cudaStream_t s);
 cudaError_t launch_p2m_adj(const TreeView& T, const int* leaves, int64_t n_leaves, const double4_32a* src,
                            const double4_32a* dip, double* mpole, int p, cudaStream_t s);
-cudaError_t launch_eval_adj(const TreeView& T, const int* leaves, int64_t n_leaves, const double4_32a* src,
+cudaError_t launch_eval_adj(const TreeView& T, const int2* items, int64_t n_items, const double4_32a* src,
                             const double4_32a* dip, const double4_32a* tgt, const uint32_t* tperm,
                             const int64_t* p2p_off, const uint32_t* p2p_src, const double* local, const double* mpole,
                             int p, int zero_mean, const void* w, int w_f32, double* phi, double* grad3,
                             unsigned long long* leaf_ctr, cudaStream_t s);
-cudaError_t launch_eval(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const double4_32a* src,
+cudaError_t launch_eval(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const double4_32a* src,
                         const double4_32a* tgt,
                         const uint32_t* tperm, const int64_t* p2p_off, const uint32_t* p2p_src, const double* local,
                         const double* mpole, int p, int zero_mean, double sigma, double* psi, double* alpha,
@@ -393,14 +394,13 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     if ((e = collect_leaves(P, T.count, P->leaves_src, &P->n_leaves, dcnt ? &dcnt->n_leaves : nullptr)))
         return cuda_fail(P, e, "leaves");
     const int64_t* d_nls = dcnt ? &dcnt->n_leaves : nullptr;
-    const int64_t* d_nlt = dcnt ? &dcnt->n_leaves_tgt : nullptr;
+    const int64_t* d_nit = dcnt ? &dcnt->n_items : nullptr;
     tm.mark();
-    // ---- join the targets; target ranges (Sec. 3.7 lookup) and target leaves
+    // ---- join the targets; target ranges (Sec. 3.7 lookup) and the evaluation's work items
     if ((e = cudaStreamWaitEvent(s, P->ev_join, 0))) return cuda_fail(P, e, "join");
     if ((e = tree_target_ranges(P, tkeys, M))) return cuda_fail(P, e, "target ranges");
     T = view(P);
-    if ((e = collect_leaves(P, T.tcount, P->leaves_tgt, &P->n_leaves_tgt, dcnt ? &dcnt->n_leaves_tgt : nullptr)))
-        return cuda_fail(P, e, "target leaves");
+    if ((e = collect_items(P, M))) return cuda_fail(P, e, "evaluation items");
     // ---- up-pass on the plan's stream while the lists (Algorithm 1) are built on
     // the auxiliary stream: neither needs the other's results, and the small
     // levels of the one leave room on the GPU for the other
@@ -472,7 +472,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         const uint64_t* p2p_t = P->p2p_alt ? P->p2p_t2.as<uint64_t>() : P->p2p_t.as<uint64_t>();
         if ((e = ensure(P->toff, (size_t)M * 32)) || (e = ensure(P->dc, (size_t)std::max<int64_t>(P->n_p2p, 1) * 32)))
             return cuda_fail(P, e, "alloc");
-        if ((e = launch_eval32_prep(T, P->leaves_tgt.as<int>(), P->n_leaves_tgt, d_nlt, P->tgt4.as<double4_32a>(),
+        if ((e = launch_eval32_prep(T, P->items.as<int2>(), P->n_items, d_nit, P->tgt4.as<double4_32a>(),
                                     P->toff.as<float4>(), p2p_t, p2p_s, P->n_p2p, P->d_p2p, P->dc.as<float4>(),
                                     P->aux)))
             return cuda_fail(P, e, "offsets");
@@ -486,7 +486,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         if ((e = ensure(P->nfbuf, (size_t)M * 48)) || (e = ensure(P->tleaf, (size_t)M * 4)))
             return cuda_fail(P, e, "alloc");
         if (P->timing) cudaEventRecord(P->ev_near[0], P->aux);
-        if ((e = launch_eval_df(T, P->leaves_tgt.as<int>(), P->n_leaves_tgt, d_nlt, P->soff.as<float4>(),
+        if ((e = launch_eval_df(T, P->items.as<int2>(), P->n_items, d_nit, P->soff.as<float4>(),
                                 P->toff.as<float4>(), P->dc.as<float4>(), P->tgt4.as<double4_32a>(), tperm,
                                 P->p2p_off.as<int64_t>(), p2p_s, P->local.p, P->mpole.p, P->logtab.as<float4>(), p,
                                 P->opt.zero_mean, psi, alpha, nullptr, nullptr, 0, nullptr, P->nfbuf.as<float4>(),
@@ -498,7 +498,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         if ((e = ensure(P->nfbuf, (size_t)M * 32)) || (e = ensure(P->tleaf, (size_t)M * 4)))
             return cuda_fail(P, e, "alloc");
         if (P->timing) cudaEventRecord(P->ev_near[0], P->aux);
-        if ((e = launch_eval32(T, P->leaves_tgt.as<int>(), P->n_leaves_tgt, d_nlt, P->soff.as<float4>(),
+        if ((e = launch_eval32(T, P->items.as<int2>(), P->n_items, d_nit, P->soff.as<float4>(),
                                P->toff.as<float4>(), P->dc.as<float4>(), P->tgt4.as<double4_32a>(), tperm,
                                P->p2p_off.as<int64_t>(), p2p_s, P->local.p, P->mpole.p, true, p, P->opt.zero_mean,
                                psi, alpha, src == tgt, P->nfbuf.as<float4>(), P->tleaf.as<int>(), P->framedf.p, M,
@@ -570,31 +570,31 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     tm.mark();
     // ---- evaluation (after the P2P list and the offsets of the auxiliary stream)
     if ((e = cudaStreamWaitEvent(s, P->ev_join, 0))) return cuda_fail(P, e, "join offsets");
-    if (adj_df) e = launch_eval_df(T, P->leaves_tgt.as<int>(), P->n_leaves_tgt, d_nlt, P->soff.as<float4>(),
+    if (adj_df) e = launch_eval_df(T, P->items.as<int2>(), P->n_items, d_nit, P->soff.as<float4>(),
                                    P->toff.as<float4>(), P->dc.as<float4>(), P->tgt4.as<double4_32a>(), tperm,
                                    P->p2p_off.as<int64_t>(), p2p_s, P->local.p, P->mpole.p, P->logtab.as<float4>(), p,
                                    P->opt.zero_mean, psi, nullptr, P->dip4.as<float4>(), adj->w, adj->w_f32,
                                    adj->grad3, nullptr, nullptr, nullptr, M, EVAL_NEAR | EVAL_FINISH, leaf_ctr, s);
-    else if (adj) e = launch_eval_adj(T, P->leaves_tgt.as<int>(), P->n_leaves_tgt, P->src4.as<double4_32a>(),
+    else if (adj) e = launch_eval_adj(T, P->items.as<int2>(), P->n_items, P->src4.as<double4_32a>(),
                                  P->dip4.as<double4_32a>(), P->tgt4.as<double4_32a>(), tperm, P->p2p_off.as<int64_t>(),
                                  p2p_s, P->local.as<double>(), P->mpole.as<double>(), p, P->opt.zero_mean, adj->w,
                                  adj->w_f32, psi, adj->grad3, leaf_ctr, s);
     else if (near32) {
         // 1e-6 path: the double-float finish on the near field's sums (the near field ran on the
         // auxiliary stream); all-FP32 path: the near field with its FP32 finish
-        e = launch_eval32(T, P->leaves_tgt.as<int>(), P->n_leaves_tgt, d_nlt, P->soff.as<float4>(),
+        e = launch_eval32(T, P->items.as<int2>(), P->n_items, d_nit, P->soff.as<float4>(),
                           P->toff.as<float4>(), P->dc.as<float4>(), P->tgt4.as<double4_32a>(), tperm,
                           P->p2p_off.as<int64_t>(), p2p_s, P->local.p, P->mpole.p, !fp32, p, P->opt.zero_mean, psi,
                           alpha, src == tgt, P->nfbuf.as<float4>(), P->tleaf.as<int>(), P->framedf.p, M,
                           near_early ? EVAL_FINISH : EVAL_NEAR | EVAL_FINISH, leaf_ctr, s);
     }
-    else if (dfe) e = launch_eval_df(T, P->leaves_tgt.as<int>(), P->n_leaves_tgt, d_nlt, P->soff.as<float4>(),
+    else if (dfe) e = launch_eval_df(T, P->items.as<int2>(), P->n_items, d_nit, P->soff.as<float4>(),
                                      P->toff.as<float4>(), P->dc.as<float4>(), P->tgt4.as<double4_32a>(), tperm,
                                      P->p2p_off.as<int64_t>(), p2p_s, P->local.p, P->mpole.p,
                                      P->logtab.as<float4>(), p, P->opt.zero_mean, psi, alpha, nullptr, nullptr, 0,
                                      nullptr, P->nfbuf.as<float4>(), P->tleaf.as<int>(), P->framedf.p, M,
                                      near_early_df ? EVAL_FINISH : EVAL_NEAR | EVAL_FINISH, leaf_ctr, s);
-    else e = launch_eval(T, P->leaves_tgt.as<int>(), P->n_leaves_tgt, d_nlt, P->src4.as<double4_32a>(),
+    else e = launch_eval(T, P->items.as<int2>(), P->n_items, d_nit, P->src4.as<double4_32a>(),
                          P->tgt4.as<double4_32a>(), tperm, P->p2p_off.as<int64_t>(), p2p_s, P->local.as<double>(),
                          P->mpole.as<double>(), p, P->opt.zero_mean, P->opt.sigma, psi, alpha, gamma, mu, leaf_ctr, s);
     if (e) return cuda_fail(P, e, "evaluation");
@@ -607,7 +607,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         // near-field source-target pairs (for the throughput of the evaluation kernel)
         unsigned long long* cnt = reinterpret_cast<unsigned long long*>(P->small.as<int64_t>() + 16);
         if ((e = cudaMemsetAsync(cnt, 0, 8, s))) return cuda_fail(P, e, "memset");
-        if ((e = launch_count_pairs(T, P->leaves_tgt.as<int>(), P->n_leaves_tgt, P->p2p_off.as<int64_t>(), p2p_s,
+        if ((e = launch_count_pairs(T, P->items.as<int2>(), P->n_items, P->p2p_off.as<int64_t>(), p2p_s,
                                     cnt, s)))
             return cuda_fail(P, e, "count pairs");
         unsigned long long h = 0;
@@ -946,7 +946,7 @@ void sfmm_destroy(sfmm_plan_t plan)
                   &plan->act, &plan->c_next, &plan->c_m2l, &plan->c_p2p, &plan->o_next, &plan->o_m2l, &plan->o_p2p,
                   &plan->m2l_t, &plan->m2l_s, &plan->m2l_t2, &plan->m2l_s2, &plan->p2p_t, &plan->p2p_s,
                   &plan->p2p_t2, &plan->p2p_s2, &plan->m2l_off, &plan->p2p_off, &plan->leaves_src,
-                  &plan->leaves_tgt, &plan->m2l_geo, &plan->m2m_geo, &plan->l2l_geo, &plan->soff,
+                  &plan->items, &plan->m2l_geo, &plan->m2m_geo, &plan->l2l_geo, &plan->soff,
                   &plan->toff, &plan->dc, &plan->leftover, &plan->geom32, &plan->macn, &plan->logtab,
                   &plan->ttmp, &plan->dip4, &plan->adj_h, &plan->adj_g, &plan->macn32, &plan->m2l_acc,
                   &plan->framedf, &plan->dcnt, &plan->nfbuf, &plan->tleaf};

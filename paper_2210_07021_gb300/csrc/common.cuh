@@ -93,6 +93,23 @@ __device__ __forceinline__ int64_t dcount(const int64_t* d, int64_t h)
     return v < h ? v : h;
 }
 
+// A work item of the evaluation kernels: a target leaf (x) and a chunk of up to
+// 64 of its targets (y: the chunk's first target, a multiple of 64, plus the
+// parts of the chunk in the low bits: ITEM_A its first 32 targets, ITEM_B the
+// rest).  A leaf can hold any number of targets (a grid's points in an empty
+// region, a clump of particles over a coarse grid), so a leaf is not a unit of
+// work; chunks are, and 64 is the number of targets one pass over the staged
+// near sources serves, so chunking changes no target's arithmetic.
+enum { ITEM_A = 1, ITEM_B = 2, ITEM_CHUNK = 64 };
+__device__ __forceinline__ int item_start(int2 it) { return it.y & ~(ITEM_CHUNK - 1); }
+// the targets [lo, hi) of the leaf that an item covers (tc: the leaf's targets)
+__device__ __forceinline__ void item_range(int2 it, int tc, int* lo, int* hi)
+{
+    const int tb = item_start(it), parts = it.y & 3;
+    *lo = tb + (parts == ITEM_B ? 32 : 0);
+    *hi = parts == ITEM_A ? tb + 32 : min(tc, tb + ITEM_CHUNK);
+}
+
 // The counts of a solve run without host synchronisation (graph mode): launches
 // are sized by the plan's capacities and every kernel reads its actual count
 // here; a kernel that would exceed a capacity sets `overflow` instead of
@@ -100,7 +117,7 @@ __device__ __forceinline__ int64_t dcount(const int64_t* d, int64_t h)
 struct DevCounts {
     int64_t nn;             // nodes
     int64_t n_leaves;       // source leaves (count > 0)
-    int64_t n_leaves_tgt;   // target leaves (tcount > 0)
+    int64_t n_items;        // work items of the evaluation (chunks of target leaves)
     int64_t overflow;       // nonzero: a capacity was exceeded
     int64_t level[32];      // level starts: nodes of level l are [level[l], level[l + 1])
 };
@@ -178,8 +195,8 @@ struct sfmm_plan_s {
     int64_t walk_cap_front = 0, walk_cap_m2l = 0, walk_cap_p2p = 0;   // list capacities that sufficed last time
     bool m2l_alt = false, p2p_alt = false;
     // node work lists
-    sfmm::Buf leaves_src, leaves_tgt;
-    int64_t n_leaves = 0, n_leaves_tgt = 0;
+    sfmm::Buf leaves_src, items;           // source leaves; evaluation items (int2, see ITEM_A)
+    int64_t n_leaves = 0, n_items = 0;
     bool skeys_alt = false, tkeys_alt = false;
     int64_t last_N = 0, last_M = 0;
 };

@@ -16,12 +16,16 @@
 //   alpha_i = (1/2pi) [ sum_j q_j (x - y_j) / d_j^2 - (x/2) sum_j q_j ]
 // with d^2 = |x - y|^2 from coordinate differences; d^2 == 0 pairs are skipped.
 //
-// One warp per target leaf.  The leaf's targets are taken in groups of tpw,
-// the largest power of two not above the targets left (at most 32), so that
-// no lane idles; each target of a group gets 32/tpw lanes that split its
+// One warp per work item, a chunk of up to 64 targets of a leaf (ITEM_CHUNK in
+// common.cuh).  (A warp per whole leaf left the chip idle behind the few leaves
+// that hold thousands of targets: 1e6 clustered sources at the 3.1e6 points of
+// an N_side 512 grid took 9.8 ms for 3.5e9 pairs, 2.7 ms with items; 1e4 sources
+// at an N_side 64 grid 3.5 ms, 0.19 ms with items.)  The targets of an item are
+// taken in groups of tpw, the largest power of two not above the targets left
+// (at most 32), so that no lane idles; each target of a group gets 32/tpw lanes that split its
 // sources and are combined by xor shuffles.  (The FP32 kernel, whose pair loop
-// is cheap next to restaging its sources per group, keeps one group size per
-// leaf: the power of two not below the leaf's targets.)
+// is cheap next to restaging its sources per group, serves two groups per pass
+// over the sources.)
 #include "common.cuh"
 #include "dfloat.cuh"
 #include "xgeo.cuh"
@@ -45,9 +49,9 @@ constexpr float INV4PI_L = (float)(INV4PI - (double)INV4PI_H);
 
 struct EvalArgs {
     TreeView T;
-    const int* leaves;        // target leaves (tcount > 0)
-    int64_t n_leaves;
-    const int64_t* d_n_leaves;      // graph mode: the leaf count on the device (n_leaves: the capacity)
+    const int2* items;        // work items: chunks of target leaves
+    int64_t n_items;
+    const int64_t* d_n_items;       // graph mode: the item count on the device (n_items: the capacity)
     const double4_32a* src;       // key-sorted sources (x, y, z, q)
     const double4_32a* tgt;       // key-sorted targets (x, y, z, -)
     const uint32_t* tperm;    // original index of each sorted target
@@ -62,7 +66,7 @@ struct EvalArgs {
     double* alpha;
     double* gamma;            // [M][2] shear (gamma_1, gamma_2) in (e_theta, e_phi), or NULL
     double* mu;               // [M] magnification 1/((1 - tr H/2)^2 - |gamma|^2), or NULL (with gamma)
-    unsigned long long* leaf_ctr;   // zero at launch: the warps take target leaves from it one at a time
+    unsigned long long* leaf_ctr;   // zero at launch: the warps take items from it one at a time
     double npm_s;             // Near Particle Model: sin^2(sigma/2) (NPM kernels only)
 };
 
@@ -87,8 +91,8 @@ __device__ __forceinline__ double group_sum(double v, int lpt)
 // f = (m(u) - u)/(1 - u), m = 2u/s - u^2/s^2 (Gauss's law on the sphere), and
 // log u replaced by log s - (1 - u/s) + ((1 - s)^2/s^2)(log1p(t) - t),
 // t = (s - u)/(1 - s) (the point-mass potential continued into the cap).
-// The next target leaf of a warp, taken from a global counter by lane 0.
-__device__ __forceinline__ int64_t next_leaf(unsigned long long* ctr, int lane)
+// The next work item of a warp, taken from a global counter by lane 0.
+__device__ __forceinline__ int64_t next_item(unsigned long long* ctr, int lane)
 {
     unsigned long long w = 0;
     if (lane == 0) w = atomicAdd(ctr, 1ull);
@@ -103,19 +107,22 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
     for (int b = 0; b < 12; ++b) qtot += A.base_mpole[(size_t)b * EXP_STRIDE + 1];
     if (A.zero_mean) shift = qtot;
     for (;;) {
-        const int64_t w = next_leaf(A.leaf_ctr, lane);
-        if (w >= dcount(A.d_n_leaves, A.n_leaves)) break;
-        const int leaf = A.leaves[w];
+        const int64_t w = next_item(A.leaf_ctr, lane);
+        if (w >= dcount(A.d_n_items, A.n_items)) break;
+        const int2 item = A.items[w];
+        const int leaf = item.x;
         const int tf = A.T.tfirst[leaf], tc = A.T.tcount[leaf];
         const double* g = A.T.geom + (size_t)leaf * GEOM_STRIDE;
         const double* L = A.local + (size_t)leaf * EXP_STRIDE;
         const int64_t nb0 = A.p2p_off[leaf], nb1 = A.p2p_off[leaf + 1];
-        for (int tb = 0, tpw = 0; tb < tc; tb += tpw) {
-            tpw = min(32, 1 << (31 - __clz(tc - tb)));     // largest power of two <= the targets left
+        int t0, t1;
+        item_range(item, tc, &t0, &t1);
+        for (int tb = t0, tpw = 0; tb < t1; tb += tpw) {
+            tpw = min(32, 1 << (31 - __clz(t1 - tb)));     // largest power of two <= the targets left
             const int lpt = 32 / tpw;
             const int slot = lane / lpt, sub = lane % lpt;
             const int ti = tb + slot;
-            const bool active = ti < tc;
+            const bool active = ti < t1;
             const double4_32a x = A.tgt[tf + (active ? ti : 0)];
             double sl = 0.0, sx = 0.0, sy = 0.0, sz = 0.0, sq = 0.0;
             double Sxx = 0.0, Syy = 0.0, Szz = 0.0, Sxy = 0.0, Sxz = 0.0, Syz = 0.0;
@@ -277,15 +284,18 @@ __global__ void __launch_bounds__(128) k_eval_adj(EvalAdjArgs AA)
     if (A.zero_mean)
         for (int b = 0; b < 12; ++b) shift += A.base_mpole[(size_t)b * EXP_STRIDE + 1];
     for (;;) {
-        const int64_t w = next_leaf(A.leaf_ctr, lane);
-        if (w >= dcount(A.d_n_leaves, A.n_leaves)) break;
-        const int leaf = A.leaves[w];
+        const int64_t w = next_item(A.leaf_ctr, lane);
+        if (w >= dcount(A.d_n_items, A.n_items)) break;
+        const int2 item = A.items[w];
+        const int leaf = item.x;
         const int tf = A.T.tfirst[leaf], tc = A.T.tcount[leaf];
         const double* g = A.T.geom + (size_t)leaf * GEOM_STRIDE;
         const double* L = A.local + (size_t)leaf * EXP_STRIDE;
         const int64_t nb0 = A.p2p_off[leaf], nb1 = A.p2p_off[leaf + 1];
-        for (int tb = 0, tpw = 0; tb < tc; tb += tpw) {
-            tpw = min(32, 1 << (31 - __clz(tc - tb)));
+        int t0, t1;
+        item_range(item, tc, &t0, &t1);
+        for (int tb = t0, tpw = 0; tb < t1; tb += tpw) {
+            tpw = min(32, 1 << (31 - __clz(t1 - tb)));
             const int lpt = 32 / tpw;
             const int slot = lane / lpt, sub = lane % lpt;
             const int ti = tb + slot;
@@ -371,14 +381,17 @@ __global__ void __launch_bounds__(128) k_eval_adj(EvalAdjArgs AA)
     }
 }
 
-__global__ void k_count_pairs(TreeView T, const int* __restrict__ leaves, int64_t n, const int64_t* __restrict__ off,
+__global__ void k_count_pairs(TreeView T, const int2* __restrict__ items, int64_t n, const int64_t* __restrict__ off,
                               const uint32_t* __restrict__ src, unsigned long long* __restrict__ out)
 {
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (int64_t)gridDim.x * blockDim.x) {
-        const int leaf = leaves[w];
+        const int2 item = items[w];
+        const int leaf = item.x;
+        int t0, t1;
+        item_range(item, T.tcount[leaf], &t0, &t1);
         unsigned long long c = 0;
         for (int64_t k = off[leaf]; k < off[leaf + 1]; ++k) c += (unsigned long long)T.count[src[k]];
-        atomicAdd(out, c * (unsigned long long)T.tcount[leaf]);
+        atomicAdd(out, c * (unsigned long long)(t1 - t0));
     }
 }
 
@@ -401,9 +414,9 @@ constexpr int STAGE32 = 192;   // FP32 kernel: smaller stage, 7 blocks of 4 warp
 
 struct Eval32Args {
     TreeView T;
-    const int* leaves;
-    int64_t n_leaves;
-    const int64_t* d_n_leaves;      // graph mode: the leaf count on the device (n_leaves: the capacity)
+    const int2* items;        // work items: chunks of target leaves
+    int64_t n_items;
+    const int64_t* d_n_items;       // graph mode: the item count on the device (n_items: the capacity)
     const float4* soff;       // [2N]: (hi offset, q), (lo offset, 0) of each source from its leaf centre
     const float4* toff;       // [2M]: (hi, x.z), (lo, 0) offset of each sorted target from its leaf centre
     const float4* dc;         // [2 n_p2p]: (hi, 0), (lo, 0) offset of each near leaf's centre from the target leaf's
@@ -420,7 +433,7 @@ struct Eval32Args {
     int zero_mean;
     double* psi;
     double* alpha;
-    unsigned long long* leaf_ctr;   // zero at launch: the warps take target leaves from it one at a time
+    unsigned long long* leaf_ctr;   // zero at launch: the warps take items from it one at a time
     // double-float far field: the near field's sums per sorted target, for k_finish_dfar:
     // nf[2t] = (x.h, x.l, y.h, y.l), nf[2t + 1] = (z.h, z.l, sum q, sum q log2 d^2), and its leaf
     float4* nf;
@@ -740,9 +753,9 @@ __device__ __forceinline__ dflt group_sum_df(dflt v, int lpt)
     return v;
 }
 
-// One warp per target leaf.  The FP32 pair loop is cheap next to staging the
+// One warp per item.  The FP32 pair loop is cheap next to staging the
 // sources, so each pass over the near sources serves two groups of targets at
-// once: group a takes the largest power of two <= the targets left (at most
+// once (an item of part A or B alone, one of them): group a takes the largest power of two <= the targets left (at most
 // 32), group b the power of two >= what a leaves (at most 32), e.g. 18 = 16 + 2
 // and 40 = 32 + 8; each target of a group gets 32/size lanes.
 // DFAR: the far field (local expansions, L2P) in double-float and the outer
@@ -763,9 +776,10 @@ __global__ void __launch_bounds__(128, 7) k_eval32(Eval32Args A)
     int* pre = s_pre[wid];
     int* fst = s_first[wid];
     for (;;) {
-        const int64_t w = next_leaf(A.leaf_ctr, lane);
-        if (w >= dcount(A.d_n_leaves, A.n_leaves)) break;
-        const int leaf = A.leaves[w];
+        const int64_t w = next_item(A.leaf_ctr, lane);
+        if (w >= dcount(A.d_n_items, A.n_items)) break;
+        const int2 item = A.items[w];
+        const int leaf = item.x;
         const int tf = A.T.tfirst[leaf], tc = A.T.tcount[leaf];
         const double* g = A.T.geom + (size_t)leaf * GEOM_STRIDE;
         const float* L = A.local + (size_t)leaf * EXP_STRIDE;
@@ -783,16 +797,18 @@ __global__ void __launch_bounds__(128, 7) k_eval32(Eval32Args A)
         }
         __syncwarp();
         const int64_t nb0 = A.p2p_off[leaf], nb1 = A.p2p_off[leaf + 1];
-        for (int tb = 0; tb < tc;) {
-            const int rem = tc - tb;
-            const int na = min(32, 1 << (31 - __clz(rem)));
-            const int rb = rem - na;
+        int t0, t1;
+        item_range(item, tc, &t0, &t1);
+        for (int tb = item_start(item); tb < t1;) {       // one pass (as a loop it compiles without spills)
+            const int rem = t1 - tb;
+            // ITEM_B alone: group a stays empty (sa past every source pair and never 0)
+            const int na = min(32, 1 << (31 - __clz(rem))), rb = rem - na;
             const int nb = rb <= 0 ? 0 : min(32, 1 << (32 - __clz(rb - 1)));   // power of two >= rb
-            const int lpa = 32 / na, sa = lane % lpa;
+            const int lpa = 32 / na, sa = (item.y & ITEM_A) ? lane % lpa : 1 << 30;
             const int lpb = nb ? 32 / nb : 32, sb = lane % lpb;
             const size_t ta = (size_t)tf + tb + lane / lpa;
             const int ib = tb + na + lane / lpb;
-            const bool act_b = nb > 0 && ib < tc;
+            const bool act_b = nb > 0 && ib < t1;
             const size_t tbx = (size_t)tf + (act_b ? ib : tb);
             const float4 tha = A.toff[2 * ta], tla = A.toff[2 * ta + 1];
             const float4 thb = A.toff[2 * tbx], tlb = A.toff[2 * tbx + 1];
@@ -938,9 +954,9 @@ __device__ __forceinline__ dflt dfl_diff(float ah, float al, float bh, float bl)
 
 struct EvalDfArgs {
     TreeView T;
-    const int* leaves;
-    int64_t n_leaves;
-    const int64_t* d_n_leaves;      // graph mode: the leaf count on the device (n_leaves: the capacity)
+    const int2* items;        // work items: chunks of target leaves
+    int64_t n_items;
+    const int64_t* d_n_items;       // graph mode: the item count on the device (n_items: the capacity)
     const float4* soff;
     const float4* toff;
     const float4* dc;
@@ -955,7 +971,7 @@ struct EvalDfArgs {
     int zero_mean;
     double* psi;
     double* alpha;
-    unsigned long long* leaf_ctr;   // zero at launch: the warps take target leaves from it one at a time
+    unsigned long long* leaf_ctr;   // zero at launch: the warps take items from it one at a time
     // the adjoint (k_eval_df<PSI, true>): the sources' tangent dipoles as (hi, lo)
     // float4 pairs, the targets' weights w (the forward masses) and the output
     // w grad Phi [M][3]; psi then receives Phi
@@ -1333,7 +1349,7 @@ __device__ __forceinline__ void finish_target_adj_df(const EvalDfArgs& A, const 
     }
 }
 
-// One warp per target leaf; each pass over the near sources serves two groups
+// One warp per item; each pass over the near sources serves two groups
 // of targets, as in k_eval32 (group a: the largest power of two <= the targets
 // left, group b: the power of two >= what a leaves; 32 / size lanes per target).
 // ADJ: the adjoint (charges and tangent dipoles at the sources, Phi and w grad
@@ -1413,9 +1429,10 @@ __global__ void __launch_bounds__(128, ADJ ? 4 : 5) k_eval_df(EvalDfArgs A)
     int* fst = s_first[wid];
     LeafFrameD2& G = s_frame2[wid];
     for (;;) {
-        const int64_t w = next_leaf(A.leaf_ctr, lane);
-        if (w >= dcount(A.d_n_leaves, A.n_leaves)) break;
-        const int leaf = A.leaves[w];
+        const int64_t w = next_item(A.leaf_ctr, lane);
+        if (w >= dcount(A.d_n_items, A.n_items)) break;
+        const int2 item = A.items[w];
+        const int leaf = item.x;
         const int tf = A.T.tfirst[leaf], tc = A.T.tcount[leaf];
         const double* g = A.T.geom + (size_t)leaf * GEOM_STRIDE;
         const dflt* L = A.local + (size_t)leaf * EXP_STRIDE;
@@ -1430,16 +1447,18 @@ __global__ void __launch_bounds__(128, ADJ ? 4 : 5) k_eval_df(EvalDfArgs A)
             if (lane == 3) G.inv_r = dflt(1.0 / g[10]);
             __syncwarp();
         }
-        for (int tb = 0; tb < tc;) {
-            const int rem = tc - tb;
-            const int na = min(32, 1 << (31 - __clz(rem)));
-            const int rb = rem - na;
+        int t0, t1;
+        item_range(item, tc, &t0, &t1);
+        for (int tb = item_start(item); tb < t1;) {       // one pass (as a loop it compiles without spills)
+            const int rem = t1 - tb;
+            // ITEM_B alone: group a stays empty (sa past every source pair and never 0)
+            const int na = min(32, 1 << (31 - __clz(rem))), rb = rem - na;
             const int nb = rb <= 0 ? 0 : min(32, 1 << (32 - __clz(rb - 1)));   // power of two >= rb
-            const int lpa = 32 / na, sa = lane % lpa;
+            const int lpa = 32 / na, sa = (item.y & ITEM_A) ? lane % lpa : 1 << 30;
             const int lpb = nb ? 32 / nb : 32, sb = lane % lpb;
             const size_t ta = (size_t)tf + tb + lane / lpa;
             const int ib = tb + na + lane / lpb;
-            const bool act_b = nb > 0 && ib < tc;
+            const bool act_b = nb > 0 && ib < t1;
             const size_t tbx = (size_t)tf + (act_b ? ib : tb);
             const float4 tha = A.toff[2 * ta], tla = A.toff[2 * ta + 1];
             const float4 thb = A.toff[2 * tbx], tlb = A.toff[2 * tbx + 1];
@@ -1586,18 +1605,20 @@ __global__ void __launch_bounds__(128, ADJ ? 4 : 5) k_eval_df(EvalDfArgs A)
 // instructions (the difference to 2^-47): each sorted target from its leaf's
 // centre, and each near leaf's centre from its target leaf's centre (one per
 // direct-act pair).
-__global__ void k_tgt_offsets(TreeView T, const int* __restrict__ leaves, int64_t n_cap, const int64_t* d_nl,
+__global__ void k_tgt_offsets(TreeView T, const int2* __restrict__ items, int64_t n_cap, const int64_t* d_nit,
                               const double4_32a* __restrict__ tgt, float4* __restrict__ off)
 {
-    const int64_t n_leaves = dcount(d_nl, n_cap);
+    const int64_t n_items = dcount(d_nit, n_cap);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t w = warp0; w < n_leaves; w += nw) {
-        const int node = leaves[w];
-        const double* g = T.geom + (size_t)node * GEOM_STRIDE;
-        const int f = T.tfirst[node], n = T.tcount[node];
-        for (int j = f + lane; j < f + n; j += 32) {
+    for (int64_t w = warp0; w < n_items; w += nw) {
+        const int2 item = items[w];
+        const double* g = T.geom + (size_t)item.x * GEOM_STRIDE;
+        const int f = T.tfirst[item.x];
+        int t0, t1;
+        item_range(item, T.tcount[item.x], &t0, &t1);
+        for (int j = f + t0 + lane; j < f + t1; j += 32) {
             const double4_32a x = tgt[j];
             const dflt dx = dfl_sub_exact(x.x, g[0]), dy = dfl_sub_exact(x.y, g[1]), dz = dfl_sub_exact(x.z, g[2]);
             off[2 * (size_t)j] = make_float4(dx.h, dy.h, dz.h, 0.f);
@@ -1621,33 +1642,33 @@ __global__ void k_pair_offsets(TreeView T, const uint64_t* __restrict__ tt, cons
     }
 }
 
-// Zero the leaf counter and size a persistent grid of 4-warp CTAs: up to
-// per_sm per SM (the CTAs an SM holds at once); every warp takes target leaves
-// from the counter until none are left, so uneven leaves leave no slot idle
+// Zero the item counter and size a persistent grid of 4-warp CTAs: up to
+// per_sm per SM (the CTAs an SM holds at once); every warp takes items
+// from the counter until none are left, so uneven items leave no slot idle
 // (CTAs beyond what the SMs hold start when others exit and find little or
 // nothing left).
-cudaError_t leaf_grid(unsigned long long* ctr, int64_t n_leaves, int per_sm, cudaStream_t s, int64_t* blocks)
+cudaError_t item_grid(unsigned long long* ctr, int64_t n_items, int per_sm, cudaStream_t s, int64_t* blocks)
 {
     cudaError_t e;
     int dev = 0, sms = 0;
     if ((e = cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), s)) || (e = cudaGetDevice(&dev)) ||
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
         return e;
-    const int64_t want = (n_leaves + 3) / 4;
+    const int64_t want = (n_items + 3) / 4;
     *blocks = want < (int64_t)sms * per_sm ? want : (int64_t)sms * per_sm;
     return cudaSuccess;
 }
 
 }  // namespace
 
-cudaError_t launch_eval32_prep(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl,
+cudaError_t launch_eval32_prep(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit,
                                const double4_32a* tgt, float4* toff, const uint64_t* p2p_t, const uint32_t* p2p_s,
                                int64_t n_p2p, const int64_t* d_np, float4* dc, cudaStream_t s)
 {
-    if (n_leaves > 0) {
-        int64_t b = (n_leaves + 7) / 8;
+    if (n_items > 0) {
+        int64_t b = (n_items + 7) / 8;
         if (b > 152 * 64) b = 152 * 64;
-        k_tgt_offsets<<<(unsigned)b, 256, 0, s>>>(T, leaves, n_leaves, d_nl, tgt, toff); count_launch();
+        k_tgt_offsets<<<(unsigned)b, 256, 0, s>>>(T, items, n_items, d_nit, tgt, toff); count_launch();
     }
     if (n_p2p > 0) {
         int64_t b = (n_p2p + 255) / 256;
@@ -1658,18 +1679,18 @@ cudaError_t launch_eval32_prep(const TreeView& T, const int* leaves, int64_t n_l
 }
 
 // local/mpole: FP32 expansions, or double-float ones when dfar (the 1e-6 path)
-cudaError_t launch_eval32(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const float4* soff,
+cudaError_t launch_eval32(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const float4* soff,
                           const float4* toff, const float4* dc, const double4_32a* tgt, const uint32_t* tperm, const int64_t* p2p_off,
                           const uint32_t* p2p_src, const void* local, const void* mpole, bool dfar, int p, int zero_mean,
                           double* psi, double* alpha, bool coincide, float4* nf, int* tleaf,
                           const void* frames, int64_t M, int what, unsigned long long* leaf_ctr, cudaStream_t s)
 {
-    if (n_leaves == 0) return cudaSuccess;
+    if (n_items == 0) return cudaSuccess;
     Eval32Args A;
     A.T = T;
-    A.leaves = leaves;
-    A.n_leaves = n_leaves;
-    A.d_n_leaves = d_nl;
+    A.items = items;
+    A.n_items = n_items;
+    A.d_n_items = d_nit;
     A.soff = soff;
     A.toff = toff;
     A.dc = dc;
@@ -1694,7 +1715,7 @@ cudaError_t launch_eval32(const TreeView& T, const int* leaves, int64_t n_leaves
     cudaError_t e;
     if (what & EVAL_NEAR) {
         int64_t blocks = 0;
-        if ((e = leaf_grid(leaf_ctr, n_leaves, 7, s, &blocks))) return e;     // 7 per SM: __launch_bounds__
+        if ((e = item_grid(leaf_ctr, n_items, 7, s, &blocks))) return e;     // 7 per SM: __launch_bounds__
 #define EVAL32_LAUNCH(PSI, MASK)                                                  \
         if (dfar) k_eval32<PSI, MASK, true><<<(unsigned)blocks, 128, 0, s>>>(A);  \
         else k_eval32<PSI, MASK, false><<<(unsigned)blocks, 128, 0, s>>>(A);
@@ -1739,7 +1760,7 @@ void fill_log_table(float* out)
     out[4 * 128 + 2] = out[4 * 128 + 3] = 0.f;
 }
 
-cudaError_t launch_eval_df(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const float4* soff,
+cudaError_t launch_eval_df(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const float4* soff,
                            const float4* toff, const float4* dc, const double4_32a* tgt, const uint32_t* tperm,
                            const int64_t* p2p_off, const uint32_t* p2p_src, const void* local, const void* mpole,
                            const float4* log_tab, int p, int zero_mean, double* psi, double* alpha,
@@ -1748,9 +1769,9 @@ cudaError_t launch_eval_df(const TreeView& T, const int* leaves, int64_t n_leave
 {
     EvalDfArgs A;
     A.T = T;
-    A.leaves = leaves;
-    A.n_leaves = n_leaves;
-    A.d_n_leaves = d_nl;
+    A.items = items;
+    A.n_items = n_items;
+    A.d_n_items = d_nit;
     A.soff = soff;
     A.toff = toff;
     A.dc = dc;
@@ -1775,9 +1796,9 @@ cudaError_t launch_eval_df(const TreeView& T, const int* leaves, int64_t n_leave
     A.frames = static_cast<const FrameDF*>(frames);
     A.M = M;
     cudaError_t e;
-    if (n_leaves > 0 && (doff || (what & EVAL_NEAR))) {
+    if (n_items > 0 && (doff || (what & EVAL_NEAR))) {
         int64_t blocks = 0;
-        if ((e = leaf_grid(leaf_ctr, n_leaves, 16, s, &blocks))) return e;
+        if ((e = item_grid(leaf_ctr, n_items, 16, s, &blocks))) return e;
         if (doff) {                // the adjoint: near field and finish in one kernel
             if (psi) k_eval_df<true, true><<<(unsigned)blocks, 128, 0, s>>>(A);
             else k_eval_df<false, true><<<(unsigned)blocks, 128, 0, s>>>(A);
@@ -1797,28 +1818,28 @@ cudaError_t launch_eval_df(const TreeView& T, const int* leaves, int64_t n_leave
     return cudaGetLastError();
 }
 
-cudaError_t launch_count_pairs(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* p2p_off,
+cudaError_t launch_count_pairs(const TreeView& T, const int2* items, int64_t n_items, const int64_t* p2p_off,
                                const uint32_t* p2p_src, unsigned long long* out, cudaStream_t s)
 {
-    if (n_leaves == 0) return cudaSuccess;
-    int64_t blocks = (n_leaves + 255) / 256;
+    if (n_items == 0) return cudaSuccess;
+    int64_t blocks = (n_items + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    k_count_pairs<<<(unsigned)blocks, 256, 0, s>>>(T, leaves, n_leaves, p2p_off, p2p_src, out); count_launch();
+    k_count_pairs<<<(unsigned)blocks, 256, 0, s>>>(T, items, n_items, p2p_off, p2p_src, out); count_launch();
     return cudaGetLastError();
 }
 
-cudaError_t launch_eval(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const double4_32a* src,
+cudaError_t launch_eval(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const double4_32a* src,
                         const double4_32a* tgt,
                         const uint32_t* tperm, const int64_t* p2p_off, const uint32_t* p2p_src, const double* local,
                         const double* mpole, int p, int zero_mean, double sigma, double* psi, double* alpha,
                         double* gamma, double* mu, unsigned long long* leaf_ctr, cudaStream_t s)
 {
-    if (n_leaves == 0) return cudaSuccess;
+    if (n_items == 0) return cudaSuccess;
     EvalArgs A;
     A.T = T;
-    A.leaves = leaves;
-    A.n_leaves = n_leaves;
-    A.d_n_leaves = d_nl;
+    A.items = items;
+    A.n_items = n_items;
+    A.d_n_items = d_nit;
     A.src = src;
     A.tgt = tgt;
     A.tperm = tperm;
@@ -1837,7 +1858,7 @@ cudaError_t launch_eval(const TreeView& T, const int* leaves, int64_t n_leaves, 
     A.leaf_ctr = leaf_ctr;
     int64_t blocks = 0;
     cudaError_t e;
-    if ((e = leaf_grid(leaf_ctr, n_leaves, 16, s, &blocks))) return e;
+    if ((e = item_grid(leaf_ctr, n_items, 16, s, &blocks))) return e;
     if (gamma) k_eval<true, false><<<(unsigned)blocks, 128, 0, s>>>(A);
     else if (sigma > 0.0) k_eval<false, true><<<(unsigned)blocks, 128, 0, s>>>(A);
     else k_eval<false, false><<<(unsigned)blocks, 128, 0, s>>>(A);
@@ -1845,19 +1866,19 @@ cudaError_t launch_eval(const TreeView& T, const int* leaves, int64_t n_leaves, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_eval_adj(const TreeView& T, const int* leaves, int64_t n_leaves, const double4_32a* src,
+cudaError_t launch_eval_adj(const TreeView& T, const int2* items, int64_t n_items, const double4_32a* src,
                             const double4_32a* dip, const double4_32a* tgt, const uint32_t* tperm,
                             const int64_t* p2p_off, const uint32_t* p2p_src, const double* local, const double* mpole,
                             int p, int zero_mean, const void* w, int w_f32, double* phi, double* grad3,
                             unsigned long long* leaf_ctr, cudaStream_t s)
 {
-    if (n_leaves == 0) return cudaSuccess;
+    if (n_items == 0) return cudaSuccess;
     EvalAdjArgs AA;
     EvalArgs& A = AA.E;
     A.T = T;
-    A.leaves = leaves;
-    A.n_leaves = n_leaves;
-    A.d_n_leaves = nullptr;
+    A.items = items;
+    A.n_items = n_items;
+    A.d_n_items = nullptr;
     A.src = src;
     A.tgt = tgt;
     A.tperm = tperm;
@@ -1879,7 +1900,7 @@ cudaError_t launch_eval_adj(const TreeView& T, const int* leaves, int64_t n_leav
     A.leaf_ctr = leaf_ctr;
     int64_t blocks = 0;
     cudaError_t e;
-    if ((e = leaf_grid(leaf_ctr, n_leaves, 16, s, &blocks))) return e;
+    if ((e = item_grid(leaf_ctr, n_items, 16, s, &blocks))) return e;
     k_eval_adj<<<(unsigned)blocks, 128, 0, s>>>(AA); count_launch();
     return cudaGetLastError();
 }

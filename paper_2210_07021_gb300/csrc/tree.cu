@@ -112,7 +112,7 @@ __global__ void k_split_flags(const int* __restrict__ count, int a, int b, int l
 __global__ void k_counts_init(DevCounts* dc)
 {
     if (threadIdx.x < 32) dc->level[threadIdx.x] = threadIdx.x == 0 ? 0 : 12;
-    if (threadIdx.x == 0) { dc->nn = 12; dc->n_leaves = 0; dc->n_leaves_tgt = 0; dc->overflow = 0; }
+    if (threadIdx.x == 0) { dc->nn = 12; dc->n_leaves = 0; dc->n_items = 0; dc->overflow = 0; }
 }
 
 // Graph mode: the next level's end from the scan of the split flags (its total),
@@ -223,6 +223,48 @@ __global__ void k_compact(int n, const int64_t* __restrict__ flags, const int64_
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         if (flags[i]) out[pos[i]] = (int)i;
+}
+
+// Evaluation items per node: a leaf's targets in chunks of 64, or (split) of 32
+// where more than 32 are left.
+__device__ __forceinline__ int64_t items_of(int tc, int split) { return split ? (tc + 31) / 32 : (tc + 63) / 64; }
+
+__global__ void k_item_counts(int n_cap, const int64_t* d_nn, const int* __restrict__ child0,
+                              const int* __restrict__ tcount, int split, int64_t* __restrict__ flags)
+{
+    const int64_t nn = dcount(d_nn, n_cap);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_cap; i += (int64_t)gridDim.x * blockDim.x)
+        flags[i] = (i < nn && child0[i] < 0) ? items_of(tcount[i], split) : 0;
+}
+
+// Items of all leaves at their scanned places: the lanes of a warp write those
+// of 32 nodes, a node with more than 4 by the whole warp (one leaf can hold
+// every target of the problem).
+__global__ void k_items(int n, const int64_t* __restrict__ flags, const int64_t* __restrict__ pos,
+                        const int* __restrict__ tcount, int split, int2* __restrict__ out)
+{
+    const int lane = threadIdx.x & 31;
+    auto item = [&](int node, int tc, int64_t k) {
+        if (!split) return make_int2(node, (int)(k * 64) | ITEM_A | ITEM_B);
+        const int tb = (int)(k / 2) * 64;
+        const int parts = (k & 1) ? ITEM_B : tc - tb > 32 ? ITEM_A : ITEM_A | ITEM_B;
+        return make_int2(node, tb | parts);
+    };
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n; i0 += step) {
+        const int64_t i = i0 + lane;
+        const int64_t c = i < n ? flags[i] : 0;
+        const int64_t at = i < n ? pos[i] : 0;
+        const int tc = i < n ? tcount[i] : 0;
+        if (c <= 4)
+            for (int64_t k = 0; k < c; ++k) out[at + k] = item((int)i, tc, k);
+        for (unsigned big = __ballot_sync(FULL, c > 4); big; big &= big - 1) {
+            const int l = __ffs(big) - 1;
+            const int64_t cl = __shfl_sync(FULL, c, l), al = __shfl_sync(FULL, at, l);
+            const int tl = __shfl_sync(FULL, tc, l);
+            for (int64_t k = lane; k < cl; k += 32) out[al + k] = item((int)(i0 + l), tl, k);
+        }
+    }
 }
 
 inline unsigned grid_for(int64_t n, int threads = 256)
@@ -350,6 +392,38 @@ cudaError_t tree_target_ranges(sfmm_plan_s* P, const uint64_t* tkeys, int64_t M)
                                                          P->n_prefix.as<uint64_t>(), P->n_level.as<int>(), tkeys, M,
                                                          P->n_tfirst.as<int>(), P->n_tcount.as<int>()); count_launch();
     return cudaGetLastError();
+}
+
+// The evaluation's work items (plan->items, plan->n_items).  Chunks are split in
+// two, at the price of staging a leaf's sources twice, when M targets make fewer
+// full chunks than the GPU holds warps (152 SMs x 28) and most chunks are full
+// (32 targets or more per node): 49,152 grid points over 447 leaves.  Where the
+// leaves hold about m targets each the halves only add staging (1e5 points at
+// their own places: 1.80 ms whole, 1.84 ms split).  Graph mode: the count
+// goes to DevCounts::n_items, plan->n_items is the capacity.
+cudaError_t collect_items(sfmm_plan_s* P, int64_t M)
+{
+    cudaError_t e;
+    const int64_t nn = P->n_nodes;
+    cudaStream_t s = P->stream;
+    const int split = M < 152 * 28 * (int64_t)ITEM_CHUNK && M >= 32 * nn;
+    const int64_t cap = nn + M / (split ? 32 : 64) + 1;       // sum of ceilings over the leaves
+    if ((e = ensure(P->flags, (size_t)nn * 8)) || (e = ensure(P->pos, (size_t)nn * 8)) ||
+        (e = ensure(P->tmp, scan_tmp_bytes(nn))) || (e = ensure(P->items, (size_t)cap * 8)))
+        return e;
+    DevCounts* dc = P->gm ? P->dcnt.as<DevCounts>() : nullptr;
+    k_item_counts<<<grid_for(nn), 256, 0, s>>>((int)nn, dc ? &dc->nn : nullptr, P->n_child0.as<int>(),
+                                               P->n_tcount.as<int>(), split, P->flags.as<int64_t>()); count_launch();
+    int64_t* total = dc ? &dc->n_items : P->small.as<int64_t>() + 1;
+    if ((e = exclusive_scan_i64(P->flags.as<int64_t>(), P->pos.as<int64_t>(), nn, total, P->tmp.p, s))) return e;
+    k_items<<<grid_for(nn), 256, 0, s>>>((int)nn, P->flags.as<int64_t>(), P->pos.as<int64_t>(), P->n_tcount.as<int>(),
+                                         split, P->items.as<int2>()); count_launch();
+    if (dc) {
+        P->n_items = cap;
+        return cudaGetLastError();
+    }
+    if ((e = cudaMemcpyAsync(&P->n_items, total, 8, cudaMemcpyDeviceToHost, s))) return e;
+    return cudaStreamSynchronize(s);
 }
 
 // Indices of the leaves whose `cnt` (source or target count) is positive.  Graph
