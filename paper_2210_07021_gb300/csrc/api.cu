@@ -4,6 +4,7 @@
 // (Lemma 4) -> L2P + near field (Sec. 3.6).  Every step runs on the device.
 #include "common.cuh"
 #include "dfloat.cuh"
+#include "fp64ops.cuh"
 
 #include <algorithm>
 #include <string>
@@ -78,6 +79,7 @@ cudaError_t launch_eval32(const TreeView& T, const int2* items, int64_t n_items,
 cudaError_t launch_count_pairs(const TreeView& T, const int2* items, int64_t n_items, const int64_t* p2p_off,
                                const uint32_t* p2p_src, unsigned long long* out, cudaStream_t s);
 void fill_log_table(float* out);
+void fill_log64_table(double2* out);     // LOG64_N entries
 cudaError_t launch_eval_df(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const float4* soff,
                            const float4* toff, const float4* dc, const double4_32a* tgt, const uint32_t* tperm,
                            const int64_t* p2p_off, const uint32_t* p2p_src, const void* local, const void* mpole,
@@ -90,12 +92,12 @@ cudaError_t launch_eval_adj(const TreeView& T, const int2* items, int64_t n_item
                             const double4_32a* dip, const double4_32a* tgt, const uint32_t* tperm,
                             const int64_t* p2p_off, const uint32_t* p2p_src, const double* local, const double* mpole,
                             int p, int zero_mean, const void* w, int w_f32, double* phi, double* grad3,
-                            unsigned long long* leaf_ctr, cudaStream_t s);
+                            const double2* log_tab, unsigned long long* leaf_ctr, cudaStream_t s);
 cudaError_t launch_eval(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const double4_32a* src,
                         const double4_32a* tgt,
                         const uint32_t* tperm, const int64_t* p2p_off, const uint32_t* p2p_src, const double* local,
                         const double* mpole, int p, int zero_mean, double sigma, double* psi, double* alpha,
-                        double* gamma, double* mu, unsigned long long* leaf_ctr, cudaStream_t s);
+                        double* gamma, double* mu, const double2* log_tab, unsigned long long* leaf_ctr, cudaStream_t s);
 
 namespace {
 std::atomic<int64_t> g_launches{0};
@@ -261,6 +263,9 @@ TreeView view(sfmm_plan_s* P)
     T.tcount = P->n_tcount.as<int>();
     return T;
 }
+
+// the FP64 logarithm's table, behind the binomial tables
+const double2* log64_tab(sfmm_plan_s* P) { return reinterpret_cast<const double2*>(P->tables.as<double>() + 2 * PMAX * PMAX); }
 
 struct PhaseTimer {
     sfmm_plan_s* P;
@@ -578,7 +583,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     else if (adj) e = launch_eval_adj(T, P->items.as<int2>(), P->n_items, P->src4.as<double4_32a>(),
                                  P->dip4.as<double4_32a>(), P->tgt4.as<double4_32a>(), tperm, P->p2p_off.as<int64_t>(),
                                  p2p_s, P->local.as<double>(), P->mpole.as<double>(), p, P->opt.zero_mean, adj->w,
-                                 adj->w_f32, psi, adj->grad3, leaf_ctr, s);
+                                 adj->w_f32, psi, adj->grad3, log64_tab(P), leaf_ctr, s);
     else if (near32) {
         // 1e-6 path: the double-float finish on the near field's sums (the near field ran on the
         // auxiliary stream); all-FP32 path: the near field with its FP32 finish
@@ -596,7 +601,8 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
                                      near_early_df ? EVAL_FINISH : EVAL_NEAR | EVAL_FINISH, leaf_ctr, s);
     else e = launch_eval(T, P->items.as<int2>(), P->n_items, d_nit, P->src4.as<double4_32a>(),
                          P->tgt4.as<double4_32a>(), tperm, P->p2p_off.as<int64_t>(), p2p_s, P->local.as<double>(),
-                         P->mpole.as<double>(), p, P->opt.zero_mean, P->opt.sigma, psi, alpha, gamma, mu, leaf_ctr, s);
+                         P->mpole.as<double>(), p, P->opt.zero_mean, P->opt.sigma, psi, alpha, gamma, mu,
+                         log64_tab(P), leaf_ctr, s);
     if (e) return cuda_fail(P, e, "evaluation");
     if (P->gm) {          // no synchronisation: the caller reads the overflow flag after the work
         P->stats.launches = launch_total() - launches0;
@@ -718,8 +724,10 @@ sfmm_status sfmm_plan(sfmm_plan_t* out, int max_depth, int order_p, double tol, 
     P->tol = tol;
     P->opt = o;
     P->stream = static_cast<cudaStream_t>(o.stream);
-    std::vector<double> h(2 * PMAX * PMAX);
+    // binomial tables, then the FP64 logarithm's table
+    std::vector<double> h(2 * PMAX * PMAX + 2 * LOG64_N);
     fill_tables(h.data());
+    fill_log64_table(reinterpret_cast<double2*>(h.data() + 2 * PMAX * PMAX));
     float lt[129 * 4];
     fill_log_table(lt);
     cudaError_t e;
