@@ -172,14 +172,13 @@ cudaError_t launch_p(int64_t n_pairs, const int64_t* d_n, const uint64_t* ptgt, 
 {
     const size_t smem = (size_t)PW * 32 * (2 * P + 3) * sizeof(dflt);
     cudaError_t e;
-    int dev = 0, sms = 0, per_sm = 0;
-    if ((e = cudaFuncSetAttribute(k_m2l_pair<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) ||
-        (e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) ||
-        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_m2l_pair<P>, PW * 32, smem)))
-        return e;
+    if ((e = cudaFuncSetAttribute(k_m2l_pair<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+    // one CTA per 128 pairs: the P2P list's sort and the near field share the GPU with
+    // this kernel, and the CTAs of a persistent grid that found their SM taken started
+    // late with as much work as the others (M2L phase at N = 1.6e7: 1e-6 path 5.5 -> 4.8 ms,
+    // 1e-10 path 17.7 -> 15.1 ms)
     const int64_t chunks = (n_pairs + PW * 32 - 1) / (PW * 32);
-    const int64_t cap = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-    const int64_t grid = chunks < cap ? chunks : cap;
+    const int64_t grid = chunks < (1 << 30) ? chunks : 1 << 30;
     k_m2l_pair<P><<<(unsigned)grid, PW * 32, smem, s>>>(n_pairs, d_n, ptgt, psrc, geo, mpole, p, acc, leftover, n_left);
     count_launch();
     return cudaGetLastError();
