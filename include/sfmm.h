@@ -92,7 +92,9 @@ typedef struct {
                               potential; far pairs also need d - R_T - R_S > sigma.  SFMM_FP64 only. */
     int wait_limit;        /* polls after which a bounded device wait (the tensor-core M2L's mbarrier waits)
                               gives up, returning SFMM_ETIMEOUT with the device context intact; 0 (default) =
-                              2^26.  A test hook: a small value makes the time-out path run. */
+                              2^26.  The radix sort's waits take the same limit (default 2^20) but need no
+                              error: a tile that gives up counts the keys before it, with the same result.
+                              A test hook: a small value makes these paths run. */
 } sfmm_options;
 
 /* Fill *opt with the defaults listed above.  Returns SFMM_EINVAL if opt is NULL. */

@@ -369,7 +369,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         return cuda_fail(P, e, "fork");
     if ((e = launch_keys(tgt, M, P->tkeys.as<uint64_t>(), P->tperm.as<uint32_t>(), s2))) return cuda_fail(P, e, "tkeys");
     if ((e = radix_sort(P->tkeys.as<uint64_t>(), P->tperm.as<uint32_t>(), P->tkeys2.as<uint64_t>(),
-                        P->tperm2.as<uint32_t>(), M, 62, P->ttmp.p, s2, &P->tkeys_alt)))
+                        P->tperm2.as<uint32_t>(), M, 62, P->ttmp.p, s2, &P->tkeys_alt, P->opt.wait_limit)))
         return cuda_fail(P, e, "sort targets");
     const uint64_t* tkeys = P->tkeys_alt ? P->tkeys2.as<uint64_t>() : P->tkeys.as<uint64_t>();
     const uint32_t* tperm = P->tkeys_alt ? P->tperm2.as<uint32_t>() : P->tperm.as<uint32_t>();
@@ -377,7 +377,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     if ((e = cudaGetLastError()) || (e = cudaEventRecord(P->ev_join, s2))) return cuda_fail(P, e, "gather targets");
     if ((e = launch_keys(src, N, P->skeys.as<uint64_t>(), P->sperm.as<uint32_t>(), s))) return cuda_fail(P, e, "keys");
     if ((e = radix_sort(P->skeys.as<uint64_t>(), P->sperm.as<uint32_t>(), P->skeys2.as<uint64_t>(),
-                        P->sperm2.as<uint32_t>(), N, 62, P->tmp.p, s, &P->skeys_alt)))
+                        P->sperm2.as<uint32_t>(), N, 62, P->tmp.p, s, &P->skeys_alt, P->opt.wait_limit)))
         return cuda_fail(P, e, "sort sources");
     const uint64_t* skeys = P->skeys_alt ? P->skeys2.as<uint64_t>() : P->skeys.as<uint64_t>();
     const uint32_t* sperm = P->skeys_alt ? P->sperm2.as<uint32_t>() : P->sperm.as<uint32_t>();

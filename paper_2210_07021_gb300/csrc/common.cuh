@@ -48,14 +48,15 @@ void release(Buf& b);
 // bytes; if `total` is non-null the sum of all n inputs is written there.
 size_t scan_tmp_bytes(int64_t n);
 cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* total, void* tmp, cudaStream_t s);
-cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total, void* tmp, cudaStream_t s);
 
 // ------------------------------------------------------------- radix sort
 // Stable LSD radix sort of (key, value) by the low `bits` bits of the key.
 // The sorted data ends in (k1, v1) if *in_alt is false, else in (k2, v2).
+// wait_limit: polls after which a tile's bounded wait gives up and the tile counts
+// the keys before it itself (same result, slower); 0 = the default.
 size_t radix_tmp_bytes(int64_t n);
 cudaError_t radix_sort(uint64_t* k1, uint32_t* v1, uint64_t* k2, uint32_t* v2, int64_t n, int bits,
-                       void* tmp, cudaStream_t s, bool* in_alt);
+                       void* tmp, cudaStream_t s, bool* in_alt, int wait_limit = 0);
 
 // ------------------------------------------------------------------- keys
 cudaError_t launch_keys(const double* xyz, int64_t n, uint64_t* keys, uint32_t* iota, cudaStream_t s);

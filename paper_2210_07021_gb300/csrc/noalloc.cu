@@ -5,8 +5,8 @@
 // affordable -- for instance a plugin inside a host application whose memory
 // pool owns the whole device, or a latency-critical pipeline that cannot accept
 // the device-wide synchronisation cudaMalloc/cudaFree may cause.  Such callers
-// provide the outputs; all scratch memory (the sort's ping-pong buffers, the
-// per-tile digit histograms and the scan's block sums) lives in one file-scope
+// provide the outputs; all scratch memory (the sort's ping-pong buffers, its
+// digit counts and its tiles' published counts) lives in one file-scope
 // static device array of fixed size that every GPU loading this library holds
 // until the process exits.
 //
@@ -15,9 +15,9 @@
 // device address is looked up once with cudaGetSymbolAddress and cached.  That
 // first call should therefore come before any stream capture.
 //
-// Every call shares the one array.  Nothing in it has to start at zero: each
-// radix pass writes the histogram, the offsets and the ping-pong buffers in
-// full before reading them.  Calls that overlap on the GPU (for example on two
+// Every call shares the one array.  Nothing in it has to start at zero: the
+// sort zeroes its counts and words, and each radix pass writes the ping-pong
+// buffers in full before they are read.  Calls that overlap on the GPU (for example on two
 // streams at once) race on the array and must be serialised by the caller.
 #include "common.cuh"
 
@@ -33,7 +33,7 @@ namespace {
 constexpr int64_t STATIC_MAX_N = int64_t(1) << 18;                 // 262,144 points
 constexpr size_t ALT_KEY_BYTES = size_t(STATIC_MAX_N) * 8;         // 2 MiB
 constexpr size_t ALT_PERM_BYTES = size_t(STATIC_MAX_N) * 4;        // 1 MiB
-constexpr size_t SORT_TMP_BYTES = size_t(1) << 19;                 // 512 KiB (histograms + scan sums)
+constexpr size_t SORT_TMP_BYTES = size_t(1) << 19;                 // 512 KiB (digit counts, tiles' words)
 constexpr size_t SCRATCH_BYTES = ALT_KEY_BYTES + ALT_PERM_BYTES + SORT_TMP_BYTES;
 
 static __device__ __align__(256) unsigned char g_static_scratch[SCRATCH_BYTES];

@@ -2,11 +2,19 @@
 //
 // Scan: reduce-then-scan in three launches (per-tile sums, a single-CTA scan of
 // the tile sums, per-tile scans with the tile offset added).
-// Sort: 8-bit digits; per pass one histogram launch (per tile of 4096 keys),
-// one scan of the digit-major histogram, and one scatter launch that ranks the
-// keys of each tile stably (warp match-any, per-warp digit counters), reorders
-// the tile by digit in shared memory and writes runs of equal digits.
+// Sort: 8-bit digits.  One launch counts the digits of every pass (the counts do
+// not depend on the order); each pass is then one launch in which a tile of
+// 1024 to 4096 keys ranks its keys stably (warp ballots, per-warp digit counters),
+// finds where its runs start by looking back over the tiles before it (each
+// publishes its digit counts, then their running totals), reorders itself by
+// digit in shared memory and writes runs of equal digits.  That is 2 + passes
+// launches; a histogram, a three-launch scan and a scatter per pass, latency-bound
+// at these sizes, took 5 per pass (62-bit keys: 4096 230 -> 60 us, 262,144 255 -> 109,
+// 1e6 285 -> 171).  Large sorts (RS_LARGE) count per tile and pass instead, in
+// three launches per pass (3.1e6 keys 433 -> 375 us; 1.6e7 1385 -> 1373).
 #include "common.cuh"
+
+#include <algorithm>
 
 namespace sfmm {
 
@@ -117,43 +125,164 @@ cudaError_t exclusive_scan_t(const T* in, T* out, int64_t n, T* total, void* tmp
 }
 
 // ---------------------------------------------------------------- radix sort
-// Tiles of RS_TILE = 4096 keys, 256 threads, 16 keys per thread.  Warp w owns
-// keys [512 w, 512 w + 512) of its tile, loaded in 16 coalesced rounds of 32.
-constexpr int RS_T = 256, RS_I = 16, RS_TILE = RS_T * RS_I, RS_W = RS_T / 32;
+// A tile is T threads x I keys; warp w owns keys [32 I w, 32 I (w + 1)) of it, loaded
+// in I coalesced rounds of 32.
+constexpr size_t RS_HEAD = 8 * 256 * 4 + 256;     // digit counts and tile counters in front of the tiles' words
+constexpr int LOOK = 4;                           // tiles whose words a look-back reads at once
+constexpr int RS_POLLS = 1 << 20;                 // polls of a look-back that found nothing new (each about 1 us)
+// Sizes at which the tile and the way to the runs' starts change (62-bit keys, us per
+// sort with the neighbouring choices): keys per thread 4 below 150,000 (4096 keys:
+// 58, with 8: 76, with 16: 93; 1e5: 93 / 93 / 122), 8 below 500,000 (262,144: 109,
+// with 16: 126), 16 above (1e6: 171, with 8: 230).  From RS_LARGE on the tiles in
+// flight are many enough that their look-backs hold one another up, and counting
+// launches take over (counting / look-back: 1.5e6 262 / 228, 2e6 295 / 300, 3.1e6
+// 375 / 420, 1.6e7 1373 / 1388).
+constexpr int64_t RS_SMALL = 150000, RS_MIDDLE = 500000, RS_LARGE = 2000000;
 constexpr int RS_WC = 257;                        // per-warp digit counters (+1 slot for keys past n)
+constexpr int RS_HT = 256;                        // threads of the counting kernel
 // the tile's keys, then its values, reordered through one 8-byte-per-key buffer,
 // plus the digit of every reordered slot
-constexpr size_t RS_SMEM = (size_t)RS_TILE * 9 + (size_t)RS_W * RS_WC * 4 + 3 * 256 * 4 + 64;
+constexpr size_t rs_smem_bytes(int T, int I) { return (size_t)T * I * 9 + (size_t)(T / 32) * RS_WC * 4 + 2 * 256 * 4 + 64; }
 
-__global__ void __launch_bounds__(RS_T) k_rs_hist(const uint64_t* __restrict__ keys, int64_t n, int shift,
-                                                 uint32_t* __restrict__ hist, int64_t ntiles)
+// A tile's published word per digit (sorts below RS_LARGE keys): its own count of
+// the digit, or the count of all keys up to and including the tile, with the flag
+// in the top two bits.  One store carries both, so no fence orders them; zero
+// means not published yet.
+constexpr uint32_t RS_OWN = 1u << 30, RS_UPTO = 2u << 30, RS_COUNT = RS_OWN - 1;
+static_assert(RS_LARGE < (int64_t)RS_COUNT, "counts and flags share a word");
+__device__ __forceinline__ uint32_t ld_word(const uint32_t* p) { return *reinterpret_cast<const volatile uint32_t*>(p); }
+__device__ __forceinline__ void st_word(uint32_t* p, uint32_t v) { *reinterpret_cast<volatile uint32_t*>(p) = v; }
+
+// the digit counts of every pass: hist[pass][digit], zero at launch
+__global__ void __launch_bounds__(RS_HT) k_rs_hist(const uint64_t* __restrict__ keys, int64_t n, int passes,
+                                                  uint32_t* __restrict__ hist)
+{
+    __shared__ uint32_t cnt[8][256];
+    for (int i = threadIdx.x; i < 8 * 256; i += RS_HT) (&cnt[0][0])[i] = 0;
+    __syncthreads();
+    for (int64_t e = (int64_t)blockIdx.x * RS_HT + threadIdx.x; e < n; e += (int64_t)gridDim.x * RS_HT) {
+        const uint64_t k = keys[e];
+        for (int p = 0; p < passes; ++p) atomicAdd(&cnt[p][(k >> (8 * p)) & 255u], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < passes * 256; i += RS_HT)
+        if (const uint32_t c = (&cnt[0][0])[i]) atomicAdd(hist + i, c);
+}
+
+// exclusive prefix sum of one value per thread over the block's 256 threads
+__device__ __forceinline__ uint32_t block_excl256(uint32_t v, uint32_t* s_warp, int lane, int warp)
+{
+    const uint32_t inc = warp_incl_scan(v, lane);
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    uint32_t before = 0;
+#pragma unroll
+    for (int w = 0; w < 7; ++w) before += w < warp ? s_warp[w] : 0u;
+    __syncthreads();
+    return before + inc - v;
+}
+
+// The keys of one digit in all tiles before `tile`, by looking back: LOOK tiles'
+// words are read at once and added up until one holds a running total.  Tiles
+// take their numbers in the order they start, so every word waited for belongs
+// to a tile that is running or done; the wait is bounded all the same, and false
+// is returned when `limit` polls found nothing (the caller then counts the keys
+// itself).
+__device__ __forceinline__ bool look_back(const uint32_t* __restrict__ words, int64_t tile, int digit, int limit,
+                                          uint32_t* before)
+{
+    uint32_t sum = 0;
+    int polls = 0;
+    for (int64_t t = tile - 1; t >= 0;) {
+        uint32_t w[LOOK];
+#pragma unroll
+        for (int i = 0; i < LOOK; ++i) w[i] = ld_word(words + (t - i < 0 ? 0 : t - i) * 256 + digit);
+        int used = 0;
+        bool go = true, done = false;
+#pragma unroll
+        for (int i = 0; i < LOOK; ++i) {
+            go = go && !done && t - i >= 0 && w[i] != 0;
+            if (go) {
+                sum += w[i] & RS_COUNT;
+                done = (w[i] & RS_UPTO) != 0;
+                used = i + 1;
+            }
+        }
+        if (done) break;
+        if (used == 0 && ++polls >= limit) return false;
+        t -= used;
+    }
+    *before = sum;
+    return true;
+}
+
+// Sorts of RS_LARGE keys and more, per pass: the tiles' digit counts,
+// counts[digit][tile], then one block per digit turns its row into exclusive
+// sums over the tiles and writes the digit's total.
+template <int T, int I>
+__global__ void __launch_bounds__(T) k_rs_tile_counts(const uint64_t* __restrict__ keys, int64_t n, int shift,
+                                                      uint32_t* __restrict__ counts, int64_t ntiles)
 {
     __shared__ uint32_t cnt[256];
-    cnt[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < 256; i += T) cnt[i] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    for (int r = 0; r < RS_I; ++r) {
-        int64_t e = base + (int64_t)r * RS_T + threadIdx.x;
+    const int64_t base = (int64_t)blockIdx.x * (T * I);
+#pragma unroll
+    for (int r = 0; r < I; ++r) {
+        const int64_t e = base + (int64_t)r * T + threadIdx.x;
         if (e < n) atomicAdd(&cnt[(keys[e] >> shift) & 255u], 1u);
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
+    for (int i = threadIdx.x; i < 256; i += T) counts[(int64_t)i * ntiles + blockIdx.x] = cnt[i];
+}
+
+__global__ void __launch_bounds__(SC_T) k_rs_rows(uint32_t* __restrict__ counts, int64_t ntiles,
+                                                  uint32_t* __restrict__ totals)
+{
+    __shared__ uint32_t s_warp[SC_T / 32];
+    __shared__ uint32_t s_total;
+    uint32_t* row = counts + (int64_t)blockIdx.x * ntiles;
+    uint32_t carry = 0;
+    for (int64_t c = 0; c < ntiles; c += SC_TILE) {
+        uint32_t v[SC_I], acc = 0;
+        const int64_t e0 = c + (int64_t)threadIdx.x * SC_I;
+#pragma unroll
+        for (int i = 0; i < SC_I; ++i) v[i] = e0 + i < ntiles ? row[e0 + i] : 0u;
+#pragma unroll
+        for (int i = 0; i < SC_I; ++i) { const uint32_t x = v[i]; v[i] = acc; acc += x; }
+        const uint32_t ex = block_excl_scan(acc, s_warp, &s_total) + carry;
+#pragma unroll
+        for (int i = 0; i < SC_I; ++i)
+            if (e0 + i < ntiles) row[e0 + i] = v[i] + ex;
+        carry += s_total;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
 }
 
 // One tile: stable rank of every key among the tile's keys of its digit
 // (warp-private counters advanced round by round; within a round the lanes of
 // equal digit are found with eight ballots, one per digit bit), counts turned
-// into per-warp offsets by a scan over (digit, warp), then the tile's keys and
-// afterwards its values reordered by digit through one shared buffer and
-// written out as runs per digit at the tile's global digit offsets (the
-// scanned histogram).  Only the digits (packed four to a register) and the
+// into per-warp offsets by a scan over (digit, warp), the start of each digit's
+// run from the look-back, then the tile's keys and afterwards its values
+// reordered by digit through one shared buffer and written out as runs per
+// digit.  Only the digits (packed four to a register) and the
 // ranks stay in registers between the phases; keys and values are read again
 // (from L2) when they are reordered, which keeps four CTAs on an SM.
-__global__ void __launch_bounds__(RS_T, 4) k_rs_scatter(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
+// words: this pass's published words (zero at launch), words_next: the next
+// pass's, zeroed here tile by tile; ticket: this pass's tile counter (zero).
+// LOOKB: the runs' starts by looking back (words, words_next, ticket, limit); else
+// from the tiles' counts (words: their exclusive sums per digit row, limit: the
+// tiles).  hist: the digits' totals in either case.
+template <int RS_T, int RS_I, int CTAS, bool LOOKB>
+__global__ void __launch_bounds__(RS_T, CTAS) k_rs_pass(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
                                                     uint64_t* __restrict__ kout, uint32_t* __restrict__ vout,
-                                                    int64_t n, int shift, const uint32_t* __restrict__ offs,
-                                                    int64_t ntiles)
+                                                    int64_t n, int shift, const uint32_t* __restrict__ hist,
+                                                    uint32_t* __restrict__ words, uint32_t* __restrict__ words_next,
+                                                    uint32_t* __restrict__ ticket, int limit)
 {
+    static_assert(RS_T == 256, "one thread per digit");
+    constexpr int RS_TILE = RS_T * RS_I, RS_W = RS_T / 32;
     extern __shared__ __align__(16) unsigned char rs_smem[];
     uint64_t* sk = reinterpret_cast<uint64_t*>(rs_smem);
     uint32_t* sv = reinterpret_cast<uint32_t*>(rs_smem);   // the same bytes, once the keys are out
@@ -163,7 +292,17 @@ __global__ void __launch_bounds__(RS_T, 4) k_rs_scatter(const uint64_t* __restri
     uint32_t* s_warp = gbase + 256;                       // scan scratch
     uint8_t* sdig = reinterpret_cast<uint8_t*>(s_warp + 16);   // digit of each reordered slot
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t tile0 = (int64_t)blockIdx.x * RS_TILE;
+    __shared__ uint32_t s_tile;
+    __shared__ int s_lost;
+    if (LOOKB) {
+        if (tid == 0) {
+            s_tile = atomicAdd(ticket, 1u);
+            s_lost = 0;
+        }
+        __syncthreads();
+    }
+    const uint32_t tile = LOOKB ? s_tile : blockIdx.x;
+    const int64_t tile0 = (int64_t)tile * RS_TILE;
     const int64_t w0 = tile0 + (int64_t)warp * (32 * RS_I);
     uint32_t dig[RS_I / 4];                               // digits, four to a register
     uint32_t loc[RS_I / 2];                               // slots (< 2^13), two to a register
@@ -178,7 +317,20 @@ __global__ void __launch_bounds__(RS_T, 4) k_rs_scatter(const uint64_t* __restri
         dig[r >> 2] |= d << (8 * (r & 3));
     }
     for (int d = lane; d < RS_WC; d += 32) wc[warp * RS_WC + d] = 0;
-    gbase[tid] = offs[(int64_t)tid * ntiles + blockIdx.x];
+    uint32_t* mine = words + (size_t)tile * 256 + tid;    // thread tid owns digit tid
+    if (LOOKB) {
+        // the tile's digit counts, published before the ranking so that later tiles find them
+        words_next[(size_t)tile * 256 + tid] = 0;
+        gbase[tid] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < RS_I; ++r)
+            if (w0 + r * 32 + lane < n) atomicAdd(&gbase[(dig[r >> 2] >> (8 * (r & 3))) & 255u], 1u);
+        __syncthreads();
+        if (tile > 0) st_word(mine, RS_OWN | gbase[tid]);
+    } else {
+        gbase[tid] = words[(size_t)tid * (unsigned)limit + (unsigned)tile];
+    }
     __syncwarp();
     const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
@@ -209,26 +361,24 @@ __global__ void __launch_bounds__(RS_T, 4) k_rs_scatter(const uint64_t* __restri
         wc[w * RS_WC + tid] = tot;
         tot += c;
     }
-    uint32_t inc = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(FULL, inc, o);
-        if (lane >= o) inc += t;
-    }
-    if (lane == 31) s_warp[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-        const uint32_t wv = lane < RS_W ? s_warp[lane] : 0u;
-        uint32_t wi = wv;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(FULL, wi, o);
-            if (lane >= o) wi += t;
+    tbase[tid] = block_excl256(tot, s_warp, lane, warp);
+    const uint32_t run0 = block_excl256(hist[tid], s_warp, lane, warp);     // the digit's first place
+    if (LOOKB) {
+        uint32_t before = 0;
+        if (!look_back(words, tile, tid, limit, &before)) s_lost = 1;
+        __syncthreads();
+        if (s_lost) {       // a wait ran out: count the keys before this tile directly
+            gbase[tid] = 0;
+            __syncthreads();
+            for (int64_t e = tid; e < tile0; e += RS_T) atomicAdd(&gbase[(kin[e] >> shift) & 255u], 1u);
+            __syncthreads();
+            before = gbase[tid];
         }
-        if (lane < RS_W) s_warp[lane] = wi - wv;
+        st_word(mine, RS_UPTO | (before + tot));
+        gbase[tid] = run0 + before;
+    } else {
+        gbase[tid] += run0;
     }
-    __syncthreads();
-    tbase[tid] = inc - tot + s_warp[warp];
     __syncthreads();
     // keys to their places in the tile's digit order (read again, from L2)
 #pragma unroll
@@ -262,6 +412,8 @@ __global__ void __launch_bounds__(RS_T, 4) k_rs_scatter(const uint64_t* __restri
     }
 }
 
+inline int64_t rs_tile(int64_t n) { return n <= RS_SMALL ? 256 * 4 : n <= RS_MIDDLE ? 256 * 8 : 256 * 16; }
+
 }  // namespace
 
 size_t scan_tmp_bytes(int64_t n)
@@ -275,46 +427,74 @@ cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64
     return exclusive_scan_t<int64_t>(in, out, n, total, tmp, s);
 }
 
-cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total, void* tmp, cudaStream_t s)
-{
-    return exclusive_scan_t<uint32_t>(in, out, n, total, tmp, s);
-}
-
+// the digit counts of 8 passes and the tile counters, then the tiles' words of even
+// and of odd passes (counting sorts use the first half); never decreasing in n (a
+// buffer sized for n serves every smaller sort)
 size_t radix_tmp_bytes(int64_t n)
 {
-    const int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
-    const int64_t nh = 256 * ntiles;
-    // histogram + scanned histogram + scan scratch
-    return (size_t)(2 * nh) * sizeof(uint32_t) + scan_tmp_bytes(nh) + 512;
+    auto need = [](int64_t m) {
+        const int64_t ntiles = (m + rs_tile(m) - 1) / rs_tile(m);
+        return RS_HEAD + (size_t)(2 * ntiles) * 256 * sizeof(uint32_t) + 512;
+    };
+    size_t b = need(n);
+    if (n > RS_SMALL) b = std::max(b, need(RS_SMALL));
+    if (n > RS_MIDDLE) b = std::max(b, need(RS_MIDDLE));
+    return b;
 }
 
-cudaError_t radix_sort(uint64_t* k1, uint32_t* v1, uint64_t* k2, uint32_t* v2, int64_t n, int bits,
-                       void* tmp, cudaStream_t s, bool* in_alt)
+namespace {
+
+template <int I, bool LOOKB>
+cudaError_t radix_sort_t(uint64_t* k1, uint32_t* v1, uint64_t* k2, uint32_t* v2, int64_t n, int bits, void* tmp,
+                         cudaStream_t s, bool* in_alt, int limit)
 {
-    *in_alt = false;
-    if (n <= 1 || bits <= 0) return cudaSuccess;
-    const int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
-    const int64_t nh = 256 * ntiles;
-    uint32_t* hist = static_cast<uint32_t*>(tmp);
-    uint32_t* offs = hist + nh;
-    void* stmp = reinterpret_cast<char*>(tmp) + (size_t)(2 * nh) * sizeof(uint32_t);
-    stmp = reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(stmp) + 255) & ~uintptr_t(255));
+    constexpr int T = 256;
+    const int64_t ntiles = (n + T * I - 1) / (T * I);
+    const int passes = (bits + 7) / 8;
+    constexpr size_t smem = rs_smem_bytes(T, I);
+    uint32_t* hist = reinterpret_cast<uint32_t*>((reinterpret_cast<uintptr_t>(tmp) + 255) & ~uintptr_t(255));
+    uint32_t* tickets = hist + 8 * 256;
+    uint32_t* words[2];
+    words[0] = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(hist) + RS_HEAD);
+    words[1] = words[0] + ntiles * 256;
     uint64_t *ka = k1, *kb = k2;
     uint32_t *va = v1, *vb = v2;
     bool alt = false;
-    cudaError_t e = cudaFuncSetAttribute(k_rs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SMEM);
-    if (e != cudaSuccess) return e;
-    for (int shift = 0; shift < bits; shift += 8) {
-        k_rs_hist<<<(unsigned)ntiles, RS_T, 0, s>>>(ka, n, shift, hist, ntiles); count_launch();
-        e = exclusive_scan_u32(hist, offs, nh, nullptr, stmp, s);
-        if (e != cudaSuccess) return e;
-        k_rs_scatter<<<(unsigned)ntiles, RS_T, RS_SMEM, s>>>(ka, va, kb, vb, n, shift, offs, ntiles); count_launch();
+    cudaError_t e;
+    auto* pass = k_rs_pass<T, I, 4, LOOKB>;
+    if ((e = cudaFuncSetAttribute(pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+    if (LOOKB) {
+        if ((e = cudaMemsetAsync(hist, 0, RS_HEAD + (size_t)ntiles * 256 * sizeof(uint32_t), s))) return e;
+        const int64_t hb = (n + RS_HT * 8 - 1) / (RS_HT * 8);
+        k_rs_hist<<<(unsigned)(hb < 152 * 8 ? hb : 152 * 8), RS_HT, 0, s>>>(ka, n, passes, hist); count_launch();
+    }
+    for (int p = 0; p < passes; ++p) {
+        if constexpr (!LOOKB) {
+            k_rs_tile_counts<T, I><<<(unsigned)ntiles, T, 0, s>>>(ka, n, 8 * p, words[0], ntiles); count_launch();
+            k_rs_rows<<<256, SC_T, 0, s>>>(words[0], ntiles, hist + 256 * p); count_launch();
+        }
+        pass<<<(unsigned)ntiles, T, smem, s>>>(ka, va, kb, vb, n, 8 * p, hist + 256 * p, words[LOOKB ? p & 1 : 0],
+                                               words[(p + 1) & 1], tickets + p, LOOKB ? limit : (int)ntiles); count_launch();
         std::swap(ka, kb);
         std::swap(va, vb);
         alt = !alt;
     }
     *in_alt = alt;
     return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t radix_sort(uint64_t* k1, uint32_t* v1, uint64_t* k2, uint32_t* v2, int64_t n, int bits,
+                       void* tmp, cudaStream_t s, bool* in_alt, int wait_limit)
+{
+    *in_alt = false;
+    if (n <= 1 || bits <= 0) return cudaSuccess;
+    const int limit = wait_limit > 0 ? wait_limit : RS_POLLS;
+    if (n <= RS_SMALL) return radix_sort_t<4, true>(k1, v1, k2, v2, n, bits, tmp, s, in_alt, limit);
+    if (n <= RS_MIDDLE) return radix_sort_t<8, true>(k1, v1, k2, v2, n, bits, tmp, s, in_alt, limit);
+    if (n < RS_LARGE) return radix_sort_t<16, true>(k1, v1, k2, v2, n, bits, tmp, s, in_alt, limit);
+    return radix_sort_t<16, false>(k1, v1, k2, v2, n, bits, tmp, s, in_alt, limit);
 }
 
 }  // namespace sfmm

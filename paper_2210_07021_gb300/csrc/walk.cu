@@ -30,8 +30,6 @@
 
 namespace sfmm {
 
-cudaError_t radix_sort(uint64_t*, uint32_t*, uint64_t*, uint32_t*, int64_t, int, void*, cudaStream_t, bool*);
-
 namespace {
 
 // Radii within this relative difference count as equal, and then the target is
@@ -487,14 +485,14 @@ cudaError_t build_lists(sfmm_plan_s* P, const TreeView& T, double c_s, double c_
         return e;
     // the M2L list first: its event (plan->ev_m2l) lets M2L start while the P2P list is sorted
     if ((e = radix_sort(P->m2l_t.as<uint64_t>(), P->m2l_s.as<uint32_t>(), P->m2l_t2.as<uint64_t>(),
-                        P->m2l_s2.as<uint32_t>(), n_m2l, bits, P->tmp.p, s, &P->m2l_alt)))
+                        P->m2l_s2.as<uint32_t>(), n_m2l, bits, P->tmp.p, s, &P->m2l_alt, P->opt.wait_limit)))
         return e;
     const uint64_t* mt = P->m2l_alt ? P->m2l_t2.as<uint64_t>() : P->m2l_t.as<uint64_t>();
     k_csr_offsets<<<grid_for(P->n_nodes + 1), 256, 0, s>>>(mt, n_m2l, P->d_m2l, (int)P->n_nodes,
                                                            P->m2l_off.as<int64_t>()); count_launch();
     if ((e = cudaEventRecord(P->ev_m2l, s))) return e;
     if ((e = radix_sort(P->p2p_t.as<uint64_t>(), P->p2p_s.as<uint32_t>(), P->p2p_t2.as<uint64_t>(),
-                        P->p2p_s2.as<uint32_t>(), n_p2p, bits, P->tmp.p, s, &P->p2p_alt)))
+                        P->p2p_s2.as<uint32_t>(), n_p2p, bits, P->tmp.p, s, &P->p2p_alt, P->opt.wait_limit)))
         return e;
     const uint64_t* pt = P->p2p_alt ? P->p2p_t2.as<uint64_t>() : P->p2p_t.as<uint64_t>();
     k_csr_offsets<<<grid_for(P->n_nodes + 1), 256, 0, s>>>(pt, n_p2p, P->d_p2p, (int)P->n_nodes,
