@@ -21,8 +21,7 @@ namespace sfmm {
 cudaError_t build_tree(sfmm_plan_s* P, const uint64_t* keys, int64_t n, int m, int max_depth);
 cudaError_t tree_geometry(sfmm_plan_s* P);
 cudaError_t tree_target_ranges(sfmm_plan_s* P, const uint64_t* tkeys, int64_t M);
-cudaError_t collect_items(sfmm_plan_s* P, int64_t M);
-cudaError_t collect_leaves(sfmm_plan_s* P, const int* cnt, Buf& out, int64_t* n_out, int64_t* d_out);
+cudaError_t collect_leaves_items(sfmm_plan_s* P, int64_t M, int64_t* d_leaves, int64_t* d_items);
 cudaError_t build_lists(sfmm_plan_s* P, const TreeView& T, double c_s, double c_t, cudaStream_t s);
 void fill_tables(double* h);
 size_t xgeo_bytes(int ek);
@@ -76,7 +75,7 @@ cudaError_t launch_eval32(const TreeView& T, const int2* items, int64_t n_items,
                           const uint32_t* p2p_src, const void* local, const void* mpole, bool dfar, int p, int zero_mean,
                           double* psi, double* alpha, bool coincide, float4* nf, int* tleaf,
                           const void* frames, int64_t M, int what, unsigned long long* leaf_ctr, cudaStream_t s);
-cudaError_t launch_count_pairs(const TreeView& T, const int2* items, int64_t n_items, const int64_t* p2p_off,
+cudaError_t launch_count_pairs(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const int64_t* p2p_off,
                                const uint32_t* p2p_src, unsigned long long* out, cudaStream_t s);
 void fill_log_table(float* out);
 void fill_log64_table(double2* out);     // LOG64_N entries
@@ -86,9 +85,9 @@ cudaError_t launch_eval_df(const TreeView& T, const int2* items, int64_t n_items
                            const float4* log_tab, int p, int zero_mean, double* psi, double* alpha,
                            const float4* doff, const void* w, int w_f32, double* grad3, float4* nf, int* tleaf,
                            const void* frames, int64_t M, int what, unsigned long long* leaf_ctr, cudaStream_t s);
-cudaError_t launch_p2m_adj(const TreeView& T, const int* leaves, int64_t n_leaves, const double4_32a* src,
+cudaError_t launch_p2m_adj(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const double4_32a* src,
                            const double4_32a* dip, double* mpole, int p, cudaStream_t s);
-cudaError_t launch_eval_adj(const TreeView& T, const int2* items, int64_t n_items, const double4_32a* src,
+cudaError_t launch_eval_adj(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const double4_32a* src,
                             const double4_32a* dip, const double4_32a* tgt, const uint32_t* tperm,
                             const int64_t* p2p_off, const uint32_t* p2p_src, const double* local, const double* mpole,
                             int p, int zero_mean, const void* w, int w_f32, double* phi, double* grad3,
@@ -349,7 +348,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     PhaseTimer tm(P);
     tm.mark();
     // ---- keys and sort (sources and targets)
-    if ((e = ensure(P->small, 64 * 8))) return cuda_fail(P, e, "alloc");
+    if ((e = ensure(P->small, SM_SLOTS * 8))) return cuda_fail(P, e, "alloc");
     if ((e = ensure(P->skeys, N * 8)) || (e = ensure(P->skeys2, N * 8)) || (e = ensure(P->sperm, N * 4)) ||
         (e = ensure(P->sperm2, N * 4)) || (e = ensure(P->src4, N * 32)))
         return cuda_fail(P, e, "alloc sources");
@@ -396,16 +395,15 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     const int64_t nn = P->n_nodes;
     if ((e = tree_geometry(P))) return cuda_fail(P, e, "geometry");
     TreeView T = view(P);
-    if ((e = collect_leaves(P, T.count, P->leaves_src, &P->n_leaves, dcnt ? &dcnt->n_leaves : nullptr)))
-        return cuda_fail(P, e, "leaves");
-    const int64_t* d_nls = dcnt ? &dcnt->n_leaves : nullptr;
-    const int64_t* d_nit = dcnt ? &dcnt->n_items : nullptr;
+    // the counts of source leaves and evaluation items stay on the device
+    int64_t* d_nls = dcnt ? &dcnt->n_leaves : P->small.as<int64_t>() + SM_COLLECT;
+    int64_t* d_nit = dcnt ? &dcnt->n_items : P->small.as<int64_t>() + SM_COLLECT + 1;
     tm.mark();
     // ---- join the targets; target ranges (Sec. 3.7 lookup) and the evaluation's work items
     if ((e = cudaStreamWaitEvent(s, P->ev_join, 0))) return cuda_fail(P, e, "join");
     if ((e = tree_target_ranges(P, tkeys, M))) return cuda_fail(P, e, "target ranges");
     T = view(P);
-    if ((e = collect_items(P, M))) return cuda_fail(P, e, "evaluation items");
+    if ((e = collect_leaves_items(P, M, d_nls, d_nit))) return cuda_fail(P, e, "leaves");
     // ---- up-pass on the plan's stream while the lists (Algorithm 1) are built on
     // the auxiliary stream: neither needs the other's results, and the small
     // levels of the one leave room on the GPU for the other
@@ -442,7 +440,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
                                     P->soff.as<float4>(), s)))
             return cuda_fail(P, e, "offsets");
     }
-    if (adj && !adj_df) e = launch_p2m_adj(T, P->leaves_src.as<int>(), P->n_leaves, P->src4.as<double4_32a>(),
+    if (adj && !adj_df) e = launch_p2m_adj(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->src4.as<double4_32a>(),
                                            P->dip4.as<double4_32a>(), P->mpole.as<double>(), p, s);
     else if (dfe) e = launch_p2m_df_leaf(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->soff.as<float4>(),
                                          adj_df ? P->dip4.as<float4>() : nullptr, P->logtab.as<float4>(), p,
@@ -484,7 +482,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     }
     // 1e-6 and 1e-10 paths: the near field needs none of the far field (their double-float
     // finish does), so it runs here, on the auxiliary stream, beside M2L and L2L
-    unsigned long long* leaf_ctr = reinterpret_cast<unsigned long long*>(P->small.as<int64_t>() + 40);
+    unsigned long long* leaf_ctr = reinterpret_cast<unsigned long long*>(P->small.as<int64_t>() + SM_ITEM_CTR);
     const bool near_early = near32 && !fp32 && !adj;
     const bool near_early_df = dfe && !near32 && !adj;
     if (near_early_df) {
@@ -518,12 +516,12 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     const uint32_t* m2l_s = P->m2l_alt ? P->m2l_s2.as<uint32_t>() : P->m2l_s.as<uint32_t>();
     const uint64_t* m2l_t = P->m2l_alt ? P->m2l_t2.as<uint64_t>() : P->m2l_t.as<uint64_t>();
     if ((e = ensure(P->m2l_geo, (size_t)std::max<int64_t>(P->n_m2l, 1) * xgeo_bytes(ek)))) return cuda_fail(P, e, "alloc");
-    int* status = reinterpret_cast<int*>(P->small.as<int64_t>() + 20);
+    int* status = reinterpret_cast<int*>(P->small.as<int64_t>() + SM_STATUS);
     if (dfe) {
         // double-float M2L, one thread per pair, summed per target box in FP64
         // accumulators; pairs with centres near antipodes go to the warp kernel
         const size_t nacc = (size_t)nn * EXP_STRIDE;
-        uint32_t* n_left = reinterpret_cast<uint32_t*>(P->small.as<int64_t>() + 21);
+        uint32_t* n_left = reinterpret_cast<uint32_t*>(P->small.as<int64_t>() + SM_LEFT);
         if ((e = ensure(P->m2l_acc, nacc * 8)) || (e = ensure(P->leftover, (size_t)std::max<int64_t>(P->n_m2l, 1) * 4)))
             return cuda_fail(P, e, "alloc");
         if ((e = cudaMemsetAsync(P->m2l_acc.p, 0, nacc * 8, s)) || (e = cudaMemsetAsync(n_left, 0, 4, s)))
@@ -543,10 +541,10 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         return cuda_fail(P, e, "pair geometry");
     } else if (fp32 && P->opt.m2l_tensor_cores) {
         // tensor-core M2L; pairs it cannot take (centres near antipodes) go to a list for the warp kernel
-        uint32_t* n_left = reinterpret_cast<uint32_t*>(P->small.as<int64_t>() + 21);
+        uint32_t* n_left = reinterpret_cast<uint32_t*>(P->small.as<int64_t>() + SM_LEFT);
         uint32_t* tile_ctr = n_left + 1;              // zeroed by the same memset
         if ((e = ensure(P->leftover, (size_t)std::max<int64_t>(P->n_m2l, 1) * 4))) return cuda_fail(P, e, "alloc");
-        if ((e = cudaMemsetAsync(P->small.as<int64_t>() + 20, 0, 16, s))) return cuda_fail(P, e, "memset");
+        if ((e = cudaMemsetAsync(P->small.as<int64_t>() + SM_STATUS, 0, 16, s))) return cuda_fail(P, e, "memset");
         if ((e = launch_m2l_tc(P->n_m2l, m2l_t, m2l_s, P->m2l_geo.p, P->mpole.p, P->local.p, p, P->leftover.as<uint32_t>(),
                                n_left, tile_ctr, status, P->opt.wait_limit, s)))
             return cuda_fail(P, e, "M2L (tensor cores)");
@@ -580,7 +578,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
                                    P->p2p_off.as<int64_t>(), p2p_s, P->local.p, P->mpole.p, P->logtab.as<float4>(), p,
                                    P->opt.zero_mean, psi, nullptr, P->dip4.as<float4>(), adj->w, adj->w_f32,
                                    adj->grad3, nullptr, nullptr, nullptr, M, EVAL_NEAR | EVAL_FINISH, leaf_ctr, s);
-    else if (adj) e = launch_eval_adj(T, P->items.as<int2>(), P->n_items, P->src4.as<double4_32a>(),
+    else if (adj) e = launch_eval_adj(T, P->items.as<int2>(), P->n_items, d_nit, P->src4.as<double4_32a>(),
                                  P->dip4.as<double4_32a>(), P->tgt4.as<double4_32a>(), tperm, P->p2p_off.as<int64_t>(),
                                  p2p_s, P->local.as<double>(), P->mpole.as<double>(), p, P->opt.zero_mean, adj->w,
                                  adj->w_f32, psi, adj->grad3, log64_tab(P), leaf_ctr, s);
@@ -611,9 +609,9 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     tm.mark();
     if (P->timing >= 2) {
         // near-field source-target pairs (for the throughput of the evaluation kernel)
-        unsigned long long* cnt = reinterpret_cast<unsigned long long*>(P->small.as<int64_t>() + 16);
+        unsigned long long* cnt = reinterpret_cast<unsigned long long*>(P->small.as<int64_t>() + SM_PAIRS);
         if ((e = cudaMemsetAsync(cnt, 0, 8, s))) return cuda_fail(P, e, "memset");
-        if ((e = launch_count_pairs(T, P->items.as<int2>(), P->n_items, P->p2p_off.as<int64_t>(), p2p_s,
+        if ((e = launch_count_pairs(T, P->items.as<int2>(), P->n_items, d_nit, P->p2p_off.as<int64_t>(), p2p_s,
                                     cnt, s)))
             return cuda_fail(P, e, "count pairs");
         unsigned long long h = 0;
@@ -634,7 +632,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         if (cudaEventElapsedTime(&ms, P->ev_near[0], P->ev_near[1]) == cudaSuccess) P->stats.near_ms = ms;
     }
     P->stats.n_nodes = nn;
-    P->stats.n_leaves = P->n_leaves;
+    P->stats.n_leaves = P->h_small[SM_COLLECT];
     P->stats.depth = depth;
     P->stats.n_m2l = P->n_m2l;
     P->stats.n_p2p = P->n_p2p;
@@ -731,7 +729,7 @@ sfmm_status sfmm_plan(sfmm_plan_t* out, int max_depth, int order_p, double tol, 
     float lt[129 * 4];
     fill_log_table(lt);
     cudaError_t e;
-    if ((e = cudaMallocHost(&P->h_status, sizeof(int))) || (e = cudaStreamCreateWithFlags(&P->aux, cudaStreamNonBlocking)) ||
+    if ((e = cudaMallocHost(&P->h_small, SM_SLOTS * 8 + sizeof(int))) || (e = cudaStreamCreateWithFlags(&P->aux, cudaStreamNonBlocking)) ||
         (e = cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming)) ||
         (e = cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming)) ||
         (e = cudaEventCreateWithFlags(&P->ev_m2l, cudaEventDisableTiming)) ||
@@ -741,6 +739,7 @@ sfmm_status sfmm_plan(sfmm_plan_t* out, int max_depth, int order_p, double tol, 
         sfmm_destroy(P);
         return SFMM_ECUDA;
     }
+    P->h_status = reinterpret_cast<int*>(P->h_small + SM_SLOTS);
     if ((e = ensure(P->tables, h.size() * 8)) ||
         (e = cudaMemcpy(P->tables.p, h.data(), h.size() * 8, cudaMemcpyHostToDevice)) ||
         (e = ensure(P->logtab, sizeof lt)) || (e = cudaMemcpy(P->logtab.p, lt, sizeof lt, cudaMemcpyHostToDevice))) {
@@ -948,10 +947,9 @@ void sfmm_destroy(sfmm_plan_t plan)
     if (!plan) return;
     Buf* all[] = {&plan->skeys, &plan->skeys2, &plan->sperm, &plan->sperm2, &plan->src4, &plan->tkeys, &plan->tkeys2,
                   &plan->tperm, &plan->tperm2, &plan->tgt4, &plan->h_src, &plan->h_q, &plan->h_tgt, &plan->h_psi,
-                  &plan->h_alpha, &plan->tmp, &plan->flags, &plan->pos, &plan->small, &plan->n_prefix,
+                  &plan->h_alpha, &plan->cwords, &plan->wwords, &plan->tmp, &plan->flags, &plan->pos, &plan->small, &plan->n_prefix,
                   &plan->n_level, &plan->n_first, &plan->n_count, &plan->n_child0, &plan->n_parent, &plan->n_geom,
                   &plan->n_tfirst, &plan->n_tcount, &plan->mpole, &plan->local, &plan->tables, &plan->fa, &plan->fb,
-                  &plan->act, &plan->c_next, &plan->c_m2l, &plan->c_p2p, &plan->o_next, &plan->o_m2l, &plan->o_p2p,
                   &plan->m2l_t, &plan->m2l_s, &plan->m2l_t2, &plan->m2l_s2, &plan->p2p_t, &plan->p2p_s,
                   &plan->p2p_t2, &plan->p2p_s2, &plan->m2l_off, &plan->p2p_off, &plan->leaves_src,
                   &plan->items, &plan->m2l_geo, &plan->m2m_geo, &plan->l2l_geo, &plan->soff,
@@ -973,7 +971,7 @@ void sfmm_destroy(sfmm_plan_t plan)
     for (cudaEvent_t ev : plan->ev_near)
         if (ev) cudaEventDestroy(ev);
     if (plan->aux) cudaStreamDestroy(plan->aux);
-    if (plan->h_status) cudaFreeHost(plan->h_status);
+    if (plan->h_small) cudaFreeHost(plan->h_small);
     delete plan;
 }
 

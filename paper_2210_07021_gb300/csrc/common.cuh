@@ -111,6 +111,19 @@ __device__ __forceinline__ void item_range(int2 it, int tc, int* lo, int* hi)
     *hi = parts == ITEM_A ? tb + 32 : min(tc, tb + ITEM_CHUNK);
 }
 
+// Slots (int64) of the plan's small buffer, its device counters.
+enum {
+    SM_TOTAL = 0,        // scan totals
+    SM_PAIRS = 16,       // near-field pairs (timing level 2)
+    SM_STATUS = 20,      // tensor-core M2L: status; SM_LEFT: leftover count (and tile counter)
+    SM_LEFT = 21,
+    SM_ITEM_CTR = 40,    // the evaluation's item counter
+    SM_TREE = 64,        // the tree's levels (TreeLevels)
+    SM_COLLECT = 112,    // source leaves, evaluation items
+    SM_WALK = 128,       // the walk's state (WalkState)
+    SM_SLOTS = 512
+};
+
 // The counts of a solve run without host synchronisation (graph mode): launches
 // are sized by the plan's capacities and every kernel reads its actual count
 // here; a kernel that would exceed a capacity sets `overflow` instead of
@@ -167,7 +180,9 @@ struct sfmm_plan_s {
     // host-array staging for sfmm_deflection_host
     sfmm::Buf h_src, h_q, h_tgt, h_psi, h_alpha;
     // scratch
-    sfmm::Buf tmp, flags, pos, small;   // small: a few int64 counters (device)
+    sfmm::Buf tmp, flags, pos, small;   // small: device counters (SM_ slots)
+    sfmm::Buf cwords, wwords;           // published words of the leaf collection and of the walk (lookback.cuh)
+    int64_t* h_small = nullptr;         // pinned host copies of small's slots
     sfmm::Buf ttmp;                     // scratch of the target sort (auxiliary stream)
     // tree (node arrays)
     sfmm::Buf n_prefix, n_level, n_first, n_count, n_child0, n_parent, n_geom, n_tfirst, n_tcount;
@@ -188,7 +203,7 @@ struct sfmm_plan_s {
     sfmm::Buf macn;                        // per-node sin/cos of the radii for the MAC
     sfmm::Buf macn32;                      // the same in FP32 with the centre as (hi, lo) pairs (first decision)
     // lists
-    sfmm::Buf fa, fb, act, c_next, c_m2l, c_p2p, o_next, o_m2l, o_p2p;
+    sfmm::Buf fa, fb;                      // the walk's frontier, two rounds' worth
     sfmm::Buf m2l_t, m2l_s, m2l_t2, m2l_s2, p2p_t, p2p_s, p2p_t2, p2p_s2, m2l_off, p2p_off;
     int64_t n_m2l = 0, n_p2p = 0;          // pair counts (graph mode: the list capacities)
     const int64_t* d_m2l = nullptr;        // graph mode: the pair counts on the device, else NULL

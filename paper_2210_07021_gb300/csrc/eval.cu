@@ -448,9 +448,11 @@ __global__ void __launch_bounds__(128) k_eval_adj(EvalAdjArgs AA)
     }
 }
 
-__global__ void k_count_pairs(TreeView T, const int2* __restrict__ items, int64_t n, const int64_t* __restrict__ off,
+__global__ void k_count_pairs(TreeView T, const int2* __restrict__ items, int64_t n_cap, const int64_t* d_nit,
+                              const int64_t* __restrict__ off,
                               const uint32_t* __restrict__ src, unsigned long long* __restrict__ out)
 {
+    const int64_t n = dcount(d_nit, n_cap);
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (int64_t)gridDim.x * blockDim.x) {
         const int2 item = items[w];
         const int leaf = item.x;
@@ -1895,13 +1897,13 @@ cudaError_t launch_eval_df(const TreeView& T, const int2* items, int64_t n_items
     return cudaGetLastError();
 }
 
-cudaError_t launch_count_pairs(const TreeView& T, const int2* items, int64_t n_items, const int64_t* p2p_off,
+cudaError_t launch_count_pairs(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const int64_t* p2p_off,
                                const uint32_t* p2p_src, unsigned long long* out, cudaStream_t s)
 {
     if (n_items == 0) return cudaSuccess;
     int64_t blocks = (n_items + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    k_count_pairs<<<(unsigned)blocks, 256, 0, s>>>(T, items, n_items, p2p_off, p2p_src, out); count_launch();
+    k_count_pairs<<<(unsigned)blocks, 256, 0, s>>>(T, items, n_items, d_nit, p2p_off, p2p_src, out); count_launch();
     return cudaGetLastError();
 }
 
@@ -1944,7 +1946,7 @@ cudaError_t launch_eval(const TreeView& T, const int2* items, int64_t n_items, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_eval_adj(const TreeView& T, const int2* items, int64_t n_items, const double4_32a* src,
+cudaError_t launch_eval_adj(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const double4_32a* src,
                             const double4_32a* dip, const double4_32a* tgt, const uint32_t* tperm,
                             const int64_t* p2p_off, const uint32_t* p2p_src, const double* local, const double* mpole,
                             int p, int zero_mean, const void* w, int w_f32, double* phi, double* grad3,
@@ -1956,7 +1958,7 @@ cudaError_t launch_eval_adj(const TreeView& T, const int2* items, int64_t n_item
     A.T = T;
     A.items = items;
     A.n_items = n_items;
-    A.d_n_items = nullptr;
+    A.d_n_items = d_nit;
     A.src = src;
     A.tgt = tgt;
     A.tperm = tperm;

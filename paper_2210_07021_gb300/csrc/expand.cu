@@ -692,10 +692,11 @@ __global__ void k_p2m(TreeView T, const int* __restrict__ leaves, int64_t n_cap,
 // (d log cos^2(theta/2) = d log((1 + x.c)/2); x.g = 0).  Stored scaled like
 // Lemma 1: A_l / r^l.
 template <int P>
-__global__ void k_p2m_adj(TreeView T, const int* __restrict__ leaves, int64_t n_leaves,
+__global__ void k_p2m_adj(TreeView T, const int* __restrict__ leaves, int64_t n_cap, const int64_t* d_nl,
                           const double4_32a* __restrict__ src, const double4_32a* __restrict__ dip,
                           double* __restrict__ mpole)
 {
+    const int64_t n_leaves = dcount(d_nl, n_cap);
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n_leaves; w += (int64_t)gridDim.x * blockDim.x) {
         const int node = leaves[w];
         const double* g = T.geom + (size_t)node * GEOM_STRIDE;
@@ -805,9 +806,10 @@ __global__ void __launch_bounds__(128) k_p2m_df(TreeView T, const int* __restric
 // FP32: from each source's FP32 offset to its leaf centre (the recentring was
 // done in FP64 when the offsets were formed).
 template <int P>
-__global__ void k_p2m32(TreeView T, const int* __restrict__ leaves, int64_t n_leaves, const float4* __restrict__ off,
+__global__ void k_p2m32(TreeView T, const int* __restrict__ leaves, int64_t n_cap, const int64_t* d_nl, const float4* __restrict__ off,
                         float* __restrict__ mpole)
 {
+    const int64_t n_leaves = dcount(d_nl, n_cap);
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n_leaves; w += (int64_t)gridDim.x * blockDim.x) {
         const int node = leaves[w];
         const double* g = T.geom + (size_t)node * GEOM_STRIDE;
@@ -1119,7 +1121,7 @@ cudaError_t launch_p2m(const TreeView& T, const int* leaves, int64_t n_leaves, c
     const unsigned g = grid_for(n_leaves, 128);
 #define P2M_CASE(PP)                                                                                       \
     case PP:                                                                                               \
-        if (ek == EXP_F32) k_p2m32<PP><<<g, 128, 0, s>>>(T, leaves, n_leaves, off, static_cast<float*>(mpole)); \
+        if (ek == EXP_F32) k_p2m32<PP><<<g, 128, 0, s>>>(T, leaves, n_leaves, d_nl, off, static_cast<float*>(mpole)); \
         else if (ek == EXP_DF) k_p2m_df<PP><<<g, 128, 0, s>>>(T, leaves, n_leaves, off, log_tab, static_cast<dflt*>(mpole)); \
         else k_p2m<PP, double><<<g, 128, 0, s>>>(T, leaves, n_leaves, d_nl, src, static_cast<double*>(mpole)); \
         count_launch();                                                                                    \
@@ -1132,14 +1134,14 @@ cudaError_t launch_p2m(const TreeView& T, const int* leaves, int64_t n_leaves, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_p2m_adj(const TreeView& T, const int* leaves, int64_t n_leaves, const double4_32a* src,
+cudaError_t launch_p2m_adj(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const double4_32a* src,
                            const double4_32a* dip, double* mpole, int p, cudaStream_t s)
 {
     if (n_leaves == 0) return cudaSuccess;
     const unsigned g = grid_for(n_leaves, 128);
 #define P2MA_CASE(PP)                                                                     \
     case PP:                                                                              \
-        k_p2m_adj<PP><<<g, 128, 0, s>>>(T, leaves, n_leaves, src, dip, mpole);            \
+        k_p2m_adj<PP><<<g, 128, 0, s>>>(T, leaves, n_leaves, d_nl, src, dip, mpole);            \
         count_launch();                                                                   \
         break;
     switch ((p + 3) / 4 * 4) {

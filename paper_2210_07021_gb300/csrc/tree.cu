@@ -15,6 +15,7 @@
 // pixel), plus 2e-15 rad for the rounding of the keys.  r = tan(R/2) is the
 // scale of the stereographic variable z = tan(theta/2) e^{i phi} inside the box.
 #include "common.cuh"
+#include "lookback.cuh"
 
 #include <algorithm>
 
@@ -132,9 +133,42 @@ __global__ void k_level_end(DevCounts* dc, int lvl, const int64_t* __restrict__ 
     dc->nn = nb;
 }
 
+struct NodeArrays {
+    uint64_t* prefix;
+    int *level, *first, *count, *child0, *parent;
+};
+
+// Child c = lane % 4 of a split node: its range by binary search of its first key
+// inside the parent's range, its end from the next child (the four lanes of a
+// node work together: one search's latency per node, not three).
+__device__ __forceinline__ void make_child(const uint64_t* __restrict__ keys, const NodeArrays& N, int node, int c0,
+                                           int lvl, bool split)
+{
+    const int c = threadIdx.x & 3;
+    const int shift = 2 * (ORDER_MAX - (lvl + 1));
+    uint64_t pf = 0;
+    int64_t lo = 0, hi = 0, start = 0;
+    if (split) {
+        pf = N.prefix[node] * 4ull + c;
+        lo = N.first[node];
+        hi = lo + N.count[node];
+        start = c == 0 ? lo : lower_bound_u64(keys, lo, hi, pf << shift);
+    }
+    const int64_t next = __shfl_down_sync(FULL, start, 1, 4);
+    if (!split) return;
+    const int64_t end = c == 3 ? hi : next;
+    const int k = c0 + c;
+    N.prefix[k] = pf;
+    N.level[k] = lvl + 1;
+    N.first[k] = (int)start;
+    N.count[k] = (int)(end - start);
+    N.child0[k] = -1;
+    N.parent[k] = node;
+    if (c == 0) N.child0[node] = c0;
+}
+
 __global__ void k_make_children(const uint64_t* __restrict__ keys, int a, int b, int lvl,
-                                const int64_t* __restrict__ flags, const int64_t* __restrict__ pos,
-                                uint64_t* prefix, int* level, int* first, int* count, int* child0, int* parent,
+                                const int64_t* __restrict__ flags, const int64_t* __restrict__ pos, NodeArrays N,
                                 const DevCounts* dc)
 {
     if (dc) {
@@ -142,26 +176,101 @@ __global__ void k_make_children(const uint64_t* __restrict__ keys, int a, int b,
         a = (int)dc->level[lvl];
         b = (int)dc->level[lvl + 1];
     }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < b - a; i += (int64_t)gridDim.x * blockDim.x) {
-        const int node = a + (int)i;
-        if (!flags[i]) continue;
-        const int c0 = b + 4 * (int)pos[i];
-        child0[node] = c0;
-        const int shift = 2 * (ORDER_MAX - (lvl + 1));
-        const uint64_t pf = prefix[node] * 4ull;
-        const int64_t lo = first[node], hi = lo + count[node];
-        int64_t starts[5];
-        starts[0] = lo;
-        starts[4] = hi;
-        for (int c = 1; c < 4; ++c) starts[c] = lower_bound_u64(keys, starts[c - 1], hi, (pf + c) << shift);
-        for (int c = 0; c < 4; ++c) {
-            prefix[c0 + c] = pf + c;
-            level[c0 + c] = lvl + 1;
-            first[c0 + c] = (int)starts[c];
-            count[c0 + c] = (int)(starts[c + 1] - starts[c]);
-            child0[c0 + c] = -1;
-            parent[c0 + c] = node;
+    const int64_t nt = 4 * (int64_t)(b - a), step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < nt; t0 += step) {
+        const int64_t i = (t0 + (threadIdx.x & 31)) >> 2;
+        const bool split = i < b - a && flags[i];
+        make_child(keys, N, a + (int)i, split ? b + 4 * (int)pos[i] : 0, lvl, split);
+    }
+}
+
+// The levels of the tree on the device: nodes of level l are [start[l], start[l + 1]),
+// levels 0..lvl exist; done when no box of level lvl is to be split.
+struct TreeLevels {
+    int64_t lvl, done;
+    int64_t start[ORDER_MAX + 3];
+};
+
+// One CTA builds the tree on from level lvl for as long as a level has at most
+// TREE_NARROW boxes (and its children fit the node capacity): the flags, their
+// scan and the children of all those levels in one launch and one host
+// synchronisation.  A level at a time costs five launches and a synchronisation,
+// 45 us: the tree of 1e4 clustered points (13 levels) took 0.58 ms without its
+// geometry, and takes 0.06 ms.
+constexpr int TREE_NARROW = 4096, TREE_T = 1024;
+
+__global__ void __launch_bounds__(TREE_T) k_tree_narrow(const uint64_t* __restrict__ keys, int64_t n, int m,
+                                                        int max_depth, int64_t node_cap, bool first, TreeLevels* L,
+                                                        NodeArrays N)
+{
+    __shared__ int s_node[TREE_NARROW];              // the level's split boxes in order
+    __shared__ int s_warp[TREE_T / 32];
+    __shared__ int s_total;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int lvl;
+    int64_t a, b;
+    if (first) {
+        if (tid < 12) {
+            const uint64_t lo = (uint64_t)tid << (2 * ORDER_MAX), hi = (uint64_t)(tid + 1) << (2 * ORDER_MAX);
+            const int64_t f = lower_bound_u64(keys, 0, n, lo), e = lower_bound_u64(keys, f, n, hi);
+            N.prefix[tid] = (uint64_t)tid;
+            N.level[tid] = 0;
+            N.first[tid] = (int)f;
+            N.count[tid] = (int)(e - f);
+            N.child0[tid] = -1;
+            N.parent[tid] = -1;
         }
+        lvl = 0;
+        a = 0;
+        b = 12;
+        if (tid == 0) { L->start[0] = 0; L->start[1] = 12; }
+        __syncthreads();
+    } else {
+        lvl = (int)L->lvl;
+        a = L->start[lvl];
+        b = L->start[lvl + 1];
+    }
+    bool done = false;
+    while (b - a <= TREE_NARROW) {
+        if (lvl >= max_depth) { done = true; break; }
+        int splits = 0;
+        for (int64_t i0 = a; i0 < b; i0 += TREE_T) {
+            const bool f = i0 + tid < b && N.count[i0 + tid] > m;
+            const unsigned mask = __ballot_sync(FULL, f);
+            if (lane == 0) s_warp[warp] = __popc(mask);
+            __syncthreads();
+            if (warp == 0) {
+                const int v = s_warp[lane];
+                int inc = v;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(FULL, inc, o);
+                    if (lane >= o) inc += t;
+                }
+                s_warp[lane] = inc - v;
+                if (lane == 31) s_total = inc;
+            }
+            __syncthreads();
+            if (f) s_node[splits + s_warp[warp] + __popc(mask & ((1u << lane) - 1u))] = (int)(i0 + tid);
+            splits += s_total;
+            __syncthreads();
+        }
+        if (splits == 0) { done = true; break; }
+        if (b + 4 * (int64_t)splits > node_cap) break;
+        for (int t0 = 0; t0 < 4 * splits; t0 += TREE_T) {
+            const int j = (t0 + tid) >> 2;
+            const bool split = j < splits;
+            make_child(keys, N, split ? s_node[j] : 0, (int)b + 4 * j, lvl, split);
+        }
+        a = b;
+        b += 4 * (int64_t)splits;
+        ++lvl;
+        if (tid == 0) L->start[lvl + 1] = b;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        L->lvl = lvl;
+        L->done = done;
     }
 }
 
@@ -210,60 +319,100 @@ __global__ void k_target_ranges(int n_cap, const int64_t* d_nn, const uint64_t* 
     }
 }
 
-// flags over the whole capacity n_cap (zero beyond the node count)
-__global__ void k_collect_leaves(int n_cap, const int64_t* d_nn, const int* __restrict__ child0,
-                                 const int* __restrict__ cnt, int64_t* __restrict__ flags)
-{
-    const int64_t nn = dcount(d_nn, n_cap);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_cap; i += (int64_t)gridDim.x * blockDim.x)
-        flags[i] = (i < nn && child0[i] < 0 && cnt[i] > 0) ? 1 : 0;
-}
-
-__global__ void k_compact(int n, const int64_t* __restrict__ flags, const int64_t* __restrict__ pos, int* __restrict__ out)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (flags[i]) out[pos[i]] = (int)i;
-}
-
 // Evaluation items per node: a leaf's targets in chunks of 64, or (split) of 32
 // where more than 32 are left.
 __device__ __forceinline__ int64_t items_of(int tc, int split) { return split ? (tc + 31) / 32 : (tc + 63) / 64; }
 
-__global__ void k_item_counts(int n_cap, const int64_t* d_nn, const int* __restrict__ child0,
-                              const int* __restrict__ tcount, int split, int64_t* __restrict__ flags)
+// The source leaves (leaves holding sources, in node order) and the evaluation's
+// items of all leaves holding targets, in one pass over the nodes: a tile of 1024
+// nodes finds its places by looking back (words: leaves and items per tile).  A
+// node with more than 4 items writes them by the whole warp (one leaf can hold
+// every target of the problem).  out: the two counts, then the tile counter.
+constexpr int CT = 256, CI = 4, CTILE = CT * CI;
+
+__device__ __forceinline__ int2 make_item(int node, int tc, int64_t k, int split)
 {
-    const int64_t nn = dcount(d_nn, n_cap);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_cap; i += (int64_t)gridDim.x * blockDim.x)
-        flags[i] = (i < nn && child0[i] < 0) ? items_of(tcount[i], split) : 0;
+    if (!split) return make_int2(node, (int)(k * 64) | ITEM_A | ITEM_B);
+    const int tb = (int)(k / 2) * 64;
+    const int parts = (k & 1) ? ITEM_B : tc - tb > 32 ? ITEM_A : ITEM_A | ITEM_B;
+    return make_int2(node, tb | parts);
 }
 
-// Items of all leaves at their scanned places: the lanes of a warp write those
-// of 32 nodes, a node with more than 4 by the whole warp (one leaf can hold
-// every target of the problem).
-__global__ void k_items(int n, const int64_t* __restrict__ flags, const int64_t* __restrict__ pos,
-                        const int* __restrict__ tcount, int split, int2* __restrict__ out)
+__global__ void __launch_bounds__(CT) k_collect(int n_cap, const int64_t* d_nn, const int* __restrict__ child0,
+                                                const int* __restrict__ count, const int* __restrict__ tcount,
+                                                int split, int* __restrict__ leaves, int2* __restrict__ items,
+                                                uint64_t* __restrict__ words, int64_t* __restrict__ n_leaves,
+                                                int64_t* __restrict__ n_items, uint32_t* __restrict__ ticket, int limit)
 {
-    const int lane = threadIdx.x & 31;
-    auto item = [&](int node, int tc, int64_t k) {
-        if (!split) return make_int2(node, (int)(k * 64) | ITEM_A | ITEM_B);
-        const int tb = (int)(k / 2) * 64;
-        const int parts = (k & 1) ? ITEM_B : tc - tb > 32 ? ITEM_A : ITEM_A | ITEM_B;
-        return make_int2(node, tb | parts);
-    };
-    const int64_t step = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n; i0 += step) {
-        const int64_t i = i0 + lane;
-        const int64_t c = i < n ? flags[i] : 0;
-        const int64_t at = i < n ? pos[i] : 0;
-        const int tc = i < n ? tcount[i] : 0;
+    __shared__ uint32_t s_tile;
+    __shared__ int64_t s_warp[2][CT / 32], s_base[2];
+    __shared__ int s_lost;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t nn = dcount(d_nn, n_cap);
+    if (threadIdx.x == 0) { s_tile = atomicAdd(ticket, 1u); s_lost = 0; }
+    __syncthreads();
+    const int64_t tile = s_tile, ntiles = ((int64_t)n_cap + CTILE - 1) / CTILE;
+    const int64_t i0 = tile * CTILE + (int64_t)threadIdx.x * CI;
+    int tc[CI];
+    bool lf[CI];
+    int64_t nl = 0, ni = 0;
+#pragma unroll
+    for (int r = 0; r < CI; ++r) {
+        const int64_t i = i0 + r;
+        const bool leaf = i < nn && child0[i] < 0;
+        lf[r] = leaf && count[i] > 0;
+        tc[r] = leaf ? tcount[i] : 0;
+        nl += lf[r];
+        ni += items_of(tc[r], split);
+    }
+    int64_t il = nl, ii = ni;                       // inclusive sums over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t x = __shfl_up_sync(FULL, il, o), y = __shfl_up_sync(FULL, ii, o);
+        if (lane >= o) { il += x; ii += y; }
+    }
+    if (lane == 31) { s_warp[0][warp] = il; s_warp[1][warp] = ii; }
+    __syncthreads();
+    int64_t bl = 0, bi = 0, tl = 0, ti = 0;
+    for (int w = 0; w < CT / 32; ++w) {
+        if (w < warp) { bl += s_warp[0][w]; bi += s_warp[1][w]; }
+        tl += s_warp[0][w];
+        ti += s_warp[1][w];
+    }
+    if (warp < 2) {                                 // warp 0: leaves, warp 1: items
+        const int64_t own = warp == 0 ? tl : ti;
+        uint64_t* w = words + 2 * tile + warp;
+        if (lane == 0) lb_publish(w, 0, LB_OWN, own);
+        int64_t before = 0;
+        const bool ok = lb_before(words + warp, 2, tile, 0, limit, &before);
+        if (!ok) {                                  // the wait ran out: count the earlier nodes
+            before = 0;
+            for (int64_t i = lane; i < tile * CTILE; i += 32)
+                if (i < nn && child0[i] < 0) before += warp == 0 ? (count[i] > 0) : items_of(tcount[i], split);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(FULL, before, o);
+        }
+        if (lane == 0) {
+            lb_publish(w, 0, LB_UPTO, before + own);
+            s_base[warp] = before;
+            if (tile == ntiles - 1) *(warp == 0 ? n_leaves : n_items) = before + own;
+        }
+    }
+    __syncthreads();
+    int64_t ol = s_base[0] + bl + il - nl, oi = s_base[1] + bi + ii - ni;
+#pragma unroll
+    for (int r = 0; r < CI; ++r) {
+        const int64_t c = items_of(tc[r], split);
+        if (lf[r]) leaves[ol++] = (int)(i0 + r);
         if (c <= 4)
-            for (int64_t k = 0; k < c; ++k) out[at + k] = item((int)i, tc, k);
+            for (int64_t k = 0; k < c; ++k) items[oi + k] = make_item((int)(i0 + r), tc[r], k, split);
         for (unsigned big = __ballot_sync(FULL, c > 4); big; big &= big - 1) {
             const int l = __ffs(big) - 1;
-            const int64_t cl = __shfl_sync(FULL, c, l), al = __shfl_sync(FULL, at, l);
-            const int tl = __shfl_sync(FULL, tc, l);
-            for (int64_t k = lane; k < cl; k += 32) out[al + k] = item((int)(i0 + l), tl, k);
+            const int64_t cl = __shfl_sync(FULL, c, l), al = __shfl_sync(FULL, oi, l), node = __shfl_sync(FULL, i0 + r, l);
+            const int tl2 = __shfl_sync(FULL, tc[r], l);
+            for (int64_t k = lane; k < cl; k += 32) items[al + k] = make_item((int)node, tl2, k, split);
         }
+        oi += c;
     }
 }
 
@@ -279,7 +428,8 @@ inline unsigned grid_for(int64_t n, int threads = 256)
 
 // Build the tree from the key-sorted source keys.  Grows the plan's node arrays
 // as needed; fills plan->level_start and plan->n_nodes.  Synchronises the
-// stream once per level (the next level's size is needed on the host).
+// stream once per run of narrow levels and once per wide level (the next level's
+// size is needed on the host).
 //
 // Graph mode (plan->gm): no synchronisation.  Every level up to the plan's level
 // capacity is launched with grids sized by the level-width capacity; the level
@@ -304,6 +454,10 @@ cudaError_t build_tree(sfmm_plan_s* P, const uint64_t* keys, int64_t n, int m, i
         P->node_cap = cap;
         return cudaSuccess;
     };
+    auto arrays = [&]() {
+        return NodeArrays{P->n_prefix.as<uint64_t>(), P->n_level.as<int>(), P->n_first.as<int>(),
+                          P->n_count.as<int>(), P->n_child0.as<int>(), P->n_parent.as<int>()};
+    };
     if (P->gm) {
         DevCounts* dc = P->dcnt.as<DevCounts>();
         const int64_t width = P->cap.width, levels = P->cap.levels;
@@ -322,52 +476,64 @@ cudaError_t build_tree(sfmm_plan_s* P, const uint64_t* keys, int64_t n, int m, i
             if ((e = exclusive_scan_i64(flags, pos, width, total, P->tmp.p, s))) return e;
             k_level_end<<<1, 1, 0, s>>>(dc, lvl, total, P->cap.nodes, lvl == levels - 1); count_launch();
             if (lvl < levels - 1) {
-                k_make_children<<<grid_for(width), 256, 0, s>>>(keys, 0, 0, lvl, flags, pos, P->n_prefix.as<uint64_t>(),
-                                                               P->n_level.as<int>(), P->n_first.as<int>(),
-                                                               P->n_count.as<int>(), P->n_child0.as<int>(),
-                                                               P->n_parent.as<int>(), dc); count_launch();
+                k_make_children<<<grid_for(4 * width), 256, 0, s>>>(keys, 0, 0, lvl, flags, pos, arrays(), dc); count_launch();
             }
         }
         P->n_nodes = P->cap.nodes;
         return cudaGetLastError();
     }
+    // narrow levels in runs by one CTA (k_tree_narrow), wide ones a level at a time
     P->n_nodes = 0;
     if ((e = grow(12 + 4 * 1024))) return e;
-    k_level0<<<1, 32, 0, s>>>(keys, n, P->n_prefix.as<uint64_t>(), P->n_level.as<int>(), P->n_first.as<int>(),
-                              P->n_count.as<int>(), P->n_child0.as<int>(), P->n_parent.as<int>()); count_launch();
-    P->n_nodes = 12;
+    TreeLevels* dL = reinterpret_cast<TreeLevels*>(P->small.as<int64_t>() + SM_TREE);
+    TreeLevels* hL = reinterpret_cast<TreeLevels*>(P->h_small + SM_TREE);
     P->level_start.assign(1, 0);
     P->level_start.push_back(12);
-    int lvl = 0;
-    int64_t max_width = 12;
+    bool first = true;
     while (true) {
-        const int a = P->level_start[lvl], b = P->level_start[lvl + 1];
-        const int width = b - a;
-        if (width == 0 || lvl >= max_depth) break;
-        max_width = std::max<int64_t>(max_width, width);
-        if ((e = ensure(P->flags, (size_t)width * 8))) return e;
-        if ((e = ensure(P->pos, (size_t)width * 8))) return e;
-        if ((e = ensure(P->tmp, scan_tmp_bytes(width)))) return e;
-        int64_t* flags = P->flags.as<int64_t>();
-        int64_t* pos = P->pos.as<int64_t>();
-        k_split_flags<<<grid_for(width), 256, 0, s>>>(P->n_count.as<int>(), a, b, lvl, m, max_depth, flags, nullptr,
-                                                       0); count_launch();
-        int64_t* total = P->small.as<int64_t>();
-        if ((e = exclusive_scan_i64(flags, pos, width, total, P->tmp.p, s))) return e;
-        int64_t splits = 0;
-        if ((e = cudaMemcpyAsync(&splits, total, 8, cudaMemcpyDeviceToHost, s))) return e;
-        if ((e = cudaStreamSynchronize(s))) return e;
-        if (splits == 0) break;
-        if ((e = grow(b + 4 * splits))) return e;
-        k_make_children<<<grid_for(width), 256, 0, s>>>(keys, a, b, lvl, flags, pos, P->n_prefix.as<uint64_t>(),
-                                                       P->n_level.as<int>(), P->n_first.as<int>(),
-                                                       P->n_count.as<int>(), P->n_child0.as<int>(),
-                                                       P->n_parent.as<int>(), nullptr); count_launch();
-        P->n_nodes = b + 4 * splits;
-        P->level_start.push_back((int)P->n_nodes);
-        ++lvl;
+        k_tree_narrow<<<1, TREE_T, 0, s>>>(keys, n, m, max_depth, P->node_cap, first, dL, arrays()); count_launch();
+        if ((e = cudaMemcpyAsync(hL, dL, sizeof *hL, cudaMemcpyDeviceToHost, s)) || (e = cudaStreamSynchronize(s)))
+            return e;
+        first = false;
+        int lvl = (int)hL->lvl;
+        P->level_start.resize(lvl + 2);
+        for (int l = 0; l <= lvl + 1; ++l) P->level_start[l] = (int)hL->start[l];
+        P->n_nodes = P->level_start[lvl + 1];
+        if (hL->done) break;
+        // this level (and the wide ones after it) with the whole GPU
+        bool end = false;
+        do {
+            const int a = P->level_start[lvl], b = P->level_start[lvl + 1];
+            const int64_t width = b - a;
+            if (lvl >= max_depth) { end = true; break; }
+            if ((e = ensure(P->flags, (size_t)width * 8)) || (e = ensure(P->pos, (size_t)width * 8)) ||
+                (e = ensure(P->tmp, scan_tmp_bytes(width))))
+                return e;
+            int64_t* flags = P->flags.as<int64_t>();
+            int64_t* pos = P->pos.as<int64_t>();
+            int64_t* total = P->small.as<int64_t>() + SM_TOTAL;
+            k_split_flags<<<grid_for(width), 256, 0, s>>>(P->n_count.as<int>(), a, b, lvl, m, max_depth, flags,
+                                                           nullptr, 0); count_launch();
+            if ((e = exclusive_scan_i64(flags, pos, width, total, P->tmp.p, s))) return e;
+            int64_t* splits = P->h_small + SM_TOTAL;
+            if ((e = cudaMemcpyAsync(splits, total, 8, cudaMemcpyDeviceToHost, s)) || (e = cudaStreamSynchronize(s)))
+                return e;
+            if (*splits == 0) { end = true; break; }
+            if ((e = grow(b + 4 * *splits))) return e;
+            k_make_children<<<grid_for(4 * width), 256, 0, s>>>(keys, a, b, lvl, flags, pos, arrays(), nullptr); count_launch();
+            P->n_nodes = b + 4 * *splits;
+            P->level_start.push_back((int)P->n_nodes);
+            ++lvl;
+        } while (P->level_start[lvl + 1] - P->level_start[lvl] > TREE_NARROW);
+        if (end) break;
+        // hand the levels so far back to the narrow kernel
+        hL->lvl = lvl;
+        for (int l = 0; l <= lvl + 1; ++l) hL->start[l] = P->level_start[l];
+        if ((e = cudaMemcpyAsync(dL, hL, sizeof *hL, cudaMemcpyHostToDevice, s))) return e;
     }
-    P->last_max_width = max_width;
+    P->last_max_width = 12;
+    for (size_t l = 0; l + 1 < P->level_start.size(); ++l)
+        P->last_max_width = std::max<int64_t>(P->last_max_width, P->level_start[l + 1] - P->level_start[l]);
     return cudaGetLastError();
 }
 
@@ -394,60 +560,36 @@ cudaError_t tree_target_ranges(sfmm_plan_s* P, const uint64_t* tkeys, int64_t M)
     return cudaGetLastError();
 }
 
-// The evaluation's work items (plan->items, plan->n_items).  Chunks are split in
-// two, at the price of staging a leaf's sources twice, when M targets make fewer
-// full chunks than the GPU holds warps (152 SMs x 28) and most chunks are full
-// (32 targets or more per node): 49,152 grid points over 447 leaves.  Where the
-// leaves hold about m targets each the halves only add staging (1e5 points at
-// their own places: 1.80 ms whole, 1.84 ms split).  Graph mode: the count
-// goes to DevCounts::n_items, plan->n_items is the capacity.
-cudaError_t collect_items(sfmm_plan_s* P, int64_t M)
+// The source leaves (plan->leaves_src) and the evaluation's work items (plan->items).
+// Their counts stay on the device (*d_leaves, *d_items), the plan holds the
+// capacities that launches over them are sized by: no host synchronisation.
+// Chunks are split in two, at the price of staging a leaf's sources twice, when M
+// targets make fewer full chunks than the GPU holds warps (152 SMs x 28) and most
+// chunks are full (32 targets or more per node): 49,152 grid points over 447
+// leaves.  Where the leaves hold about m targets each the halves only add staging
+// (1e5 points at their own places: 1.80 ms whole, 1.84 ms split).
+cudaError_t collect_leaves_items(sfmm_plan_s* P, int64_t M, int64_t* d_leaves, int64_t* d_items)
 {
     cudaError_t e;
     const int64_t nn = P->n_nodes;
     cudaStream_t s = P->stream;
     const int split = M < 152 * 28 * (int64_t)ITEM_CHUNK && M >= 32 * nn;
     const int64_t cap = nn + M / (split ? 32 : 64) + 1;       // sum of ceilings over the leaves
-    if ((e = ensure(P->flags, (size_t)nn * 8)) || (e = ensure(P->pos, (size_t)nn * 8)) ||
-        (e = ensure(P->tmp, scan_tmp_bytes(nn))) || (e = ensure(P->items, (size_t)cap * 8)))
+    const int64_t ntiles = (nn + CTILE - 1) / CTILE;
+    // the published words, then the tile counter
+    const size_t wb = (size_t)(2 * ntiles + 1) * 8;
+    if ((e = ensure(P->items, (size_t)cap * 8)) || (e = ensure(P->leaves_src, (size_t)nn * 4)) ||
+        (e = ensure(P->cwords, wb)) || (e = cudaMemsetAsync(P->cwords.p, 0, wb, s)))
         return e;
-    DevCounts* dc = P->gm ? P->dcnt.as<DevCounts>() : nullptr;
-    k_item_counts<<<grid_for(nn), 256, 0, s>>>((int)nn, dc ? &dc->nn : nullptr, P->n_child0.as<int>(),
-                                               P->n_tcount.as<int>(), split, P->flags.as<int64_t>()); count_launch();
-    int64_t* total = dc ? &dc->n_items : P->small.as<int64_t>() + 1;
-    if ((e = exclusive_scan_i64(P->flags.as<int64_t>(), P->pos.as<int64_t>(), nn, total, P->tmp.p, s))) return e;
-    k_items<<<grid_for(nn), 256, 0, s>>>((int)nn, P->flags.as<int64_t>(), P->pos.as<int64_t>(), P->n_tcount.as<int>(),
-                                         split, P->items.as<int2>()); count_launch();
-    if (dc) {
-        P->n_items = cap;
-        return cudaGetLastError();
-    }
-    if ((e = cudaMemcpyAsync(&P->n_items, total, 8, cudaMemcpyDeviceToHost, s))) return e;
-    return cudaStreamSynchronize(s);
-}
-
-// Indices of the leaves whose `cnt` (source or target count) is positive.  Graph
-// mode: the count goes to *d_out on the device (no synchronisation).
-cudaError_t collect_leaves(sfmm_plan_s* P, const int* cnt, sfmm::Buf& out, int64_t* n_out, int64_t* d_out)
-{
-    cudaError_t e;
-    const int64_t nn = P->n_nodes;
-    cudaStream_t s = P->stream;
-    if ((e = ensure(P->flags, (size_t)nn * 8))) return e;
-    if ((e = ensure(P->pos, (size_t)nn * 8))) return e;
-    if ((e = ensure(P->tmp, scan_tmp_bytes(nn)))) return e;
-    if ((e = ensure(out, (size_t)nn * 4))) return e;
-    const int64_t* d_nn = P->gm ? &P->dcnt.as<DevCounts>()->nn : nullptr;
-    k_collect_leaves<<<grid_for(nn), 256, 0, s>>>((int)nn, d_nn, P->n_child0.as<int>(), cnt, P->flags.as<int64_t>()); count_launch();
-    int64_t* total = P->gm ? d_out : P->small.as<int64_t>() + 1;
-    if ((e = exclusive_scan_i64(P->flags.as<int64_t>(), P->pos.as<int64_t>(), nn, total, P->tmp.p, s))) return e;
-    k_compact<<<grid_for(nn), 256, 0, s>>>((int)nn, P->flags.as<int64_t>(), P->pos.as<int64_t>(), out.as<int>()); count_launch();
-    if (P->gm) {
-        *n_out = nn;          // the capacity: launches over the leaves read *d_out
-        return cudaGetLastError();
-    }
-    if ((e = cudaMemcpyAsync(n_out, total, 8, cudaMemcpyDeviceToHost, s))) return e;
-    return cudaStreamSynchronize(s);
+    uint64_t* words = P->cwords.as<uint64_t>();
+    k_collect<<<(unsigned)ntiles, CT, 0, s>>>((int)nn, P->gm ? &P->dcnt.as<DevCounts>()->nn : nullptr,
+                                              P->n_child0.as<int>(), P->n_count.as<int>(), P->n_tcount.as<int>(), split,
+                                              P->leaves_src.as<int>(), P->items.as<int2>(), words, d_leaves, d_items,
+                                              reinterpret_cast<uint32_t*>(words + 2 * ntiles),
+                                              P->opt.wait_limit > 0 ? P->opt.wait_limit : LB_POLLS); count_launch();
+    P->n_leaves = nn;
+    P->n_items = cap;
+    return cudaGetLastError();
 }
 
 }  // namespace sfmm

@@ -18,15 +18,20 @@
 // contribute nothing).  The lists are then grouped by target box with a stable
 // radix sort, giving CSR offsets per box.
 //
-// A round is three launches: classify (+ per-tile sums of the three output
-// counts), a single-CTA scan of the tile sums that also advances the running
-// list totals and checks capacities, and emit (in-tile scan + scatter).  The
-// frontier size lives on the device, so the rounds run back to back without
-// host synchronisation; 2 * depth + 4 rounds always suffice (every split makes
-// one side, or for B_S == B_T both, one level deeper).  If an output would
-// exceed its buffer, an overflow flag is set, nothing more is written, and the
-// host grows the buffers and runs the walk again.
+// A round is one launch: a tile of the frontier classifies its pairs, finds the
+// places of its outputs by looking back over the tiles before it (lookback.cuh,
+// one published word per output), and writes them.  The frontier's size and the
+// lists' lengths live on the device, one record per round, so the rounds run
+// back to back without host synchronisation; 2 * depth + 4 rounds always suffice
+// (every split makes one side, or for B_S == B_T both, one level deeper).  A tile
+// whose outputs would exceed a buffer writes nothing of them, the round's last
+// tile sets the overflow flag and empties the frontier, and the host grows the
+// buffers and runs the walk again.  (Classify, scan and emit as three launches
+// read the frontier twice and cost 17 us per round where it is small:
+// 30 rounds over 1e4 clustered points 0.51 -> 0.24 ms, 34 rounds at N = M = 1.6e7
+// 1.69 -> 1.34 ms.)
 #include "common.cuh"
+#include "lookback.cuh"
 
 namespace sfmm {
 
@@ -39,10 +44,20 @@ constexpr double RADIUS_TIE = 1e-12;
 
 enum : uint8_t { A_DROP = 0, A_SELF = 1, A_LEAFSELF = 2, A_M2L = 3, A_SPLIT_S = 4, A_SPLIT_T = 5, A_P2P = 6 };
 
-constexpr int WT = 256, WI = 8, WTILE = WT * WI;
+constexpr int WT = 256, WI = 4, WTILE = WT * WI;
+constexpr int MAX_ROUNDS = 2 * ORDER_MAX + 4;
 
-// device counters (in the plan's small buffer, int64 slots)
-enum { C_FRONT0 = 0, C_FRONT1 = 1, C_M2L = 2, C_P2P = 3, C_OVERFLOW = 4, C_ROUNDS = 5 };
+// The walk's state (in the plan's small buffer): round r reads rec[r] and leaves
+// rec[r + 1]; a round's tiles take their numbers from its counter.
+struct WalkRec {
+    int64_t front, m2l, p2p;        // pairs of the frontier; lengths of the two lists
+};
+struct WalkState {
+    int64_t overflow;
+    uint32_t ticket[MAX_ROUNDS + 2];
+    WalkRec rec[MAX_ROUNDS + 1];
+};
+static_assert(sizeof(WalkState) % 8 == 0 && SM_WALK + sizeof(WalkState) / 8 <= SM_SLOTS, "the walk's state fits its slots");
 
 struct WalkCaps {
     int64_t front, m2l, p2p;
@@ -191,122 +206,103 @@ __device__ __forceinline__ int3 block_excl3(int3 v, int3* s_w, int3* total)
     return make_int3(inc.x - v.x + wb.x, inc.y - v.y + wb.y, inc.z - v.z + wb.z);
 }
 
-__global__ void k_init_frontier(int2* f, int64_t* ctr)
+__global__ void k_init_frontier(int2* f, WalkState* S)
 {
     const int i = threadIdx.x;
     if (i < 144) f[i] = make_int2(i / 12, i % 12);
+    if (i < MAX_ROUNDS + 2) S->ticket[i] = 0;
     if (i == 0) {
-        ctr[C_FRONT0] = 144;
-        ctr[C_FRONT1] = 0;
-        ctr[C_M2L] = 0;
-        ctr[C_P2P] = 0;
-        ctr[C_OVERFLOW] = 0;
-        ctr[C_ROUNDS] = 0;
+        S->overflow = 0;
+        S->rec[0].front = 144;
+        S->rec[0].m2l = S->rec[0].p2p = 0;
     }
 }
 
-__global__ void __launch_bounds__(WT) k_walk_classify(TreeView T, const MacNode* __restrict__ mac,
-                                                      const MacNode32* __restrict__ mac32,
-                                                      const int2* __restrict__ front,
-                                                      const int64_t* __restrict__ n_front_p, double c_s, double sigma,
-                                                      uint8_t* __restrict__ act, int3* __restrict__ tile_sums)
+__global__ void __launch_bounds__(WT) k_walk_round(TreeView T, const MacNode* __restrict__ mac,
+                                                   const MacNode32* __restrict__ mac32, double c_s, double sigma,
+                                                   const int2* __restrict__ front, int2* __restrict__ next,
+                                                   WalkState* S, int round, WalkCaps caps, uint64_t* __restrict__ words,
+                                                   int limit, uint64_t* __restrict__ m2l_t, uint32_t* __restrict__ m2l_s,
+                                                   uint64_t* __restrict__ p2p_t, uint32_t* __restrict__ p2p_s)
 {
     __shared__ int3 s_w[WT / 32];
     __shared__ int3 s_tot;
-    const int64_t n = *n_front_p;
-    const int64_t ntiles = (n + WTILE - 1) / WTILE;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        int3 acc = make_int3(0, 0, 0);
-        for (int r = 0; r < WI; ++r) {
-            const int64_t i = tile * WTILE + (int64_t)r * WT + threadIdx.x;
-            if (i < n) {
-                const int2 pr = front[i];
-                const uint8_t a = classify(T, mac, mac32, pr.x, pr.y, c_s, sigma);
-                act[i] = a;
-                acc = add3(acc, counts_of(a));
-            }
-        }
-        block_excl3(acc, s_w, &s_tot);
-        if (threadIdx.x == 0) tile_sums[tile] = s_tot;
-        __syncthreads();
-    }
-}
-
-// single CTA: exclusive scan of the tile sums; bases of this round's outputs
-__global__ void __launch_bounds__(WT) k_walk_top(int3* __restrict__ tile_sums, const int64_t* __restrict__ n_front_p,
-                                                 int64_t* __restrict__ n_next_p, int64_t* __restrict__ ctr,
-                                                 int64_t* __restrict__ bases, WalkCaps caps)
-{
-    __shared__ int3 s_w[WT / 32];
-    __shared__ int3 s_tot;
-    const int64_t n = *n_front_p;
-    const int64_t ntiles = (n + WTILE - 1) / WTILE;
-    int64_t cx = 0, cy = 0, cz = 0;
-    for (int64_t c0 = 0; c0 < ntiles; c0 += WT) {
-        const int64_t e = c0 + threadIdx.x;
-        const int3 v = e < ntiles ? tile_sums[e] : make_int3(0, 0, 0);
-        const int3 ex = block_excl3(v, s_w, &s_tot);
-        // tile offsets fit in int: a round's outputs are far below 2^31
-        if (e < ntiles) tile_sums[e] = make_int3((int)(ex.x + cx), (int)(ex.y + cy), (int)(ex.z + cz));
-        cx += s_tot.x; cy += s_tot.y; cz += s_tot.z;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const int64_t m0 = ctr[C_M2L], p0 = ctr[C_P2P];
-        bases[0] = m0;
-        bases[1] = p0;
-        if (cx > caps.front || m0 + cy > caps.m2l || p0 + cz > caps.p2p || ctr[C_OVERFLOW]) {
-            ctr[C_OVERFLOW] = 1;
-            *n_next_p = 0;            // stop the walk; the host grows the buffers and reruns it
-            bases[2] = 1;
-        } else {
-            ctr[C_M2L] = m0 + cy;
-            ctr[C_P2P] = p0 + cz;
-            *n_next_p = cx;
-            bases[2] = 0;
-        }
-        ctr[C_ROUNDS] += 1;
-    }
-}
-
-__global__ void __launch_bounds__(WT) k_walk_emit(TreeView T, const int2* __restrict__ front,
-                                                  const int64_t* __restrict__ n_front_p, const uint8_t* __restrict__ act,
-                                                  const int3* __restrict__ tile_off, const int64_t* __restrict__ bases,
-                                                  int2* __restrict__ next, uint64_t* __restrict__ m2l_t,
-                                                  uint32_t* __restrict__ m2l_s, uint64_t* __restrict__ p2p_t,
-                                                  uint32_t* __restrict__ p2p_s)
-{
-    __shared__ int3 s_w[WT / 32];
-    __shared__ int3 s_tot;
+    __shared__ int2 s_pair[WTILE];
     __shared__ uint8_t s_act[WTILE];
-    if (bases[2]) return;         // overflow: write nothing
-    const int64_t n = *n_front_p;
+    __shared__ int64_t s_base[3];
+    __shared__ uint32_t s_tile;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const WalkRec R = S->rec[round];
+    const int64_t n = R.front;
     const int64_t ntiles = (n + WTILE - 1) / WTILE;
-    const int64_t mb = bases[0], pb = bases[1];
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_tile = atomicAdd(&S->ticket[round], 1u);
+        __syncthreads();
+        const int64_t tile = s_tile;
+        if (tile >= ntiles) {
+            if (n == 0 && tile == 0 && threadIdx.x == 0) S->rec[round + 1] = R;     // the walk has ended
+            return;
+        }
         const int64_t t0 = tile * WTILE;
         for (int r = 0; r < WI; ++r) {
-            const int64_t i = t0 + (int64_t)r * WT + threadIdx.x;
-            s_act[r * WT + threadIdx.x] = i < n ? act[i] : A_DROP;
+            const int k = r * WT + threadIdx.x;
+            const int64_t i = t0 + k;
+            uint8_t a = A_DROP;
+            if (i < n) {
+                const int2 pr = front[i];
+                a = classify(T, mac, mac32, pr.x, pr.y, c_s, sigma);
+                s_pair[k] = pr;
+            }
+            s_act[k] = a;
         }
         __syncthreads();
         // thread-local run of WI consecutive items (blocked), then a block scan
         int3 loc[WI];
         int3 acc = make_int3(0, 0, 0);
+#pragma unroll
         for (int r = 0; r < WI; ++r) {
             loc[r] = acc;
             acc = add3(acc, counts_of(s_act[threadIdx.x * WI + r]));
         }
         const int3 ex = block_excl3(acc, s_w, &s_tot);
-        const int3 to = tile_off[tile];
+        if (warp < 3) {          // warp 0: the next frontier, 1: M2L, 2: P2P
+            const int64_t own = warp == 0 ? s_tot.x : warp == 1 ? s_tot.y : s_tot.z;
+            const int64_t from = warp == 0 ? 0 : warp == 1 ? R.m2l : R.p2p;
+            uint64_t* w = words + 3 * tile + warp;
+            if (lane == 0) lb_publish(w, round, LB_OWN, own);
+            int64_t before = 0;
+            if (!lb_before(words + warp, 3, tile, round, limit, &before)) {
+                before = 0;      // the wait ran out: classify the earlier pairs here
+                for (int64_t i = lane; i < t0; i += 32) {
+                    const int3 c = counts_of(classify(T, mac, mac32, front[i].x, front[i].y, c_s, sigma));
+                    before += warp == 0 ? c.x : warp == 1 ? c.y : c.z;
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(FULL, before, o);
+            }
+            if (lane == 0) {
+                lb_publish(w, round, LB_UPTO, before + own);
+                s_base[warp] = from + before;
+            }
+        }
+        __syncthreads();
+        const int64_t bn = s_base[0], bm = s_base[1], bp = s_base[2];
+        const bool fits = bn + s_tot.x <= caps.front && bm + s_tot.y <= caps.m2l && bp + s_tot.z <= caps.p2p;
+        if (tile == ntiles - 1 && threadIdx.x == 0) {
+            if (!fits) S->overflow = 1;       // stop the walk; the host grows the buffers and reruns it
+            S->rec[round + 1].front = fits ? bn + s_tot.x : 0;
+            S->rec[round + 1].m2l = fits ? bm + s_tot.y : R.m2l;
+            S->rec[round + 1].p2p = fits ? bp + s_tot.z : R.p2p;
+        }
+        if (!fits) continue;
+#pragma unroll
         for (int r = 0; r < WI; ++r) {
-            const int64_t i = t0 + (int64_t)threadIdx.x * WI + r;
-            if (i >= n) break;
             const uint8_t a = s_act[threadIdx.x * WI + r];
             if (a == A_DROP) continue;
-            const int2 pr = front[i];
+            const int2 pr = s_pair[threadIdx.x * WI + r];
             const int s = pr.x, t = pr.y;
-            const int64_t on = (int64_t)to.x + ex.x + loc[r].x;
+            const int64_t on = bn + ex.x + loc[r].x;
             if (a == A_SELF) {
                 const int c = T.child0[s];
                 int2* o = next + on;
@@ -319,16 +315,15 @@ __global__ void __launch_bounds__(WT) k_walk_emit(TreeView T, const int2* __rest
                 const int c = T.child0[t];
                 for (int u = 0; u < 4; ++u) next[on + u] = make_int2(s, c + u);
             } else if (a == A_M2L) {
-                const int64_t om = mb + to.y + ex.y + loc[r].y;
+                const int64_t om = bm + ex.y + loc[r].y;
                 m2l_t[om] = (uint64_t)t;
                 m2l_s[om] = (uint32_t)s;
             } else {
-                const int64_t op = pb + to.z + ex.z + loc[r].z;
+                const int64_t op = bp + ex.z + loc[r].z;
                 p2p_t[op] = (uint64_t)t;
                 p2p_s[op] = (uint32_t)s;
             }
         }
-        __syncthreads();
     }
 }
 
@@ -359,9 +354,9 @@ __global__ void k_pad_pairs(uint64_t* __restrict__ t, uint32_t* __restrict__ src
 }
 
 // Graph mode: a walk that overflowed its capacities or left a frontier voids the solve.
-__global__ void k_walk_check(const int64_t* __restrict__ ctr, int left_slot, DevCounts* dc)
+__global__ void k_walk_check(const WalkState* __restrict__ S, int rounds, DevCounts* dc)
 {
-    if (ctr[C_OVERFLOW] || ctr[left_slot] != 0) dc->overflow = 1;
+    if (S->overflow || S->rec[rounds].front != 0) dc->overflow = 1;
 }
 
 inline unsigned grid_for(int64_t n, int threads = 256)
@@ -392,12 +387,12 @@ cudaError_t build_lists(sfmm_plan_s* P, const TreeView& T, double c_s, double c_
     cudaError_t e;
     const int depth = P->gm ? (int)P->cap.levels : (int)P->level_start.size() - 2;
     const int rounds = 2 * depth + 4;
-    int64_t* ctr = P->small.as<int64_t>() + 24;      // [24..29] counters, [30..32] bases
-    int64_t* bases = ctr + 6;
+    WalkState* S = reinterpret_cast<WalkState*>(P->small.as<int64_t>() + SM_WALK);
+    const int limit = P->opt.wait_limit > 0 ? P->opt.wait_limit : LB_POLLS;
     // capacities: start from the last solve's needs, or from the node count
     int64_t cap_front = std::max<int64_t>(P->walk_cap_front, std::max<int64_t>(4096, 32 * P->n_nodes));
     int64_t cap_m2l = std::max<int64_t>(P->walk_cap_m2l, std::max<int64_t>(4096, 48 * P->n_nodes));
-    int64_t cap_p2p = std::max<int64_t>(P->walk_cap_p2p, std::max<int64_t>(4096, 16 * P->n_nodes));
+    int64_t cap_p2p = std::max<int64_t>(P->walk_cap_p2p, std::max<int64_t>(4096, 24 * P->n_nodes));
     if (P->gm) {
         cap_front = P->cap.front;
         cap_m2l = P->cap.m2l;
@@ -410,50 +405,43 @@ cudaError_t build_lists(sfmm_plan_s* P, const TreeView& T, double c_s, double c_
                                                      P->macn32.as<MacNode32>());
     count_launch();
     for (int attempt = 0; attempt < 8; ++attempt) {
+        const size_t wb = (size_t)((cap_front + WTILE - 1) / WTILE) * 3 * 8;
         if ((e = ensure(P->fa, (size_t)cap_front * 8)) || (e = ensure(P->fb, (size_t)cap_front * 8)) ||
-            (e = ensure(P->act, (size_t)cap_front)) ||
-            (e = ensure(P->c_next, (size_t)((cap_front + WTILE - 1) / WTILE + 1) * sizeof(int3))) ||
+            (e = ensure(P->wwords, wb)) || (e = cudaMemsetAsync(P->wwords.p, 0, wb, s)) ||
             (e = ensure(P->m2l_t, (size_t)cap_m2l * 8)) || (e = ensure(P->m2l_s, (size_t)cap_m2l * 4)) ||
             (e = ensure(P->p2p_t, (size_t)cap_p2p * 8)) || (e = ensure(P->p2p_s, (size_t)cap_p2p * 4)))
             return e;
-        k_init_frontier<<<1, 160, 0, s>>>(P->fa.as<int2>(), ctr); count_launch();
+        k_init_frontier<<<1, 160, 0, s>>>(P->fa.as<int2>(), S); count_launch();
         WalkCaps caps{cap_front, cap_m2l, cap_p2p};
-        const unsigned grid = 152 * 4;
         for (int r = 0; r < rounds; ++r) {
-            const int2* front = (r & 1) ? P->fb.as<int2>() : P->fa.as<int2>();
-            int2* next = (r & 1) ? P->fa.as<int2>() : P->fb.as<int2>();
-            int64_t* nf = ctr + ((r & 1) ? C_FRONT1 : C_FRONT0);
-            int64_t* nn = ctr + ((r & 1) ? C_FRONT0 : C_FRONT1);
-            k_walk_classify<<<grid, WT, 0, s>>>(T, P->macn.as<MacNode>(), P->macn32.as<MacNode32>(), front, nf, c_s,
-                                                P->opt.sigma,
-                                                P->act.as<uint8_t>(),
-                                                P->c_next.as<int3>());
-            count_launch();
-            k_walk_top<<<1, WT, 0, s>>>(P->c_next.as<int3>(), nf, nn, ctr, bases, caps); count_launch();
-            k_walk_emit<<<grid, WT, 0, s>>>(T, front, nf, P->act.as<uint8_t>(), P->c_next.as<int3>(), bases, next,
-                                            P->m2l_t.as<uint64_t>(), P->m2l_s.as<uint32_t>(), P->p2p_t.as<uint64_t>(),
-                                            P->p2p_s.as<uint32_t>());
-            count_launch();
+            int2* f[2] = {P->fa.as<int2>(), P->fb.as<int2>()};
+            k_walk_round<<<152 * 4, WT, 0, s>>>(T, P->macn.as<MacNode>(), P->macn32.as<MacNode32>(), c_s, P->opt.sigma,
+                                                f[r & 1], f[(r + 1) & 1], S, r, caps, P->wwords.as<uint64_t>(), limit,
+                                                P->m2l_t.as<uint64_t>(), P->m2l_s.as<uint32_t>(),
+                                                P->p2p_t.as<uint64_t>(), P->p2p_s.as<uint32_t>()); count_launch();
         }
         if ((e = cudaGetLastError())) return e;
         if (P->gm) {
-            k_walk_check<<<1, 1, 0, s>>>(ctr, (rounds & 1) ? C_FRONT1 : C_FRONT0, P->dcnt.as<DevCounts>()); count_launch();
+            k_walk_check<<<1, 1, 0, s>>>(S, rounds, P->dcnt.as<DevCounts>()); count_launch();
             P->n_m2l = cap_m2l;
             P->n_p2p = cap_p2p;
-            P->d_m2l = ctr + C_M2L;
-            P->d_p2p = ctr + C_P2P;
+            P->d_m2l = &S->rec[rounds].m2l;
+            P->d_p2p = &S->rec[rounds].p2p;
             break;
         }
-        int64_t h[6];
-        if ((e = cudaMemcpyAsync(h, ctr, sizeof h, cudaMemcpyDeviceToHost, s))) return e;
+        // the walk's state, and with it the counts of leaves and items (SM_COLLECT)
+        const WalkState* h = reinterpret_cast<const WalkState*>(P->h_small + SM_WALK);
+        if ((e = cudaMemcpyAsync(P->h_small + SM_COLLECT, P->small.as<int64_t>() + SM_COLLECT,
+                                 (SM_WALK - SM_COLLECT) * 8 + sizeof(WalkState), cudaMemcpyDeviceToHost, s)))
+            return e;
         if ((e = cudaStreamSynchronize(s))) return e;
-        const int64_t left = h[(rounds & 1) ? C_FRONT1 : C_FRONT0];
-        if (!h[C_OVERFLOW] && left == 0) {
-            P->n_m2l = h[C_M2L];
-            P->n_p2p = h[C_P2P];
+        const WalkRec& end = h->rec[rounds];
+        if (!h->overflow && end.front == 0) {
+            P->n_m2l = end.m2l;
+            P->n_p2p = end.p2p;
             break;
         }
-        if (!h[C_OVERFLOW] && left != 0) return cudaErrorUnknown;   // cannot happen: the round bound is exact
+        if (!h->overflow) return cudaErrorUnknown;   // cannot happen: the round bound is exact
         cap_front *= 2;
         cap_m2l *= 2;
         cap_p2p *= 2;
