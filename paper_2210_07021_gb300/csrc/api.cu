@@ -31,9 +31,8 @@ cudaError_t launch_pair_geo(const TreeView& T, const float* g32, const uint64_t*
 cudaError_t launch_child_geo(const TreeView& T, const float* g32, void* m2m, void* l2l, int ek, cudaStream_t s);
 cudaError_t launch_src_offsets(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl,
                                const double4_32a* src, float4* off, cudaStream_t s);
-cudaError_t launch_p2m(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl,
-                       const double4_32a* src, const float4* off, const float4* log_tab, void* mpole, int p, int ek,
-                       cudaStream_t s);
+cudaError_t launch_p2m32(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const float4* off,
+                         float* mpole, int p, cudaStream_t s);
 cudaError_t launch_m2m(const TreeView& T, int a, int b, int lvl, int p, const double* tables, const void* geo,
                        void* mpole, int ek, cudaStream_t s);
 cudaError_t launch_m2m_narrow(const TreeView& T, int a, int b, int lvl, int p, const void* tables, const void* geo,
@@ -42,9 +41,15 @@ cudaError_t launch_l2l_df_narrow(const TreeView& T, int a, int b, int lvl, int p
                                  const double* acc, void* local, cudaStream_t s);
 cudaError_t launch_m2l(const TreeView& T, const int64_t* off, const uint32_t* srcs, int p, const double* tables,
                        const void* geo, const void* mpole, void* local, int ek, cudaStream_t s);
+size_t m2l64_part_bytes(int64_t n_pairs);
+cudaError_t launch_m2l_pair64(const TreeView& T, int64_t n_pairs, const int64_t* d_n, const uint64_t* ptgt,
+                              const uint32_t* psrc, const int64_t* off, const void* geo, const double* mpole, int p,
+                              double* local, double* part, uint32_t* leftover, uint32_t* n_left, cudaStream_t s);
+cudaError_t launch_p2m64_leaf(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl,
+                              const double4_32a* src, int p, double* mpole, cudaStream_t s);
 cudaError_t launch_m2l_list(const uint64_t* ptgt, const uint32_t* psrc, const uint32_t* list, const uint32_t* n_list,
                             int64_t max_list, int p, const double* tables, const void* geo, const void* mpole,
-                            void* local, cudaStream_t s);
+                            void* local, int ek, cudaStream_t s);
 cudaError_t launch_m2l_tc(int64_t n_pairs, const uint64_t* ptgt, const uint32_t* psrc, const void* geo,
                           const void* mpole, void* local, int p, uint32_t* leftover, uint32_t* n_leftover,
                           uint32_t* tile_ctr, int* status, int wait_limit, cudaStream_t s);
@@ -461,8 +466,10 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     else if (dfe) e = launch_p2m_df_leaf(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->soff.as<float4>(),
                                          adj_df ? P->dip4.as<float4>() : nullptr, P->logtab.as<float4>(), p,
                                          P->mpole.p, s);
-    else e = launch_p2m(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->src4.as<double4_32a>(),
-                        P->soff.as<float4>(), P->logtab.as<float4>(), P->mpole.p, p, ek, s);
+    else if (fp32) e = launch_p2m32(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->soff.as<float4>(),
+                                    P->mpole.as<float>(), p, s);
+    else e = launch_p2m64_leaf(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->src4.as<double4_32a>(), p,
+                               P->mpole.as<double>(), s);
     if (e) return cuda_fail(P, e, "P2M");
     // graph mode: every level up to the capacity, each launch sized by the level-width capacity
     const int depth = P->gm ? (int)P->cap.levels : (int)P->level_start.size() - 2;
@@ -552,6 +559,22 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         if ((e = launch_m2l_left_df(T, m2l_t, m2l_s, P->leftover.as<uint32_t>(), n_left, P->n_m2l, p,
                                     P->tables.as<double>(), P->mpole.p, P->m2l_acc.as<double>(), s)))
             return cuda_fail(P, e, "M2L (pairs near antipodes)");
+    } else if (!fp32) {
+        // FP64: one thread per pair, each box's sum in the list's order; pairs with centres
+        // antipodal to rounding go to the warp kernel
+        uint32_t* n_left = reinterpret_cast<uint32_t*>(P->small.as<int64_t>() + SM_LEFT);
+        if ((e = ensure(P->m2l_acc, std::max<size_t>(m2l64_part_bytes(P->n_m2l), 8))) ||
+            (e = ensure(P->leftover, (size_t)std::max<int64_t>(P->n_m2l, 1) * 4)))
+            return cuda_fail(P, e, "alloc");
+        if ((e = cudaMemsetAsync(n_left, 0, 4, s))) return cuda_fail(P, e, "memset");
+        if ((e = launch_pair_geo(T, P->geom32.as<float>(), m2l_t, m2l_s, P->n_m2l, P->d_m2l, P->m2l_geo.p, ek, s)))
+            return cuda_fail(P, e, "pair geometry");
+        if ((e = launch_m2l_pair64(T, P->n_m2l, P->d_m2l, m2l_t, m2l_s, P->m2l_off.as<int64_t>(), P->m2l_geo.p,
+                                   P->mpole.as<double>(), p, P->local.as<double>(), P->m2l_acc.as<double>(),
+                                   P->leftover.as<uint32_t>(), n_left, s)) ||
+            (e = launch_m2l_list(m2l_t, m2l_s, P->leftover.as<uint32_t>(), n_left, P->n_m2l, p, P->tables.as<double>(),
+                                 P->m2l_geo.p, P->mpole.p, P->local.p, ek, s)))
+            return cuda_fail(P, e, "M2L");
     } else if ((e = cudaMemsetAsync(P->local.p, 0, (size_t)nn * EXP_STRIDE * esz, s)) ||
                (e = launch_pair_geo(T, P->geom32.as<float>(), m2l_t, m2l_s, P->n_m2l, P->d_m2l, P->m2l_geo.p, ek,
                                     s))) {
@@ -566,7 +589,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
                                n_left, tile_ctr, status, P->opt.wait_limit, s)))
             return cuda_fail(P, e, "M2L (tensor cores)");
         if ((e = launch_m2l_list(m2l_t, m2l_s, P->leftover.as<uint32_t>(), n_left, P->n_m2l, p, P->tables.as<double>(),
-                                 P->m2l_geo.p, P->mpole.p, P->local.p, s)))
+                                 P->m2l_geo.p, P->mpole.p, P->local.p, ek, s)))
             return cuda_fail(P, e, "M2L (leftover pairs)");
     } else if ((e = launch_m2l(T, P->m2l_off.as<int64_t>(), m2l_s, p, P->tables.as<double>(), P->m2l_geo.p, P->mpole.p,
                                P->local.p, ek, s))) {

@@ -14,6 +14,7 @@ __device__ __forceinline__ dflt add_lazy(dflt a, dflt b)
     const dflt s = dfl_two_sum(a.h, b.h);
     return dflt(s.h, __fadd_rn(__fadd_rn(a.l, b.l), s.l));
 }
+__device__ __forceinline__ double add_lazy(double a, double b) { return a + b; }
 // renormalisation safe for any magnitudes of the two parts
 __device__ __forceinline__ dflt renorm(dflt a) { return dfl_two_sum(a.h, a.l); }
 
@@ -38,8 +39,8 @@ __device__ __forceinline__ void cmul_df(dflt ar, dflt ai, dflt br, dflt bi, dflt
 // registers) and its passes are a runtime loop, with the j < i positions
 // left alone: about a quarter of the code of fully unrolled passes (which
 // overflows the instruction cache at P = 20), for about 15 % more additions.
-template <int P>
-__device__ __forceinline__ void pascal_up(dflt* c)
+template <int P, typename R>
+__device__ __forceinline__ void pascal_up(R* c)
 {
 #pragma unroll
     for (int g = 0; g < P; g += 4) {
@@ -54,8 +55,8 @@ __device__ __forceinline__ void pascal_up(dflt* c)
 
 // Its dual on x_m = c[m + 1], m = 0..P-1: for i = 1..P-1, for j = P-1 down to i,
 // x_j += x_{j-1} (x_k = sum_{m <= k} C(k, m) x_m), grouped the same way.
-template <int P>
-__device__ __forceinline__ void pascal_down(dflt* c)
+template <int P, typename R>
+__device__ __forceinline__ void pascal_down(R* c)
 {
 #pragma unroll
     for (int g = 1; g < P; g += 4) {

@@ -36,6 +36,8 @@
 #include "dfloat.cuh"
 #include "xgeo.cuh"
 
+#include <algorithm>
+
 namespace sfmm {
 
 namespace {
@@ -648,53 +650,6 @@ __device__ __forceinline__ void atomic_exp(ST* e, int lane, int p, R C, R Q, cx<
 }
 
 // ----------------------------------------------------------------- P2M
-// FP64: from the key-sorted FP64 positions.
-template <int P, typename ST>
-__global__ void k_p2m(TreeView T, const int* __restrict__ leaves, int64_t n_cap, const int64_t* d_nl,
-                      const double4_32a* __restrict__ src, ST* __restrict__ mpole)
-{
-    const int64_t n_leaves = dcount(d_nl, n_cap);
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n_leaves; w += (int64_t)gridDim.x * blockDim.x) {
-        const int node = leaves[w];
-        const double* g = T.geom + (size_t)node * GEOM_STRIDE;
-        const double cx_ = g[0], cy = g[1], cz = g[2];
-        const double inv_r = 1.0 / g[10];
-        cd A[P];
-#pragma unroll
-        for (int l = 0; l < P; ++l) A[l] = mk(0.0, 0.0);
-        double Csum = 0.0, Qsum = 0.0;
-        const int f = T.first[node], n = T.count[node];
-        for (int j = f; j < f + n; ++j) {
-            const double4_32a y = src[j];
-            const double dx = y.x - cx_, dy = y.y - cy, dz = y.z - cz;
-            const double d2 = dx * dx + dy * dy + dz * dz;
-            const double den = 2.0 - 0.5 * d2;   // 1 + y.c
-            const double zr = (dx * g[3] + dy * g[4] + dz * g[5]) / den * inv_r;
-            const double zi = (dx * g[6] + dy * g[7] + dz * g[8]) / den * inv_r;
-            const double q = y.w;
-            Qsum += q;
-            Csum += q * log1p(-0.25 * d2);        // 2 log cos(theta/2)
-            cd zp = mk(q, 0.0);
-#pragma unroll
-            for (int l = 0; l < P; ++l) {
-                zp = cmul(zp, mk(zr, zi));
-                A[l] = cadd(A[l], zp);
-            }
-        }
-        ST* e = mpole + (size_t)node * EXP_STRIDE;
-        const double Q = INV4PI * Qsum;
-        e[0] = ST(INV4PI * Csum - Q * LOG2);
-        e[1] = ST(Q);
-#pragma unroll
-        for (int l = 0; l < P; ++l) {
-            const double s = -INV4PI / (double)(l + 1);
-            e[2 + 2 * l] = ST(s * A[l].x);
-            e[3 + 2 * l] = ST(s * A[l].y);
-        }
-        for (int l = P; l < PMAX; ++l) { e[2 + 2 * l] = ST(0.0); e[3 + 2 * l] = ST(0.0); }
-    }
-}
-
 // Adjoint (FP64): charges h and tangent dipoles g at the sources.  A dipole's
 // potential g . grad_x G(x, y) is the derivative of the point-mass potential
 // along g, so its multipole is the derivative of Lemma 1 along g: with
@@ -755,63 +710,6 @@ __global__ void k_p2m_adj(TreeView T, const int* __restrict__ leaves, int64_t n_
             e[3 + 2 * l] = -INV4PI * (s * A[l].y + B[l].y);
         }
         for (int l = P; l < PMAX; ++l) { e[2 + 2 * l] = 0.0; e[3 + 2 * l] = 0.0; }
-    }
-}
-
-// Double-float (1e-10 mixed path): from each source's (hi, lo) offset to its
-// leaf centre, z^l by repeated double-float products, log(1 - d^2/4) = 2 log
-// cos(theta/2) by the table-driven double-float logarithm (tab: as in the
-// evaluation).  One thread per leaf.
-template <int P>
-__global__ void __launch_bounds__(128) k_p2m_df(TreeView T, const int* __restrict__ leaves, int64_t n_leaves,
-                                                const float4* __restrict__ off, const float4* __restrict__ log_tab,
-                                                dflt* __restrict__ mpole)
-{
-    __shared__ float4 s_tab[129];
-    for (int i = threadIdx.x; i < 129; i += blockDim.x) s_tab[i] = log_tab[i];
-    __syncthreads();
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n_leaves; w += (int64_t)gridDim.x * blockDim.x) {
-        const int node = leaves[w];
-        const double* g = T.geom + (size_t)node * GEOM_STRIDE;
-        const dflt etx(g[3]), ety(g[4]), etz(g[5]), epx(g[6]), epy(g[7]), epz(g[8]);
-        const dflt inv_r(1.0 / g[10]);
-        dflt Ar[P], Ai[P];
-#pragma unroll
-        for (int l = 0; l < P; ++l) { Ar[l] = dflt(0.f, 0.f); Ai[l] = dflt(0.f, 0.f); }
-        dflt Csum(0.f, 0.f), Qsum(0.f, 0.f);
-        const int f = T.first[node], n = T.count[node];
-        for (int j = f; j < f + n; ++j) {
-            const float4 h = off[2 * (size_t)j], lo = off[2 * (size_t)j + 1];
-            const dflt dx(h.x, lo.x), dy(h.y, lo.y), dz(h.z, lo.z), q(h.w, lo.w);
-            const dflt d2 = dx * dx + dy * dy + dz * dz;
-            const dflt sc = inv_r / (dflt(2.f, 0.f) - d2 * 0.5f);            // 1/(r (1 + y.c))
-            const dflt zr = (dx * etx + dy * ety + dz * etz) * sc;
-            const dflt zi = (dx * epx + dy * epy + dz * epz) * sc;
-            Qsum += q;
-            dfl_mac(Csum, q, dfl_log_lazy(dflt(1.f, 0.f) - d2 * 0.25f, s_tab));   // 2 log cos(theta/2)
-            dflt pr = q, pi(0.f, 0.f);
-#pragma unroll
-            for (int l = 0; l < P; ++l) {
-                const dflt nr = pr * zr - pi * zi, ni = pr * zi + pi * zr;
-                pr = nr;
-                pi = ni;
-                Ar[l] += pr;
-                Ai[l] += pi;
-            }
-        }
-        Csum = dfl_norm(Csum);
-        dflt* e = mpole + (size_t)node * EXP_STRIDE;
-        const dflt i4p(INV4PI), l2(LOG2);
-        const dflt Q = i4p * Qsum;
-        e[0] = i4p * Csum - Q * l2;
-        e[1] = Q;
-#pragma unroll
-        for (int l = 0; l < P; ++l) {
-            const dflt sl = -(i4p / dflt(l + 1));
-            e[2 + 2 * l] = sl * Ar[l];
-            e[3 + 2 * l] = sl * Ai[l];
-        }
-        for (int l = P; l < PMAX; ++l) { e[2 + 2 * l] = dflt(0.f, 0.f); e[3 + 2 * l] = dflt(0.f, 0.f); }
     }
 }
 
@@ -1203,19 +1101,12 @@ cudaError_t launch_src_offsets(const TreeView& T, const int* leaves, int64_t n_l
 }
 
 // mpole: double (FP64 path), float (mixed path) or double-float storage (1e-10 mixed path)
-cudaError_t launch_p2m(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl,
-                       const double4_32a* src, const float4* off, const float4* log_tab, void* mpole, int p, int ek,
-                       cudaStream_t s)
+cudaError_t launch_p2m32(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const float4* off,
+                         float* mpole, int p, cudaStream_t s)
 {
     if (n_leaves == 0) return cudaSuccess;
     const unsigned g = grid_for(n_leaves, 128);
-#define P2M_CASE(PP)                                                                                       \
-    case PP:                                                                                               \
-        if (ek == EXP_F32) k_p2m32<PP><<<g, 128, 0, s>>>(T, leaves, n_leaves, d_nl, off, static_cast<float*>(mpole)); \
-        else if (ek == EXP_DF) k_p2m_df<PP><<<g, 128, 0, s>>>(T, leaves, n_leaves, off, log_tab, static_cast<dflt*>(mpole)); \
-        else k_p2m<PP, double><<<g, 128, 0, s>>>(T, leaves, n_leaves, d_nl, src, static_cast<double*>(mpole)); \
-        count_launch();                                                                                    \
-        break;
+#define P2M_CASE(PP) case PP: k_p2m32<PP><<<g, 128, 0, s>>>(T, leaves, n_leaves, d_nl, off, mpole); count_launch(); break;
     switch ((p + 3) / 4 * 4) {
         P2M_CASE(4) P2M_CASE(8) P2M_CASE(12) P2M_CASE(16) P2M_CASE(20) P2M_CASE(24) P2M_CASE(28) P2M_CASE(32)
         default: return cudaErrorInvalidValue;
@@ -1295,24 +1186,27 @@ cudaError_t launch_m2l(const TreeView& T, const int64_t* off, const uint32_t* sr
     if (ek == EXP_F32)
         k_m2l<float, XGeo32, float><<<g, 128, 0, s>>>(T, off, srcs, p, tables, static_cast<const XGeo32*>(geo),
                                                       static_cast<const float*>(mpole), static_cast<float*>(local));
-    else if (ek == EXP_DF)
-        k_m2l<dflt, XGeoDF, dflt><<<g, 128, 0, s>>>(T, off, srcs, p, tables, static_cast<const XGeoDF*>(geo),
-                                                    static_cast<const dflt*>(mpole), static_cast<dflt*>(local));
     else
-        k_m2l<double, XGeo, double><<<g, 128, 0, s>>>(T, off, srcs, p, tables, static_cast<const XGeo*>(geo),
-                                                      static_cast<const double*>(mpole), static_cast<double*>(local));
+        return cudaErrorInvalidValue;             // the FP64 and double-float paths: one thread per pair
     count_launch();
     return cudaGetLastError();
 }
 
 cudaError_t launch_m2l_list(const uint64_t* ptgt, const uint32_t* psrc, const uint32_t* list, const uint32_t* n_list,
                             int64_t max_list, int p, const double* tables, const void* geo, const void* mpole,
-                            void* local, cudaStream_t s)
+                            void* local, int ek, cudaStream_t s)
 {
     if (max_list == 0) return cudaSuccess;
-    k_m2l_list<float, XGeo32, float><<<grid_for(max_list < 152 * 64 ? max_list : 152 * 64, 4), 128, 0, s>>>(
-        ptgt, psrc, list, n_list, p, tables, static_cast<const XGeo32*>(geo), static_cast<const float*>(mpole),
-        static_cast<float*>(local));
+    // FP64 lists hold a few antipodal pairs at most
+    const unsigned g = grid_for(ek == EXP_F64 ? std::min<int64_t>(max_list, 152 * 4) : std::min<int64_t>(max_list, 152 * 64), 4);
+    if (ek == EXP_F64)
+        k_m2l_list<double, XGeo, double><<<g, 128, 0, s>>>(ptgt, psrc, list, n_list, p, tables,
+                                                           static_cast<const XGeo*>(geo),
+                                                           static_cast<const double*>(mpole), static_cast<double*>(local));
+    else
+        k_m2l_list<float, XGeo32, float><<<g, 128, 0, s>>>(ptgt, psrc, list, n_list, p, tables,
+                                                           static_cast<const XGeo32*>(geo),
+                                                           static_cast<const float*>(mpole), static_cast<float*>(local));
     count_launch();
     return cudaGetLastError();
 }
