@@ -259,9 +259,10 @@ int sfmm_order(sfmm_plan_t plan);
  *   ms[8]                    : device time of the phases on the plan's stream (only
  *                              while timing is on): keys+sort, tree+geometry, up-pass,
  *                              lists, M2L, L2L, evaluation, total
- *   near_ms                  : SFMM_MIXED: device time of the near-field kernel, which
- *                              runs on the auxiliary stream beside M2L and L2L (its
- *                              evaluation phase is then the double-float finish); else 0
+ *   near_ms                  : device time of the near-field kernel where it runs on the
+ *                              auxiliary stream beside M2L and L2L (every forward solve
+ *                              but SFMM_FP32's; the evaluation phase is then L2P and the
+ *                              combination); else 0
  */
 typedef struct {
     int64_t n_nodes, n_leaves, depth, n_m2l, n_p2p, p2p_interactions, launches;

@@ -105,7 +105,9 @@ cudaError_t launch_eval(const TreeView& T, const int2* items, int64_t n_items, c
                         const double4_32a* tgt,
                         const uint32_t* tperm, const int64_t* p2p_off, const uint32_t* p2p_src, const double* local,
                         const double* mpole, int p, int zero_mean, double sigma, double* psi, double* alpha,
-                        double* gamma, double* mu, const double2* log_tab, unsigned long long* leaf_ctr, cudaStream_t s);
+                        double* gamma, double* mu, const double2* log_tab, double* nf, int* tleaf, int64_t M, int what,
+                        unsigned long long* leaf_ctr, cudaStream_t s);
+size_t near64_bytes(bool shear, bool npm);
 
 namespace {
 std::atomic<int64_t> g_launches{0};
@@ -471,6 +473,8 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     else e = launch_p2m64_leaf(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->src4.as<double4_32a>(), p,
                                P->mpole.as<double>(), s);
     if (e) return cuda_fail(P, e, "P2M");
+    const bool near_early64 = !fp32 && !dfe && !adj;
+    if (near_early64 && (e = cudaEventRecord(P->ev_p2m, s))) return cuda_fail(P, e, "event");
     // graph mode: every level up to the capacity, each launch sized by the level-width capacity
     const int depth = P->gm ? (int)P->cap.levels : (int)P->level_start.size() - 2;
     const int W = (int)P->cap.width;
@@ -504,11 +508,24 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
                                     P->aux)))
             return cuda_fail(P, e, "offsets");
     }
-    // 1e-6 and 1e-10 paths: the near field needs none of the far field (their double-float
-    // finish does), so it runs here, on the auxiliary stream, beside M2L and L2L
+    // the near field needs none of the far field but the leaves' masses (the finish does), so
+    // it runs here, on the auxiliary stream, beside M2L and L2L (all-FP32 path and adjoint: not)
     unsigned long long* leaf_ctr = reinterpret_cast<unsigned long long*>(P->small.as<int64_t>() + SM_ITEM_CTR);
     const bool near_early = near32 && !fp32 && !adj;
     const bool near_early_df = dfe && !near32 && !adj;
+    if (near_early64) {
+        if ((e = ensure(P->nfbuf, (size_t)M * near64_bytes(gamma, P->opt.sigma > 0.0))) ||
+            (e = ensure(P->tleaf, (size_t)M * 4)))
+            return cuda_fail(P, e, "alloc");
+        if ((e = cudaStreamWaitEvent(P->aux, P->ev_p2m, 0))) return cuda_fail(P, e, "wait");
+        if (P->timing) cudaEventRecord(P->ev_near[0], P->aux);
+        if ((e = launch_eval(T, P->items.as<int2>(), P->n_items, d_nit, P->src4.as<double4_32a>(),
+                             P->tgt4.as<double4_32a>(), tperm, P->p2p_off.as<int64_t>(), p2p_s, P->local.as<double>(),
+                             P->mpole.as<double>(), p, P->opt.zero_mean, P->opt.sigma, psi, alpha, gamma, mu,
+                             log64_tab(P), P->nfbuf.as<double>(), P->tleaf.as<int>(), M, EVAL_NEAR, leaf_ctr, P->aux)))
+            return cuda_fail(P, e, "near field");
+        if (P->timing) cudaEventRecord(P->ev_near[1], P->aux);
+    }
     if (near_early_df) {
         if ((e = ensure(P->nfbuf, (size_t)M * 48)) || (e = ensure(P->tleaf, (size_t)M * 4)))
             return cuda_fail(P, e, "alloc");
@@ -642,7 +659,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     else e = launch_eval(T, P->items.as<int2>(), P->n_items, d_nit, P->src4.as<double4_32a>(),
                          P->tgt4.as<double4_32a>(), tperm, P->p2p_off.as<int64_t>(), p2p_s, P->local.as<double>(),
                          P->mpole.as<double>(), p, P->opt.zero_mean, P->opt.sigma, psi, alpha, gamma, mu,
-                         log64_tab(P), leaf_ctr, s);
+                         log64_tab(P), P->nfbuf.as<double>(), P->tleaf.as<int>(), M, EVAL_FINISH, leaf_ctr, s);
     if (e) return cuda_fail(P, e, "evaluation");
     if (P->gm) {          // no synchronisation: the caller reads the overflow flag after the work
         P->stats.launches = launch_total() - launches0;
@@ -669,7 +686,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     if (tc_status && *P->h_status)
         return fail(P, SFMM_ETIMEOUT, "a bounded wait of the tensor-core M2L kernel ran out");
     tm.finish();
-    if (P->timing && (near_early || near_early_df)) {
+    if (P->timing && (near_early || near_early_df || near_early64)) {
         float ms = 0.f;
         if (cudaEventElapsedTime(&ms, P->ev_near[0], P->ev_near[1]) == cudaSuccess) P->stats.near_ms = ms;
     }
@@ -778,6 +795,7 @@ sfmm_status sfmm_plan(sfmm_plan_t* out, int max_depth, int order_p, double tol, 
         (e = cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming)) ||
         (e = cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming)) ||
         (e = cudaEventCreateWithFlags(&P->ev_m2l, cudaEventDisableTiming)) ||
+        (e = cudaEventCreateWithFlags(&P->ev_p2m, cudaEventDisableTiming)) ||
         (e = cudaEventCreate(&P->ev_near[0])) || (e = cudaEventCreate(&P->ev_near[1]))) {
         std::lock_guard<std::mutex> g(g_err_mu);
         g_plan_err = std::string("CUDA error at plan time: ") + cudaGetErrorString(e);
@@ -1013,6 +1031,7 @@ void sfmm_destroy(sfmm_plan_t plan)
     if (plan->ev_fork) cudaEventDestroy(plan->ev_fork);
     if (plan->ev_join) cudaEventDestroy(plan->ev_join);
     if (plan->ev_m2l) cudaEventDestroy(plan->ev_m2l);
+    if (plan->ev_p2m) cudaEventDestroy(plan->ev_p2m);
     for (cudaEvent_t ev : plan->ev_near)
         if (ev) cudaEventDestroy(ev);
     if (plan->aux) cudaStreamDestroy(plan->aux);

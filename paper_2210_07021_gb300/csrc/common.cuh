@@ -65,8 +65,8 @@ cudaError_t launch_keys(const double* xyz, int64_t n, uint64_t* keys, uint32_t* 
 // Number format of the expansions and translations: FP64, FP32 (mixed path)
 // or double-float pairs of FP32 (1e-10 mixed path).
 enum { EXP_F64 = 0, EXP_F32 = 1, EXP_DF = 2 };
-// the parts launch_eval32 / launch_eval_df launch: the near-field kernel, the
-// double-float finish (L2P and the combination, one thread per target)
+// the parts launch_eval / launch_eval32 / launch_eval_df launch: the near-field
+// kernel, the finish (L2P and the combination, one thread per target)
 enum { EVAL_NEAR = 1, EVAL_FINISH = 2 };
 
 // --------------------------------------------------------------- the tree
@@ -155,7 +155,8 @@ struct sfmm_plan_s {
     std::vector<sfmm_plan_s*> lanes;       // batch lanes: solvers on their own streams
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaEvent_t ev_m2l = nullptr;          // the M2L list is sorted (recorded by build_lists)
-    cudaEvent_t ev_near[2] = {nullptr, nullptr};   // timing: around the 1e-6 path's near-field kernel
+    cudaEvent_t ev_p2m = nullptr;          // P2M is done (the FP64 near field reads the leaves' masses)
+    cudaEvent_t ev_near[2] = {nullptr, nullptr};   // timing: around the near-field kernel on the auxiliary stream
     bool forked = false;                   // the next solve finds the auxiliary stream already forked
                                            // (the host entry point copies the targets there)
     std::string err;
@@ -168,7 +169,7 @@ struct sfmm_plan_s {
         int64_t nodes = 0, width = 0, levels = 0, m2l = 0, p2p = 0, front = 0;
     } cap;
     sfmm::Buf dcnt;
-    sfmm::Buf nfbuf, tleaf;                // 1e-6 path: near-field sums and leaf per sorted target
+    sfmm::Buf nfbuf, tleaf;                // near-field sums and leaf per sorted target
     int64_t last_max_width = 0;            // widest tree level of the last synchronised solve
     sfmm::GraphState* graph = nullptr;     // graph-launched shells (graph.cu), or NULL
     sfmm_stats stats{};

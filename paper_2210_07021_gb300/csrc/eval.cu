@@ -70,6 +70,9 @@ struct EvalArgs {
     unsigned long long* leaf_ctr;   // zero at launch: the warps take items from it one at a time
     double npm_s;             // Near Particle Model: sin^2(sigma/2) (NPM kernels only)
     const double2* log_tab;   // (1/c_j, log c_j), see fp64ops.cuh
+    double* nf;               // near-field sums per sorted target (near_width doubles each)
+    int* tleaf;               // and its leaf
+    int64_t M;                // sorted targets
 };
 
 __device__ __forceinline__ double group_sum(double v, int lpt)
@@ -127,29 +130,46 @@ __device__ __noinline__ double near_mass_of(const EvalArgs& A, int64_t nb0, int6
     return q;
 }
 
+// Near-field sums of one target as k_eval writes them and k_finish64 reads them: sums
+// of q d / d^2 (3), of q, of q log d^2; then the NPM sum of f q, or the shear's six sums
+// of q d d^T / d^4 and the mass left out.
+__host__ __device__ constexpr int near_width(bool shear, bool npm) { return shear ? 12 : npm ? 6 : 5; }
+
 // The FP64 pipe bounds this kernel (fp64ops.cuh): 13 FP64 instructions per pair of
 // a run of equal masses (3 differences, 3 for d^2, 3 for 1/d^2, 1 for the log
 // product, 3 accumulations), 22 where every mass differs, against about 49 with
 // a division, a library logarithm and the mass sum per pair.  1e6 clustered points
-// at p = 32, m = 32 (5.1e8 pairs, equal masses): 58.6 -> 20.7 ms.
-template <bool SHEAR, bool NPM>
+// at p = 32, m = 32 (5.1e8 pairs, equal masses): 58.6 -> 20.7 ms.  L2P and the
+// combination run in k_finish64, a thread per target: 420 FP64 instructions per
+// target group that the groups of 1 to 16 targets left to a few lanes (20.7 -> 15.3 ms
+// with 1.0 ms there).  TEAM: the four warps of a CTA share an item, each taking every
+// fourth near leaf, for problems with fewer items than the GPU has warps to run
+// (4096 points, 195 items: 0.57 -> 0.23 ms; the line is four items per warp
+// slot of the SMs' FP64 pipes).
+template <bool SHEAR, bool NPM, bool TEAM>
 __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
 {
+    constexpr int NW = near_width(SHEAR, NPM);
     __shared__ double2 s_tab[LOG64_N];
+    __shared__ double s_part[TEAM ? 4 : 1][TEAM ? 32 * NW : 1];
+    __shared__ unsigned long long s_item;
     for (int i = threadIdx.x; i < LOG64_N; i += blockDim.x) s_tab[i] = A.log_tab[i];
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    double shift = 0.0, qtot = 0.0;        // qtot = sum q / 4pi (the base boxes' Q)
-    for (int b = 0; b < 12; ++b) qtot += A.base_mpole[(size_t)b * EXP_STRIDE + 1];
-    if (A.zero_mean) shift = qtot;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (;;) {
-        const int64_t w = next_item(A.leaf_ctr, lane);
+        int64_t w;
+        if (TEAM) {
+            __syncthreads();
+            if (threadIdx.x == 0) s_item = atomicAdd(A.leaf_ctr, 1ull);
+            __syncthreads();
+            w = (int64_t)s_item;
+        } else {
+            w = next_item(A.leaf_ctr, lane);
+        }
         if (w >= dcount(A.d_n_items, A.n_items)) break;
         const int2 item = A.items[w];
         const int leaf = item.x;
         const int tf = A.T.tfirst[leaf], tc = A.T.tcount[leaf];
-        const double* g = A.T.geom + (size_t)leaf * GEOM_STRIDE;
-        const double* L = A.local + (size_t)leaf * EXP_STRIDE;
         const int64_t nb0 = A.p2p_off[leaf], nb1 = A.p2p_off[leaf + 1];
         const double mass = near_mass(A, nb0, nb1, lane);
         int t0, t1;
@@ -159,15 +179,14 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
             const int lpt = 32 / tpw;
             const int slot = lane / lpt, sub = lane % lpt;
             const int ti = tb + slot;
-            const bool active = ti < t1;
-            const double4_32a x = A.tgt[tf + (active ? ti : 0)];
+            const double4_32a x = A.tgt[tf + ti];
             double sx = 0.0, sy = 0.0, sz = 0.0;
             double skip = 0.0;                // mass of the sources left out (d = 0)
             double Sxx = 0.0, Syy = 0.0, Szz = 0.0, Sxy = 0.0, Sxz = 0.0, Syz = 0.0;
             double qfd = 0.0;                 // NPM: sum of (f - 1) q inside the caps
             LogSum ls;
             ls.init();
-            for (int64_t k = nb0; k < nb1; ++k) {
+            for (int64_t k = nb0 + (TEAM ? wid : 0); k < nb1; k += TEAM ? 4 : 1) {
                 const int sleaf = (int)A.p2p_src[k];
                 const int f = A.T.first[sleaf], n = A.T.count[sleaf];
                 for (int j = f + sub; j < f + n; j += lpt) {
@@ -219,90 +238,131 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
             }
             if (A.want_psi) ls.flush(s_tab);
             double sl = ls.sum;
+            double v[NW];                     // this target's sums (near_width)
+            v[0] = group_sum(sx, lpt);
+            v[1] = group_sum(sy, lpt);
+            v[2] = group_sum(sz, lpt);
             const double sqs = group_sum(skip, lpt);       // masses at the target's position (left out)
-            const double sq = isfinite(mass) ? mass - sqs : group_sum(near_mass_of(A, nb0, nb1, x, sub, lpt), lpt);
-            const double sqa = NPM ? sq + group_sum(qfd, lpt) : sq;   // the alpha part of sum q
-            sx = group_sum(sx, lpt);
-            sy = group_sum(sy, lpt);
-            sz = group_sum(sz, lpt);
-            if (A.want_psi) sl = group_sum(sl, lpt);
+            // the mass once per target (TEAM: by warp 0), less what is left out
+            v[3] = isfinite(mass) ? (TEAM && wid > 0 ? 0.0 : mass) - sqs
+                                  : TEAM && wid > 0 ? 0.0 : group_sum(near_mass_of(A, nb0, nb1, x, sub, lpt), lpt);
+            v[4] = A.want_psi ? group_sum(sl, lpt) : 0.0;
+            if (NPM) v[NW - 1] = v[3] + group_sum(qfd, lpt);              // the alpha part of sum q
             if (SHEAR) {
-                Sxx = group_sum(Sxx, lpt); Syy = group_sum(Syy, lpt); Szz = group_sum(Szz, lpt);
-                Sxy = group_sum(Sxy, lpt); Sxz = group_sum(Sxz, lpt); Syz = group_sum(Syz, lpt);
+                v[5] = group_sum(Sxx, lpt); v[6] = group_sum(Syy, lpt); v[7] = group_sum(Szz, lpt);
+                v[8] = group_sum(Sxy, lpt); v[9] = group_sum(Sxz, lpt); v[10] = group_sum(Syz, lpt);
+                v[NW - 1] = sqs;
             }
-            if (!active || sub != 0) continue;
-            // ---- L2P in the leaf frame
-            const double Dx = x.x - g[0], Dy = x.y - g[1], Dz = x.z - g[2];
-            const double D2 = Dx * Dx + Dy * Dy + Dz * Dz;
-            const double den = 2.0 - 0.5 * D2;                  // 1 + x.c
-            const double wu = (Dx * g[3] + Dy * g[4] + Dz * g[5]) / den;
-            const double wv = (Dx * g[6] + Dy * g[7] + Dz * g[8]) / den;
-            const double inv_r = 1.0 / g[10];
-            const cd om = mk(wu * inv_r, wv * inv_r);
-            cd f = mk(0.0, 0.0), fd = mk(0.0, 0.0), fdd = mk(0.0, 0.0);
-            for (int l = A.p; l >= 1; --l) {
-                const cd a = mk(L[2 * l], L[2 * l + 1]);
-                f = cadd(cmul(f, om), a);
-                fd = cadd(cmul(fd, om), cscale(a, (double)l));
-                if (SHEAR && l >= 2) fdd = cadd(cmul(fdd, om), cscale(a, (double)(l * (l - 1))));
+            if (TEAM) {
+                __syncthreads();
+                if (sub == 0)
+                    for (int c = 0; c < NW; ++c) s_part[wid][slot * NW + c] = v[c];
+                __syncthreads();
+                for (int i = threadIdx.x; i < tpw * NW; i += 128)
+                    A.nf[(size_t)(tf + tb) * NW + i] = (s_part[0][i] + s_part[1][i]) + (s_part[2][i] + s_part[3][i]);
+                if (threadIdx.x < tpw) A.tleaf[tf + tb + threadIdx.x] = leaf;
+            } else if (sub == 0) {
+                for (int c = 0; c < NW; ++c) A.nf[(size_t)(tf + ti) * NW + c] = v[c];
+                A.tleaf[tf + ti] = leaf;
             }
-            const cd F = cmul(f, om);
-            const cd Fp = cscale(fd, inv_r);                    // dF/dw
-            const double C = L[0], Q = L[1];
-            const double w2 = wu * wu + wv * wv;
-            const double au = (1.0 + w2) * Fp.x - Q * wu;
-            const double av = -(1.0 + w2) * Fp.y - Q * wv;
-            const double cxx = g[0] + x.x, cyy = g[1] + x.y, czz = g[2] + x.z;
-            double a3x = au * (g[3] - wu * cxx) + av * (g[6] - wv * cxx);
-            double a3y = au * (g[4] - wu * cyy) + av * (g[7] - wv * cyy);
-            double a3z = au * (g[5] - wu * czz) + av * (g[8] - wv * czz);
-            // ---- near field
-            a3x += INV2PI * (sx - 0.5 * x.x * sqa);
-            a3y += INV2PI * (sy - 0.5 * x.y * sqa);
-            a3z += INV2PI * (sz - 0.5 * x.z * sqa);
-            const double rho = sqrt(x.x * x.x + x.y * x.y);
-            double cp = 1.0, sp = 0.0;
-            if (rho > 0.0) { cp = x.x / rho; sp = x.y / rho; }
-            const uint32_t o = A.tperm[tf + ti];
-            if (A.alpha) {
-                A.alpha[2 * (size_t)o] = a3x * (x.z * cp) + a3y * (x.z * sp) - a3z * rho;
-                A.alpha[2 * (size_t)o + 1] = -a3x * sp + a3y * cp;
-            }
-            if (A.want_psi) {
-                const double psi_e = C + Q * (LOG2 + log1p(-0.25 * D2)) + 2.0 * F.x;
-                A.psi[o] = psi_e + INV4PI * (sl - LOG4 * sq) + shift;
-            }
-            if (SHEAR) {
-                // far field: chart-frame trace-free Hessian, then onto (e_theta, e_phi)
-                const cd Fpp = cscale(fdd, inv_r * inv_r);
-                const double opw = 1.0 + w2;
-                const cd wb = mk(wu, -wv);
-                const cd t1 = cadd(Fpp, cscale(cmul(wb, Fp), 2.0 / opw));
-                const cd wb2 = cmul(wb, wb);
-                const double gr = 0.5 * opw * opw * t1.x - 0.5 * Q * wb2.x;
-                const double gi = 0.5 * opw * opw * t1.y - 0.5 * Q * wb2.y;
-                const double huu = gr, huv = -gi;                        // H_vv = -H_uu (trace-free part)
-                const double eux = g[3] - wu * cxx, euy = g[4] - wu * cyy, euz = g[5] - wu * czz;
-                const double evx = g[6] - wv * cxx, evy = g[7] - wv * cyy, evz = g[8] - wv * czz;
-                const double etx = x.z * cp, ety = x.z * sp, etz = -rho, epx = -sp, epy = cp;
-                const double c1 = eux * etx + euy * ety + euz * etz, s1 = eux * epx + euy * epy;
-                const double c2 = evx * etx + evy * ety + evz * etz, s2 = evx * epx + evy * epy;
-                double g1 = 0.5 * (huu * (c1 * c1 - s1 * s1 - c2 * c2 + s2 * s2)) + huv * (c1 * c2 - s1 * s2);
-                double g2 = huu * (c1 * s1 - c2 * s2) + huv * (c1 * s2 + c2 * s1);
-                // near field: -(e_a^T S e_b)/pi
-                const double stt = etx * (Sxx * etx + Sxy * ety + Sxz * etz) + ety * (Sxy * etx + Syy * ety + Syz * etz) +
-                                   etz * (Sxz * etx + Syz * ety + Szz * etz);
-                const double spp = epx * (Sxx * epx + Sxy * epy) + epy * (Sxy * epx + Syy * epy);
-                const double stp = epx * (Sxx * etx + Sxy * ety + Sxz * etz) + epy * (Sxy * etx + Syy * ety + Syz * etz);
-                g1 -= 0.5 * (stt - spp) / PI;
-                g2 -= stp / PI;
-                A.gamma[2 * (size_t)o] = g1;
-                A.gamma[2 * (size_t)o + 1] = g2;
-                if (A.mu) {       // tr H = kappa - kappa_bar = -(sum q of the masses not at x) / 4pi
-                    const double trh = -qtot + INV4PI * sqs;
-                    const double a = 1.0 - 0.5 * trh;
-                    A.mu[o] = 1.0 / (a * a - g1 * g1 - g2 * g2);
-                }
+        }
+    }
+}
+
+// L2P of the leaf's local expansion and the combination with the near field's sums,
+// one thread per sorted target.
+template <bool SHEAR, bool NPM>
+__global__ void __launch_bounds__(128) k_finish64(EvalArgs A)
+{
+    constexpr int NW = near_width(SHEAR, NPM);
+    __shared__ double s_qtot;
+    if (threadIdx.x == 0) {
+        double qt = 0.0;                      // sum q / 4pi (the base boxes' Q)
+        for (int b = 0; b < 12; ++b) qt += A.base_mpole[(size_t)b * EXP_STRIDE + 1];
+        s_qtot = qt;
+    }
+    __syncthreads();
+    const double qtot = s_qtot, shift = A.zero_mean ? qtot : 0.0;
+    for (int64_t tix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; tix < A.M;
+         tix += (int64_t)gridDim.x * blockDim.x) {
+        const int leaf = A.tleaf[tix];
+        const double* g = A.T.geom + (size_t)leaf * GEOM_STRIDE;
+        const double* L = A.local + (size_t)leaf * EXP_STRIDE;
+        const double4_32a x = A.tgt[tix];
+        const double* v = A.nf + (size_t)tix * NW;
+        const double sx = v[0], sy = v[1], sz = v[2], sq = v[3], sl = v[4], sqa = NPM ? v[NW - 1] : sq;
+        // ---- L2P in the leaf frame
+        const double Dx = x.x - g[0], Dy = x.y - g[1], Dz = x.z - g[2];
+        const double D2 = Dx * Dx + Dy * Dy + Dz * Dz;
+        const double den = 2.0 - 0.5 * D2;                  // 1 + x.c
+        const double wu = (Dx * g[3] + Dy * g[4] + Dz * g[5]) / den;
+        const double wv = (Dx * g[6] + Dy * g[7] + Dz * g[8]) / den;
+        const double inv_r = 1.0 / g[10];
+        const cd om = mk(wu * inv_r, wv * inv_r);
+        cd f = mk(0.0, 0.0), fd = mk(0.0, 0.0), fdd = mk(0.0, 0.0);
+        for (int l = A.p; l >= 1; --l) {
+            const cd a = mk(L[2 * l], L[2 * l + 1]);
+            if (A.want_psi) f = cadd(cmul(f, om), a);
+            fd = cadd(cmul(fd, om), cscale(a, (double)l));
+            if (SHEAR && l >= 2) fdd = cadd(cmul(fdd, om), cscale(a, (double)(l * (l - 1))));
+        }
+        const cd F = cmul(f, om);
+        const cd Fp = cscale(fd, inv_r);                    // dF/dw
+        const double C = L[0], Q = L[1];
+        const double w2 = wu * wu + wv * wv;
+        const double au = (1.0 + w2) * Fp.x - Q * wu;
+        const double av = -(1.0 + w2) * Fp.y - Q * wv;
+        const double cxx = g[0] + x.x, cyy = g[1] + x.y, czz = g[2] + x.z;
+        double a3x = au * (g[3] - wu * cxx) + av * (g[6] - wv * cxx);
+        double a3y = au * (g[4] - wu * cyy) + av * (g[7] - wv * cyy);
+        double a3z = au * (g[5] - wu * czz) + av * (g[8] - wv * czz);
+        // ---- near field
+        a3x += INV2PI * (sx - 0.5 * x.x * sqa);
+        a3y += INV2PI * (sy - 0.5 * x.y * sqa);
+        a3z += INV2PI * (sz - 0.5 * x.z * sqa);
+        const double rho = sqrt(x.x * x.x + x.y * x.y);
+        double cp = 1.0, sp = 0.0;
+        if (rho > 0.0) { cp = x.x / rho; sp = x.y / rho; }
+        const uint32_t o = A.tperm[tix];
+        if (A.alpha) {
+            A.alpha[2 * (size_t)o] = a3x * (x.z * cp) + a3y * (x.z * sp) - a3z * rho;
+            A.alpha[2 * (size_t)o + 1] = -a3x * sp + a3y * cp;
+        }
+        if (A.want_psi) {
+            const double psi_e = C + Q * (LOG2 + log1p(-0.25 * D2)) + 2.0 * F.x;
+            A.psi[o] = psi_e + INV4PI * (sl - LOG4 * sq) + shift;
+        }
+        if (SHEAR) {
+            // far field: chart-frame trace-free Hessian, then onto (e_theta, e_phi)
+            const cd Fpp = cscale(fdd, inv_r * inv_r);
+            const double opw = 1.0 + w2;
+            const cd wb = mk(wu, -wv);
+            const cd t1 = cadd(Fpp, cscale(cmul(wb, Fp), 2.0 / opw));
+            const cd wb2 = cmul(wb, wb);
+            const double gr = 0.5 * opw * opw * t1.x - 0.5 * Q * wb2.x;
+            const double gi = 0.5 * opw * opw * t1.y - 0.5 * Q * wb2.y;
+            const double huu = gr, huv = -gi;                        // H_vv = -H_uu (trace-free part)
+            const double eux = g[3] - wu * cxx, euy = g[4] - wu * cyy, euz = g[5] - wu * czz;
+            const double evx = g[6] - wv * cxx, evy = g[7] - wv * cyy, evz = g[8] - wv * czz;
+            const double etx = x.z * cp, ety = x.z * sp, etz = -rho, epx = -sp, epy = cp;
+            const double c1 = eux * etx + euy * ety + euz * etz, s1 = eux * epx + euy * epy;
+            const double c2 = evx * etx + evy * ety + evz * etz, s2 = evx * epx + evy * epy;
+            double g1 = 0.5 * (huu * (c1 * c1 - s1 * s1 - c2 * c2 + s2 * s2)) + huv * (c1 * c2 - s1 * s2);
+            double g2 = huu * (c1 * s1 - c2 * s2) + huv * (c1 * s2 + c2 * s1);
+            // near field: -(e_a^T S e_b)/pi
+            const double Sxx = v[5], Syy = v[6], Szz = v[7], Sxy = v[8], Sxz = v[9], Syz = v[10], sqs = v[NW - 1];
+            const double stt = etx * (Sxx * etx + Sxy * ety + Sxz * etz) + ety * (Sxy * etx + Syy * ety + Syz * etz) +
+                               etz * (Sxz * etx + Syz * ety + Szz * etz);
+            const double spp = epx * (Sxx * epx + Sxy * epy) + epy * (Sxy * epx + Syy * epy);
+            const double stp = epx * (Sxx * etx + Sxy * ety + Sxz * etz) + epy * (Sxy * etx + Syy * ety + Syz * etz);
+            g1 -= 0.5 * (stt - spp) / PI;
+            g2 -= stp / PI;
+            A.gamma[2 * (size_t)o] = g1;
+            A.gamma[2 * (size_t)o + 1] = g2;
+            if (A.mu) {       // tr H = kappa - kappa_bar = -(sum q of the masses not at x) / 4pi
+                const double trh = -qtot + INV4PI * sqs;
+                const double a = 1.0 - 0.5 * trh;
+                A.mu[o] = 1.0 / (a * a - g1 * g1 - g2 * g2);
             }
         }
     }
@@ -1911,7 +1971,8 @@ cudaError_t launch_eval(const TreeView& T, const int2* items, int64_t n_items, c
                         const double4_32a* tgt,
                         const uint32_t* tperm, const int64_t* p2p_off, const uint32_t* p2p_src, const double* local,
                         const double* mpole, int p, int zero_mean, double sigma, double* psi, double* alpha,
-                        double* gamma, double* mu, const double2* log_tab, unsigned long long* leaf_ctr, cudaStream_t s)
+                        double* gamma, double* mu, const double2* log_tab, double* nf, int* tleaf, int64_t M, int what,
+                        unsigned long long* leaf_ctr, cudaStream_t s)
 {
     if (n_items == 0) return cudaSuccess;
     EvalArgs A;
@@ -1935,16 +1996,38 @@ cudaError_t launch_eval(const TreeView& T, const int2* items, int64_t n_items, c
     A.mu = mu;
     A.npm_s = sin(0.5 * sigma) * sin(0.5 * sigma);
     A.log_tab = log_tab;
+    A.nf = nf;
+    A.tleaf = tleaf;
+    A.M = M;
     A.leaf_ctr = leaf_ctr;
-    int64_t blocks = 0;
     cudaError_t e;
-    if ((e = item_grid(leaf_ctr, n_items, 16, s, &blocks))) return e;
-    if (gamma) k_eval<true, false><<<(unsigned)blocks, 128, 0, s>>>(A);
-    else if (sigma > 0.0) k_eval<false, true><<<(unsigned)blocks, 128, 0, s>>>(A);
-    else k_eval<false, false><<<(unsigned)blocks, 128, 0, s>>>(A);
-    count_launch();
+    if (what & EVAL_NEAR) {
+        // fewer items than four per SM sub-partition's warp: a CTA per item (TEAM)
+        const bool team = n_items <= 152 * 16;
+        int64_t blocks = 0;
+        if ((e = item_grid(leaf_ctr, team ? 4 * n_items : n_items, 16, s, &blocks))) return e;
+#define EVAL64(SH, NP)                                                               \
+        if (team) k_eval<SH, NP, true><<<(unsigned)blocks, 128, 0, s>>>(A);          \
+        else k_eval<SH, NP, false><<<(unsigned)blocks, 128, 0, s>>>(A);
+        if (gamma) { EVAL64(true, false) }
+        else if (sigma > 0.0) { EVAL64(false, true) }
+        else { EVAL64(false, false) }
+#undef EVAL64
+        count_launch();
+    }
+    if ((what & EVAL_FINISH) && M > 0) {
+        int64_t fb = (M + 127) / 128;
+        if (fb > 152 * 16) fb = 152 * 16;
+        if (gamma) k_finish64<true, false><<<(unsigned)fb, 128, 0, s>>>(A);
+        else if (sigma > 0.0) k_finish64<false, true><<<(unsigned)fb, 128, 0, s>>>(A);
+        else k_finish64<false, false><<<(unsigned)fb, 128, 0, s>>>(A);
+        count_launch();
+    }
     return cudaGetLastError();
 }
+
+// bytes per target of the sums between the two kernels of launch_eval
+size_t near64_bytes(bool shear, bool npm) { return near_width(shear, npm) * sizeof(double); }
 
 cudaError_t launch_eval_adj(const TreeView& T, const int2* items, int64_t n_items, const int64_t* d_nit, const double4_32a* src,
                             const double4_32a* dip, const double4_32a* tgt, const uint32_t* tperm,

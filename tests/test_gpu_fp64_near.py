@@ -70,3 +70,19 @@ def test_a_mass_that_is_not_finite_is_left_out_where_it_coincides():
     rp, ra, mp, ma = direct(src[keep], q[keep], src[3:4])
     assert np.all(np.abs(psi.cpu().numpy() - rp) <= TOL * mp)
     assert np.all(np.abs(alpha.cpu().numpy() - ra) <= TOL * ma[:, None])
+
+
+@pytest.mark.parametrize("what", ["deflection", "shear", "npm"])
+def test_few_and_many_targets_give_the_same(what):
+    """A few targets' items are each shared by a CTA's warps, many targets' are not: the
+    same sums in another order (rounding, 2^-45 of the largest; mu, a reciprocal of a
+    difference of these, is not a sum)."""
+    rng = np.random.default_rng(3)
+    src, tgt = unit(rng.normal(size=(600, 3))), unit(rng.normal(size=(160_000, 3)))
+    q = dev(rng.lognormal(0, 0.5, 600))
+    plan = sfmm.Plan(p=12, leaf_size=8, sigma=0.05 if what == "npm" else 0.0)
+    call = (lambda t: plan.shear(dev(src), q, t, True, True)[:3]) if what == "shear" else \
+        (lambda t: plan.deflection(dev(src), q, t))
+    for a, b in zip(call(dev(tgt[:300])), call(dev(tgt))):
+        a, b = a.cpu().numpy(), b.cpu().numpy()[:300]
+        assert np.abs(a - b).max() <= TOL * np.abs(b).max()
