@@ -150,15 +150,13 @@ struct sfmm_plan_s {
     double tol = 0;
     sfmm_options opt{};
     cudaStream_t stream = nullptr;
-    cudaStream_t aux = nullptr;            // target keys + sort run here, overlapping the source tree
+    cudaStream_t aux = nullptr;            // target keys + sort run here, beside the tree; then the lists and the near field
     bool owns_stream = false;              // a batch lane's own stream (destroyed with the plan)
     std::vector<sfmm_plan_s*> lanes;       // batch lanes: solvers on their own streams
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaEvent_t ev_m2l = nullptr;          // the M2L list is sorted (recorded by build_lists)
     cudaEvent_t ev_p2m = nullptr;          // P2M is done (the FP64 near field reads the leaves' masses)
     cudaEvent_t ev_near[2] = {nullptr, nullptr};   // timing: around the near-field kernel on the auxiliary stream
-    bool forked = false;                   // the next solve finds the auxiliary stream already forked
-                                           // (the host entry point copies the targets there)
     std::string err;
     int timing = 0;                        // 0 off, 1 phase times, 2 also the near-field pair count
     int* h_status = nullptr;               // pinned host word: the tensor-core M2L's status of the last solve
