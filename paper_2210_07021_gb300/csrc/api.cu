@@ -35,10 +35,12 @@ cudaError_t launch_p2m32(const TreeView& T, const int* leaves, int64_t n_leaves,
                          float* mpole, int p, cudaStream_t s);
 cudaError_t launch_m2m(const TreeView& T, int a, int b, int lvl, int p, const double* tables, const void* geo,
                        void* mpole, int ek, cudaStream_t s);
-cudaError_t launch_m2m_narrow(const TreeView& T, int a, int b, int lvl, int p, const void* tables, const void* geo,
-                              void* mpole, int ek, cudaStream_t s);
-cudaError_t launch_l2l_df_narrow(const TreeView& T, int a, int b, int lvl, int p, const void* tables, const void* geo,
-                                 const double* acc, void* local, cudaStream_t s);
+cudaError_t launch_m2m_narrow(const TreeView& T, int a, int b, int lvl, int p, const double* tables, const void* geo,
+                              double* mpole, cudaStream_t s);
+cudaError_t launch_m2m_df_narrow(const TreeView& T, int a, int b, int lvl, int p, const void* geo, void* mpole,
+                                 cudaStream_t s);
+cudaError_t launch_l2l_df_narrow(const TreeView& T, int a, int b, int lvl, int p, const void* geo, const double* acc,
+                                 void* local, cudaStream_t s);
 cudaError_t launch_m2l(const TreeView& T, const int64_t* off, const uint32_t* srcs, int p, const double* tables,
                        const void* geo, const void* mpole, void* local, int ek, cudaStream_t s);
 size_t m2l64_part_bytes(int64_t n_pairs);
@@ -277,13 +279,10 @@ TreeView view(sfmm_plan_s* P)
 // the FP64 logarithm's table, behind the binomial tables
 const double2* log64_tab(sfmm_plan_s* P) { return reinterpret_cast<const double2*>(P->tables.as<double>() + 2 * PMAX * PMAX); }
 
-// the binomials as double-float pairs, behind that
-const void* tables_df(sfmm_plan_s* P) { return P->tables.as<double>() + 2 * PMAX * PMAX + 2 * LOG64_N; }
-
 // Levels of up to this many nodes take a warp per translation in the up- and
 // down-pass (M2M of the double-float and FP64 paths, L2L of the double-float ones): a
 // thread's translation takes 28 us at p = 20 and 60 to 85 us at p = 28 however few
-// there are, a warp's 5 us, but five times the instructions.  1e4 clustered points
+// there are, a warp's 8 to 14 us, but several times the instructions.  1e4 clustered points
 // (13 levels, 48 to 200 nodes each): up-pass 0.41 -> 0.20 ms, L2L 0.34 -> 0.12 ms; 1e5
 // points at p = 28 with lines at 0 / 1024 / 4096 / 16384 nodes: 1.27 / 1.12 / 1.11 /
 // 1.17 ms per solve; 1e6 on the N_side 512 grid: 5.94 / 5.87 / 5.81 / 5.85.
@@ -481,9 +480,11 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         // parents [a, b) of level l, children the nodes of level l + 1
         const int a = P->gm ? 0 : P->level_start[l], b = P->gm ? W : P->level_start[l + 1];
         const int c1 = P->gm ? W : P->level_start[l + 2];
-        if (!fp32 && (P->gm ? W : c1 - b) <= NARROW_NODES)
-            e = launch_m2m_narrow(T, a, b, l, p, dfe ? tables_df(P) : P->tables.p, P->m2m_geo.p, P->mpole.p, ek, s);
+        const bool narrow = (P->gm ? W : c1 - b) <= NARROW_NODES;
+        if (dfe && narrow) e = launch_m2m_df_narrow(T, a, b, l, p, P->m2m_geo.p, P->mpole.p, s);
         else if (dfe) e = launch_m2m_df(T, P->gm ? 0 : b, c1, l, p, P->m2m_geo.p, P->mpole.p, s);
+        else if (!fp32 && narrow)
+            e = launch_m2m_narrow(T, a, b, l, p, P->tables.as<double>(), P->m2m_geo.p, P->mpole.as<double>(), s);
         else e = launch_m2m(T, a, b, l, p, P->tables.as<double>(), P->m2m_geo.p, P->mpole.p, ek, s);
         if (e) return cuda_fail(P, e, "M2M");
     }
@@ -617,7 +618,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         for (int l = 0; l <= depth; ++l) {
             const int a = P->gm ? 0 : P->level_start[l], b = P->gm ? W : P->level_start[l + 1];
             if (b - a <= NARROW_NODES)
-                e = launch_l2l_df_narrow(T, a, b, l, p, tables_df(P), P->l2l_geo.p, P->m2l_acc.as<double>(), P->local.p, s);
+                e = launch_l2l_df_narrow(T, a, b, l, p, P->l2l_geo.p, P->m2l_acc.as<double>(), P->local.p, s);
             else e = launch_l2l_df(T, a, b, l, p, P->l2l_geo.p, P->m2l_acc.as<double>(), P->local.p, s);
             if (e) return cuda_fail(P, e, "L2L");
         }
@@ -780,13 +781,10 @@ sfmm_status sfmm_plan(sfmm_plan_t* out, int max_depth, int order_p, double tol, 
     P->tol = tol;
     P->opt = o;
     P->stream = static_cast<cudaStream_t>(o.stream);
-    // binomial tables, the FP64 logarithm's table, then the binomials as double-float pairs
-    std::vector<double> h(2 * PMAX * PMAX + 2 * LOG64_N + 2 * PMAX * PMAX);
+    // binomial tables, then the FP64 logarithm's table
+    std::vector<double> h(2 * PMAX * PMAX + 2 * LOG64_N);
     fill_tables(h.data());
     fill_log64_table(reinterpret_cast<double2*>(h.data() + 2 * PMAX * PMAX));
-    static_assert(sizeof(dflt) == sizeof(double), "one slot per pair");
-    dflt* hdf = reinterpret_cast<dflt*>(h.data() + 2 * PMAX * PMAX + 2 * LOG64_N);
-    for (int i = 0; i < 2 * PMAX * PMAX; ++i) hdf[i] = dflt(h[i]);
     float lt[129 * 4];
     fill_log_table(lt);
     cudaError_t e;

@@ -446,18 +446,6 @@ template <typename R> __device__ __forceinline__ void load_tables(Tables<R>* st,
     __syncthreads();
 }
 
-// The tables as the narrow-level kernels read them: double, or double-float pairs
-// rounded once at plan time (converting 2048 doubles per CTA would cost it 2 us of
-// the FP64 pipe).
-__device__ __forceinline__ void load_tables_as(Tables<double>* st, const double* g) { load_tables<double>(st, g); }
-__device__ __forceinline__ void load_tables_as(Tables<dflt>* st, const dflt* g)
-{
-    const float4* in = reinterpret_cast<const float4*>(g);
-    float4* out = reinterpret_cast<float4*>(&st->t1[0]);
-    for (int i = threadIdx.x; i < PMAX * PMAX; i += blockDim.x) out[i] = in[i];     // two entries at a time
-    __syncthreads();
-}
-
 // One translation by the whole warp.  Input expansion (Cin, Qin, X = lane's
 // coefficient); accumulates into (accC, accQ, accY).
 template <typename R, typename GR>
@@ -795,80 +783,40 @@ __global__ void k_m2m(TreeView T, int a, int b, int lvl, int p, const double* __
 }
 
 // Narrow levels (launch_m2m_narrow): one CTA per parent, one warp per child, so
-// that the level takes one translation's latency; R double or dflt.
-template <typename R, typename GR>
-__global__ void __launch_bounds__(128) k_m2m_narrow(TreeView T, int a, int b, int lvl, int p, const R* __restrict__ tables,
-                                                    const GR* __restrict__ geo, R* __restrict__ mpole)
+// that the level takes one translation's latency (FP64; the double-float one is in
+// updown_df.cu).
+__global__ void __launch_bounds__(128) k_m2m_narrow(TreeView T, int a, int b, int lvl, int p, const double* __restrict__ tables,
+                                                    const XGeo* __restrict__ geo, double* __restrict__ mpole)
 {
     if (T.d_level) {              // graph mode: the parents are the nodes of level lvl
         a = (int)T.d_level[lvl];
         b = (int)T.d_level[lvl + 1];
     }
-    __shared__ Tables<R> tb;
-    __shared__ WarpSmem<R> ws[4];
-    __shared__ R s_sum[4][2 * PMAX + 2];
-    load_tables_as(&tb, tables);
+    __shared__ Tables<double> tb;
+    __shared__ WarpSmem<double> ws[4];
+    __shared__ double s_sum[4][2 * PMAX + 2];
+    load_tables<double>(&tb, tables);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int64_t node = a + blockIdx.x; node < b; node += gridDim.x) {
         const int c0 = T.child0[node];
         if (c0 < 0 || T.count[node] == 0) continue;
-        const R zero = R(0);
-        R accC = zero, accQ = zero;
-        cx<R> accY = cmk<R>(zero, zero);
+        const double zero = 0.0;
+        double accC = zero, accQ = zero;
+        cx<double> accY = cmk<double>(zero, zero);
         if (T.count[c0 + wid] > 0) {
-            R C, Q;
-            cx<R> X;
-            load_exp<R>(mpole + (size_t)(c0 + wid) * EXP_STRIDE, lane, p, &C, &Q, &X);
-            warp_translate<R>(p, lane, geo[c0 + wid], C, Q, X, &tb, &ws[wid], &accC, &accQ, &accY);
+            double C, Q;
+            cx<double> X;
+            load_exp<double>(mpole + (size_t)(c0 + wid) * EXP_STRIDE, lane, p, &C, &Q, &X);
+            warp_translate<double>(p, lane, geo[c0 + wid], C, Q, X, &tb, &ws[wid], &accC, &accQ, &accY);
         }
         if (lane == 0) { s_sum[wid][0] = accC; s_sum[wid][1] = accQ; }
         s_sum[wid][2 + 2 * lane] = accY.x;
         s_sum[wid][3 + 2 * lane] = accY.y;
         __syncthreads();
-        R* out = mpole + (size_t)node * EXP_STRIDE;
+        double* out = mpole + (size_t)node * EXP_STRIDE;
         for (int k = threadIdx.x; k < 2 * p + 2; k += 128)
             out[k] = (s_sum[0][k] + s_sum[1][k]) + (s_sum[2][k] + s_sum[3][k]);
         __syncthreads();
-    }
-}
-
-// Narrow levels of the double-float down-pass: one warp per node; local = M2L sum +
-// the parent's local translated (as k_l2l_df).
-__global__ void __launch_bounds__(128) k_l2l_df_narrow(TreeView T, int a, int b, int lvl, int p,
-                                                       const dflt* __restrict__ tables, const XGeoDF* __restrict__ geo,
-                                                       const double* __restrict__ acc, dflt* __restrict__ local)
-{
-    if (T.d_level) {              // graph mode: the nodes of level lvl
-        a = (int)T.d_level[lvl];
-        b = (int)T.d_level[lvl + 1];
-    }
-    __shared__ Tables<dflt> tb;
-    __shared__ WarpSmem<dflt> ws[4];
-    load_tables_as(&tb, tables);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int ncol = 2 * p + 2;
-    for (int64_t node = a + (int64_t)blockIdx.x * 4 + wid; node < b; node += (int64_t)gridDim.x * 4) {
-        const double* m = acc + (size_t)node * EXP_STRIDE;
-        dflt* out = local + (size_t)node * EXP_STRIDE;
-        const int par = T.parent[node];
-        if (T.tcount[node] == 0 || par < 0) {      // never evaluated: zero; level 0: the M2L sum alone
-            for (int k = lane; k < ncol; k += 32) out[k] = T.tcount[node] == 0 ? dflt(0.f, 0.f) : dflt(m[k]);
-            continue;
-        }
-        dflt C, Q;
-        cx<dflt> X;
-        load_exp<dflt>(local + (size_t)par * EXP_STRIDE, lane, p, &C, &Q, &X);
-        dflt accC(0.f, 0.f), accQ(0.f, 0.f);
-        cx<dflt> accY = cmk<dflt>(accC, accC);
-        warp_translate<dflt>(p, lane, geo[node], C, Q, X, &tb, &ws[wid], &accC, &accQ, &accY);
-        if (lane == 0) {
-            out[0] = dflt(m[0]) + accC;
-            out[1] = dflt(m[1]) + accQ;
-        }
-        if (lane < p) {
-            out[2 + 2 * lane] = dflt(m[2 + 2 * lane]) + accY.x;
-            out[3 + 2 * lane] = dflt(m[3 + 2 * lane]) + accY.y;
-        }
     }
 }
 
@@ -1152,29 +1100,13 @@ cudaError_t launch_m2m(const TreeView& T, int a, int b, int lvl, int p, const do
     return cudaGetLastError();
 }
 
-// as launch_m2m, for FP64 or double-float expansions (tables in that format) and levels
-// narrow enough that one translation's latency, not the arithmetic, is the cost
-cudaError_t launch_m2m_narrow(const TreeView& T, int a, int b, int lvl, int p, const void* tables, const void* geo,
-                              void* mpole, int ek, cudaStream_t s)
+// as launch_m2m, for FP64 expansions and levels narrow enough that one translation's
+// latency, not the arithmetic, is the cost
+cudaError_t launch_m2m_narrow(const TreeView& T, int a, int b, int lvl, int p, const double* tables, const void* geo,
+                              double* mpole, cudaStream_t s)
 {
     if (b <= a) return cudaSuccess;
-    const unsigned g = grid_for(b - a, 1);
-    if (ek == EXP_DF)
-        k_m2m_narrow<dflt, XGeoDF><<<g, 128, 0, s>>>(T, a, b, lvl, p, static_cast<const dflt*>(tables),
-                                                     static_cast<const XGeoDF*>(geo), static_cast<dflt*>(mpole));
-    else
-        k_m2m_narrow<double, XGeo><<<g, 128, 0, s>>>(T, a, b, lvl, p, static_cast<const double*>(tables),
-                                                     static_cast<const XGeo*>(geo), static_cast<double*>(mpole));
-    count_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t launch_l2l_df_narrow(const TreeView& T, int a, int b, int lvl, int p, const void* tables, const void* geo,
-                                 const double* acc, void* local, cudaStream_t s)
-{
-    if (b <= a) return cudaSuccess;
-    k_l2l_df_narrow<<<grid_for(b - a, 4), 128, 0, s>>>(T, a, b, lvl, p, static_cast<const dflt*>(tables),
-                                                       static_cast<const XGeoDF*>(geo), acc, static_cast<dflt*>(local));
+    k_m2m_narrow<<<grid_for(b - a, 1), 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeo*>(geo), mpole);
     count_launch();
     return cudaGetLastError();
 }

@@ -187,6 +187,150 @@ __global__ void __launch_bounds__(128) k_l2l_df(TreeView T, int a, int b, int lv
     }
 }
 
+// ------------------------------------------------------- narrow levels
+// One translation by a whole warp, lane l - 1 holding coefficient l: the operations of
+// translate_row, each on the same operands in the same order, so the result is the
+// same to the last bit (the 1e-6 path rounds its outputs to FP32, where one bit here
+// can move one there by an FP32 unit), spread over the lanes.  A level with few
+// translations waits for one translation's chain: 28 us at p = 20 and 60 to 85 us at
+// p = 28 by one thread, 8 and 14 us by a warp.
+//   Powers: every lane forms the four chains and keeps its own members.
+//   Shift by a (pascal_up_mul2): in pass i, c_j takes a c_{j+1} of the same pass, so lane
+//   j runs pass i in step i + P - 1 - j, one step behind its neighbour: P steps.
+//   Its dual (pascal_down_mul2): in a pass, c_{j+1} takes b c_j of the pass before, all
+//   lanes at once: P - 1 steps.
+__device__ __forceinline__ dflt2 shfl_down2(dflt2 v)
+{
+    return dflt2{make_float2(__shfl_down_sync(FULL, v.h.x, 1), __shfl_down_sync(FULL, v.h.y, 1)),
+                 make_float2(__shfl_down_sync(FULL, v.l.x, 1), __shfl_down_sync(FULL, v.l.y, 1))};
+}
+__device__ __forceinline__ dflt2 shfl_up2(dflt2 v)
+{
+    return dflt2{make_float2(__shfl_up_sync(FULL, v.h.x, 1), __shfl_up_sync(FULL, v.h.y, 1)),
+                 make_float2(__shfl_up_sync(FULL, v.l.x, 1), __shfl_up_sync(FULL, v.l.y, 1))};
+}
+
+// xr, xi: the lane's X_l (zero beyond p); returns Y_l in *yr, *yi and C' (lane 0) in *Cout
+__device__ __forceinline__ void translate_warp(int p, int lane, const XGeoDF& G, dflt C, dflt Q, dflt xr, dflt xi,
+                                               dflt* yr, dflt* yi, dflt* Cout)
+{
+    const int P = (p + 3) / 4 * 4, L = lane + 1;         // translate_row's instance
+    dflt z1r = G.p1x, z1i = G.p1y, z2r = G.p2x, z2i = G.p2y, gp = G.g, bp = G.b;
+    dflt m1r = z1r, m1i = z1i, m2r = z2r, m2i = z2i, mg = gp, mb = bp;      // the lane's members
+#pragma unroll 1
+    for (int l = 2; l <= P; ++l) {
+        dflt nr, ni;
+        cmul_df(z1r, z1i, G.p1x, G.p1y, &nr, &ni);
+        z1r = nr;
+        z1i = ni;
+        cmul_df(z2r, z2i, G.p2x, G.p2y, &nr, &ni);
+        z2r = nr;
+        z2i = ni;
+        gp = gp * G.g;
+        bp = bp * G.b;
+        if (l == L) { m1r = z1r; m1i = z1i; m2r = z2r; m2i = z2i; mg = gp; mb = bp; }
+    }
+    dflt ur(0.f, 0.f), ui(0.f, 0.f);
+    if (L <= p) cmul_df(m1r, m1i, xr, xi, &ur, &ui);
+    dflt2 c{make_float2(ur.h, ui.h), make_float2(ur.l, ui.l)};
+    dflt2 c0{f2s(0.f), f2s(0.f)};
+#pragma unroll 1
+    for (int t = 0; t < P; ++t) {
+        const dflt2 nb = shfl_down2(c);
+        const int i = t - (P - 1 - L);
+        if (t == P - 1 && lane == 0) c0 = mac_lazy2(c0, G.a, c);     // c_0 takes part in pass 0 only
+        if (i >= 0 && i <= L && L < P) c = mac_lazy2(c, G.a, nb);
+    }
+    const dflt v0 = renorm(dflt(c0.h.x, c0.l.x));
+    c = mul2_df(renorm2(c), mg);
+#pragma unroll 1
+    for (int i = 1; i < P; ++i) {
+        const dflt2 nb = shfl_up2(c);
+        if (L >= i + 1 && L <= P) c = mac_lazy2(c, G.b, nb);
+    }
+    c = renorm2(c);
+    const float fl = (float)L, il = 1.f / fl;
+    const dflt qb = Q * mb;
+    const float q1 = __fmul_rn(qb.h, il);                        // Q b^l / l
+    const float rq = __fadd_rn(__fmaf_rn(-q1, fl, qb.h), qb.l);
+    const dflt ql = dfl_fast_two_sum(q1, __fmul_rn(rq, il));
+    const dflt orr = dflt(c.h.x, c.l.x) - ql, oi = dflt(c.h.y, c.l.y);
+    cmul_df(m2r, m2i, orr, oi, yr, yi);
+    const dflt two(2.f, 0.f);
+    *Cout = C + two * (Q * G.logk + v0);
+}
+
+// M2M: one CTA per parent (the nodes of level lvl), one warp per child
+__global__ void __launch_bounds__(128) k_m2m_df_narrow(TreeView T, int a, int b, int lvl, int p,
+                                                       const XGeoDF* __restrict__ geo, dflt* __restrict__ mpole)
+{
+    if (T.d_level) {              // graph mode
+        a = (int)T.d_level[lvl];
+        b = (int)T.d_level[lvl + 1];
+    }
+    __shared__ dflt s_row[4][2 * PMAX + 2];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int ncol = 2 * p + 2;
+    for (int64_t node = a + blockIdx.x; node < b; node += gridDim.x) {
+        const int c0 = T.child0[node];
+        if (c0 < 0) continue;
+        const int ch = c0 + wid;
+        const dflt zero(0.f, 0.f);
+        dflt yr = zero, yi = zero, Cp = zero, Q = zero;
+        if (T.count[ch] > 0) {
+            const dflt* e = mpole + (size_t)ch * EXP_STRIDE;
+            dflt xi = zero;
+            const dflt xr = lane < p ? ld_dflt2(e + 2 + 2 * lane, &xi) : zero;
+            Q = e[1];
+            translate_warp(p, lane, geo[ch], e[0], Q, xr, xi, &yr, &yi, &Cp);
+        }
+        s_row[wid][2 + 2 * lane] = yr;
+        s_row[wid][3 + 2 * lane] = yi;
+        if (lane == 0) { s_row[wid][0] = Cp; s_row[wid][1] = Q; }
+        __syncthreads();
+        dflt* out = mpole + (size_t)node * EXP_STRIDE;
+        for (int k = threadIdx.x; k < ncol; k += 128)
+            out[k] = renorm(add_lazy(add_lazy(s_row[0][k], s_row[1][k]), add_lazy(s_row[2][k], s_row[3][k])));
+        __syncthreads();
+    }
+}
+
+// L2L: one warp per node of level lvl (as k_l2l_df)
+__global__ void __launch_bounds__(128) k_l2l_df_narrow(TreeView T, int a, int b, int lvl, int p,
+                                                       const XGeoDF* __restrict__ geo, const double* __restrict__ acc,
+                                                       dflt* __restrict__ local)
+{
+    if (T.d_level) {              // graph mode
+        a = (int)T.d_level[lvl];
+        b = (int)T.d_level[lvl + 1];
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int ncol = 2 * p + 2;
+    for (int64_t node = a + (int64_t)blockIdx.x * 4 + wid; node < b; node += (int64_t)gridDim.x * 4) {
+        const double* m = acc + (size_t)node * EXP_STRIDE;
+        dflt* out = local + (size_t)node * EXP_STRIDE;
+        const int par = T.parent[node];
+        const dflt zero(0.f, 0.f);
+        if (T.tcount[node] == 0 || par < 0) {      // never evaluated: zero; level 0: the M2L sum alone
+            for (int k = lane; k < ncol; k += 32) out[k] = T.tcount[node] == 0 ? zero : dflt(m[k]);
+            continue;
+        }
+        const dflt* e = local + (size_t)par * EXP_STRIDE;
+        dflt xi = zero, yr, yi, Cp;
+        const dflt xr = lane < p ? ld_dflt2(e + 2 + 2 * lane, &xi) : zero;
+        const dflt Q = e[1];
+        translate_warp(p, lane, geo[node], e[0], Q, xr, xi, &yr, &yi, &Cp);
+        if (lane == 0) {
+            out[0] = dflt(m[0]) + Cp;
+            out[1] = dflt(m[1]) + Q;
+        }
+        if (lane < p) {
+            out[2 + 2 * lane] = dflt(m[2 + 2 * lane]) + yr;
+            out[3 + 2 * lane] = dflt(m[3 + 2 * lane]) + yi;
+        }
+    }
+}
+
 // ----------------------------------------------------------------- P2M
 // One warp per leaf, one lane per source (in rounds of 32): z = tan(theta/2)
 // e^{i phi} in the leaf frame from the source's (hi, lo) offset D,
@@ -382,6 +526,28 @@ cudaError_t launch_l2l_df(const TreeView& T, int a, int b, int lvl, int p, const
 #define CALL(PP) l2l_p<PP>(T, a, b, lvl, p, geo, acc, local, s)
     SFMM_P_SWITCH(CALL)
 #undef CALL
+}
+
+// the same for levels narrow enough that one translation's latency is the cost:
+// parents a..b-1 (level lvl); nodes a..b-1 (level lvl)
+cudaError_t launch_m2m_df_narrow(const TreeView& T, int a, int b, int lvl, int p, const void* geo, void* mpole,
+                                 cudaStream_t s)
+{
+    if (b <= a) return cudaSuccess;
+    k_m2m_df_narrow<<<grid_of(b - a, 1, 152 * 64), 128, 0, s>>>(T, a, b, lvl, p, static_cast<const XGeoDF*>(geo),
+                                                                static_cast<dflt*>(mpole));
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_l2l_df_narrow(const TreeView& T, int a, int b, int lvl, int p, const void* geo, const double* acc,
+                                 void* local, cudaStream_t s)
+{
+    if (b <= a) return cudaSuccess;
+    k_l2l_df_narrow<<<grid_of(b - a, 4, 152 * 64), 128, 0, s>>>(T, a, b, lvl, p, static_cast<const XGeoDF*>(geo), acc,
+                                                                static_cast<dflt*>(local));
+    count_launch();
+    return cudaGetLastError();
 }
 
 // doff: NULL, or the sources' tangent dipoles as (hi, lo) float4 pairs (the adjoint)
