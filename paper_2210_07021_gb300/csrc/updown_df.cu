@@ -345,6 +345,13 @@ __global__ void __launch_bounds__(128) k_l2l_df_narrow(TreeView T, int a, int b,
 // 1 + x.c = 2 - |D|^2/2, dz = [(g.e_theta + i g.e_phi) - z (g.c)] / (1 + x.c)
 // (scaled by 1/r like z), dC = (1/4pi) (g.c) / (1 + x.c), dQ = 0 and
 // dA_l = -(1/4pi) z^(l-1) dz; the row holds q z^l + l z^(l-1) dz for column l.
+// The rows hold HP coefficients at a time (half the order): the powers of a round's
+// sources run on in registers while the columns of one half are summed, and half the
+// shared memory per warp lets twice as many warps wait for their chains (p = 20: 20 of 64
+// warps per SM with whole rows; N = 1.6e7: 1.84 -> 1.59 ms, p = 28 2.80 -> 2.18 ms).
+constexpr int p2m_half(int P) { return P > 4 ? P / 2 : P; }
+constexpr int p2m_stride(int P) { return 2 * p2m_half(P) + 3; }       // odd: conflict-free row access
+
 template <int P, bool DIP>
 __global__ void __launch_bounds__(128) k_p2m_df_leaf(TreeView T, const int* __restrict__ leaves, int64_t n_cap,
                                                      const int64_t* d_nl, const float4* __restrict__ off,
@@ -352,7 +359,8 @@ __global__ void __launch_bounds__(128) k_p2m_df_leaf(TreeView T, const int* __re
                                                      const float4* __restrict__ log_tab, int p, dflt* __restrict__ mpole)
 {
     const int64_t n_leaves = dcount(d_nl, n_cap);
-    constexpr int RS = 2 * P + 3;
+    constexpr int HP = p2m_half(P), NH = P / HP, RS = p2m_stride(P);
+    constexpr int NC = (2 * HP + 2 + 31) / 32;      // a lane's columns per half
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float4 s_tab[129];
     for (int i = threadIdx.x; i < 129; i += blockDim.x) s_tab[i] = log_tab[i];
@@ -360,7 +368,6 @@ __global__ void __launch_bounds__(128) k_p2m_df_leaf(TreeView T, const int* __re
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     dflt* rows = reinterpret_cast<dflt*>(smem_raw) + (size_t)wid * 32 * RS;
     dflt* row = rows + lane * RS;
-    const int ncol = 2 * p + 2;
     for (int64_t w = (int64_t)blockIdx.x * UW + wid; w < n_leaves; w += (int64_t)gridDim.x * UW) {
         const int node = leaves[w];
         const double* g = T.geom + (size_t)node * GEOM_STRIDE;
@@ -368,72 +375,86 @@ __global__ void __launch_bounds__(128) k_p2m_df_leaf(TreeView T, const int* __re
         const dflt inv_r(1.0 / g[10]);
         const dflt ccx(g[0]), ccy(g[1]), ccz(g[2]);
         const int f = T.first[node], n = T.count[node];
-        dflt sc[3] = {dflt(0.f, 0.f), dflt(0.f, 0.f), dflt(0.f, 0.f)};   // this lane's columns lane + 32 i (2p + 2 <= 66)
+        // this lane's columns: of half h, lane + 32 i; column 0 = sum q log(..), 1 = sum q (half 0),
+        // then (Re, Im) of the half's coefficients
+        dflt sc[NH * NC];
+#pragma unroll
+        for (int i = 0; i < NH * NC; ++i) sc[i] = dflt(0.f, 0.f);
         for (int j0 = 0; j0 < n; j0 += 32) {
             const int j = j0 + lane;
+            dflt zr(0.f, 0.f), zi(0.f, 0.f), pr(0.f, 0.f), pi(0.f, 0.f);
+            dflt qr(0.f, 0.f), qi(0.f, 0.f);         // z^(l-1) dz (DIP)
             if (j < n) {
                 const float4 h = off[2 * (size_t)(f + j)], lo = off[2 * (size_t)(f + j) + 1];
                 const dflt dx(h.x, lo.x), dy(h.y, lo.y), dz(h.z, lo.z), q(h.w, lo.w);
                 const dflt d2 = dx * dx + dy * dy + dz * dz;
                 const dflt opc = dflt(2.f, 0.f) - d2 * 0.5f;                         // 1 + x.c
                 const dflt inv = DIP ? dflt(1.f, 0.f) / opc : dflt(0.f, 0.f);
-                const dflt sc = inv_r / opc;
-                const dflt zr = (dx * etx + dy * ety + dz * etz) * sc;
-                const dflt zi = (dx * epx + dy * epy + dz * epz) * sc;
+                const dflt sc_ = inv_r / opc;
+                zr = (dx * etx + dy * ety + dz * etz) * sc_;
+                zi = (dx * epx + dy * epy + dz * epz) * sc_;
                 row[0] = q * dfl_norm(dfl_log_lazy(dflt(1.f, 0.f) - d2 * 0.25f, s_tab));
                 row[1] = q;
-                dflt pr = q, pi(0.f, 0.f);
-                dflt qr(0.f, 0.f), qi(0.f, 0.f);     // z^(l-1) dz (DIP)
+                pr = q;
                 if (DIP) {
                     const float4 gh = doff[2 * (size_t)(f + j)], gl = doff[2 * (size_t)(f + j) + 1];
                     const dflt gx(gh.x, gl.x), gy(gh.y, gl.y), gz(gh.z, gl.z);
                     const dflt gc = gx * ccx + gy * ccy + gz * ccz;
                     const dflt gci = gc * inv;
                     row[0] = row[0] + gci;
-                    qr = (gx * etx + gy * ety + gz * etz) * sc - zr * gci;
-                    qi = (gx * epx + gy * epy + gz * epz) * sc - zi * gci;
-                }
-#pragma unroll 1
-                for (int l = 1; l <= p; ++l) {
-                    dflt nr, ni;
-                    cmul_df(pr, pi, zr, zi, &nr, &ni);
-                    pr = nr;
-                    pi = ni;
-                    if (DIP) {
-                        row[2 * l] = pr + qr * (float)l;
-                        row[2 * l + 1] = pi + qi * (float)l;
-                        cmul_df(qr, qi, zr, zi, &nr, &ni);
-                        qr = nr;
-                        qi = ni;
-                    } else {
-                        row[2 * l] = pr;
-                        row[2 * l + 1] = pi;
-                    }
+                    qr = (gx * etx + gy * ety + gz * etz) * sc_ - zr * gci;
+                    qi = (gx * epx + gy * epy + gz * epz) * sc_ - zi * gci;
                 }
             }
-            __syncwarp();
             const int nr = min(32, n - j0);
-            // only the columns this lane owns (c < ncol < RS): every index stays below 32 RS
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
-                if (lane + 32 * i < ncol)
-                    for (int r = 0; r < nr; ++r) sc[i] = add_lazy(sc[i], rows[r * RS + lane + 32 * i]);
-            __syncwarp();
+            for (int hf = 0; hf < NH; ++hf) {
+                const int l0 = hf * HP, lh = min(HP, p - l0);      // coefficients l0 + 1 .. l0 + lh
+                if (j < n) {
+#pragma unroll 1
+                    for (int l = 1; l <= lh; ++l) {
+                        dflt nr_, ni_;
+                        cmul_df(pr, pi, zr, zi, &nr_, &ni_);
+                        pr = nr_;
+                        pi = ni_;
+                        if (DIP) {
+                            row[2 * l] = pr + qr * (float)(l0 + l);
+                            row[2 * l + 1] = pi + qi * (float)(l0 + l);
+                            cmul_df(qr, qi, zr, zi, &nr_, &ni_);
+                            qr = nr_;
+                            qi = ni_;
+                        } else {
+                            row[2 * l] = pr;
+                            row[2 * l + 1] = pi;
+                        }
+                    }
+                }
+                __syncwarp();
+                // only the half's columns: every index stays below 32 RS
+#pragma unroll
+                for (int i = 0; i < NC; ++i) {
+                    const int k = lane + 32 * i;
+                    if (k < 2 * lh + 2 && (hf == 0 || k >= 2))
+                        for (int r = 0; r < nr; ++r) sc[hf * NC + i] = add_lazy(sc[hf * NC + i], rows[r * RS + k]);
+                }
+                __syncwarp();
+            }
         }
         dflt* e = mpole + (size_t)node * EXP_STRIDE;
         const dflt i4p(INV4PI);
-        // column k: 0 = sum q log(..), 1 = sum q, 2l / 2l+1 = sum q z^l (Re / Im)
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const int k = lane + 32 * i;
-            if (k < ncol) {
-                const dflt sk = renorm(sc[i]);
-                e[k] = k < 2 ? i4p * sk : -(sk * (i4p / dflt(k >> 1)));
+        for (int hf = 0; hf < NH; ++hf)
+#pragma unroll
+            for (int i = 0; i < NC; ++i) {
+                const int c = lane + 32 * i, k = c + 2 * hf * HP;      // 2l / 2l + 1 = sum q z^l (Re / Im)
+                if (c < 2 * min(HP, p - hf * HP) + 2 && (hf == 0 || c >= 2)) {
+                    const dflt sk = renorm(sc[hf * NC + i]);
+                    e[k] = k < 2 ? i4p * sk : -(sk * (i4p / dflt(k >> 1)));
+                }
             }
-        }
         __syncwarp();
         if (lane == 0) e[0] = e[0] - e[1] * dflt(LOG2);      // C = (1/4pi) sum q log(..) - Q log 2
-        for (int k = ncol + lane; k < EXP_STRIDE; k += 32) e[k] = dflt(0.f, 0.f);
+        for (int k = 2 * p + 2 + lane; k < EXP_STRIDE; k += 32) e[k] = dflt(0.f, 0.f);
     }
 }
 
@@ -480,7 +501,7 @@ template <int P>
 cudaError_t p2m_p(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl, const float4* off,
                   const float4* doff, const float4* log_tab, int p, void* mpole, cudaStream_t s)
 {
-    const size_t smem = (size_t)UW * 32 * (2 * P + 3) * sizeof(dflt);
+    const size_t smem = (size_t)UW * 32 * p2m_stride(P) * sizeof(dflt);
     cudaError_t e;
     const unsigned grid = grid_of(n_leaves, UW, 152 * 32);
     if (doff) {
