@@ -47,6 +47,9 @@ size_t m2l64_part_bytes(int64_t n_pairs);
 cudaError_t launch_m2l_pair64(const TreeView& T, int64_t n_pairs, const int64_t* d_n, const uint64_t* ptgt,
                               const uint32_t* psrc, const int64_t* off, const void* geo, const double* mpole, int p,
                               double* local, double* part, uint32_t* leftover, uint32_t* n_left, cudaStream_t s);
+cudaError_t launch_m2m64(const TreeView& T, int c0, int c1, int lvl, int p, const void* geo, double* mpole,
+                         cudaStream_t s);
+cudaError_t launch_l2l64(const TreeView& T, int a, int b, int lvl, int p, const void* geo, double* local, cudaStream_t s);
 cudaError_t launch_p2m64_leaf(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl,
                               const double4_32a* src, int p, double* mpole, cudaStream_t s);
 cudaError_t launch_m2l_list(const uint64_t* ptgt, const uint32_t* psrc, const uint32_t* list, const uint32_t* n_list,
@@ -280,8 +283,7 @@ TreeView view(sfmm_plan_s* P)
 const double2* log64_tab(sfmm_plan_s* P) { return reinterpret_cast<const double2*>(P->tables.as<double>() + 2 * PMAX * PMAX); }
 
 // Levels of up to this many nodes take a warp per translation in the up- and
-// down-pass (M2M of the double-float and FP64 paths, L2L of the double-float ones): a
-// thread's translation takes 28 us at p = 20 and 60 to 85 us at p = 28 however few
+// down-pass of the double-float and FP64 paths: a thread's translation takes 28 us at p = 20 and 60 to 85 us at p = 28 however few
 // there are, a warp's 8 to 14 us, but several times the instructions.  1e4 clustered points
 // (13 levels, 48 to 200 nodes each): up-pass 0.41 -> 0.20 ms, L2L 0.34 -> 0.12 ms; 1e5
 // points at p = 28 with lines at 0 / 1024 / 4096 / 16384 nodes: 1.27 / 1.12 / 1.11 /
@@ -485,6 +487,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         else if (dfe) e = launch_m2m_df(T, P->gm ? 0 : b, c1, l, p, P->m2m_geo.p, P->mpole.p, s);
         else if (!fp32 && narrow)
             e = launch_m2m_narrow(T, a, b, l, p, P->tables.as<double>(), P->m2m_geo.p, P->mpole.as<double>(), s);
+        else if (!fp32) e = launch_m2m64(T, P->gm ? 0 : b, c1, l, p, P->m2m_geo.p, P->mpole.as<double>(), s);
         else e = launch_m2m(T, a, b, l, p, P->tables.as<double>(), P->m2m_geo.p, P->mpole.p, ek, s);
         if (e) return cuda_fail(P, e, "M2M");
     }
@@ -623,11 +626,12 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
             if (e) return cuda_fail(P, e, "L2L");
         }
     } else {
-        for (int l = 1; l <= depth; ++l)
-            if ((e = P->gm ? launch_l2l(T, 0, W, l, p, P->tables.as<double>(), P->l2l_geo.p, P->local.p, ek, s)
-                           : launch_l2l(T, P->level_start[l], P->level_start[l + 1], l, p, P->tables.as<double>(),
-                                        P->l2l_geo.p, P->local.p, ek, s)))
-                return cuda_fail(P, e, "L2L");
+        for (int l = 1; l <= depth; ++l) {
+            const int a = P->gm ? 0 : P->level_start[l], b = P->gm ? W : P->level_start[l + 1];
+            if (!fp32 && b - a > NARROW_NODES) e = launch_l2l64(T, a, b, l, p, P->l2l_geo.p, P->local.as<double>(), s);
+            else e = launch_l2l(T, a, b, l, p, P->tables.as<double>(), P->l2l_geo.p, P->local.p, ek, s);
+            if (e) return cuda_fail(P, e, "L2L");
+        }
     }
     tm.mark();
     // ---- evaluation (after the P2P list and the offsets of the auxiliary stream)

@@ -86,10 +86,12 @@ __device__ __forceinline__ dflt mac_lazy(dflt acc, dflt a, dflt b)
     return dflt(s.h, __fadd_rn(acc.l, __fadd_rn(s.l, e)));
 }
 
+__device__ __forceinline__ double mac_lazy(double acc, double a, double b) { return fma(a, b, acc); }
+
 // The Taylor shift by a: for i < P, for j = P-1 down to i, c_j += a c_{j+1}
 // (c_n = sum_{l >= n} C(l, n) a^(l-n) c_l), grouped as pascal_up.
-template <int P>
-__device__ __forceinline__ void pascal_up_mul(dflt* c, dflt a)
+template <int P, typename R>
+__device__ __forceinline__ void pascal_up_mul(R* c, R a)
 {
 #pragma unroll
     for (int g = 0; g < P; g += 4) {
@@ -104,8 +106,8 @@ __device__ __forceinline__ void pascal_up_mul(dflt* c, dflt a)
 
 // Its dual with multiplier b on x_m = c[m + 1]: for i = 1..P-1, for j = P-1
 // down to i, x_j += b x_{j-1} (x_k = sum_{m <= k} C(k, m) b^(k-m) x_m).
-template <int P>
-__device__ __forceinline__ void pascal_down_mul(dflt* c, dflt b)
+template <int P, typename R>
+__device__ __forceinline__ void pascal_down_mul(R* c, R b)
 {
 #pragma unroll
     for (int g = 1; g < P; g += 4) {

@@ -1090,12 +1090,8 @@ cudaError_t launch_m2m(const TreeView& T, int a, int b, int lvl, int p, const do
     if (ek == EXP_F32)
         k_m2m<float, XGeo32, float><<<g, 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeo32*>(geo),
                                                       static_cast<float*>(mpole));
-    else if (ek == EXP_DF)
-        k_m2m<dflt, XGeoDF, dflt><<<g, 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeoDF*>(geo),
-                                                    static_cast<dflt*>(mpole));
     else
-        k_m2m<double, XGeo, double><<<g, 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeo*>(geo),
-                                                      static_cast<double*>(mpole));
+        return cudaErrorInvalidValue;             // the FP64 and double-float paths: kernels of their own
     count_launch();
     return cudaGetLastError();
 }
@@ -1200,9 +1196,6 @@ cudaError_t launch_l2l(const TreeView& T, int a, int b, int lvl, int p, const do
     if (ek == EXP_F32)
         k_l2l<float, XGeo32, float><<<g, 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeo32*>(geo),
                                                       static_cast<float*>(local));
-    else if (ek == EXP_DF)
-        k_l2l<dflt, XGeoDF, dflt><<<g, 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeoDF*>(geo),
-                                                    static_cast<dflt*>(local));
     else
         k_l2l<double, XGeo, double><<<g, 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeo*>(geo),
                                                       static_cast<double*>(local));

@@ -1,4 +1,5 @@
-// M2L (Lemma 3) and P2M (Lemma 1) of the FP64 path.
+// M2L (Lemma 3), P2M (Lemma 1) and the wide levels' M2M and L2L (Lemmas 2, 4) of the
+// FP64 path.
 //
 // M2L, one thread per FMM-act pair, in the form of m2l_pair.cu: with
 // u~_l = (a ph1)^l X_l and rho = g/(a b),
@@ -180,8 +181,9 @@ __global__ void __launch_bounds__(128) k_m2l_runs(TreeView T, const int64_t* __r
     }
 }
 
-// few pairs (one warp of single lanes for every SM sub-partition or less): two lanes
-// per pair, CTAs of one warp, so that the pairs spread over the SMs' FP64 pipes
+// few pairs or translations (one warp of single lanes for every SM sub-partition or
+// less): two lanes for each, pairs in CTAs of one warp, so that they spread over the SMs'
+// FP64 pipes
 inline bool few_pairs(int64_t n) { return n <= 152 * 4 * 32; }
 
 template <int P, int L>
@@ -196,6 +198,172 @@ cudaError_t launch_p(int64_t n_pairs, const int64_t* d_n, const uint64_t* ptgt, 
     const int64_t ctas = (n_pairs + nw * ch - 1) / (nw * ch);
     k_m2l_pair64<P, L><<<(unsigned)(ctas < (1 << 30) ? ctas : 1 << 30), nw * 32, smem, s>>>(
         n_pairs, d_n, ptgt, psrc, off, geo, mpole, p, local, part, leftover, n_left);
+    count_launch();
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------- M2M and L2L
+// One thread per translation in the general form of expand.cu (a and b as multipliers
+// of the passes: folded into the vectors they would underflow at deep levels):
+//     u_l = ph1^l X_l,  v_n = sum_{l >= n} C(l, n) a^(l-n) u_l,  w_n = g^n v_n,
+//     Y_l = ph2^l ( -Q b^l / l + sum_{n <= l} C(l-1, n-1) b^(l-n) w_n ),
+//     C'  = C + 2 Q log k + 2 Re v_0,   Q' = Q,
+// 88 FP64 warp instructions per translation at p = 32 against about 260 by a warp, which
+// levels too narrow to fill the GPU keep (1e6 clustered points: M2M 1.77 -> 1.12 ms, L2L
+// 2.21 -> 1.18 + 0.21 in the narrow ones; the whole call 29.4 -> 28.2 ms).  One lane
+// would leave half of the sub-partitions idle at 4e3 to 2e4 nodes (1.64 and 1.72 ms);
+// above that two lanes repeat the turns and cost more (4e6 points, levels over 2e4 nodes:
+// 3.03 and 3.04 ms with two lanes, 2.47 and 2.59 with one).
+// L lanes per translation (1 or 2, sub: this lane's): with two, each takes one part of
+// the passes.  on: the lanes of the warp that translate, both of a pair or neither.
+template <int P, int L>
+__device__ __forceinline__ void translate_row64(double* row, int p, int sub, unsigned on, const XGeo& G, double C,
+                                                double Q, double* Cout)
+{
+    {   // u_l, in place (the caller zeroes p < l <= P)
+        double zr = G.p1x, zi = G.p1y;
+#pragma unroll 1
+        for (int l = 1; l <= p; ++l) {
+            const double xr = row[2 * l], xi = row[2 * l + 1];
+            if (L > 1) __syncwarp(on);
+            if (L == 1 || sub == 0) row[2 * l] = zr * xr - zi * xi;
+            if (L == 1 || sub == 1) row[2 * l + 1] = zr * xi + zi * xr;
+            cmul64(zr, zi, G.p1x, G.p1y);
+        }
+    }
+    double v0 = 0.0;
+#pragma unroll 1
+    for (int prt = sub; prt < 2; prt += L) {
+        double c[P + 1];
+        c[0] = 0.0;
+#pragma unroll
+        for (int l = 1; l <= P; ++l) c[l] = row[2 * l + prt];
+        pascal_up_mul<P>(c, G.a);
+        if (prt == 0) v0 = c[0];
+        double gp = G.g;
+#pragma unroll
+        for (int n = 1; n <= P; ++n) {
+            c[n] *= gp;
+            if (n < P) gp *= G.g;
+        }
+        pascal_down_mul<P>(c, G.b);
+#pragma unroll
+        for (int l = 1; l <= P; ++l) row[2 * l + prt] = c[l];
+    }
+    if (L > 1) __syncwarp(on);
+    {
+        double zr = G.p2x, zi = G.p2y, bp = G.b;
+#pragma unroll 1
+        for (int l = 1; l <= p; ++l) {
+            const double orr = row[2 * l] - Q * bp * kInv64.v[l], oi = row[2 * l + 1];
+            if (L > 1) __syncwarp(on);
+            if (L == 1 || sub == 0) row[2 * l] = zr * orr - zi * oi;
+            if (L == 1 || sub == 1) row[2 * l + 1] = zr * oi + zi * orr;
+            cmul64(zr, zi, G.p2x, G.p2y);
+            bp *= G.b;
+        }
+    }
+    *Cout = C + 2.0 * (Q * G.logk + v0);        // of sub == 0
+}
+
+// X_l of e into the row (zero for p < l <= P), by the translation's lanes
+template <int P, int L>
+__device__ __forceinline__ void ld_row64(double* row, const double* e, int p, int sub)
+{
+    for (int k = 2 + sub; k < 2 * P + 2; k += L) row[k] = k < 2 * p + 2 ? e[k] : 0.0;
+}
+
+// L lanes per child of a level; the four siblings' lanes sum their rows into the parent
+template <int P, int L>
+__global__ void __launch_bounds__(128, 3) k_m2m64(TreeView T, int c0, int c1, int lvl, int p,
+                                                  const XGeo* __restrict__ geo, double* __restrict__ mpole)
+{
+    if (T.d_level) {              // graph mode: the children are the nodes of level lvl + 1
+        c0 = (int)T.d_level[lvl + 1];
+        c1 = (int)T.d_level[lvl + 2];
+    }
+    constexpr int RS = 2 * P + 3, CH = 32 / L;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int slot = threadIdx.x / L, sub = threadIdx.x % L;
+    double* rows = reinterpret_cast<double*>(smem_raw);
+    double* row = rows + slot * RS;
+    const int ncol = 2 * p + 2;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x / L);
+    // rounded up to whole warps, so that all lanes of a sibling group take part
+    for (int64_t c = c0 + (int64_t)blockIdx.x * (blockDim.x / L) + slot; c - c0 < ((int64_t)(c1 - c0) + CH - 1) / CH * CH;
+         c += step) {
+        const bool use = c < c1 && T.count[c] > 0;
+        const unsigned on = __ballot_sync(FULL, use);
+        if (use) {
+            const double* e = mpole + (size_t)c * EXP_STRIDE;
+            ld_row64<P, L>(row, e, p, sub);
+            if (L > 1) __syncwarp(on);
+            double Cp;
+            translate_row64<P, L>(row, p, sub, on, geo[c], e[0], e[1], &Cp);
+            if (sub == 0) {
+                row[0] = Cp;
+                row[1] = e[1];
+            }
+        } else {
+            for (int k = sub; k < ncol; k += L) row[k] = 0.0;
+        }
+        __syncwarp();
+        const int r = threadIdx.x & (4 * L - 1);
+        const double* g0 = rows + (slot & ~3) * RS;
+        const int64_t first = c - (slot & 3);     // the group's first child
+        if (first < c1) {
+            double* out = mpole + (size_t)T.parent[first] * EXP_STRIDE;
+            for (int k = r; k < ncol; k += 4 * L) out[k] = (g0[k] + g0[RS + k]) + (g0[2 * RS + k] + g0[3 * RS + k]);
+        }
+        __syncwarp();
+    }
+}
+
+// L lanes per node of a level holding targets: local += the parent's local translated
+template <int P, int L>
+__global__ void __launch_bounds__(128, 3) k_l2l64(TreeView T, int a, int b, int lvl, int p,
+                                                  const XGeo* __restrict__ geo, double* __restrict__ local)
+{
+    if (T.d_level) {              // graph mode: the nodes of level lvl
+        a = (int)T.d_level[lvl];
+        b = (int)T.d_level[lvl + 1];
+    }
+    constexpr int RS = 2 * P + 3, CH = 32 / L;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int slot = threadIdx.x / L, sub = threadIdx.x % L;
+    double* row = reinterpret_cast<double*>(smem_raw) + slot * RS;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x / L);
+    for (int64_t node = a + (int64_t)blockIdx.x * (blockDim.x / L) + slot;
+         node - a < ((int64_t)(b - a) + CH - 1) / CH * CH; node += step) {
+        const bool use = node < b && T.tcount[node] > 0 && T.parent[node] >= 0;
+        const unsigned on = __ballot_sync(FULL, use);
+        if (use) {
+            const double* e = local + (size_t)T.parent[node] * EXP_STRIDE;
+            double* out = local + (size_t)node * EXP_STRIDE;
+            ld_row64<P, L>(row, e, p, sub);
+            if (L > 1) __syncwarp(on);
+            double Cp;
+            translate_row64<P, L>(row, p, sub, on, geo[node], e[0], e[1], &Cp);
+            if (L > 1) __syncwarp(on);
+            if (sub == 0) {
+                out[0] += Cp;
+                out[1] += e[1];
+            }
+            for (int k = 2 + sub; k < 2 * p + 2; k += L) out[k] += row[k];
+        }
+        __syncwarp();
+    }
+}
+
+template <int P, typename K, typename... Args>
+cudaError_t level_p(K kern, int64_t n, int lanes, cudaStream_t s, Args... args)
+{
+    const int per = 128 / lanes;             // translations of a CTA
+    const size_t smem = (size_t)per * (2 * P + 3) * sizeof(double);
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+    const int64_t blocks = (n + per - 1) / per;
+    kern<<<(unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 128, smem, s>>>(args...);
     count_launch();
     return cudaGetLastError();
 }
@@ -320,6 +488,29 @@ cudaError_t launch_m2l_pair64(const TreeView& T, int64_t n_pairs, const int64_t*
     if (b > 152 * 64) b = 152 * 64;
     k_m2l_runs<<<(unsigned)(b > 0 ? b : 1), 128, 0, s>>>(T, off, p, few_pairs(n_pairs) ? 16 : 32, part, local); count_launch();
     return cudaGetLastError();
+}
+
+// children c0..c1-1 (the nodes of level lvl + 1) -> their parents; nodes a..b-1 (level lvl).
+// Graph mode: the bounds from the device, the given ones the capacity.
+cudaError_t launch_m2m64(const TreeView& T, int c0, int c1, int lvl, int p, const void* geo, double* mpole,
+                         cudaStream_t s)
+{
+    if (c1 <= c0) return cudaSuccess;
+    const XGeo* G = static_cast<const XGeo*>(geo);
+#define CALL(PP) few_pairs(c1 - c0) ? level_p<PP>(k_m2m64<PP, 2>, c1 - c0, 2, s, T, c0, c1, lvl, p, G, mpole) \
+                                    : level_p<PP>(k_m2m64<PP, 1>, c1 - c0, 1, s, T, c0, c1, lvl, p, G, mpole)
+    SFMM_P_SWITCH(CALL)
+#undef CALL
+}
+
+cudaError_t launch_l2l64(const TreeView& T, int a, int b, int lvl, int p, const void* geo, double* local, cudaStream_t s)
+{
+    if (b <= a) return cudaSuccess;
+    const XGeo* G = static_cast<const XGeo*>(geo);
+#define CALL(PP) few_pairs(b - a) ? level_p<PP>(k_l2l64<PP, 2>, b - a, 2, s, T, a, b, lvl, p, G, local) \
+                                  : level_p<PP>(k_l2l64<PP, 1>, b - a, 1, s, T, a, b, lvl, p, G, local)
+    SFMM_P_SWITCH(CALL)
+#undef CALL
 }
 
 cudaError_t launch_p2m64_leaf(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl,
