@@ -283,10 +283,10 @@ TreeView view(sfmm_plan_s* P)
 const double2* log64_tab(sfmm_plan_s* P) { return reinterpret_cast<const double2*>(P->tables.as<double>() + 2 * PMAX * PMAX); }
 
 // Levels of up to this many nodes take a warp per translation in the up- and
-// down-pass of the double-float and FP64 paths: a thread's translation takes 28 us at p = 20 and 60 to 85 us at p = 28 however few
-// there are, a warp's 8 to 14 us, but several times the instructions.  1e4 clustered points
-// (13 levels, 48 to 200 nodes each): up-pass 0.41 -> 0.20 ms, L2L 0.34 -> 0.12 ms; 1e5
-// points at p = 28 with lines at 0 / 1024 / 4096 / 16384 nodes: 1.27 / 1.12 / 1.11 /
+// down-pass of the double-float and FP64 paths: a thread's translation takes 28 us at
+// p = 20 and 60 to 85 us at p = 28 however few there are, a warp's 8 to 14 us, but
+// several times the instructions.  1e4 clustered points (13 levels, 48 to 200 nodes
+// each): up-pass 0.41 -> 0.20 ms, L2L 0.34 -> 0.12 ms; 1e5 points at p = 28 with lines at 0 / 1024 / 4096 / 16384 nodes: 1.27 / 1.12 / 1.11 /
 // 1.17 ms per solve; 1e6 on the N_side 512 grid: 5.94 / 5.87 / 5.81 / 5.85.
 constexpr int64_t NARROW_NODES = 4096;
 
