@@ -96,7 +96,9 @@ __global__ void k_mac_nodes(TreeView T, double c_s, double c_t, double sigma, Ma
         const double a = R / c_t;
         m.t2 = a < 3.141592653589793 ? 2.0 * sin(0.5 * a) : 3.0;
         m.R = R;
-        sincos(0.5 * (R + sigma), &m.s3, &m.c3);
+        m.s3 = m.s1;
+        m.c3 = m.c1;
+        if (sigma != 0.0) sincos(0.5 * (R + sigma), &m.s3, &m.c3);
         out[i] = m;
         const double* g = T.geom + (size_t)i * GEOM_STRIDE;
         MacNode32 f;
