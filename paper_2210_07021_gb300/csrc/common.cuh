@@ -29,6 +29,37 @@ __host__ __device__ __forceinline__ cd cconj(cd a) { return mk(a.x, -a.y); }
 // Every kernel launch of the library bumps this counter (reported per solve in
 // sfmm_stats.launches).
 void count_launch(int n = 1);
+
+// A launch whose blocks are set up while the last blocks of the kernel before it on the
+// stream end: the kernel calls after_previous() before it touches anything that an earlier
+// kernel writes; the call returns when that kernel has ended and its writes can be seen.
+// (Pointers that such a kernel reads through are not __restrict__: the compiler may move
+// their loads above the call.)  For chains of short kernels, where the gap between two
+// launches, about 2 us, is what a launch costs: sorts of up to 2e6 keys, the walk's rounds, narrow
+// levels.  262144 keys (9 launches) 117 -> 93 us, 1e4 clustered points (103 launches)
+// 0.77 -> 0.68 ms, 4096 points 0.75 -> 0.70 ms, 1e6 on the N_side 512 grid 5.26 -> 5.01 ms, 16
+// shells 12.95 -> 12.51 ms.  Launching yet earlier (griddepcontrol.launch_dependents at the
+// start of each kernel) gained no more on one stream, and the waiting blocks took places
+// from the other streams' kernels (16 shells 13.15 ms).
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    count_launch();
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
 int64_t launch_total();
 
 // ------------------------------------------------------------ device buffers

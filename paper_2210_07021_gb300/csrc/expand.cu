@@ -785,9 +785,10 @@ __global__ void k_m2m(TreeView T, int a, int b, int lvl, int p, const double* __
 // Narrow levels (launch_m2m_narrow): one CTA per parent, one warp per child, so
 // that the level takes one translation's latency (FP64; the double-float one is in
 // updown_df.cu).
-__global__ void __launch_bounds__(128) k_m2m_narrow(TreeView T, int a, int b, int lvl, int p, const double* __restrict__ tables,
-                                                    const XGeo* __restrict__ geo, double* __restrict__ mpole)
+__global__ void __launch_bounds__(128) k_m2m_narrow(TreeView T, int a, int b, int lvl, int p, const double* tables,
+                                                    const XGeo* geo, double* mpole)
 {
+    after_previous();
     if (T.d_level) {              // graph mode: the parents are the nodes of level lvl
         a = (int)T.d_level[lvl];
         b = (int)T.d_level[lvl + 1];
@@ -850,9 +851,10 @@ __global__ void k_m2l(TreeView T, const int64_t* __restrict__ off, const uint32_
 // ----------------------------------------------------------------- L2L
 // One warp per node of one level holding targets: local += L2L(parent local).
 template <typename R, typename GR, typename ST>
-__global__ void k_l2l(TreeView T, int a, int b, int lvl, int p, const double* __restrict__ tables,
-                      const GR* __restrict__ geo, ST* __restrict__ local)
+__global__ void k_l2l(TreeView T, int a, int b, int lvl, int p, const double* tables,
+                      const GR* geo, ST* local)
 {
+    after_previous();
     if (T.d_level) {              // graph mode: the nodes of level lvl
         a = (int)T.d_level[lvl];
         b = (int)T.d_level[lvl + 1];
@@ -1102,8 +1104,7 @@ cudaError_t launch_m2m_narrow(const TreeView& T, int a, int b, int lvl, int p, c
                               double* mpole, cudaStream_t s)
 {
     if (b <= a) return cudaSuccess;
-    k_m2m_narrow<<<grid_for(b - a, 1), 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeo*>(geo), mpole);
-    count_launch();
+    launch_chained(k_m2m_narrow, grid_for(b - a, 1), 128, 0, s, T, a, b, lvl, p, tables, static_cast<const XGeo*>(geo), mpole);
     return cudaGetLastError();
 }
 
@@ -1194,12 +1195,11 @@ cudaError_t launch_l2l(const TreeView& T, int a, int b, int lvl, int p, const do
     if (b <= a) return cudaSuccess;
     const unsigned g = grid_for(b - a, 4);
     if (ek == EXP_F32)
-        k_l2l<float, XGeo32, float><<<g, 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeo32*>(geo),
+        launch_chained(k_l2l<float, XGeo32, float>, g, 128, 0, s, T, a, b, lvl, p, tables, static_cast<const XGeo32*>(geo),
                                                       static_cast<float*>(local));
     else
-        k_l2l<double, XGeo, double><<<g, 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeo*>(geo),
+        launch_chained(k_l2l<double, XGeo, double>, g, 128, 0, s, T, a, b, lvl, p, tables, static_cast<const XGeo*>(geo),
                                                       static_cast<double*>(local));
-    count_launch();
     return cudaGetLastError();
 }
 

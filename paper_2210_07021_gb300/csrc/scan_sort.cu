@@ -154,9 +154,10 @@ __device__ __forceinline__ uint32_t ld_word(const uint32_t* p) { return *reinter
 __device__ __forceinline__ void st_word(uint32_t* p, uint32_t v) { *reinterpret_cast<volatile uint32_t*>(p) = v; }
 
 // the digit counts of every pass: hist[pass][digit], zero at launch
-__global__ void __launch_bounds__(RS_HT) k_rs_hist(const uint64_t* __restrict__ keys, int64_t n, int passes,
-                                                  uint32_t* __restrict__ hist)
+__global__ void __launch_bounds__(RS_HT) k_rs_hist(const uint64_t* keys, int64_t n, int passes,
+                                                  uint32_t* hist)
 {
+    after_previous();
     __shared__ uint32_t cnt[8][256];
     for (int i = threadIdx.x; i < 8 * 256; i += RS_HT) (&cnt[0][0])[i] = 0;
     __syncthreads();
@@ -275,12 +276,13 @@ __global__ void __launch_bounds__(SC_T) k_rs_rows(uint32_t* __restrict__ counts,
 // from the tiles' counts (words: their exclusive sums per digit row, limit: the
 // tiles).  hist: the digits' totals in either case.
 template <int RS_T, int RS_I, int CTAS, bool LOOKB>
-__global__ void __launch_bounds__(RS_T, CTAS) k_rs_pass(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                                                    uint64_t* __restrict__ kout, uint32_t* __restrict__ vout,
-                                                    int64_t n, int shift, const uint32_t* __restrict__ hist,
-                                                    uint32_t* __restrict__ words, uint32_t* __restrict__ words_next,
-                                                    uint32_t* __restrict__ ticket, int limit)
+__global__ void __launch_bounds__(RS_T, CTAS) k_rs_pass(const uint64_t* kin, const uint32_t* vin,
+                                                    uint64_t* kout, uint32_t* vout,
+                                                    int64_t n, int shift, const uint32_t* hist,
+                                                    uint32_t* words, uint32_t* words_next,
+                                                    uint32_t* ticket, int limit)
 {
+    after_previous();
     static_assert(RS_T == 256, "one thread per digit");
     constexpr int RS_TILE = RS_T * RS_I, RS_W = RS_T / 32;
     extern __shared__ __align__(16) unsigned char rs_smem[];
@@ -466,15 +468,20 @@ cudaError_t radix_sort_t(uint64_t* k1, uint32_t* v1, uint64_t* k2, uint32_t* v2,
     if (LOOKB) {
         if ((e = cudaMemsetAsync(hist, 0, RS_HEAD + (size_t)ntiles * 256 * sizeof(uint32_t), s))) return e;
         const int64_t hb = (n + RS_HT * 8 - 1) / (RS_HT * 8);
-        k_rs_hist<<<(unsigned)(hb < 152 * 8 ? hb : 152 * 8), RS_HT, 0, s>>>(ka, n, passes, hist); count_launch();
+        launch_chained(k_rs_hist, (unsigned)(hb < 152 * 8 ? hb : 152 * 8), RS_HT, 0, s, ka, n, passes, hist);
     }
     for (int p = 0; p < passes; ++p) {
         if constexpr (!LOOKB) {
             k_rs_tile_counts<T, I><<<(unsigned)ntiles, T, 0, s>>>(ka, n, 8 * p, words[0], ntiles); count_launch();
             k_rs_rows<<<256, SC_T, 0, s>>>(words[0], ntiles, hist + 256 * p); count_launch();
         }
-        pass<<<(unsigned)ntiles, T, smem, s>>>(ka, va, kb, vb, n, 8 * p, hist + 256 * p, words[LOOKB ? p & 1 : 0],
-                                               words[(p + 1) & 1], tickets + p, LOOKB ? limit : (int)ntiles); count_launch();
+        uint32_t *w = words[LOOKB ? p & 1 : 0], *wn = words[(p + 1) & 1];
+        if (LOOKB) {
+            launch_chained(pass, (unsigned)ntiles, T, smem, s, ka, va, kb, vb, n, 8 * p, hist + 256 * p, w, wn, tickets + p, limit);
+        } else {
+            pass<<<(unsigned)ntiles, T, smem, s>>>(ka, va, kb, vb, n, 8 * p, hist + 256 * p, w, wn, tickets + p, (int)ntiles);
+            count_launch();
+        }
         std::swap(ka, kb);
         std::swap(va, vb);
         alt = !alt;

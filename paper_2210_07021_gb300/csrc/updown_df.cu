@@ -262,8 +262,9 @@ __device__ __forceinline__ void translate_warp(int p, int lane, const XGeoDF& G,
 
 // M2M: one CTA per parent (the nodes of level lvl), one warp per child
 __global__ void __launch_bounds__(128) k_m2m_df_narrow(TreeView T, int a, int b, int lvl, int p,
-                                                       const XGeoDF* __restrict__ geo, dflt* __restrict__ mpole)
+                                                       const XGeoDF* geo, dflt* mpole)
 {
+    after_previous();
     if (T.d_level) {              // graph mode
         a = (int)T.d_level[lvl];
         b = (int)T.d_level[lvl + 1];
@@ -297,9 +298,10 @@ __global__ void __launch_bounds__(128) k_m2m_df_narrow(TreeView T, int a, int b,
 
 // L2L: one warp per node of level lvl (as k_l2l_df)
 __global__ void __launch_bounds__(128) k_l2l_df_narrow(TreeView T, int a, int b, int lvl, int p,
-                                                       const XGeoDF* __restrict__ geo, const double* __restrict__ acc,
-                                                       dflt* __restrict__ local)
+                                                       const XGeoDF* geo, const double* acc,
+                                                       dflt* local)
 {
+    after_previous();
     if (T.d_level) {              // graph mode
         a = (int)T.d_level[lvl];
         b = (int)T.d_level[lvl + 1];
@@ -555,9 +557,8 @@ cudaError_t launch_m2m_df_narrow(const TreeView& T, int a, int b, int lvl, int p
                                  cudaStream_t s)
 {
     if (b <= a) return cudaSuccess;
-    k_m2m_df_narrow<<<grid_of(b - a, 1, 152 * 64), 128, 0, s>>>(T, a, b, lvl, p, static_cast<const XGeoDF*>(geo),
+    launch_chained(k_m2m_df_narrow, grid_of(b - a, 1, 152 * 64), 128, 0, s, T, a, b, lvl, p, static_cast<const XGeoDF*>(geo),
                                                                 static_cast<dflt*>(mpole));
-    count_launch();
     return cudaGetLastError();
 }
 
@@ -565,9 +566,8 @@ cudaError_t launch_l2l_df_narrow(const TreeView& T, int a, int b, int lvl, int p
                                  void* local, cudaStream_t s)
 {
     if (b <= a) return cudaSuccess;
-    k_l2l_df_narrow<<<grid_of(b - a, 4, 152 * 64), 128, 0, s>>>(T, a, b, lvl, p, static_cast<const XGeoDF*>(geo), acc,
+    launch_chained(k_l2l_df_narrow, grid_of(b - a, 4, 152 * 64), 128, 0, s, T, a, b, lvl, p, static_cast<const XGeoDF*>(geo), acc,
                                                                 static_cast<dflt*>(local));
-    count_launch();
     return cudaGetLastError();
 }
 

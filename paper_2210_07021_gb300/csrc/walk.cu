@@ -222,7 +222,7 @@ __global__ void k_init_frontier(int2* f, WalkState* S)
 
 __global__ void __launch_bounds__(WT) k_walk_round(TreeView T, const MacNode* __restrict__ mac,
                                                    const MacNode32* __restrict__ mac32, double c_s, double sigma,
-                                                   const int2* __restrict__ front, int2* __restrict__ next,
+                                                   const int2* front, int2* __restrict__ next,
                                                    WalkState* S, int round, WalkCaps caps, uint64_t* __restrict__ words,
                                                    int limit, uint64_t* __restrict__ m2l_t, uint32_t* __restrict__ m2l_s,
                                                    uint64_t* __restrict__ p2p_t, uint32_t* __restrict__ p2p_s)
@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(WT) k_walk_round(TreeView T, const MacNode* __
     __shared__ int64_t s_base[3];
     __shared__ uint32_t s_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    after_previous();
     const WalkRec R = S->rec[round];
     const int64_t n = R.front;
     const int64_t ntiles = (n + WTILE - 1) / WTILE;
@@ -417,10 +418,10 @@ cudaError_t build_lists(sfmm_plan_s* P, const TreeView& T, double c_s, double c_
         WalkCaps caps{cap_front, cap_m2l, cap_p2p};
         for (int r = 0; r < rounds; ++r) {
             int2* f[2] = {P->fa.as<int2>(), P->fb.as<int2>()};
-            k_walk_round<<<152 * 4, WT, 0, s>>>(T, P->macn.as<MacNode>(), P->macn32.as<MacNode32>(), c_s, P->opt.sigma,
-                                                f[r & 1], f[(r + 1) & 1], S, r, caps, P->wwords.as<uint64_t>(), limit,
-                                                P->m2l_t.as<uint64_t>(), P->m2l_s.as<uint32_t>(),
-                                                P->p2p_t.as<uint64_t>(), P->p2p_s.as<uint32_t>()); count_launch();
+            launch_chained(k_walk_round, 152 * 4, WT, 0, s, T, P->macn.as<MacNode>(), P->macn32.as<MacNode32>(), c_s,
+                           P->opt.sigma, f[r & 1], f[(r + 1) & 1], S, r, caps, P->wwords.as<uint64_t>(), limit,
+                           P->m2l_t.as<uint64_t>(), P->m2l_s.as<uint32_t>(), P->p2p_t.as<uint64_t>(),
+                           P->p2p_s.as<uint32_t>());
         }
         if ((e = cudaGetLastError())) return e;
         if (P->gm) {
