@@ -161,9 +161,10 @@ namespace {
 std::mutex g_err_mu;
 std::string g_plan_err;
 
-__global__ void k_gather_src(const double* __restrict__ xyz, const void* __restrict__ q, int q_f32,
-                             const uint32_t* __restrict__ perm, int64_t n, double4_32a* __restrict__ out)
+__global__ void k_gather_src(const double* xyz, const void* q, int q_f32,
+                             const uint32_t* perm, int64_t n, double4_32a* out)
 {
+    after_previous();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t j = perm[i];
         const double qq = q_f32 ? (double)static_cast<const float*>(q)[j] : static_cast<const double*>(q)[j];
@@ -220,9 +221,10 @@ __global__ void k_fill(double* __restrict__ p, int64_t n, double v)
         p[i] = v;
 }
 
-__global__ void k_gather_tgt(const double* __restrict__ xyz, const uint32_t* __restrict__ perm, int64_t n,
-                             double4_32a* __restrict__ out)
+__global__ void k_gather_tgt(const double* xyz, const uint32_t* perm, int64_t n,
+                             double4_32a* out)
 {
+    after_previous();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t j = perm[i];
         out[i] = make_double4_32a(xyz[3 * (size_t)j], xyz[3 * (size_t)j + 1], xyz[3 * (size_t)j + 2], 0.0);
@@ -387,7 +389,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         return cuda_fail(P, e, "sort sources");
     const uint64_t* skeys = P->skeys_alt ? P->skeys2.as<uint64_t>() : P->skeys.as<uint64_t>();
     const uint32_t* sperm = P->skeys_alt ? P->sperm2.as<uint32_t>() : P->sperm.as<uint32_t>();
-    k_gather_src<<<grid_for(N), 256, 0, s>>>(src, q, q_f32, sperm, N, P->src4.as<double4_32a>()); count_launch();
+    launch_chained(k_gather_src, grid_for(N), 256, 0, s, src, q, q_f32, sperm, N, P->src4.as<double4_32a>());
     if (adj_df) {
         if ((e = ensure(P->dip4, (size_t)N * 32))) return cuda_fail(P, e, "alloc dipoles");
         k_gather_dip_df<<<grid_for(N), 256, 0, s>>>(adj->dip, sperm, N, P->dip4.as<float4>()); count_launch();
@@ -410,7 +412,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         return cuda_fail(P, e, "sort targets");
     const uint64_t* tkeys = P->tkeys_alt ? P->tkeys2.as<uint64_t>() : P->tkeys.as<uint64_t>();
     const uint32_t* tperm = P->tkeys_alt ? P->tperm2.as<uint32_t>() : P->tperm.as<uint32_t>();
-    k_gather_tgt<<<grid_for(M), 256, 0, s2>>>(tgt, tperm, M, P->tgt4.as<double4_32a>()); count_launch();
+    launch_chained(k_gather_tgt, grid_for(M), 256, 0, s2, tgt, tperm, M, P->tgt4.as<double4_32a>());
     if ((e = cudaGetLastError()) || (e = cudaEventRecord(P->ev_join, s2))) return cuda_fail(P, e, "gather targets");
     tm.mark();
     // ---- tree and geometry (sources)

@@ -1729,9 +1729,10 @@ __global__ void __launch_bounds__(128, ADJ ? 4 : 5) k_eval_df(EvalDfArgs A)
 // instructions (the difference to 2^-47): each sorted target from its leaf's
 // centre, and each near leaf's centre from its target leaf's centre (one per
 // direct-act pair).
-__global__ void k_tgt_offsets(TreeView T, const int2* __restrict__ items, int64_t n_cap, const int64_t* d_nit,
-                              const double4_32a* __restrict__ tgt, float4* __restrict__ off)
+__global__ void k_tgt_offsets(TreeView T, const int2* items, int64_t n_cap, const int64_t* d_nit,
+                              const double4_32a* tgt, float4* off)
 {
+    after_previous();
     const int64_t n_items = dcount(d_nit, n_cap);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1752,9 +1753,10 @@ __global__ void k_tgt_offsets(TreeView T, const int2* __restrict__ items, int64_
 }
 
 // per direct-act pair: (hi offset, first source of the near leaf), (lo offset, its source count)
-__global__ void k_pair_offsets(TreeView T, const uint64_t* __restrict__ tt, const uint32_t* __restrict__ ss,
-                               int64_t n_cap, const int64_t* d_n, float4* __restrict__ dc)
+__global__ void k_pair_offsets(TreeView T, const uint64_t* tt, const uint32_t* ss,
+                               int64_t n_cap, const int64_t* d_n, float4* dc)
 {
+    after_previous();
     const int64_t n = dcount(d_n, n_cap);
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t sl = ss[k];
@@ -1792,12 +1794,12 @@ cudaError_t launch_eval32_prep(const TreeView& T, const int2* items, int64_t n_i
     if (n_items > 0) {
         int64_t b = (n_items + 7) / 8;
         if (b > 152 * 64) b = 152 * 64;
-        k_tgt_offsets<<<(unsigned)b, 256, 0, s>>>(T, items, n_items, d_nit, tgt, toff); count_launch();
+        launch_chained(k_tgt_offsets, (unsigned)b, 256, 0, s, T, items, n_items, d_nit, tgt, toff);
     }
     if (n_p2p > 0) {
         int64_t b = (n_p2p + 255) / 256;
         if (b > 152 * 64) b = 152 * 64;
-        k_pair_offsets<<<(unsigned)b, 256, 0, s>>>(T, p2p_t, p2p_s, n_p2p, d_np, dc); count_launch();
+        launch_chained(k_pair_offsets, (unsigned)b, 256, 0, s, T, p2p_t, p2p_s, n_p2p, d_np, dc);
     }
     return cudaGetLastError();
 }

@@ -174,8 +174,9 @@ __device__ __forceinline__ XGeo32 make_geo32(int kind, const double* gS, const d
 }
 
 // FP32 frame vectors and scale of every node (e_theta, e_phi, r, padding)
-__global__ void k_geom32(int n_nodes, const double* __restrict__ geom, float* __restrict__ g32)
+__global__ void k_geom32(int n_nodes, const double* geom, float* g32)
 {
+    after_previous();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes; i += (int64_t)gridDim.x * blockDim.x) {
         const double* g = geom + (size_t)i * GEOM_STRIDE;
         float* o = g32 + (size_t)i * 8;
@@ -185,10 +186,11 @@ __global__ void k_geom32(int n_nodes, const double* __restrict__ geom, float* __
     }
 }
 
-__global__ void k_pair_geo32(TreeView T, const float* __restrict__ g32, const uint64_t* __restrict__ tt,
-                             const uint32_t* __restrict__ ss, int64_t n_cap, const int64_t* d_n,
-                             XGeo32* __restrict__ out)
+__global__ void k_pair_geo32(TreeView T, const float* g32, const uint64_t* tt,
+                             const uint32_t* ss, int64_t n_cap, const int64_t* d_n,
+                             XGeo32* out)
 {
+    after_previous();
     const int64_t n = dcount(d_n, n_cap);
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t s = ss[k], t = (uint32_t)tt[k];
@@ -197,9 +199,10 @@ __global__ void k_pair_geo32(TreeView T, const float* __restrict__ g32, const ui
     }
 }
 
-__global__ void k_child_geo32(TreeView T, const float* __restrict__ g32, XGeo32* __restrict__ m2m,
-                              XGeo32* __restrict__ l2l)
+__global__ void k_child_geo32(TreeView T, const float* g32, XGeo32* m2m,
+                              XGeo32* l2l)
 {
+    after_previous();
     const int64_t nn = dcount(T.d_nn, T.n_nodes);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += (int64_t)gridDim.x * blockDim.x) {
         const int par = T.parent[i];
@@ -212,9 +215,10 @@ __global__ void k_child_geo32(TreeView T, const float* __restrict__ g32, XGeo32*
 }
 
 template <typename GR>
-__global__ void k_pair_geo(TreeView T, const uint64_t* __restrict__ tt, const uint32_t* __restrict__ ss, int64_t n_cap,
-                           const int64_t* d_n, GR* __restrict__ out)
+__global__ void k_pair_geo(TreeView T, const uint64_t* tt, const uint32_t* ss, int64_t n_cap,
+                           const int64_t* d_n, GR* out)
 {
+    after_previous();
     const int64_t n = dcount(d_n, n_cap);
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const double* gS = T.geom + (size_t)ss[k] * GEOM_STRIDE;
@@ -232,8 +236,9 @@ __global__ void k_pair_geo(TreeView T, const uint64_t* __restrict__ tt, const ui
 // log sin(theta/2) are double-float (the table logarithm of the evaluation).
 // The azimuths come from the shorter of D and E as in pair_geometry.
 
-__global__ void k_frame_df(int n_cap, const int64_t* d_nn, const double* __restrict__ geom, FrameDF* __restrict__ out)
+__global__ void k_frame_df(int n_cap, const int64_t* d_nn, const double* geom, FrameDF* out)
 {
+    after_previous();
     const int64_t n_nodes = dcount(d_nn, n_cap);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes; i += (int64_t)gridDim.x * blockDim.x) {
         const double* g = geom + (size_t)i * GEOM_STRIDE;
@@ -280,10 +285,11 @@ __device__ __forceinline__ PairGeoDF pair_geometry_df(const double* gS, const do
 
 // M2L parameters of the thread-per-pair double-float kernel (m2l_pair.cu):
 // a ph1, b ph2, rho = g/(a b) = 1/cos^2(theta/2), log sin(theta/2).
-__global__ void k_pair_geo_rho(TreeView T, const FrameDF* __restrict__ fr, const float4* __restrict__ log_tab,
-                               const uint64_t* __restrict__ tt, const uint32_t* __restrict__ ss, int64_t n_cap,
-                               const int64_t* d_n, XGeoRho* __restrict__ out)
+__global__ void k_pair_geo_rho(TreeView T, const FrameDF* fr, const float4* log_tab,
+                               const uint64_t* tt, const uint32_t* ss, int64_t n_cap,
+                               const int64_t* d_n, XGeoRho* out)
 {
+    after_previous();
     __shared__ float4 s_tab[129];
     for (int i = threadIdx.x; i < 129; i += blockDim.x) s_tab[i] = log_tab[i];
     __syncthreads();
@@ -314,9 +320,10 @@ __global__ void k_pair_geo_rho(TreeView T, const FrameDF* __restrict__ fr, const
 }
 
 // M2M and L2L parameters per node with a parent (the double-float paths)
-__global__ void k_child_geo_df(TreeView T, const FrameDF* __restrict__ fr, const float4* __restrict__ log_tab,
-                               XGeoDF* __restrict__ m2m, XGeoDF* __restrict__ l2l)
+__global__ void k_child_geo_df(TreeView T, const FrameDF* fr, const float4* log_tab,
+                               XGeoDF* m2m, XGeoDF* l2l)
 {
+    after_previous();
     __shared__ float4 s_tab[129];
     for (int i = threadIdx.x; i < 129; i += blockDim.x) s_tab[i] = log_tab[i];
     __syncthreads();
@@ -357,8 +364,9 @@ __global__ void k_child_geo_df(TreeView T, const FrameDF* __restrict__ fr, const
 
 // per node with a parent: child -> parent (M2M) and parent -> child (L2L)
 template <typename GR>
-__global__ void k_child_geo(TreeView T, GR* __restrict__ m2m, GR* __restrict__ l2l)
+__global__ void k_child_geo(TreeView T, GR* m2m, GR* l2l)
 {
+    after_previous();
     const int64_t nn = dcount(T.d_nn, T.n_nodes);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += (int64_t)gridDim.x * blockDim.x) {
         const int par = T.parent[i];
@@ -753,9 +761,10 @@ __global__ void k_p2m32(TreeView T, const int* __restrict__ leaves, int64_t n_ca
 // One warp per internal node of one level: sum of its children's multipoles
 // (pipelined over the non-empty children).
 template <typename R, typename GR, typename ST>
-__global__ void k_m2m(TreeView T, int a, int b, int lvl, int p, const double* __restrict__ tables,
-                      const GR* __restrict__ geo, ST* __restrict__ mpole)
+__global__ void k_m2m(TreeView T, int a, int b, int lvl, int p, const double* tables,
+                      const GR* geo, ST* mpole)
 {
+    after_previous();
     if (T.d_level) {              // graph mode: the parents are the nodes of level lvl
         a = (int)T.d_level[lvl];
         b = (int)T.d_level[lvl + 1];
@@ -910,11 +919,12 @@ __global__ void k_m2l_list(const uint64_t* __restrict__ ptgt, const uint32_t* __
 // at or near antipodes): one warp per listed pair, in double-float from the
 // a, b, g form, its parameters formed from the node centres in FP64; the
 // result is added to the FP64 accumulators of the target box.
-__global__ void k_m2l_left_df(TreeView T, const uint64_t* __restrict__ ptgt, const uint32_t* __restrict__ psrc,
-                              const uint32_t* __restrict__ list, const uint32_t* __restrict__ n_list, int p,
-                              const double* __restrict__ tables, const dflt* __restrict__ mpole,
-                              double* __restrict__ acc)
+__global__ void k_m2l_left_df(TreeView T, const uint64_t* ptgt, const uint32_t* psrc,
+                              const uint32_t* list, const uint32_t* n_list, int p,
+                              const double* tables, const dflt* mpole,
+                              double* acc)
 {
+    after_previous();
     __shared__ Tables<dflt> tb;
     __shared__ WarpSmem<dflt> ws[4];
     load_tables<dflt>(&tb, tables);
@@ -947,9 +957,10 @@ __global__ void k_acc_to_df(int64_t n, const double* __restrict__ acc, dflt* __r
 // FP32 offset of every key-sorted source from the centre of its leaf as an
 // (hi, lo) pair (the difference to 2^-47, formed without FP64 instructions),
 // plus its mass split the same way: off[2j] = (hi, q_hi), off[2j+1] = (lo, q_lo).
-__global__ void k_src_offsets(TreeView T, const int* __restrict__ leaves, int64_t n_cap, const int64_t* d_nl,
-                              const double4_32a* __restrict__ src, float4* __restrict__ off)
+__global__ void k_src_offsets(TreeView T, const int* leaves, int64_t n_cap, const int64_t* d_nl,
+                              const double4_32a* src, float4* off)
 {
+    after_previous();
     const int64_t n_leaves = dcount(d_nl, n_cap);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1017,7 +1028,7 @@ void fill_tables(double* h)   // [2][PMAX][PMAX]
 
 cudaError_t launch_geom32(int n_nodes, const double* geom, float* g32, cudaStream_t s)
 {
-    k_geom32<<<grid_for(n_nodes, 256), 256, 0, s>>>(n_nodes, geom, g32); count_launch();
+    launch_chained(k_geom32, grid_for(n_nodes, 256), 256, 0, s, n_nodes, geom, g32);
     return cudaGetLastError();
 }
 
@@ -1025,20 +1036,18 @@ cudaError_t launch_pair_geo(const TreeView& T, const float* g32, const uint64_t*
                             const int64_t* d_n, void* out, int ek, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    if (ek == EXP_F32) k_pair_geo32<<<grid_for(n, 256), 256, 0, s>>>(T, g32, tt, ss, n, d_n, static_cast<XGeo32*>(out));
-    else if (ek == EXP_DF) k_pair_geo<XGeoDF><<<grid_for(n, 256), 256, 0, s>>>(T, tt, ss, n, d_n, static_cast<XGeoDF*>(out));
-    else k_pair_geo<XGeo><<<grid_for(n, 256), 256, 0, s>>>(T, tt, ss, n, d_n, static_cast<XGeo*>(out));
-    count_launch();
+    if (ek == EXP_F32) launch_chained(k_pair_geo32, grid_for(n, 256), 256, 0, s, T, g32, tt, ss, n, d_n, static_cast<XGeo32*>(out));
+    else if (ek == EXP_DF) launch_chained(k_pair_geo<XGeoDF>, grid_for(n, 256), 256, 0, s, T, tt, ss, n, d_n, static_cast<XGeoDF*>(out));
+    else launch_chained(k_pair_geo<XGeo>, grid_for(n, 256), 256, 0, s, T, tt, ss, n, d_n, static_cast<XGeo*>(out));
     return cudaGetLastError();
 }
 
 cudaError_t launch_child_geo(const TreeView& T, const float* g32, void* m2m, void* l2l, int ek, cudaStream_t s)
 {
     const unsigned g = grid_for(T.n_nodes, 256);
-    if (ek == EXP_F32) k_child_geo32<<<g, 256, 0, s>>>(T, g32, static_cast<XGeo32*>(m2m), static_cast<XGeo32*>(l2l));
-    else if (ek == EXP_DF) k_child_geo<XGeoDF><<<g, 256, 0, s>>>(T, static_cast<XGeoDF*>(m2m), static_cast<XGeoDF*>(l2l));
-    else k_child_geo<XGeo><<<g, 256, 0, s>>>(T, static_cast<XGeo*>(m2m), static_cast<XGeo*>(l2l));
-    count_launch();
+    if (ek == EXP_F32) launch_chained(k_child_geo32, g, 256, 0, s, T, g32, static_cast<XGeo32*>(m2m), static_cast<XGeo32*>(l2l));
+    else if (ek == EXP_DF) launch_chained(k_child_geo<XGeoDF>, g, 256, 0, s, T, static_cast<XGeoDF*>(m2m), static_cast<XGeoDF*>(l2l));
+    else launch_chained(k_child_geo<XGeo>, g, 256, 0, s, T, static_cast<XGeo*>(m2m), static_cast<XGeo*>(l2l));
     return cudaGetLastError();
 }
 
@@ -1046,7 +1055,7 @@ cudaError_t launch_src_offsets(const TreeView& T, const int* leaves, int64_t n_l
                                const double4_32a* src, float4* off, cudaStream_t s)
 {
     if (n_leaves == 0) return cudaSuccess;
-    k_src_offsets<<<grid_for(n_leaves, 8), 256, 0, s>>>(T, leaves, n_leaves, d_nl, src, off); count_launch();
+    launch_chained(k_src_offsets, grid_for(n_leaves, 8), 256, 0, s, T, leaves, n_leaves, d_nl, src, off);
     return cudaGetLastError();
 }
 
@@ -1090,7 +1099,7 @@ cudaError_t launch_m2m(const TreeView& T, int a, int b, int lvl, int p, const do
     if (b <= a) return cudaSuccess;
     const unsigned g = grid_for(b - a, 4);
     if (ek == EXP_F32)
-        k_m2m<float, XGeo32, float><<<g, 128, 0, s>>>(T, a, b, lvl, p, tables, static_cast<const XGeo32*>(geo),
+        launch_chained(k_m2m<float, XGeo32, float>, g, 128, 0, s, T, a, b, lvl, p, tables, static_cast<const XGeo32*>(geo),
                                                       static_cast<float*>(mpole));
     else
         return cudaErrorInvalidValue;             // the FP64 and double-float paths: kernels of their own
@@ -1145,8 +1154,7 @@ size_t frame_df_bytes() { return sizeof(FrameDF); }
 cudaError_t launch_frame_df(int n_nodes, const int64_t* d_nn, const double* geom, void* out, cudaStream_t s)
 {
     if (n_nodes == 0) return cudaSuccess;
-    k_frame_df<<<grid_for(n_nodes, 256), 256, 0, s>>>(n_nodes, d_nn, geom, static_cast<FrameDF*>(out));
-    count_launch();
+    launch_chained(k_frame_df, grid_for(n_nodes, 256), 256, 0, s, n_nodes, d_nn, geom, static_cast<FrameDF*>(out));
     return cudaGetLastError();
 }
 
@@ -1154,18 +1162,16 @@ cudaError_t launch_pair_geo_rho(const TreeView& T, const void* frames, const flo
                                 const uint32_t* ss, int64_t n, const int64_t* d_n, void* out, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    k_pair_geo_rho<<<grid_for(n, 256), 256, 0, s>>>(T, static_cast<const FrameDF*>(frames), log_tab, tt, ss, n, d_n,
+    launch_chained(k_pair_geo_rho, grid_for(n, 256), 256, 0, s, T, static_cast<const FrameDF*>(frames), log_tab, tt, ss, n, d_n,
                                                      static_cast<XGeoRho*>(out));
-    count_launch();
     return cudaGetLastError();
 }
 
 cudaError_t launch_child_geo_df(const TreeView& T, const void* frames, const float4* log_tab, void* m2m, void* l2l,
                                 cudaStream_t s)
 {
-    k_child_geo_df<<<grid_for(T.n_nodes, 256), 256, 0, s>>>(T, static_cast<const FrameDF*>(frames), log_tab,
+    launch_chained(k_child_geo_df, grid_for(T.n_nodes, 256), 256, 0, s, T, static_cast<const FrameDF*>(frames), log_tab,
                                                              static_cast<XGeoDF*>(m2m), static_cast<XGeoDF*>(l2l));
-    count_launch();
     return cudaGetLastError();
 }
 
@@ -1174,9 +1180,8 @@ cudaError_t launch_m2l_left_df(const TreeView& T, const uint64_t* ptgt, const ui
                                const void* mpole, double* acc, cudaStream_t s)
 {
     if (max_list == 0) return cudaSuccess;
-    k_m2l_left_df<<<grid_for(max_list < 152 * 64 ? max_list : 152 * 64, 4), 128, 0, s>>>(
+    launch_chained(k_m2l_left_df, grid_for(max_list < 152 * 64 ? max_list : 152 * 64, 4), 128, 0, s,
         T, ptgt, psrc, list, n_list, p, tables, static_cast<const dflt*>(mpole), acc);
-    count_launch();
     return cudaGetLastError();
 }
 

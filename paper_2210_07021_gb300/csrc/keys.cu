@@ -517,9 +517,10 @@ __device__ __noinline__ uint64_t key29_exact(double x, double y, double z)
     return key_from_floors(cap, (uint32_t)trunc_scaled(vp, ORDER_MAX), (uint32_t)trunc_scaled(vm, ORDER_MAX), ntt, nonneg(z));
 }
 
-__global__ void __launch_bounds__(256) k_keys(const double* __restrict__ xyz, int64_t n, uint64_t* __restrict__ keys,
-                                              uint32_t* __restrict__ iota)
+__global__ void __launch_bounds__(256) k_keys(const double* xyz, int64_t n, uint64_t* keys,
+                                              uint32_t* iota)
 {
+    after_previous();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
         uint64_t k;
@@ -536,7 +537,7 @@ cudaError_t launch_keys(const double* xyz, int64_t n, uint64_t* keys, uint32_t* 
     if (n <= 0) return cudaSuccess;
     int64_t blocks = (n + 255) / 256;
     if (blocks > 152 * 32) blocks = 152 * 32;
-    k_keys<<<(unsigned)blocks, 256, 0, s>>>(xyz, n, keys, iota); count_launch();
+    launch_chained(k_keys, (unsigned)blocks, 256, 0, s, xyz, n, keys, iota);
     return cudaGetLastError();
 }
 

@@ -276,8 +276,9 @@ __device__ __forceinline__ void ld_row64(double* row, const double* e, int p, in
 // L lanes per child of a level; the four siblings' lanes sum their rows into the parent
 template <int P, int L>
 __global__ void __launch_bounds__(128, 3) k_m2m64(TreeView T, int c0, int c1, int lvl, int p,
-                                                  const XGeo* __restrict__ geo, double* __restrict__ mpole)
+                                                  const XGeo* geo, double* mpole)
 {
+    after_previous();
     if (T.d_level) {              // graph mode: the children are the nodes of level lvl + 1
         c0 = (int)T.d_level[lvl + 1];
         c1 = (int)T.d_level[lvl + 2];
@@ -322,8 +323,9 @@ __global__ void __launch_bounds__(128, 3) k_m2m64(TreeView T, int c0, int c1, in
 // L lanes per node of a level holding targets: local += the parent's local translated
 template <int P, int L>
 __global__ void __launch_bounds__(128, 3) k_l2l64(TreeView T, int a, int b, int lvl, int p,
-                                                  const XGeo* __restrict__ geo, double* __restrict__ local)
+                                                  const XGeo* geo, double* local)
 {
+    after_previous();
     if (T.d_level) {              // graph mode: the nodes of level lvl
         a = (int)T.d_level[lvl];
         b = (int)T.d_level[lvl + 1];
@@ -363,8 +365,7 @@ cudaError_t level_p(K kern, int64_t n, int lanes, cudaStream_t s, Args... args)
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
     const int64_t blocks = (n + per - 1) / per;
-    kern<<<(unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 128, smem, s>>>(args...);
-    count_launch();
+    launch_chained(kern, (unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 128, smem, s, args...);
     return cudaGetLastError();
 }
 

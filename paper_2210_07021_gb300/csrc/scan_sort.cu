@@ -53,8 +53,9 @@ __device__ __forceinline__ T block_excl_scan(T v, T* s_warp, T* total)
 }
 
 template <typename T>
-__global__ void k_scan_reduce(const T* __restrict__ in, int64_t n, T* __restrict__ bsum)
+__global__ void k_scan_reduce(const T* in, int64_t n, T* bsum)
 {
+    after_previous();
     __shared__ T s_warp[SC_T / 32];
     __shared__ T s_total;
     const int64_t base = (int64_t)blockIdx.x * SC_TILE;
@@ -68,8 +69,9 @@ __global__ void k_scan_reduce(const T* __restrict__ in, int64_t n, T* __restrict
 }
 
 template <typename T>
-__global__ void k_scan_top(T* __restrict__ bsum, int64_t nb, T* __restrict__ total)
+__global__ void k_scan_top(T* bsum, int64_t nb, T* total)
 {
+    after_previous();
     __shared__ T s_warp[SC_T / 32];
     __shared__ T s_total;
     T carry = 0;
@@ -85,8 +87,9 @@ __global__ void k_scan_top(T* __restrict__ bsum, int64_t nb, T* __restrict__ tot
 }
 
 template <typename T>
-__global__ void k_scan_down(const T* __restrict__ in, T* __restrict__ out, int64_t n, const T* __restrict__ bsum)
+__global__ void k_scan_down(const T* in, T* out, int64_t n, const T* bsum)
 {
+    after_previous();
     __shared__ T s_tile[SC_TILE];
     __shared__ T s_warp[SC_T / 32];
     __shared__ T s_total;
@@ -118,9 +121,9 @@ cudaError_t exclusive_scan_t(const T* in, T* out, int64_t n, T* total, void* tmp
     }
     const int64_t nb = (n + SC_TILE - 1) / SC_TILE;
     T* bsum = static_cast<T*>(tmp);
-    k_scan_reduce<T><<<(unsigned)nb, SC_T, 0, s>>>(in, n, bsum); count_launch();
-    k_scan_top<T><<<1, SC_T, 0, s>>>(bsum, nb, total); count_launch();
-    k_scan_down<T><<<(unsigned)nb, SC_T, 0, s>>>(in, out, n, bsum); count_launch();
+    launch_chained(k_scan_reduce<T>, (unsigned)nb, SC_T, 0, s, in, n, bsum);
+    launch_chained(k_scan_top<T>, 1, SC_T, 0, s, bsum, nb, total);
+    launch_chained(k_scan_down<T>, (unsigned)nb, SC_T, 0, s, in, out, n, bsum);
     return cudaGetLastError();
 }
 
@@ -221,9 +224,10 @@ __device__ __forceinline__ bool look_back(const uint32_t* __restrict__ words, in
 // counts[digit][tile], then one block per digit turns its row into exclusive
 // sums over the tiles and writes the digit's total.
 template <int T, int I>
-__global__ void __launch_bounds__(T) k_rs_tile_counts(const uint64_t* __restrict__ keys, int64_t n, int shift,
-                                                      uint32_t* __restrict__ counts, int64_t ntiles)
+__global__ void __launch_bounds__(T) k_rs_tile_counts(const uint64_t* keys, int64_t n, int shift,
+                                                      uint32_t* counts, int64_t ntiles)
 {
+    after_previous();
     __shared__ uint32_t cnt[256];
     for (int i = threadIdx.x; i < 256; i += T) cnt[i] = 0;
     __syncthreads();
@@ -237,9 +241,10 @@ __global__ void __launch_bounds__(T) k_rs_tile_counts(const uint64_t* __restrict
     for (int i = threadIdx.x; i < 256; i += T) counts[(int64_t)i * ntiles + blockIdx.x] = cnt[i];
 }
 
-__global__ void __launch_bounds__(SC_T) k_rs_rows(uint32_t* __restrict__ counts, int64_t ntiles,
-                                                  uint32_t* __restrict__ totals)
+__global__ void __launch_bounds__(SC_T) k_rs_rows(uint32_t* counts, int64_t ntiles,
+                                                  uint32_t* totals)
 {
+    after_previous();
     __shared__ uint32_t s_warp[SC_T / 32];
     __shared__ uint32_t s_total;
     uint32_t* row = counts + (int64_t)blockIdx.x * ntiles;
@@ -472,16 +477,12 @@ cudaError_t radix_sort_t(uint64_t* k1, uint32_t* v1, uint64_t* k2, uint32_t* v2,
     }
     for (int p = 0; p < passes; ++p) {
         if constexpr (!LOOKB) {
-            k_rs_tile_counts<T, I><<<(unsigned)ntiles, T, 0, s>>>(ka, n, 8 * p, words[0], ntiles); count_launch();
-            k_rs_rows<<<256, SC_T, 0, s>>>(words[0], ntiles, hist + 256 * p); count_launch();
+            launch_chained(k_rs_tile_counts<T, I>, (unsigned)ntiles, T, 0, s, ka, n, 8 * p, words[0], ntiles);
+            launch_chained(k_rs_rows, 256, SC_T, 0, s, words[0], ntiles, hist + 256 * p);
         }
         uint32_t *w = words[LOOKB ? p & 1 : 0], *wn = words[(p + 1) & 1];
-        if (LOOKB) {
-            launch_chained(pass, (unsigned)ntiles, T, smem, s, ka, va, kb, vb, n, 8 * p, hist + 256 * p, w, wn, tickets + p, limit);
-        } else {
-            pass<<<(unsigned)ntiles, T, smem, s>>>(ka, va, kb, vb, n, 8 * p, hist + 256 * p, w, wn, tickets + p, (int)ntiles);
-            count_launch();
-        }
+        launch_chained(pass, (unsigned)ntiles, T, smem, s, ka, va, kb, vb, n, 8 * p, hist + 256 * p, w, wn, tickets + p,
+                       LOOKB ? limit : (int)ntiles);
         std::swap(ka, kb);
         std::swap(va, vb);
         alt = !alt;

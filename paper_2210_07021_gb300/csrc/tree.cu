@@ -108,9 +108,10 @@ __global__ void k_level0(const uint64_t* __restrict__ keys, int64_t n, uint64_t*
 // Graph mode (dc != NULL): the level's bounds come from dc->level, the launch
 // covers `width` (the level-width capacity) and the flags beyond the level are
 // zero, so that a scan over the whole capacity is the scan of the level.
-__global__ void k_split_flags(const int* __restrict__ count, int a, int b, int lvl, int m, int max_depth,
-                              int64_t* __restrict__ flags, DevCounts* dc, int64_t width)
+__global__ void k_split_flags(const int* count, int a, int b, int lvl, int m, int max_depth,
+                              int64_t* flags, DevCounts* dc, int64_t width)
 {
+    after_previous();
     if (dc) {
         a = (int)dc->level[lvl];
         b = (int)dc->level[lvl + 1];
@@ -131,8 +132,9 @@ __global__ void k_counts_init(DevCounts* dc)
 // Graph mode: the next level's end from the scan of the split flags (its total),
 // or an overflow if the nodes would not fit the capacity (`last`: the deepest
 // level the capacity allows; a split there is an overflow too).
-__global__ void k_level_end(DevCounts* dc, int lvl, const int64_t* __restrict__ total, int64_t node_cap, int last)
+__global__ void k_level_end(DevCounts* dc, int lvl, const int64_t* total, int64_t node_cap, int last)
 {
+    after_previous();
     const int64_t b = dc->level[lvl + 1];
     int64_t nb = b + 4 * *total;
     // after an overflow the tree stops growing: the nodes built so far stay a
@@ -179,10 +181,11 @@ __device__ __forceinline__ void make_child(const uint64_t* __restrict__ keys, co
     if (c == 0) N.child0[node] = c0;
 }
 
-__global__ void k_make_children(const uint64_t* __restrict__ keys, int a, int b, int lvl,
-                                const int64_t* __restrict__ flags, const int64_t* __restrict__ pos, NodeArrays N,
+__global__ void k_make_children(const uint64_t* keys, int a, int b, int lvl,
+                                const int64_t* flags, const int64_t* pos, NodeArrays N,
                                 const DevCounts* dc)
 {
+    after_previous();
     if (dc) {
         if (dc->overflow) return;
         a = (int)dc->level[lvl];
@@ -211,10 +214,11 @@ struct TreeLevels {
 // geometry, and takes 0.06 ms.
 constexpr int TREE_NARROW = 4096, TREE_T = 1024;
 
-__global__ void __launch_bounds__(TREE_T) k_tree_narrow(const uint64_t* __restrict__ keys, int64_t n, int m,
+__global__ void __launch_bounds__(TREE_T) k_tree_narrow(const uint64_t* keys, int64_t n, int m,
                                                         int max_depth, int64_t node_cap, bool first, TreeLevels* L,
                                                         NodeArrays N)
 {
+    after_previous();
     __shared__ int s_node[TREE_NARROW];              // the level's split boxes in order
     __shared__ int s_warp[TREE_T / 32];
     __shared__ int s_total;
@@ -286,9 +290,10 @@ __global__ void __launch_bounds__(TREE_T) k_tree_narrow(const uint64_t* __restri
     }
 }
 
-__global__ void k_geometry(int n_cap, const int64_t* d_nn, const uint64_t* __restrict__ prefix,
-                           const int* __restrict__ level, double* __restrict__ geom)
+__global__ void k_geometry(int n_cap, const int64_t* d_nn, const uint64_t* prefix,
+                           const int* level, double* geom)
 {
+    after_previous();
     const int64_t n_nodes = dcount(d_nn, n_cap);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes; i += (int64_t)gridDim.x * blockDim.x) {
         const int order = level[i];
@@ -326,10 +331,11 @@ __global__ void k_geometry(int n_cap, const int64_t* d_nn, const uint64_t* __res
     }
 }
 
-__global__ void k_target_ranges(int n_cap, const int64_t* d_nn, const uint64_t* __restrict__ prefix,
-                                const int* __restrict__ level, const uint64_t* __restrict__ tkeys, int64_t M,
-                                int* __restrict__ tfirst, int* __restrict__ tcount)
+__global__ void k_target_ranges(int n_cap, const int64_t* d_nn, const uint64_t* prefix,
+                                const int* level, const uint64_t* tkeys, int64_t M,
+                                int* tfirst, int* tcount)
 {
+    after_previous();
     const int64_t n_nodes = dcount(d_nn, n_cap);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes; i += (int64_t)gridDim.x * blockDim.x) {
         const int shift = 2 * (ORDER_MAX - level[i]);
@@ -360,12 +366,13 @@ __device__ __forceinline__ int2 make_item(int node, int tc, int64_t k, int split
     return make_int2(node, tb | parts);
 }
 
-__global__ void __launch_bounds__(CT) k_collect(int n_cap, const int64_t* d_nn, const int* __restrict__ child0,
-                                                const int* __restrict__ count, const int* __restrict__ tcount,
-                                                int split, int* __restrict__ leaves, int2* __restrict__ items,
-                                                uint64_t* __restrict__ words, int64_t* __restrict__ n_leaves,
-                                                int64_t* __restrict__ n_items, uint32_t* __restrict__ ticket, int limit)
+__global__ void __launch_bounds__(CT) k_collect(int n_cap, const int64_t* d_nn, const int* child0,
+                                                const int* count, const int* tcount,
+                                                int split, int* leaves, int2* items,
+                                                uint64_t* words, int64_t* n_leaves,
+                                                int64_t* n_items, uint32_t* ticket, int limit)
 {
+    after_previous();
     __shared__ uint32_t s_tile;
     __shared__ int64_t s_warp[2][CT / 32], s_base[2];
     __shared__ int s_lost;
@@ -493,12 +500,12 @@ cudaError_t build_tree(sfmm_plan_s* P, const uint64_t* keys, int64_t n, int m, i
                                   P->n_count.as<int>(), P->n_child0.as<int>(), P->n_parent.as<int>()); count_launch();
         k_counts_init<<<1, 32, 0, s>>>(dc); count_launch();
         for (int lvl = 0; lvl < levels; ++lvl) {
-            k_split_flags<<<grid_for(width), 256, 0, s>>>(P->n_count.as<int>(), 0, 0, lvl, m, max_depth, flags, dc,
-                                                           width); count_launch();
+            launch_chained(k_split_flags, grid_for(width), 256, 0, s, P->n_count.as<int>(), 0, 0, lvl, m, max_depth, flags, dc,
+                                                           width);
             if ((e = exclusive_scan_i64(flags, pos, width, total, P->tmp.p, s))) return e;
-            k_level_end<<<1, 1, 0, s>>>(dc, lvl, total, P->cap.nodes, lvl == levels - 1); count_launch();
+            launch_chained(k_level_end, 1, 1, 0, s, dc, lvl, total, P->cap.nodes, lvl == levels - 1);
             if (lvl < levels - 1) {
-                k_make_children<<<grid_for(4 * width), 256, 0, s>>>(keys, 0, 0, lvl, flags, pos, arrays(), dc); count_launch();
+                launch_chained(k_make_children, grid_for(4 * width), 256, 0, s, keys, 0, 0, lvl, flags, pos, arrays(), dc);
             }
         }
         P->n_nodes = P->cap.nodes;
@@ -513,7 +520,7 @@ cudaError_t build_tree(sfmm_plan_s* P, const uint64_t* keys, int64_t n, int m, i
     P->level_start.push_back(12);
     bool first = true;
     while (true) {
-        k_tree_narrow<<<1, TREE_T, 0, s>>>(keys, n, m, max_depth, P->node_cap, first, dL, arrays()); count_launch();
+        launch_chained(k_tree_narrow, 1, TREE_T, 0, s, keys, n, m, max_depth, P->node_cap, first, dL, arrays());
         if ((e = cudaMemcpyAsync(hL, dL, sizeof *hL, cudaMemcpyDeviceToHost, s)) || (e = cudaStreamSynchronize(s)))
             return e;
         first = false;
@@ -534,15 +541,15 @@ cudaError_t build_tree(sfmm_plan_s* P, const uint64_t* keys, int64_t n, int m, i
             int64_t* flags = P->flags.as<int64_t>();
             int64_t* pos = P->pos.as<int64_t>();
             int64_t* total = P->small.as<int64_t>() + SM_TOTAL;
-            k_split_flags<<<grid_for(width), 256, 0, s>>>(P->n_count.as<int>(), a, b, lvl, m, max_depth, flags,
-                                                           nullptr, 0); count_launch();
+            launch_chained(k_split_flags, grid_for(width), 256, 0, s, P->n_count.as<int>(), a, b, lvl, m, max_depth, flags,
+                                                           nullptr, 0);
             if ((e = exclusive_scan_i64(flags, pos, width, total, P->tmp.p, s))) return e;
             int64_t* splits = P->h_small + SM_TOTAL;
             if ((e = cudaMemcpyAsync(splits, total, 8, cudaMemcpyDeviceToHost, s)) || (e = cudaStreamSynchronize(s)))
                 return e;
             if (*splits == 0) { end = true; break; }
             if ((e = grow(b + 4 * *splits))) return e;
-            k_make_children<<<grid_for(4 * width), 256, 0, s>>>(keys, a, b, lvl, flags, pos, arrays(), nullptr); count_launch();
+            launch_chained(k_make_children, grid_for(4 * width), 256, 0, s, keys, a, b, lvl, flags, pos, arrays(), nullptr);
             P->n_nodes = b + 4 * *splits;
             P->level_start.push_back((int)P->n_nodes);
             ++lvl;
@@ -564,9 +571,9 @@ cudaError_t tree_geometry(sfmm_plan_s* P)
     cudaError_t e;
     const int64_t nn = P->n_nodes;
     if ((e = ensure(P->n_geom, (size_t)nn * GEOM_STRIDE * 8))) return e;
-    k_geometry<<<grid_for(nn), 256, 0, P->stream>>>((int)nn, P->gm ? &P->dcnt.as<DevCounts>()->nn : nullptr,
+    launch_chained(k_geometry, grid_for(nn), 256, 0, P->stream, (int)nn, P->gm ? &P->dcnt.as<DevCounts>()->nn : nullptr,
                                                     P->n_prefix.as<uint64_t>(), P->n_level.as<int>(),
-                                                    P->n_geom.as<double>()); count_launch();
+                                                    P->n_geom.as<double>());
     return cudaGetLastError();
 }
 
@@ -576,9 +583,9 @@ cudaError_t tree_target_ranges(sfmm_plan_s* P, const uint64_t* tkeys, int64_t M)
     const int64_t nn = P->n_nodes;
     if ((e = ensure(P->n_tfirst, (size_t)nn * 4))) return e;
     if ((e = ensure(P->n_tcount, (size_t)nn * 4))) return e;
-    k_target_ranges<<<grid_for(nn), 256, 0, P->stream>>>((int)nn, P->gm ? &P->dcnt.as<DevCounts>()->nn : nullptr,
+    launch_chained(k_target_ranges, grid_for(nn), 256, 0, P->stream, (int)nn, P->gm ? &P->dcnt.as<DevCounts>()->nn : nullptr,
                                                          P->n_prefix.as<uint64_t>(), P->n_level.as<int>(), tkeys, M,
-                                                         P->n_tfirst.as<int>(), P->n_tcount.as<int>()); count_launch();
+                                                         P->n_tfirst.as<int>(), P->n_tcount.as<int>());
     return cudaGetLastError();
 }
 
@@ -604,11 +611,11 @@ cudaError_t collect_leaves_items(sfmm_plan_s* P, int64_t M, int64_t* d_leaves, i
         (e = ensure(P->cwords, wb)) || (e = cudaMemsetAsync(P->cwords.p, 0, wb, s)))
         return e;
     uint64_t* words = P->cwords.as<uint64_t>();
-    k_collect<<<(unsigned)ntiles, CT, 0, s>>>((int)nn, P->gm ? &P->dcnt.as<DevCounts>()->nn : nullptr,
+    launch_chained(k_collect, (unsigned)ntiles, CT, 0, s, (int)nn, P->gm ? &P->dcnt.as<DevCounts>()->nn : nullptr,
                                               P->n_child0.as<int>(), P->n_count.as<int>(), P->n_tcount.as<int>(), split,
                                               P->leaves_src.as<int>(), P->items.as<int2>(), words, d_leaves, d_items,
                                               reinterpret_cast<uint32_t*>(words + 2 * ntiles),
-                                              P->opt.wait_limit > 0 ? P->opt.wait_limit : LB_POLLS); count_launch();
+                                              P->opt.wait_limit > 0 ? P->opt.wait_limit : LB_POLLS);
     P->n_leaves = nn;
     P->n_items = cap;
     return cudaGetLastError();

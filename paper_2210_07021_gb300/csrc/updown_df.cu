@@ -110,8 +110,9 @@ __device__ __forceinline__ void ld_row(dflt* row, const dflt* e, int p, int P)
 // ----------------------------------------------------------------- M2M
 template <int P>
 __global__ void __launch_bounds__(128) k_m2m_df(TreeView T, int c0, int c1, int lvl, int p,
-                                                const XGeoDF* __restrict__ geo, dflt* __restrict__ mpole)
+                                                const XGeoDF* geo, dflt* mpole)
 {
+    after_previous();
     if (T.d_level) {              // graph mode: the children are the nodes of level lvl + 1
         c0 = (int)T.d_level[lvl + 1];
         c1 = (int)T.d_level[lvl + 2];
@@ -153,9 +154,10 @@ __global__ void __launch_bounds__(128) k_m2m_df(TreeView T, int c0, int c1, int 
 // ----------------------------------------------------------------- L2L
 template <int P>
 __global__ void __launch_bounds__(128) k_l2l_df(TreeView T, int a, int b, int lvl, int p,
-                                                const XGeoDF* __restrict__ geo, const double* __restrict__ acc,
-                                                dflt* __restrict__ local)
+                                                const XGeoDF* geo, const double* acc,
+                                                dflt* local)
 {
+    after_previous();
     if (T.d_level) {              // graph mode: the nodes of level lvl
         a = (int)T.d_level[lvl];
         b = (int)T.d_level[lvl + 1];
@@ -480,9 +482,8 @@ cudaError_t m2m_p(const TreeView& T, int c0, int c1, int lvl, int p, const void*
     const size_t smem = (size_t)128 * (2 * P + 3) * sizeof(dflt);
     cudaError_t e;
     if ((e = smem_attr(k_m2m_df<P>, smem))) return e;
-    k_m2m_df<P><<<grid_of(c1 - c0, 128, 152 * 16), 128, smem, s>>>(T, c0, c1, lvl, p, static_cast<const XGeoDF*>(geo),
+    launch_chained(k_m2m_df<P>, grid_of(c1 - c0, 128, 152 * 16), 128, smem, s, T, c0, c1, lvl, p, static_cast<const XGeoDF*>(geo),
                                                                    static_cast<dflt*>(mpole));
-    count_launch();
     return cudaGetLastError();
 }
 
@@ -493,9 +494,8 @@ cudaError_t l2l_p(const TreeView& T, int a, int b, int lvl, int p, const void* g
     const size_t smem = (size_t)128 * (2 * P + 3) * sizeof(dflt);
     cudaError_t e;
     if ((e = smem_attr(k_l2l_df<P>, smem))) return e;
-    k_l2l_df<P><<<grid_of(b - a, 128, 152 * 16), 128, smem, s>>>(T, a, b, lvl, p, static_cast<const XGeoDF*>(geo), acc,
+    launch_chained(k_l2l_df<P>, grid_of(b - a, 128, 152 * 16), 128, smem, s, T, a, b, lvl, p, static_cast<const XGeoDF*>(geo), acc,
                                                                  static_cast<dflt*>(local));
-    count_launch();
     return cudaGetLastError();
 }
 

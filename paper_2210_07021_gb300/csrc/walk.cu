@@ -84,9 +84,10 @@ struct __align__(64) MacNode32 {
     int count, tcount, child0, pad;
 };
 
-__global__ void k_mac_nodes(TreeView T, double c_s, double c_t, double sigma, MacNode* __restrict__ out,
-                            MacNode32* __restrict__ out32)
+__global__ void k_mac_nodes(TreeView T, double c_s, double c_t, double sigma, MacNode* out,
+                            MacNode32* out32)
 {
+    after_previous();
     const int64_t nn = dcount(T.d_nn, T.n_nodes);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += (int64_t)gridDim.x * blockDim.x) {
         const double R = T.geom[(size_t)i * GEOM_STRIDE + 9];
@@ -210,6 +211,7 @@ __device__ __forceinline__ int3 block_excl3(int3 v, int3* s_w, int3* total)
 
 __global__ void k_init_frontier(int2* f, WalkState* S)
 {
+    after_previous();
     const int i = threadIdx.x;
     if (i < 144) f[i] = make_int2(i / 12, i % 12);
     if (i < MAX_ROUNDS + 2) S->ticket[i] = 0;
@@ -330,9 +332,10 @@ __global__ void __launch_bounds__(WT) k_walk_round(TreeView T, const MacNode* __
     }
 }
 
-__global__ void k_csr_offsets(const uint64_t* __restrict__ sorted_t, int64_t n_cap, const int64_t* d_np, int n_nodes,
-                              int64_t* __restrict__ off)
+__global__ void k_csr_offsets(const uint64_t* sorted_t, int64_t n_cap, const int64_t* d_np, int n_nodes,
+                              int64_t* off)
 {
+    after_previous();
     const int64_t n_pairs = dcount(d_np, n_cap);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= n_nodes; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t lo = 0, hi = n_pairs;
@@ -404,9 +407,8 @@ cudaError_t build_lists(sfmm_plan_s* P, const TreeView& T, double c_s, double c_
     if ((e = ensure(P->macn, (size_t)P->n_nodes * sizeof(MacNode))) ||
         (e = ensure(P->macn32, (size_t)P->n_nodes * sizeof(MacNode32))))
         return e;
-    k_mac_nodes<<<grid_for(P->n_nodes), 256, 0, s>>>(T, c_s, c_t, P->opt.sigma, P->macn.as<MacNode>(),
+    launch_chained(k_mac_nodes, grid_for(P->n_nodes), 256, 0, s, T, c_s, c_t, P->opt.sigma, P->macn.as<MacNode>(),
                                                      P->macn32.as<MacNode32>());
-    count_launch();
     for (int attempt = 0; attempt < 8; ++attempt) {
         const size_t wb = (size_t)((cap_front + WTILE - 1) / WTILE) * 3 * 8;
         if ((e = ensure(P->fa, (size_t)cap_front * 8)) || (e = ensure(P->fb, (size_t)cap_front * 8)) ||
@@ -414,7 +416,7 @@ cudaError_t build_lists(sfmm_plan_s* P, const TreeView& T, double c_s, double c_
             (e = ensure(P->m2l_t, (size_t)cap_m2l * 8)) || (e = ensure(P->m2l_s, (size_t)cap_m2l * 4)) ||
             (e = ensure(P->p2p_t, (size_t)cap_p2p * 8)) || (e = ensure(P->p2p_s, (size_t)cap_p2p * 4)))
             return e;
-        k_init_frontier<<<1, 160, 0, s>>>(P->fa.as<int2>(), S); count_launch();
+        launch_chained(k_init_frontier, 1, 160, 0, s, P->fa.as<int2>(), S);
         WalkCaps caps{cap_front, cap_m2l, cap_p2p};
         for (int r = 0; r < rounds; ++r) {
             int2* f[2] = {P->fa.as<int2>(), P->fb.as<int2>()};
@@ -479,15 +481,15 @@ cudaError_t build_lists(sfmm_plan_s* P, const TreeView& T, double c_s, double c_
                         P->m2l_s2.as<uint32_t>(), n_m2l, bits, P->tmp.p, s, &P->m2l_alt, P->opt.wait_limit)))
         return e;
     const uint64_t* mt = P->m2l_alt ? P->m2l_t2.as<uint64_t>() : P->m2l_t.as<uint64_t>();
-    k_csr_offsets<<<grid_for(P->n_nodes + 1), 256, 0, s>>>(mt, n_m2l, P->d_m2l, (int)P->n_nodes,
-                                                           P->m2l_off.as<int64_t>()); count_launch();
+    launch_chained(k_csr_offsets, grid_for(P->n_nodes + 1), 256, 0, s, mt, n_m2l, P->d_m2l, (int)P->n_nodes,
+                                                           P->m2l_off.as<int64_t>());
     if ((e = cudaEventRecord(P->ev_m2l, s))) return e;
     if ((e = radix_sort(P->p2p_t.as<uint64_t>(), P->p2p_s.as<uint32_t>(), P->p2p_t2.as<uint64_t>(),
                         P->p2p_s2.as<uint32_t>(), n_p2p, bits, P->tmp.p, s, &P->p2p_alt, P->opt.wait_limit)))
         return e;
     const uint64_t* pt = P->p2p_alt ? P->p2p_t2.as<uint64_t>() : P->p2p_t.as<uint64_t>();
-    k_csr_offsets<<<grid_for(P->n_nodes + 1), 256, 0, s>>>(pt, n_p2p, P->d_p2p, (int)P->n_nodes,
-                                                           P->p2p_off.as<int64_t>()); count_launch();
+    launch_chained(k_csr_offsets, grid_for(P->n_nodes + 1), 256, 0, s, pt, n_p2p, P->d_p2p, (int)P->n_nodes,
+                                                           P->p2p_off.as<int64_t>());
     return cudaGetLastError();
 }
 
