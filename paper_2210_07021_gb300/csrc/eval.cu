@@ -130,6 +130,39 @@ __device__ __noinline__ double near_mass_of(const EvalArgs& A, int64_t nb0, int6
     return q;
 }
 
+// A lane's place in the sources of near leaves k, k + step, ...: source j of the leaf
+// that begins at f and holds n.  The leaf after it is read ahead.
+struct NearCursor {
+    int k, nk, step, f, n, f2, n2, j;
+    __device__ __forceinline__ void leaf_at(const EvalArgs& A, int64_t nb0, int i, int* first, int* count) const
+    {
+        if (i < nk) {
+            const int s = (int)A.p2p_src[nb0 + i];
+            *first = A.T.first[s];
+            *count = A.T.count[s];
+        }
+    }
+    __device__ __forceinline__ NearCursor(const EvalArgs& A, int64_t nb0, int leaves, int k0, int step_, int j0)
+        : k(k0), nk(leaves), step(step_), f(0), n(0), f2(0), n2(0), j(j0)
+    {
+        leaf_at(A, nb0, k, &f, &n);
+        leaf_at(A, nb0, k + step, &f2, &n2);
+    }
+    __device__ __forceinline__ bool done() const { return k >= nk; }
+    // on to the leaf that holds j; false past the last one
+    __device__ __forceinline__ bool seek(const EvalArgs& A, int64_t nb0)
+    {
+        while (k < nk && j >= n) {
+            j -= n;
+            k += step;
+            f = f2;
+            n = n2;
+            leaf_at(A, nb0, k + step, &f2, &n2);
+        }
+        return k < nk;
+    }
+};
+
 // Near-field sums of one target as k_eval writes them and k_finish64 reads them: sums
 // of q d / d^2 (3), of q, of q log d^2; then the NPM sum of f q, or the shear's six sums
 // of q d d^T / d^4 and the mass left out.
@@ -142,7 +175,8 @@ __host__ __device__ constexpr int near_width(bool shear, bool npm) { return shea
 // at p = 32, m = 32 (5.1e8 pairs, equal masses): 58.6 -> 20.7 ms.  L2P and the
 // combination run in k_finish64, a thread per target: 420 FP64 instructions per
 // target group that the groups of 1 to 16 targets left to a few lanes (20.7 -> 15.3 ms
-// with 1.0 ms there).  TEAM: the four warps of a CTA share an item, each taking every
+// with 1.0 ms there).  The lanes of a target walk the near sources as one list: leaf by
+// leaf the last step of each (20 sources by 2 to 32 lanes) had idle ones (15.2 -> 13.8 ms).  TEAM: the four warps of a CTA share an item, each taking every
 // fourth near leaf, for problems with fewer items than the GPU has warps to run
 // (4096 points, 195 items: 0.57 -> 0.23 ms; the line is four items per warp
 // slot of the SMs' FP64 pipes).
@@ -186,11 +220,10 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
             double qfd = 0.0;                 // NPM: sum of (f - 1) q inside the caps
             LogSum ls;
             ls.init();
-            for (int64_t k = nb0 + (TEAM ? wid : 0); k < nb1; k += TEAM ? 4 : 1) {
-                const int sleaf = (int)A.p2p_src[k];
-                const int f = A.T.first[sleaf], n = A.T.count[sleaf];
-                for (int j = f + sub; j < f + n; j += lpt) {
-                    const double4_32a y = A.src[j];
+            NearCursor at(A, nb0, (int)(nb1 - nb0), TEAM ? wid : 0, TEAM ? 4 : 1, sub);
+            while (__any_sync(FULL, at.seek(A, nb0))) {
+                if (!at.done()) {
+                    const double4_32a y = A.src[at.f + at.j];
                     const double dx = x.x - y.x, dy = x.y - y.y, dz = x.z - y.z;
                     const double d2 = dx * dx + dy * dy + dz * dz;
                     const bool cap = NPM && __double_as_longlong(d2) < __double_as_longlong(4.0 * A.npm_s);
@@ -234,6 +267,7 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
                     } else {
                         skip += y.w;
                     }
+                    at.j += lpt;
                 }
             }
             if (A.want_psi) ls.flush(s_tab);
