@@ -51,8 +51,8 @@ OPS_PER_PAIR = 14
 MUFU_PER_PAIR = 2           # rcp and lg2 (the FP32 pair loop's special-function operations)
 DTYPES = {"mixed": "f32+f32x2", "mixed_df": "f32x2+f64", "fp64": "f64", "fp32": "f32+bf16"}
 EVAL_KERNEL = {"mixed": "k_eval32 (FP32 near field; its double-float L2P and combination are k_finish_dfar)",
-               "mixed_df": "k_eval_df (near field and L2P in double-float)",
-               "fp64": "k_eval (near field and L2P in FP64)",
+               "mixed_df": "k_eval_df (double-float near field; its L2P and combination are k_finish_df)",
+               "fp64": "k_eval (FP64 near field; its L2P and combination are k_finish64)",
                "fp32": "k_eval32 (near field and L2P in FP32)"}
 # DRAM bytes of one k_eval32 launch of the headline path (p = 20, m = 96, c_s = 1.5 at N = M = 1.6e7):
 # ncu at N = M = 2e6 (profiles/k_eval32_mixed_clustered_2e6.md), scaled by the near-field pairs
