@@ -168,6 +168,12 @@ struct NearCursor {
 // of q d d^T / d^4 and the mass left out.
 __host__ __device__ constexpr int near_width(bool shear, bool npm) { return shear ? 12 : npm ? 6 : 5; }
 
+// TEAM: the parts of an item's targets that CTAs take one by one.  Whole items (195 at 4096
+// points) leave some SMs' FP64 pipes twice the work of others: the solve with 1 / 2 / 4 parts
+// 654 / 658 / 606 us, of 20,000 random points 1.48 / 1.27 / 1.23 ms, of 4096 clustered ones
+// 1.27 / 1.03 / 1.00 ms; 50,000 points 3.49 / 3.47 / 3.49 ms.
+constexpr int TEAM_PARTS = 4;
+
 // The FP64 pipe bounds this kernel (fp64ops.cuh): 13 FP64 instructions per pair of
 // a run of equal masses (3 differences, 3 for d^2, 3 for 1/d^2, 1 for the log
 // product, 3 accumulations), 22 where every mass differs, against about 49 with
@@ -178,7 +184,7 @@ __host__ __device__ constexpr int near_width(bool shear, bool npm) { return shea
 // with 1.0 ms there).  The lanes of a target walk the near sources as one list: leaf by
 // leaf the last step of each (20 sources by 2 to 32 lanes) had idle ones (15.2 -> 13.8 ms).  TEAM: the four warps of a CTA share an item, each taking every
 // fourth near leaf, for problems with fewer items than the GPU has warps to run
-// (4096 points, 195 items: 0.57 -> 0.23 ms; the line is four items per warp
+// (4096 points, 195 items: 0.57 -> 0.23 ms, in parts 0.17; the line is four items per warp
 // slot of the SMs' FP64 pipes).
 template <bool SHEAR, bool NPM, bool TEAM>
 __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
@@ -200,14 +206,19 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
         } else {
             w = next_item(A.leaf_ctr, lane);
         }
-        if (w >= dcount(A.d_n_items, A.n_items)) break;
-        const int2 item = A.items[w];
+        if (w >= dcount(A.d_n_items, A.n_items) * (TEAM ? TEAM_PARTS : 1)) break;
+        const int2 item = A.items[TEAM ? w / TEAM_PARTS : w];
         const int leaf = item.x;
         const int tf = A.T.tfirst[leaf], tc = A.T.tcount[leaf];
         const int64_t nb0 = A.p2p_off[leaf], nb1 = A.p2p_off[leaf + 1];
         const double mass = near_mass(A, nb0, nb1, lane);
         int t0, t1;
         item_range(item, tc, &t0, &t1);
+        if (TEAM) {                           // this part of the item's targets
+            const int part = (int)(w % TEAM_PARTS), n = t1 - t0, b = t0;
+            t0 = b + n * part / TEAM_PARTS;
+            t1 = b + n * (part + 1) / TEAM_PARTS;
+        }
         for (int tb = t0, tpw = 0; tb < t1; tb += tpw) {
             tpw = min(32, 1 << (31 - __clz(t1 - tb)));     // largest power of two <= the targets left
             const int lpt = 32 / tpw;
@@ -2036,7 +2047,7 @@ cudaError_t launch_eval(const TreeView& T, const int2* items, int64_t n_items, c
         // fewer items than four per SM sub-partition's warp: a CTA per item (TEAM)
         const bool team = n_items <= 152 * 16;
         int64_t blocks = 0;
-        if ((e = item_grid(leaf_ctr, team ? 4 * n_items : n_items, 16, s, &blocks))) return e;
+        if ((e = item_grid(leaf_ctr, team ? 4 * TEAM_PARTS * n_items : n_items, 16, s, &blocks))) return e;
 #define EVAL64(SH, NP)                                                               \
         if (team) k_eval<SH, NP, true><<<(unsigned)blocks, 128, 0, s>>>(A);          \
         else k_eval<SH, NP, false><<<(unsigned)blocks, 128, 0, s>>>(A);
