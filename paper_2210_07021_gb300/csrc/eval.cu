@@ -182,10 +182,11 @@ constexpr int TEAM_PARTS = 4;
 // combination run in k_finish64, a thread per target: 420 FP64 instructions per
 // target group that the groups of 1 to 16 targets left to a few lanes (20.7 -> 15.3 ms
 // with 1.0 ms there).  The lanes of a target walk the near sources as one list: leaf by
-// leaf the last step of each (20 sources by 2 to 32 lanes) had idle ones (15.2 -> 13.8 ms).  TEAM: the four warps of a CTA share an item, each taking every
-// fourth near leaf, for problems with fewer items than the GPU has warps to run
-// (4096 points, 195 items: 0.57 -> 0.23 ms, in parts 0.17; the line is four items per warp
-// slot of the SMs' FP64 pipes).
+// leaf the last step of each (20 sources by 2 to 32 lanes) had idle ones (15.2 -> 13.8
+// ms).  TEAM: the four warps of a CTA share a part of an item, each taking every fourth
+// near leaf, for problems with fewer items than the GPU has warps to run (4096 points,
+// 195 items: 0.57 -> 0.23 ms, in parts 0.17; the line is four items per warp slot of the
+// SMs' FP64 pipes).
 template <bool SHEAR, bool NPM, bool TEAM>
 __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
 {
