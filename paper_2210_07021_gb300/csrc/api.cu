@@ -52,12 +52,13 @@ cudaError_t launch_m2m64(const TreeView& T, int c0, int c1, int lvl, int p, cons
 cudaError_t launch_l2l64(const TreeView& T, int a, int b, int lvl, int p, const void* geo, double* local, cudaStream_t s);
 cudaError_t launch_p2m64_leaf(const TreeView& T, const int* leaves, int64_t n_leaves, const int64_t* d_nl,
                               const double4_32a* src, int p, double* mpole, cudaStream_t s);
-cudaError_t launch_m2l_list(const uint64_t* ptgt, const uint32_t* psrc, const uint32_t* list, const uint32_t* n_list,
-                            int64_t max_list, int p, const double* tables, const void* geo, const void* mpole,
+cudaError_t launch_m2l_list(const uint64_t* ptgt, const uint32_t* psrc, const int64_t* off, const uint32_t* list,
+                            const uint32_t* n_list, int64_t max_list, int p, const double* tables, const void* geo, const void* mpole,
                             void* local, int ek, cudaStream_t s);
-cudaError_t launch_m2l_tc(int64_t n_pairs, const uint64_t* ptgt, const uint32_t* psrc, const void* geo,
-                          const void* mpole, void* local, int p, uint32_t* leftover, uint32_t* n_leftover,
-                          uint32_t* tile_ctr, int* status, int wait_limit, cudaStream_t s);
+size_t m2l_tc_row_bytes(int64_t n_pairs);
+cudaError_t launch_m2l_tc(int64_t n_pairs, const uint64_t* ptgt, const uint32_t* psrc, const int64_t* off,
+                          const void* geo, const void* mpole, void* local, float* rows, int p, uint32_t* leftover,
+                          uint32_t* n_leftover, uint32_t* tile_ctr, int* status, int wait_limit, cudaStream_t s);
 cudaError_t launch_l2l(const TreeView& T, int a, int b, int lvl, int p, const double* tables, const void* geo,
                        void* local, int ek, cudaStream_t s);
 size_t frame_df_bytes();
@@ -594,7 +595,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         if ((e = launch_m2l_pair64(T, P->n_m2l, P->d_m2l, m2l_t, m2l_s, P->m2l_off.as<int64_t>(), P->m2l_geo.p,
                                    P->mpole.as<double>(), p, P->local.as<double>(), P->m2l_acc.as<double>(),
                                    P->leftover.as<uint32_t>(), n_left, s)) ||
-            (e = launch_m2l_list(m2l_t, m2l_s, P->leftover.as<uint32_t>(), n_left, P->n_m2l, p, P->tables.as<double>(),
+            (e = launch_m2l_list(m2l_t, m2l_s, P->m2l_off.as<int64_t>(), P->leftover.as<uint32_t>(), n_left, P->n_m2l, p, P->tables.as<double>(),
                                  P->m2l_geo.p, P->mpole.p, P->local.p, ek, s)))
             return cuda_fail(P, e, "M2L");
     } else if ((e = cudaMemsetAsync(P->local.p, 0, (size_t)nn * EXP_STRIDE * esz, s)) ||
@@ -605,12 +606,14 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         // tensor-core M2L; pairs it cannot take (centres near antipodes) go to a list for the warp kernel
         uint32_t* n_left = reinterpret_cast<uint32_t*>(P->small.as<int64_t>() + SM_LEFT);
         uint32_t* tile_ctr = n_left + 1;              // zeroed by the same memset
-        if ((e = ensure(P->leftover, (size_t)std::max<int64_t>(P->n_m2l, 1) * 4))) return cuda_fail(P, e, "alloc");
+        if ((e = ensure(P->leftover, (size_t)std::max<int64_t>(P->n_m2l, 1) * 4)) ||
+            (e = ensure(P->m2l_acc, std::max<size_t>(m2l_tc_row_bytes(P->n_m2l), 8))))
+            return cuda_fail(P, e, "alloc");
         if ((e = cudaMemsetAsync(P->small.as<int64_t>() + SM_STATUS, 0, 16, s))) return cuda_fail(P, e, "memset");
-        if ((e = launch_m2l_tc(P->n_m2l, m2l_t, m2l_s, P->m2l_geo.p, P->mpole.p, P->local.p, p, P->leftover.as<uint32_t>(),
-                               n_left, tile_ctr, status, P->opt.wait_limit, s)))
+        if ((e = launch_m2l_tc(P->n_m2l, m2l_t, m2l_s, P->m2l_off.as<int64_t>(), P->m2l_geo.p, P->mpole.p, P->local.p,
+                               P->m2l_acc.as<float>(), p, P->leftover.as<uint32_t>(), n_left, tile_ctr, status, P->opt.wait_limit, s)))
             return cuda_fail(P, e, "M2L (tensor cores)");
-        if ((e = launch_m2l_list(m2l_t, m2l_s, P->leftover.as<uint32_t>(), n_left, P->n_m2l, p, P->tables.as<double>(),
+        if ((e = launch_m2l_list(m2l_t, m2l_s, P->m2l_off.as<int64_t>(), P->leftover.as<uint32_t>(), n_left, P->n_m2l, p, P->tables.as<double>(),
                                  P->m2l_geo.p, P->mpole.p, P->local.p, ek, s)))
             return cuda_fail(P, e, "M2L (leftover pairs)");
     } else if ((e = launch_m2l(T, P->m2l_off.as<int64_t>(), m2l_s, p, P->tables.as<double>(), P->m2l_geo.p, P->mpole.p,

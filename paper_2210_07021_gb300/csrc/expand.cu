@@ -637,14 +637,6 @@ __device__ __forceinline__ void store_exp(ST* e, int lane, int p, R C, R Q, cx<R
     }
 }
 
-// atomic accumulation (leftover M2L pairs of the tensor-core kernel)
-template <typename R, typename ST>
-__device__ __forceinline__ void atomic_exp(ST* e, int lane, int p, R C, R Q, cx<R> Y)
-{
-    if (lane == 0) { atomicAdd(e, (ST)C); atomicAdd(e + 1, (ST)Q); }
-    if (lane < p) { atomicAdd(e + 2 + 2 * lane, (ST)Y.x); atomicAdd(e + 3 + 2 * lane, (ST)Y.y); }
-}
-
 // ----------------------------------------------------------------- P2M
 // Adjoint (FP64): charges h and tangent dipoles g at the sources.  A dipole's
 // potential g . grad_x G(x, y) is the derivative of the point-mass potential
@@ -888,13 +880,15 @@ __global__ void k_l2l(TreeView T, int a, int b, int lvl, int p, const double* ta
 }
 
 // ------------------------------------------------------ M2L, listed pairs
-// One warp per pair of a list (the pairs the tensor-core M2L leaves out); the
-// result is added atomically to the target's local expansion.
+// The pairs that the tensor-core and the FP64 thread-per-pair M2L leave out, one warp per
+// target box: the warp of the first listed pair of a box takes all of the box's, in the
+// order of the box's list, and adds each to the local expansion (so the sum does not depend
+// on the order in which the pairs were listed).
 template <typename R, typename GR, typename ST>
 __global__ void k_m2l_list(const uint64_t* __restrict__ ptgt, const uint32_t* __restrict__ psrc,
-                           const uint32_t* __restrict__ list, const uint32_t* __restrict__ n_list, int p,
-                           const double* __restrict__ tables, const GR* __restrict__ geo, const ST* __restrict__ mpole,
-                           ST* __restrict__ local)
+                           const int64_t* __restrict__ off, const uint32_t* __restrict__ list,
+                           const uint32_t* __restrict__ n_list, int p, const double* __restrict__ tables,
+                           const GR* __restrict__ geo, const ST* __restrict__ mpole, ST* __restrict__ local)
 {
     __shared__ Tables<R> tb;
     __shared__ WarpSmem<R> ws[4];
@@ -902,16 +896,25 @@ __global__ void k_m2l_list(const uint64_t* __restrict__ ptgt, const uint32_t* __
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t n = *n_list;
     for (int64_t w = (int64_t)blockIdx.x * 4 + wid; w < n; w += (int64_t)gridDim.x * 4) {
-        const uint32_t k = list[w];
-        const int s = (int)psrc[k], t = (int)ptgt[k];
-        const GR G = geo[k];
-        R C, Q;
-        cx<R> X;
-        load_exp<R>(mpole + (size_t)s * EXP_STRIDE, lane, p, &C, &Q, &X);
-        R accC = 0, accQ = 0;
-        cx<R> accY = cmk<R>(0, 0);
-        warp_translate<R>(p, lane, G, C, Q, X, &tb, &ws[wid], &accC, &accQ, &accY);
-        atomic_exp<R>(local + (size_t)t * EXP_STRIDE, lane, p, accC, accQ, accY);
+        const int64_t k = list[w];
+        const int t = (int)ptgt[k];
+        const int64_t lo = off[t], hi = off[t + 1];
+        bool later = false;                     // an earlier pair of the box is listed too
+        for (int64_t i = lo + lane; i < k; i += 32) later = later || left_out(geo[i]);
+        if (__any_sync(FULL, later)) continue;
+        for (int64_t i0 = k; i0 < hi; i0 += 32) {
+            const bool out = i0 + lane < hi && left_out(geo[i0 + lane]);
+            for (unsigned m = __ballot_sync(FULL, out); m; m &= m - 1) {
+                const int64_t i = i0 + __ffs(m) - 1;
+                R C, Q;
+                cx<R> X;
+                load_exp<R>(mpole + (size_t)psrc[i] * EXP_STRIDE, lane, p, &C, &Q, &X);
+                R accC = 0, accQ = 0;
+                cx<R> accY = cmk<R>(0, 0);
+                warp_translate<R>(p, lane, geo[i], C, Q, X, &tb, &ws[wid], &accC, &accQ, &accY);
+                store_exp<R>(local + (size_t)t * EXP_STRIDE, lane, p, accC, accQ, accY, true);
+            }
+        }
     }
 }
 
@@ -1130,19 +1133,19 @@ cudaError_t launch_m2l(const TreeView& T, const int64_t* off, const uint32_t* sr
     return cudaGetLastError();
 }
 
-cudaError_t launch_m2l_list(const uint64_t* ptgt, const uint32_t* psrc, const uint32_t* list, const uint32_t* n_list,
-                            int64_t max_list, int p, const double* tables, const void* geo, const void* mpole,
+cudaError_t launch_m2l_list(const uint64_t* ptgt, const uint32_t* psrc, const int64_t* off, const uint32_t* list,
+                            const uint32_t* n_list, int64_t max_list, int p, const double* tables, const void* geo, const void* mpole,
                             void* local, int ek, cudaStream_t s)
 {
     if (max_list == 0) return cudaSuccess;
     // FP64 lists hold a few antipodal pairs at most
     const unsigned g = grid_for(ek == EXP_F64 ? std::min<int64_t>(max_list, 152 * 4) : std::min<int64_t>(max_list, 152 * 64), 4);
     if (ek == EXP_F64)
-        k_m2l_list<double, XGeo, double><<<g, 128, 0, s>>>(ptgt, psrc, list, n_list, p, tables,
+        k_m2l_list<double, XGeo, double><<<g, 128, 0, s>>>(ptgt, psrc, off, list, n_list, p, tables,
                                                            static_cast<const XGeo*>(geo),
                                                            static_cast<const double*>(mpole), static_cast<double*>(local));
     else
-        k_m2l_list<float, XGeo32, float><<<g, 128, 0, s>>>(ptgt, psrc, list, n_list, p, tables,
+        k_m2l_list<float, XGeo32, float><<<g, 128, 0, s>>>(ptgt, psrc, off, list, n_list, p, tables,
                                                            static_cast<const XGeo32*>(geo),
                                                            static_cast<const float*>(mpole), static_cast<float*>(local));
     count_launch();

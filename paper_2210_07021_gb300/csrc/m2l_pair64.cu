@@ -17,9 +17,9 @@
 // column over the runs of equal target.  A run that is its target's whole list
 // is stored; the others go to two partial rows per warp (slot 0: a run that began
 // before these 32 pairs, slot 1: one that goes on after them), which k_m2l_runs
-// adds in order: no atomics, the same result every time.  Pairs with a below
-// 2^-30 or rho above 2^30 (centres antipodal to rounding: rho^32 would leave the
-// FP64 range) are listed for the warp kernel of expand.cu.
+// adds in order: no atomics, the same result every time.  Pairs with centres
+// antipodal to rounding (left_out in xgeo.cuh) are listed for the warp kernel of
+// expand.cu.
 #include "common.cuh"
 #include "dfops.cuh"
 #include "xgeo.cuh"
@@ -29,7 +29,6 @@ namespace sfmm {
 namespace {
 
 constexpr int PW = 4;            // warps per CTA
-constexpr double TINY = 1.0 / (1 << 30), HUGE_RHO = 1 << 30;
 
 // 1/l, l = 1..32
 struct InvTab64 {
@@ -79,7 +78,7 @@ k_m2l_pair64(int64_t n_cap, const int64_t* d_n, const uint64_t* __restrict__ ptg
         if (k < n_pairs) {
             G = geo[k];
             tnode = (int)ptgt[k];
-            on = G.a > TINY && G.b > 0.0 && G.g < HUGE_RHO * (G.a * G.b);
+            on = !left_out(G);
             if (!on && sub == 0) leftover[atomicAdd(n_left, 1u)] = (uint32_t)k;
         }
         if (on) {

@@ -15,9 +15,11 @@
 // tensor memory (≈ 2^-24 relative, the FP32 level).  The diagonal scalings,
 // the splits and the constant term C' = C + 2Q log sin(theta/2) + 2 Re sum u_l
 // are done by the CTA's threads; each tile's outputs, staged in the bytes of
-// its A tiles once the MMAs are complete, are summed per target segment (each
-// half of the tile by its own thread per coefficient) and added to the (FP32)
-// local expansions with atomics.
+// its A tiles once the MMAs are complete, are summed per run of equal target (each
+// half of the tile by its own thread per coefficient): a run that is its target's
+// whole list is the (FP32) local expansion, the others go to two partial rows per
+// half (0: a run that began before it, 1: one that goes on after it), which
+// k_m2l_tc_runs adds up.
 //
 // rho = 1/cos^2(theta/2) grows without bound as the two centres approach
 // antipodes; pairs with rho^PK beyond 2^100 are appended to a leftover list and
@@ -37,6 +39,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstring>
 
 namespace sfmm {
@@ -44,6 +47,7 @@ namespace sfmm {
 namespace {
 
 constexpr int TILE = 64;                 // pairs per tile
+constexpr int HALF = TILE / 2;           // pairs summed by one thread per coefficient
 constexpr int TC_CTAS = 5;               // CTAs per SM: registers capped for 5; 5 x 64 TMEM columns <= 512
 constexpr int WAIT_LIMIT = 1 << 26;
 
@@ -127,7 +131,7 @@ template <int PK> struct TcSmem {
     };
     unsigned char b2[SB][BBYTES];
     unsigned char b1[SB][BBYTES];
-    int tgt[TILE];
+    int dst[TILE];                                    // where the run ending at a pair goes (run_end)
     uint64_t mbar;
     uint32_t tmem;
     uint32_t next;                                    // the CTA's next tile
@@ -234,10 +238,24 @@ __device__ __forceinline__ void tc_sync()
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// Where the sum over the run of equal target that ends at pair k goes: the target's row of
+// the locals (the run is its whole list), or ~row of the partial rows; NO_END: the run goes
+// on in this half of the tile.
+constexpr int NO_END = INT_MIN;
+__device__ __forceinline__ int run_end(int64_t k, int t, const int64_t* __restrict__ off)
+{
+    const int64_t next = k + 1, base = k / HALF * HALF;
+    const int64_t lo = off[t], hi = off[t + 1];
+    if (next < base + HALF && next < hi) return NO_END;
+    if (lo >= base && hi <= base + HALF) return t;
+    return ~(int)(2 * (k / HALF) + (lo < base ? 0 : 1));
+}
+
 template <int PK, int PL>
 __global__ void __launch_bounds__(128, TC_CTAS) k_m2l_tc(int64_t n_pairs, const uint64_t* __restrict__ ptgt,
                                                 const uint32_t* __restrict__ psrc, const XGeo32* __restrict__ geo,
-                                                const float* __restrict__ mpole, float* __restrict__ local, int p,
+                                                const int64_t* __restrict__ off, const float* __restrict__ mpole,
+                                                float* __restrict__ local, float* __restrict__ rows, int p,
                                                 uint32_t* __restrict__ leftover, uint32_t* __restrict__ n_leftover,
                                                 uint32_t* __restrict__ tile_ctr, int* __restrict__ status,
                                                 int wait_limit)
@@ -336,7 +354,7 @@ __global__ void __launch_bounds__(128, TC_CTAS) k_m2l_tc(int64_t n_pairs, const 
         }
         // the MMAs of the previous tile have been waited for (or none were issued)
         store_row<PK, PL>(S, tid, u);
-        if (part == 0) S->tgt[j] = valid ? t_node : -1;
+        if (part == 0) S->dst[j] = valid ? run_end(k, t_node, off) : NO_END;
         tc_sync();
         // ---------------- stage 1 GEMM: D1 = A * B2^T
         if (tid == 0) issue_stage<PK>(S, S->b2, 0);
@@ -390,25 +408,22 @@ __global__ void __launch_bounds__(128, TC_CTAS) k_m2l_tc(int64_t n_pairs, const 
             }
         }
         __syncthreads();
-        // ---------------- per-target segment sums over each half of the tile, atomically added to the locals
+        // ---------------- sums over the runs of equal target of each half of the tile
         for (int it = tid; it < 2 * ncol; it += blockDim.x) {
             const int half = it >= ncol ? 1 : 0;
             const int c = it - half * ncol;
-            const int j0 = half * (TILE / 2);
-            int cur = -1;
+            const int j0 = half * HALF;
             float acc = 0.f;
 #pragma unroll 4
-            for (int jj = j0; jj < j0 + TILE / 2; ++jj) {
-                const int tn = S->tgt[jj];
-                const float x = S->out[jj][c];
-                if (tn != cur) {
-                    if (cur >= 0 && acc != 0.f) atomicAdd(local + (size_t)cur * EXP_STRIDE + c, acc);
-                    cur = tn;
+            for (int jj = j0; jj < j0 + HALF; ++jj) {
+                const int d = S->dst[jj];
+                acc += S->out[jj][c];
+                if (d != NO_END) {
+                    float* row = d >= 0 ? local + (size_t)d * EXP_STRIDE : rows + (size_t)~d * EXP_STRIDE;
+                    row[c] = acc;
                     acc = 0.f;
                 }
-                acc += x;             // rows of absent pairs hold zeros
             }
-            if (cur >= 0 && acc != 0.f) atomicAdd(local + (size_t)cur * EXP_STRIDE + c, acc);
         }
         if (tid == 0) S->next = atomicAdd(tile_ctr, 1u);     // every thread read this tile's index before
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -424,9 +439,42 @@ __global__ void __launch_bounds__(128, TC_CTAS) k_m2l_tc(int64_t n_pairs, const 
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(S->tmem), "r"(TCOLS) : "memory");
 }
 
+// Locals of boxes whose list spans several half tiles: the sum of the partial rows, always
+// in the same order, so that the path gives the same bits every time.  One warp per half,
+// for the box whose list begins in it and goes on after it.
+// The order is the one in which the atomic additions to the locals that stood here mostly
+// arrived (the halves' loops run side by side: a run that ends inside its half came before
+// those that fill theirs, first halves before second ones), which keeps the results where
+// they were.  Those additions' order changed from call to call: 4e6 clustered points,
+// relative change of psi 3e-13 or, where a coarse box's C was rounded the other way, up to
+// 4.4e-9.  Against five calls of that build on each of 16 skies, psi and alpha lie within
+// the spread of those calls but for one sky's alpha (4.9e-10, spread 8e-11); summed in
+// plain list order, psi was 1.6e-9 and 2e-9 from all five calls on two of twelve skies.
+// Cost at 4e6 points (2.75e6 pairs): k_m2l_tc 505 -> 515 us, this kernel 35 us with cold
+// caches, the solve 6.30 -> 6.35 ms.
+__global__ void __launch_bounds__(128) k_m2l_tc_runs(int64_t n_pairs, const uint64_t* ptgt, const int64_t* off, int p,
+                                                     const float* rows, float* local)
+{
+    after_previous();
+    const int lane = threadIdx.x & 31;
+    const int64_t c0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, next = (c0 + 1) * HALF;
+    if (next >= n_pairs) return;
+    const int64_t t = (int64_t)ptgt[next];
+    const int64_t lo = off[t], hi = off[t + 1], c1 = (hi - 1) / HALF;
+    if (lo < c0 * HALF || lo >= next) return;            // it begins in an earlier half, or in the next one
+    const bool inside = hi < (c1 + 1) * HALF;
+    for (int c = lane; c < 2 * p + 2; c += 32) {
+        float a = inside ? rows[(size_t)(2 * c1) * EXP_STRIDE + c] : 0.f;
+        for (int half = 0; half < 2; ++half)
+            for (int64_t k = c0 + ((c0 ^ half) & 1); k < c1 + !inside; k += 2)
+                a += rows[(size_t)(2 * k + (k == c0)) * EXP_STRIDE + c];
+        local[(size_t)t * EXP_STRIDE + c] = a;
+    }
+}
+
 template <int PK, int PL>
 cudaError_t launch_inst(int64_t n_pairs, const uint64_t* ptgt, const uint32_t* psrc, const XGeo32* geo,
-                        const float* mpole, float* local, int p, uint32_t* leftover, uint32_t* n_leftover,
+                        const int64_t* off, const float* mpole, float* local, float* rows, int p, uint32_t* leftover, uint32_t* n_leftover,
                         uint32_t* tile_ctr, int* status, int wait_limit, cudaStream_t s)
 {
     const size_t smem = sizeof(TcSmem<PK>) + 128;
@@ -443,27 +491,42 @@ cudaError_t launch_inst(int64_t n_pairs, const uint64_t* ptgt, const uint32_t* p
     const int64_t n_tiles = (n_pairs + TILE - 1) / TILE;
     const int64_t cap = (int64_t)sms * TC_CTAS;
     const int64_t grid = n_tiles < cap ? n_tiles : cap;
-    k_m2l_tc<PK, PL><<<(unsigned)grid, 128, smem, s>>>(n_pairs, ptgt, psrc, geo, mpole, local, p, leftover, n_leftover,
-                                                        tile_ctr, status, wait_limit);
+    k_m2l_tc<PK, PL><<<(unsigned)grid, 128, smem, s>>>(n_pairs, ptgt, psrc, geo, off, mpole, local, rows, p, leftover,
+                                                        n_leftover, tile_ctr, status, wait_limit);
     count_launch();
     return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_m2l_tc(int64_t n_pairs, const uint64_t* ptgt, const uint32_t* psrc, const void* geo,
-                          const void* mpole, void* local, int p, uint32_t* leftover, uint32_t* n_leftover,
-                          uint32_t* tile_ctr, int* status, int wait_limit, cudaStream_t s)
+// bytes of the partial rows for n pairs
+size_t m2l_tc_row_bytes(int64_t n_pairs)
+{
+    return (size_t)((n_pairs + HALF - 1) / HALF) * 2 * EXP_STRIDE * sizeof(float);
+}
+
+// Locals of every box = the sum of its M2Ls, but for the pairs put on the leftover list
+// (*n_leftover of them, zero at the call).  local: zero at the call; rows: m2l_tc_row_bytes(n_pairs).
+cudaError_t launch_m2l_tc(int64_t n_pairs, const uint64_t* ptgt, const uint32_t* psrc, const int64_t* off,
+                          const void* geo, const void* mpole, void* local, float* rows, int p, uint32_t* leftover,
+                          uint32_t* n_leftover, uint32_t* tile_ctr, int* status, int wait_limit, cudaStream_t s)
 {
     if (n_pairs == 0) return cudaSuccess;
     if (wait_limit <= 0 || wait_limit > WAIT_LIMIT) wait_limit = WAIT_LIMIT;
     const XGeo32* G = static_cast<const XGeo32*>(geo);
     const float* mp = static_cast<const float*>(mpole);
     float* lc = static_cast<float*>(local);
-    if (p <= 8) return launch_inst<16, 8>(n_pairs, ptgt, psrc, G, mp, lc, p, leftover, n_leftover, tile_ctr, status, wait_limit, s);
-    if (p <= 16) return launch_inst<16, 16>(n_pairs, ptgt, psrc, G, mp, lc, p, leftover, n_leftover, tile_ctr, status, wait_limit, s);
-    if (p <= 24) return launch_inst<32, 24>(n_pairs, ptgt, psrc, G, mp, lc, p, leftover, n_leftover, tile_ctr, status, wait_limit, s);
-    return launch_inst<32, 32>(n_pairs, ptgt, psrc, G, mp, lc, p, leftover, n_leftover, tile_ctr, status, wait_limit, s);
+    cudaError_t e;
+#define INST(PK, PL) launch_inst<PK, PL>(n_pairs, ptgt, psrc, G, off, mp, lc, rows, p, leftover, n_leftover, tile_ctr, status, wait_limit, s)
+    if (p <= 8) e = INST(16, 8);
+    else if (p <= 16) e = INST(16, 16);
+    else if (p <= 24) e = INST(32, 24);
+    else e = INST(32, 32);
+#undef INST
+    if (e) return e;
+    const int64_t halves = (n_pairs + HALF - 1) / HALF;
+    launch_chained(k_m2l_tc_runs, (unsigned)((halves + 3) / 4), 128, 0, s, n_pairs, ptgt, off, p, rows, lc);
+    return cudaGetLastError();
 }
 
 }  // namespace sfmm

@@ -36,6 +36,16 @@ struct __align__(16) XGeo32 {
     float pad[2];
 };
 
+// Pairs that the tensor-core and the FP64 thread-per-pair M2L leave to the warp kernel:
+// centres near antipodes; FP64 only antipodal ones up to rounding (a below 2^-30 or rho
+// above 2^30: rho^32 would leave the FP64 range).
+__device__ __forceinline__ bool left_out(const XGeo32& G) { return G.big != 0; }
+__device__ __forceinline__ bool left_out(const XGeo& G)
+{
+    constexpr double TINY = 1.0 / (1 << 30), HUGE_RHO = 1 << 30;
+    return !(G.a > TINY && G.b > 0.0 && G.g < HUGE_RHO * (G.a * G.b));
+}
+
 // The FP64 parameters rounded to double-float pairs.
 struct __align__(16) XGeoDF {
     dflt a, b, g, logk;
