@@ -437,6 +437,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     const bool dfe = precision == SFMM_MIXED || precision == SFMM_MIXED_DF;   // ... in double-float
     const bool near32 = precision == SFMM_FP32 || precision == SFMM_MIXED;    // FP32 near field
     const bool offsets = fp32 || dfe;                  // FP32 (hi, lo) offsets feed the near field
+    const bool near_aux = !fp32 && !adj;               // the near field runs on the auxiliary stream
     const int ek = fp32 ? EXP_F32 : dfe ? EXP_DF : EXP_F64;
     const size_t esz = fp32 ? 4 : 8;                   // expansion storage: float, double or double-float
     if ((e = ensure(P->mpole, (size_t)nn * EXP_STRIDE * esz)) || (e = ensure(P->local, (size_t)nn * EXP_STRIDE * esz)))
@@ -465,6 +466,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
         if ((e = launch_src_offsets(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->src4.as<double4_32a>(),
                                     P->soff.as<float4>(), s)))
             return cuda_fail(P, e, "offsets");
+        if (near_aux && (e = cudaEventRecord(P->ev_src, s))) return cuda_fail(P, e, "event");
     }
     if (adj && !adj_df) e = launch_p2m_adj(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->src4.as<double4_32a>(),
                                            P->dip4.as<double4_32a>(), P->mpole.as<double>(), p, s);
@@ -476,8 +478,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     else e = launch_p2m64_leaf(T, P->leaves_src.as<int>(), P->n_leaves, d_nls, P->src4.as<double4_32a>(), p,
                                P->mpole.as<double>(), s);
     if (e) return cuda_fail(P, e, "P2M");
-    const bool near_early64 = !fp32 && !dfe && !adj;
-    if (near_early64 && (e = cudaEventRecord(P->ev_p2m, s))) return cuda_fail(P, e, "event");
+    if (near_aux && !offsets && (e = cudaEventRecord(P->ev_src, s))) return cuda_fail(P, e, "event");
     // graph mode: every level up to the capacity, each launch sized by the level-width capacity
     const int depth = P->gm ? (int)P->cap.levels : (int)P->level_start.size() - 2;
     const int W = (int)P->cap.width;
@@ -514,16 +515,18 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
                                     P->aux)))
             return cuda_fail(P, e, "offsets");
     }
-    // the near field needs none of the far field but the leaves' masses (the finish does), so
-    // it runs here, on the auxiliary stream, beside M2L and L2L (all-FP32 path and adjoint: not)
+    // the near field needs none of the far field (the finish does), so it runs here, on the
+    // auxiliary stream, beside M2L and L2L (all-FP32 path and adjoint: not); what it reads of the
+    // sources, their offsets or in FP64 their leaves' masses, is written on the plan's stream
+    // after the fork (ev_src)
+    if (near_aux && (e = cudaStreamWaitEvent(P->aux, P->ev_src, 0))) return cuda_fail(P, e, "wait");
     unsigned long long* leaf_ctr = reinterpret_cast<unsigned long long*>(P->small.as<int64_t>() + SM_ITEM_CTR);
-    const bool near_early = near32 && !fp32 && !adj;
-    const bool near_early_df = dfe && !near32 && !adj;
+    const bool near_early = near32 && near_aux, near_early_df = dfe && !near32 && near_aux;
+    const bool near_early64 = !dfe && near_aux;
     if (near_early64) {
         if ((e = ensure(P->nfbuf, (size_t)M * near64_bytes(gamma, P->opt.sigma > 0.0))) ||
             (e = ensure(P->tleaf, (size_t)M * 4)))
             return cuda_fail(P, e, "alloc");
-        if ((e = cudaStreamWaitEvent(P->aux, P->ev_p2m, 0))) return cuda_fail(P, e, "wait");
         if (P->timing) cudaEventRecord(P->ev_near[0], P->aux);
         if ((e = launch_eval(T, P->items.as<int2>(), P->n_items, d_nit, P->src4.as<double4_32a>(),
                              P->tgt4.as<double4_32a>(), tperm, P->p2p_off.as<int64_t>(), p2p_s, P->local.as<double>(),
@@ -695,7 +698,7 @@ sfmm_status solve(sfmm_plan_s* P, const double* src, const void* q, int64_t N, c
     if (tc_status && *P->h_status)
         return fail(P, SFMM_ETIMEOUT, "a bounded wait of the tensor-core M2L kernel ran out");
     tm.finish();
-    if (P->timing && (near_early || near_early_df || near_early64)) {
+    if (P->timing && near_aux) {
         float ms = 0.f;
         if (cudaEventElapsedTime(&ms, P->ev_near[0], P->ev_near[1]) == cudaSuccess) P->stats.near_ms = ms;
     }
@@ -801,7 +804,7 @@ sfmm_status sfmm_plan(sfmm_plan_t* out, int max_depth, int order_p, double tol, 
         (e = cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming)) ||
         (e = cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming)) ||
         (e = cudaEventCreateWithFlags(&P->ev_m2l, cudaEventDisableTiming)) ||
-        (e = cudaEventCreateWithFlags(&P->ev_p2m, cudaEventDisableTiming)) ||
+        (e = cudaEventCreateWithFlags(&P->ev_src, cudaEventDisableTiming)) ||
         (e = cudaEventCreate(&P->ev_near[0])) || (e = cudaEventCreate(&P->ev_near[1]))) {
         std::lock_guard<std::mutex> g(g_err_mu);
         g_plan_err = std::string("CUDA error at plan time: ") + cudaGetErrorString(e);
@@ -1035,7 +1038,7 @@ void sfmm_destroy(sfmm_plan_t plan)
     if (plan->ev_fork) cudaEventDestroy(plan->ev_fork);
     if (plan->ev_join) cudaEventDestroy(plan->ev_join);
     if (plan->ev_m2l) cudaEventDestroy(plan->ev_m2l);
-    if (plan->ev_p2m) cudaEventDestroy(plan->ev_p2m);
+    if (plan->ev_src) cudaEventDestroy(plan->ev_src);
     for (cudaEvent_t ev : plan->ev_near)
         if (ev) cudaEventDestroy(ev);
     if (plan->aux) cudaStreamDestroy(plan->aux);

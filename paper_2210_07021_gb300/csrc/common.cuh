@@ -187,7 +187,7 @@ struct sfmm_plan_s {
     std::vector<sfmm_plan_s*> lanes;       // batch lanes: solvers on their own streams
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaEvent_t ev_m2l = nullptr;          // the M2L list is sorted (recorded by build_lists)
-    cudaEvent_t ev_p2m = nullptr;          // P2M is done (the FP64 near field reads the leaves' masses)
+    cudaEvent_t ev_src = nullptr;          // the near field's inputs from the sources are written (offsets; FP64: the leaves' masses)
     cudaEvent_t ev_near[2] = {nullptr, nullptr};   // timing: around the near-field kernel on the auxiliary stream
     std::string err;
     int timing = 0;                        // 0 off, 1 phase times, 2 also the near-field pair count
