@@ -117,6 +117,7 @@ k_m2l_pair64(int64_t n_cap, const int64_t* d_n, const uint64_t* __restrict__ ptg
             }
         }
         const unsigned onm = __ballot_sync(FULL, on);       // both lanes of a pair, or neither
+        if (L > 1) __syncwarp();                            // each lane reads the part that the other wrote
         if (on) {
             // Y_l = (b ph2)^l (-Q/l + o_l)
             const double br = G.b * G.p2x, bi = G.b * G.p2y;
