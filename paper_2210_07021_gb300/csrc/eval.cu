@@ -104,22 +104,22 @@ __device__ __forceinline__ int64_t next_item(unsigned long long* ctr, int lane)
     return (int64_t)__shfl_sync(FULL, w, 0);
 }
 
-// The near leaves' total mass (4 pi times the Q of their multipoles), the same for
-// every target of the leaf: the pair loops then only subtract what a target skips.
-__device__ __forceinline__ double near_mass(const EvalArgs& A, int64_t nb0, int64_t nb1, int lane)
+// The total mass of near leaves k0, k0 + step, ... (4 pi times the Q of their multipoles), the
+// same for every target of the leaf: the pair loops then only subtract what a target skips.
+__device__ __forceinline__ double near_mass(const EvalArgs& A, int64_t k0, int64_t nb1, int step, int lane)
 {
     double q = 0.0;
-    for (int64_t k = nb0 + lane; k < nb1; k += 32) q += A.base_mpole[(size_t)A.p2p_src[k] * EXP_STRIDE + 1];
+    for (int64_t k = k0 + (int64_t)lane * step; k < nb1; k += 32 * step)
+        q += A.base_mpole[(size_t)A.p2p_src[k] * EXP_STRIDE + 1];
     return 4.0 * PI * group_sum(q, 32);
 }
 
-// The mass of the near sources a target does not coincide with, summed pair by
-// pair: where the near leaves' total is not finite, a skipped mass cannot be
-// subtracted from it.
-__device__ __noinline__ double near_mass_of(const EvalArgs& A, int64_t nb0, int64_t nb1, double4_32a x, int sub, int lpt)
+// The mass of the sources of these leaves that a target does not coincide with, summed pair by pair.
+__device__ __noinline__ double near_mass_of(const EvalArgs& A, int64_t k0, int64_t nb1, int step, double4_32a x, int sub,
+                                            int lpt)
 {
     double q = 0.0;
-    for (int64_t k = nb0; k < nb1; ++k) {
+    for (int64_t k = k0; k < nb1; k += step) {
         const int sleaf = (int)A.p2p_src[k], f = A.T.first[sleaf], n = A.T.count[sleaf];
         for (int j = f + sub; j < f + n; j += lpt) {
             const double4_32a y = A.src[j];
@@ -128,6 +128,45 @@ __device__ __noinline__ double near_mass_of(const EvalArgs& A, int64_t nb0, int6
         }
     }
     return q;
+}
+
+// What a target skips, the masses at its own position (d = 0): their sum; and the largest
+// of them and of the others, as the leading words of their magnitudes, so that the pair loop
+// compares them on the integer pipe.
+__device__ __forceinline__ unsigned mag_word(double q) { return (unsigned)__double2hiint(q) & 0x7fffffffu; }
+struct Skipped {
+    double sum;
+    unsigned own, others;
+    __device__ __forceinline__ void init() { sum = 0.0; own = others = 0; }
+    __device__ __forceinline__ void acts(double q) { others = max(others, mag_word(q)); }
+    __device__ __forceinline__ void skip(double q) { sum += q; own = max(own, mag_word(q)); }
+};
+
+// The mass of the near sources a target does not skip, by all lanes of the warp: mass (near_mass)
+// less the skipped (returned in *skipped).  That leaves the rounding of the skipped masses behind,
+// so the masses are summed pair by pair where the skipped ones outweigh the heaviest other 16
+// times, as one of them or as their sum (a target on one heavy mass: psi was off by 1e-16 of it,
+// whatever the others weigh), and where the total is not finite.
+__device__ __forceinline__ double mass_acting(const EvalArgs& A, int64_t k0, int64_t nb1, int step, double mass,
+                                              const Skipped& sk, double4_32a x, int sub, int lpt, double* skipped)
+{
+    constexpr unsigned TIMES16 = 4u << 20;             // four steps of the exponent
+    const double sum = group_sum(sk.sum, lpt);
+    double sq = mass - sum;
+    if (__any_sync(FULL, sk.own != 0 || !isfinite(mass))) {
+        unsigned own = sk.own, others = sk.others;
+        for (int o = lpt >> 1; o > 0; o >>= 1) {
+            own = max(own, __shfl_xor_sync(FULL, own, o));
+            others = max(others, __shfl_xor_sync(FULL, others, o));
+        }
+        const bool apart = !isfinite(mass) || max(own, mag_word(sum)) > others + TIMES16;
+        if (__any_sync(FULL, apart)) {
+            const double s = group_sum(near_mass_of(A, k0, nb1, step, x, sub, lpt), lpt);
+            if (apart) sq = s;
+        }
+    }
+    *skipped = sum;
+    return sq;
 }
 
 // A lane's place in the sources of near leaves k, k + step, ...: source j of the leaf
@@ -186,9 +225,10 @@ constexpr int TEAM_PARTS = 4;
 // ms).  TEAM: the four warps of a CTA share a part of an item, each taking every fourth
 // near leaf, for problems with fewer items than the GPU has warps to run (4096 points,
 // 195 items: 0.57 -> 0.23 ms, in parts 0.17; the line is four items per warp slot of the
-// SMs' FP64 pipes).
+// SMs' FP64 pipes).  Its plain form is held to 64 registers: at the 72 it takes by itself it
+// runs no slower, but leaves M2L beside it less room (the solve 611 against 619 us).
 template <bool SHEAR, bool NPM, bool TEAM>
-__global__ void __launch_bounds__(128) k_eval(EvalArgs A)
+__global__ void __launch_bounds__(128, TEAM && !SHEAR && !NPM ? 8 : 1) k_eval(EvalArgs A)
 {
     constexpr int NW = near_width(SHEAR, NPM);
     __shared__ double2 s_tab[LOG64_N];
@@ -212,7 +252,9 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
         const int leaf = item.x;
         const int tf = A.T.tfirst[leaf], tc = A.T.tcount[leaf];
         const int64_t nb0 = A.p2p_off[leaf], nb1 = A.p2p_off[leaf + 1];
-        const double mass = near_mass(A, nb0, nb1, lane);
+        const int64_t k0 = nb0 + (TEAM ? wid : 0);      // the near leaves of this warp: k0, k0 + step, ...
+        constexpr int step = TEAM ? 4 : 1;
+        const double mass = near_mass(A, k0, nb1, step, lane);
         int t0, t1;
         item_range(item, tc, &t0, &t1);
         if (TEAM) {                           // this part of the item's targets
@@ -227,12 +269,13 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
             const int ti = tb + slot;
             const double4_32a x = A.tgt[tf + ti];
             double sx = 0.0, sy = 0.0, sz = 0.0;
-            double skip = 0.0;                // mass of the sources left out (d = 0)
+            Skipped sk;
+            sk.init();
             double Sxx = 0.0, Syy = 0.0, Szz = 0.0, Sxy = 0.0, Sxz = 0.0, Syz = 0.0;
             double qfd = 0.0;                 // NPM: sum of (f - 1) q inside the caps
             LogSum ls;
             ls.init();
-            NearCursor at(A, nb0, (int)(nb1 - nb0), TEAM ? wid : 0, TEAM ? 4 : 1, sub);
+            NearCursor at(A, nb0, (int)(nb1 - nb0), TEAM ? wid : 0, step, sub);
             while (__any_sync(FULL, at.seek(A, nb0))) {
                 if (!at.done()) {
                     const double4_32a y = A.src[at.f + at.j];
@@ -240,6 +283,7 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
                     const double d2 = dx * dx + dy * dy + dz * dz;
                     const bool cap = NPM && __double_as_longlong(d2) < __double_as_longlong(4.0 * A.npm_s);
                     if (f64_plain(d2) && !cap) {
+                        sk.acts(y.w);
                         double u;
                         const double r0 = rcp_series(d2, &u);
                         const double t = y.w * r0;
@@ -255,6 +299,7 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
                             Sxy += wx * dy; Sxz += wx * dz; Syz += wy * dz;
                         }
                     } else if (d2 > 0.0) {    // inside a cap, or outside the fast paths' range
+                        sk.acts(y.w);
                         double fq = 1.0, lg;
                         if (cap) {
                             const double s = A.npm_s, u = 0.25 * d2;
@@ -277,7 +322,7 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
                             Sxy += w4 * dx * dy; Sxz += w4 * dx * dz; Syz += w4 * dy * dz;
                         }
                     } else {
-                        skip += y.w;
+                        sk.skip(y.w);
                     }
                     at.j += lpt;
                 }
@@ -288,10 +333,8 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A)
             v[0] = group_sum(sx, lpt);
             v[1] = group_sum(sy, lpt);
             v[2] = group_sum(sz, lpt);
-            const double sqs = group_sum(skip, lpt);       // masses at the target's position (left out)
-            // the mass once per target (TEAM: by warp 0), less what is left out
-            v[3] = isfinite(mass) ? (TEAM && wid > 0 ? 0.0 : mass) - sqs
-                                  : TEAM && wid > 0 ? 0.0 : group_sum(near_mass_of(A, nb0, nb1, x, sub, lpt), lpt);
+            double sqs;                       // masses at the target's position (left out)
+            v[3] = mass_acting(A, k0, nb1, step, mass, sk, x, sub, lpt, &sqs);
             v[4] = A.want_psi ? group_sum(sl, lpt) : 0.0;
             if (NPM) v[NW - 1] = v[3] + group_sum(qfd, lpt);              // the alpha part of sum q
             if (SHEAR) {
@@ -449,7 +492,7 @@ __global__ void __launch_bounds__(128) k_eval_adj(EvalAdjArgs AA)
         const double* g = A.T.geom + (size_t)leaf * GEOM_STRIDE;
         const double* L = A.local + (size_t)leaf * EXP_STRIDE;
         const int64_t nb0 = A.p2p_off[leaf], nb1 = A.p2p_off[leaf + 1];
-        const double mass = near_mass(A, nb0, nb1, lane);
+        const double mass = near_mass(A, nb0, nb1, 1, lane);
         int t0, t1;
         item_range(item, tc, &t0, &t1);
         for (int tb = t0, tpw = 0; tb < t1; tb += tpw) {
@@ -458,8 +501,10 @@ __global__ void __launch_bounds__(128) k_eval_adj(EvalAdjArgs AA)
             const int slot = lane / lpt, sub = lane % lpt;
             const int ti = tb + slot;
             const double4_32a x = A.tgt[tf + ti];
-            double sx = 0.0, sy = 0.0, sz = 0.0, skip = 0.0;             // charges (as k_eval)
+            double sx = 0.0, sy = 0.0, sz = 0.0;                         // charges (as k_eval)
             double sd = 0.0, vx = 0.0, vy = 0.0, vz = 0.0;               // dipoles
+            Skipped sk;
+            sk.init();
             LogSum ls;
             ls.init();
             for (int64_t k = nb0; k < nb1; ++k) {
@@ -471,6 +516,7 @@ __global__ void __launch_bounds__(128) k_eval_adj(EvalAdjArgs AA)
                     const double dx = x.x - y.x, dy = x.y - y.y, dz = x.z - y.z;
                     const double d2 = dx * dx + dy * dy + dz * dz;
                     if (d2 > 0.0) {
+                        sk.acts(y.w);
                         double inv;
                         if (f64_plain(d2)) {
                             double u;
@@ -493,14 +539,14 @@ __global__ void __launch_bounds__(128) k_eval_adj(EvalAdjArgs AA)
                         vy += c2 * dy - gd.y * inv;
                         vz += c2 * dz - gd.z * inv;
                     } else {
-                        skip += y.w;
+                        sk.skip(y.w);
                     }
                 }
             }
             if (A.want_psi) ls.flush(s_tab);
             double sl = ls.sum;
-            const double sqs = group_sum(skip, lpt);
-            const double sq = isfinite(mass) ? mass - sqs : group_sum(near_mass_of(A, nb0, nb1, x, sub, lpt), lpt);
+            double sqs;
+            const double sq = mass_acting(A, nb0, nb1, 1, mass, sk, x, sub, lpt, &sqs);
             sx = group_sum(sx, lpt);
             sy = group_sum(sy, lpt);
             sz = group_sum(sz, lpt);
