@@ -1106,7 +1106,6 @@ cudaError_t launch_m2m(const TreeView& T, int a, int b, int lvl, int p, const do
                                                       static_cast<float*>(mpole));
     else
         return cudaErrorInvalidValue;             // the FP64 and double-float paths: kernels of their own
-    count_launch();
     return cudaGetLastError();
 }
 

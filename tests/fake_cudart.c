@@ -1,7 +1,7 @@
 /* A CUDA runtime without a device, for the host code's order of work (test_stream_order.py):
    device memory is host memory, copies and fills take place at once, a kernel launch is
    written down and does nothing.  Only the tree kernel's answer, which the host reads, is
-   given: level 0 with its 12 boxes, done. */
+   given: levels 0 and 1 with 12 and 48 boxes, done. */
 #include <stdarg.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -33,10 +33,11 @@ static int launch(const void* host, void** args, void* stream)
     say("launch %p %s\n", stream, name);
     if (strstr(name, "k_tree_narrow")) {
         long long* levels = *(long long**)args[6];
-        levels[0] = 0;
+        levels[0] = 1;
         levels[1] = 1;
         levels[2] = 0;
         levels[3] = 12;
+        levels[4] = 60;
     }
     return 0;
 }

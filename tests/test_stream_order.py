@@ -1,7 +1,7 @@
 """A solve's work on its two streams: what a kernel reads has been written before it, by
-the order of a stream, an event or a host synchronisation, whatever the timing.  The host
-code runs against a CUDA runtime without a device that writes the calls down
-(fake_cudart.c)."""
+the order of a stream, an event or a host synchronisation, whatever the timing; and every
+launch is counted once.  The host code runs against a CUDA runtime without a device that
+writes the calls down (fake_cudart.c)."""
 import ctypes
 import glob
 import os
@@ -29,11 +29,13 @@ def lib(tmp_path_factory):
     return L
 
 
-def trace(lib, call, precision):
-    """[(kernel or operation, the operations that are done before it)] of one call."""
+def trace(lib, call, precision, **options):
+    """[(kernel or operation, the operations that are done before it)] of one call, and its launch count."""
     o = sfmm.Options()
     lib.sfmm_default_options(ctypes.byref(o))
     o.precision = precision
+    for k, v in options.items():
+        setattr(o, k, v)
     h = ctypes.c_void_p()
     lib.sfmm_plan(ctypes.byref(h), 29, 8, ctypes.c_double(0), ctypes.byref(o))
     a = [np.zeros(8192) for _ in range(7)]
@@ -60,8 +62,10 @@ def trace(lib, call, precision):
         else:
             done[s] = before | 1 << len(ops)
             ops.append((more[0] if what == "launch" else what, before))
+    stats = sfmm.Stats()
+    lib.sfmm_get_stats(h, ctypes.byref(stats))
     lib.sfmm_destroy(h)
-    return ops
+    return ops, stats.launches
 
 
 # what the near-field kernel of each path reads, beside the lists and the targets
@@ -79,7 +83,7 @@ def test_near_field_comes_after_what_it_reads(lib, call, precision):
         near, written = NEAR[sfmm.SFMM_FP64]
     elif call == "adjoint":
         near, written = NEAR[sfmm.SFMM_MIXED_DF] if precision != sfmm.SFMM_FP64 else ("k_eval_adj", ["k_gather_dip", "k_p2m_adj"])
-    ops = trace(lib, call, precision)
+    ops, _ = trace(lib, call, precision)
     is_ = lambda name, k: f"{len(k)}{k}" in name        # a mangled name holds its length
     reads = [i for i, (name, _) in enumerate(ops) if is_(name, near)]
     assert reads
@@ -94,3 +98,13 @@ def test_near_field_comes_after_what_it_reads(lib, call, precision):
         if "k_m2l" in name or "k_pair_geo" in name:
             assert all(before >> i & 1 for i in walk)
     assert ops[-1][1] == (1 << len(ops) - 1) - 1
+
+
+@pytest.mark.parametrize("precision", sorted(NEAR))
+@pytest.mark.parametrize("call", ["sfmm_deflection", "sfmm_deflection_host", "shear"])
+@pytest.mark.parametrize("options", [{}, {"m2l_tensor_cores": 0}, {"sigma": 0.1}])
+def test_every_launch_is_counted_once(lib, call, precision, options):
+    if "sigma" in options and (precision != sfmm.SFMM_FP64 or call == "shear"):
+        pytest.skip("the Near Particle Model runs in FP64, without shear")
+    ops, launches = trace(lib, call, precision, **options)
+    assert launches == sum(name.startswith("_Z") for name, _ in ops)
