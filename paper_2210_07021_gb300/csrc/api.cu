@@ -73,7 +73,6 @@ cudaError_t launch_m2l_pair(int64_t n_pairs, const int64_t* d_n, const uint64_t*
 cudaError_t launch_m2l_left_df(const TreeView& T, const uint64_t* ptgt, const uint32_t* psrc, const uint32_t* list,
                                const uint32_t* n_list, int64_t max_list, int p, const double* tables,
                                const void* mpole, double* acc, cudaStream_t s);
-cudaError_t launch_acc_to_df(int64_t n, const double* acc, void* out, cudaStream_t s);
 cudaError_t launch_m2m_df(const TreeView& T, int c0, int c1, int lvl, int p, const void* geo, void* mpole,
                           cudaStream_t s);
 cudaError_t launch_l2l_df(const TreeView& T, int a, int b, int lvl, int p, const void* geo, const double* acc,

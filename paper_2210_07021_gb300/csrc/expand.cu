@@ -117,7 +117,6 @@ __device__ __forceinline__ XGeo make_geo(int kind, const double* gS, const doubl
     return G;
 }
 
-__device__ __forceinline__ void store_geo(XGeo* out, const XGeo& G) { *out = G; }
 __device__ __forceinline__ void store_geo(XGeoDF* out, const XGeo& G)
 {
     XGeoDF D;
@@ -214,16 +213,15 @@ __global__ void k_child_geo32(TreeView T, const float* g32, XGeo32* m2m,
     }
 }
 
-template <typename GR>
 __global__ void k_pair_geo(TreeView T, const uint64_t* tt, const uint32_t* ss, int64_t n_cap,
-                           const int64_t* d_n, GR* out)
+                           const int64_t* d_n, XGeo* out)
 {
     after_previous();
     const int64_t n = dcount(d_n, n_cap);
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const double* gS = T.geom + (size_t)ss[k] * GEOM_STRIDE;
         const double* gT = T.geom + (size_t)tt[k] * GEOM_STRIDE;
-        store_geo(out + k, make_geo(K_M2L, gS, gT));
+        out[k] = make_geo(K_M2L, gS, gT);
     }
 }
 
@@ -363,8 +361,7 @@ __global__ void k_child_geo_df(TreeView T, const FrameDF* fr, const float4* log_
 }
 
 // per node with a parent: child -> parent (M2M) and parent -> child (L2L)
-template <typename GR>
-__global__ void k_child_geo(TreeView T, GR* m2m, GR* l2l)
+__global__ void k_child_geo(TreeView T, XGeo* m2m, XGeo* l2l)
 {
     after_previous();
     const int64_t nn = dcount(T.d_nn, T.n_nodes);
@@ -373,8 +370,8 @@ __global__ void k_child_geo(TreeView T, GR* m2m, GR* l2l)
         if (par < 0) continue;
         const double* gC = T.geom + (size_t)i * GEOM_STRIDE;
         const double* gP = T.geom + (size_t)par * GEOM_STRIDE;
-        store_geo(m2m + i, make_geo(K_M2M, gC, gP));
-        store_geo(l2l + i, make_geo(K_L2L, gP, gC));
+        m2m[i] = make_geo(K_M2M, gC, gP);
+        l2l[i] = make_geo(K_L2L, gP, gC);
     }
 }
 
@@ -950,13 +947,6 @@ __global__ void k_m2l_left_df(TreeView T, const uint64_t* ptgt, const uint32_t* 
     }
 }
 
-// FP64 accumulators -> double-float expansions (every entry)
-__global__ void k_acc_to_df(int64_t n, const double* __restrict__ acc, dflt* __restrict__ out)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = dflt(acc[i]);
-}
-
 // FP32 offset of every key-sorted source from the centre of its leaf as an
 // (hi, lo) pair (the difference to 2^-47, formed without FP64 instructions),
 // plus its mass split the same way: off[2j] = (hi, q_hi), off[2j+1] = (lo, q_lo).
@@ -1040,8 +1030,7 @@ cudaError_t launch_pair_geo(const TreeView& T, const float* g32, const uint64_t*
 {
     if (n == 0) return cudaSuccess;
     if (ek == EXP_F32) launch_chained(k_pair_geo32, grid_for(n, 256), 256, 0, s, T, g32, tt, ss, n, d_n, static_cast<XGeo32*>(out));
-    else if (ek == EXP_DF) launch_chained(k_pair_geo<XGeoDF>, grid_for(n, 256), 256, 0, s, T, tt, ss, n, d_n, static_cast<XGeoDF*>(out));
-    else launch_chained(k_pair_geo<XGeo>, grid_for(n, 256), 256, 0, s, T, tt, ss, n, d_n, static_cast<XGeo*>(out));
+    else launch_chained(k_pair_geo, grid_for(n, 256), 256, 0, s, T, tt, ss, n, d_n, static_cast<XGeo*>(out));
     return cudaGetLastError();
 }
 
@@ -1049,8 +1038,7 @@ cudaError_t launch_child_geo(const TreeView& T, const float* g32, void* m2m, voi
 {
     const unsigned g = grid_for(T.n_nodes, 256);
     if (ek == EXP_F32) launch_chained(k_child_geo32, g, 256, 0, s, T, g32, static_cast<XGeo32*>(m2m), static_cast<XGeo32*>(l2l));
-    else if (ek == EXP_DF) launch_chained(k_child_geo<XGeoDF>, g, 256, 0, s, T, static_cast<XGeoDF*>(m2m), static_cast<XGeoDF*>(l2l));
-    else launch_chained(k_child_geo<XGeo>, g, 256, 0, s, T, static_cast<XGeo*>(m2m), static_cast<XGeo*>(l2l));
+    else launch_chained(k_child_geo, g, 256, 0, s, T, static_cast<XGeo*>(m2m), static_cast<XGeo*>(l2l));
     return cudaGetLastError();
 }
 
@@ -1184,14 +1172,6 @@ cudaError_t launch_m2l_left_df(const TreeView& T, const uint64_t* ptgt, const ui
     if (max_list == 0) return cudaSuccess;
     launch_chained(k_m2l_left_df, grid_for(max_list < 152 * 64 ? max_list : 152 * 64, 4), 128, 0, s,
         T, ptgt, psrc, list, n_list, p, tables, static_cast<const dflt*>(mpole), acc);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_acc_to_df(int64_t n, const double* acc, void* out, cudaStream_t s)
-{
-    if (n == 0) return cudaSuccess;
-    k_acc_to_df<<<grid_for(n, 256), 256, 0, s>>>(n, acc, static_cast<dflt*>(out));
-    count_launch();
     return cudaGetLastError();
 }
 

@@ -375,10 +375,9 @@ __global__ void __launch_bounds__(CT) k_collect(int n_cap, const int64_t* d_nn, 
     after_previous();
     __shared__ uint32_t s_tile;
     __shared__ int64_t s_warp[2][CT / 32], s_base[2];
-    __shared__ int s_lost;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nn = dcount(d_nn, n_cap);
-    if (threadIdx.x == 0) { s_tile = atomicAdd(ticket, 1u); s_lost = 0; }
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
     __syncthreads();
     const int64_t tile = s_tile, ntiles = ((int64_t)n_cap + CTILE - 1) / CTILE;
     const int64_t i0 = tile * CTILE + (int64_t)threadIdx.x * CI;
