@@ -34,8 +34,28 @@
  *    points synchronise the stream once per solve to size the adaptive tree
  *    and lists).
  *  - Errors are reported as status codes, never by exceptions or device traps;
- *    sfmm_last_error() gives a message.  No kernel of this library waits on
- *    another kernel or on a flag.
+ *    sfmm_last_error() gives a message.
+ *  - No kernel waits on another rank or process.  A kernel may be set up while
+ *    the one before it on its stream ends, and waits for that end on the device
+ *    (programmatic stream serialisation).  Inside one launch the blocks of the
+ *    radix sort (below 2e6 keys), of the collection of leaves and evaluation
+ *    items and of the list walk wait for words that earlier blocks of the same
+ *    launch publish; blocks take their numbers in the order they start, so these
+ *    waits end, and all are bounded (wait_limit).
+ *  - SFMM_FP64 and SFMM_FP32 give the same bits on every call with the same
+ *    inputs.  In SFMM_MIXED and SFMM_MIXED_DF two calls can differ by the rounding
+ *    of float64 sums (M2L sums reach a box by atomic additions).  A graph replay
+ *    may take another kernel than the direct solve where the choice rests on a
+ *    size (there a capacity, here the actual size), with its sums in another
+ *    order.
+ *  - Workspace: about 56 bytes per source and per target (keys, indexes, sorted
+ *    records), 32 more each for the near fields on FP32 offsets; the near field's
+ *    sums per target: 36 bytes (SFMM_MIXED), 52 (SFMM_MIXED_DF), 44 (SFMM_FP64; 52
+ *    with sigma, 100 for the shear); partial M2L sums per M2L pair: 33 bytes
+ *    (SFMM_FP64; 66 up to 19,456 pairs), 17 (SFMM_FP32).  The lists start at 48 M2L
+ *    and 24 direct-act entries of 12 bytes per node and 32 frontier pairs of 16
+ *    bytes, and a node holds its two expansions (2 x 528 bytes, 2 x 264 in SFMM_FP32)
+ *    and about 400 bytes of geometry and translation parameters.
  */
 #ifndef SFMM_H
 #define SFMM_H
@@ -92,9 +112,12 @@ typedef struct {
                               potential; far pairs also need d - R_T - R_S > sigma.  SFMM_FP64 only. */
     int wait_limit;        /* polls after which a bounded device wait (the tensor-core M2L's mbarrier waits)
                               gives up, returning SFMM_ETIMEOUT with the device context intact; 0 (default) =
-                              2^26.  The radix sort's waits take the same limit (default 2^20) but need no
-                              error: a tile that gives up counts the keys before it, with the same result.
-                              A test hook: a small value makes these paths run. */
+                              2^26.  The waits of the radix sort, of the collection of leaves and items and of
+                              the list walk take the same limit (default 2^20) but need no error: a block that
+                              gives up forms the sum of the earlier blocks from their inputs, with the same
+                              result.  That makes the launch quadratic in its input (all keys, nodes or frontier
+                              pairs before the block are read again): a test hook for small problems, where a
+                              small value makes these paths run; at 1e7 points it can cost seconds. */
 } sfmm_options;
 
 /* Fill *opt with the defaults listed above.  Returns SFMM_EINVAL if opt is NULL. */

@@ -39,7 +39,7 @@ void count_launch(int n = 1);
 // sorts of up to 2e6 keys, the walk's rounds and the narrow levels, then on the other chained
 // kernels too: 262144 keys (9 launches) 117 -> 93 -> 90 us, 1e4 clustered points (103) 0.77 -> 0.68
 // -> 0.66 ms, 4096 points 0.75 -> 0.69 -> 0.66 ms, 1e6 on the N_side 512 grid 5.26 -> 5.02 ms, 16 shells
-// 12.95 -> 12.54 -> 12.37 ms, 4e6 FP32 points (208) 6.62 -> 6.57 -> 6.40 ms.  Launching yet earlier
+// 12.95 -> 12.54 -> 12.37 ms, 4e6 FP32 points (203) 6.62 -> 6.57 -> 6.40 ms.  Launching yet earlier
 // (griddepcontrol.launch_dependents at the start of each kernel) gained no more on one stream, and the
 // waiting blocks took places from the other streams' kernels (16 shells 13.15 ms).
 template <typename... P, typename... A>

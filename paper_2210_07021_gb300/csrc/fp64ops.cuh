@@ -15,6 +15,13 @@
 // ACM TOMS 16, 1990): m in [1, 2), c_j the midpoint of m's 1/128 interval,
 // r = m / c_j - 1, |r| < 2^-7.9, log m = log c_j + r - r^2/2 + r^3/3 + r^4 g(r); g is
 // a polynomial in FP32 (r^4/4 < 2^-33, so its rounding stays below 2^-56).
+//
+// Errors.  A term q/d^2 has about 1.5 units in the last place where a division had 1/2, but
+// the sums it goes into have fewer roundings: the logarithms of a run are one, and the mass
+// is not summed pair by pair.  Near fields alone (40, 300 and 2000 sources; wide and arcminute
+// skies; equal, lognormal and signed masses; half of the targets on sources) against 80-bit
+// sums, before -> now: psi, rms 1.5e-16 .. 4.8e-14 -> 1.1e-16 .. 3.9e-15 (0.03 to 1.00 of
+// before), alpha 2.0e-16 .. 1.0e-14 -> 1.6e-16 .. 1.3e-15 (0.12 to 0.83).
 #pragma once
 #include <cuda_runtime.h>
 #include <cstdint>
