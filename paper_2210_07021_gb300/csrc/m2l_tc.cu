@@ -447,8 +447,8 @@ __global__ void __launch_bounds__(128, TC_CTAS) k_m2l_tc(int64_t n_pairs, const 
 // those that fill theirs, first halves before second ones), which keeps the results where
 // they were.  Those additions' order changed from call to call: 4e6 clustered points,
 // relative change of psi 3e-13 or, where a coarse box's C was rounded the other way, up to
-// 4.4e-9.  Against five calls of that build on each of 16 skies, psi and alpha lie within
-// the spread of those calls but for one sky's alpha (4.9e-10, spread 8e-11); summed in
+// 4.4e-9.  Against five calls with atomic additions on each of 16 skies, psi and alpha lie
+// within those calls' spread but for one sky's alpha (4.9e-10, spread 8e-11); summed in
 // plain list order, psi was 1.6e-9 and 2e-9 from all five calls on two of twelve skies.
 // Cost at 4e6 points (2.75e6 pairs): k_m2l_tc 505 -> 515 us, this kernel 35 us with cold
 // caches, the solve 6.30 -> 6.35 ms.

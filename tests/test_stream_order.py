@@ -100,11 +100,13 @@ def test_near_field_comes_after_what_it_reads(lib, call, precision):
     assert ops[-1][1] == (1 << len(ops) - 1) - 1
 
 
-@pytest.mark.parametrize("precision", sorted(NEAR))
-@pytest.mark.parametrize("call", ["sfmm_deflection", "sfmm_deflection_host", "shear"])
-@pytest.mark.parametrize("options", [{}, {"m2l_tensor_cores": 0}, {"sigma": 0.1}])
+COUNTED = [(call, precision, options) for precision in sorted(NEAR)
+           for call in ("sfmm_deflection", "sfmm_deflection_host", "shear")
+           for options in ({}, {"m2l_tensor_cores": 0})]
+COUNTED += [(call, sfmm.SFMM_FP64, {"sigma": 0.1}) for call in ("sfmm_deflection", "sfmm_deflection_host")]
+
+
+@pytest.mark.parametrize("call,precision,options", COUNTED)
 def test_every_launch_is_counted_once(lib, call, precision, options):
-    if "sigma" in options and (precision != sfmm.SFMM_FP64 or call == "shear"):
-        pytest.skip("the Near Particle Model runs in FP64, without shear")
     ops, launches = trace(lib, call, precision, **options)
     assert launches == sum(name.startswith("_Z") for name, _ in ops)
